@@ -745,7 +745,7 @@ def bench_stress(B, torch, peaks, flush, steps, traffic):
                                      ws=ws_a), max(5, min(reps, 10)))
     # Allocation step (Sec. 4.3-4.4): the paper's group size (G = 16) for 64
     # prompts of one RL step, and the 4096 x 64 stress size. Latency bound
-    # (a fixed number of small fp64 Newton systems per group).
+    # (some ten interior-point steps per group, fp64).
     alloc = {}
     for nb, ga in ((64, 16), (4096, 64)):
         ai = synth.make_alloc_inputs(77, nb, ga)
@@ -759,7 +759,7 @@ def bench_stress(B, torch, peaks, flush, steps, traffic):
             "ms": t_al, "groups_per_s": nb / (t_al / 1e3),
             "newton_mean": float(s_al[:, 3].mean()), "newton_max": int(s_al[:, 3].max()),
             "solved": int((s_al[:, 4] == 0).sum()),
-            "bound": "latency (fp64 log-barrier Newton, one CTA per group)"}
+            "bound": "fp64 pipe and latency (primal-dual interior point, one CTA per group)"}
     bytes_p = Bn * (4 * G + G + 4 * G + 4 * G + G + 16)
     bytes_d = 4 * D * n_act + Bn * (4 * G * (G - 1) // 2 + 4 * G + G) + 4 * Bn * D + 4 * Bn * G
     gbs_c = bytes_c / (t_c / 1e3) / 1e9

@@ -277,7 +277,7 @@ PAIR_API pair_status pair_estimate_dense(int32_t B, int32_t G, int32_t D,
  * the disagreement p_i (1 - p_j) + (1 - p_i) p_j of the predicted success
  * probabilities (Eq. disagreement), times ((m_i + m_j) / 2)^2 when score-norm
  * predictions m are given. Solved per group in fp64 to a duality-gap bound
- * of 1e-12 Phi (log-barrier Newton, one CTA per group); the group's case is
+ * of 1e-12 Phi (primal-dual interior point, one CTA per group); the group's case is
  * classified first from the fp64 sum of c in index order:
  *     PAIR_ALLOC_SLACK       budget >= sum c: pi = 1 (x = 0 minimises Phi)
  *     PAIR_ALLOC_FLOOR       budget == pi_min sum c: pi = pi_min
@@ -285,7 +285,7 @@ PAIR_API pair_status pair_estimate_dense(int32_t B, int32_t G, int32_t D,
  *                            PAIR_DEV_ERR_ALLOC_INFEASIBLE is raised
  *     PAIR_ALLOC_FLAT        every a_ij and b_i is 0: pi = budget / sum c
  *     PAIR_ALLOC_OK          solved
- *     PAIR_ALLOC_FALLBACK    Newton did not converge: pi = budget / sum c
+ *     PAIR_ALLOC_FALLBACK    the solver did not converge: pi = budget / sum c
  *                            (uniform, same expected cost; App. C)
  *     PAIR_ALLOC_INVALID     a non-finite or out-of-range input: pi = NaN,
  *                            PAIR_DEV_ERR_ALLOC_INPUT is raised.
@@ -296,8 +296,8 @@ PAIR_API pair_status pair_estimate_dense(int32_t B, int32_t G, int32_t D,
  *      the expected suffix cost); 0 < pi_min <= 1. All device pointers.
  * Out: pi [B][G] float; stats [B][PAIR_ALLOC_NSTATS] double (nullable):
  *      [PAIR_ALLOC_PHI] objective at pi, [PAIR_ALLOC_SPENT] sum c pi,
- *      [PAIR_ALLOC_GAP] duality-gap bound (2G + 1) / t, [PAIR_ALLOC_NEWTON]
- *      Newton steps, [PAIR_ALLOC_STATUS] the status above.
+ *      [PAIR_ALLOC_GAP] duality gap (<= 1e-12 Phi), [PAIR_ALLOC_NEWTON]
+ *      Newton (interior-point) steps, [PAIR_ALLOC_STATUS] the status above.
  * dev_err required. Deterministic. No workspace, no allocation.
  */
 #define PAIR_ALLOC_OK 0

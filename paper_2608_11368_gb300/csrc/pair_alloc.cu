@@ -6,23 +6,46 @@
 //     s.t.   sum_i c_i e^(-x_i) <= budget,   0 <= x_i <= -log pi_min,
 // with pi_i = e^(-x_i).
 //
-// Solver (one CTA per group, fp64): a log-barrier path-following method,
-//     F_t(x) = t Phi(x) - log(budget - sum c e^-x) - sum log x_i - sum log(X - x_i),
-// Newton steps on F_t (gradient and Hessian in closed form, the G x G system
-// factorised by Cholesky in shared memory, backtracking line search kept
-// strictly feasible), t multiplied by 32 (G <= 24) or 16 after each centring,
-// with a predictor step along the central path's tangent from the factor of
-// the centred point, until the duality-gap bound (2G + 1) / t is below
-// 1e-12 Phi. The paper solves the
-// same program with SLSQP on the CPU (App. C); any method reaching its
-// unique optimum is equivalent, and a barrier method maps onto one CTA with
-// a fixed, small number of dense factorisations. Cases the program leaves
-// without an interior (budget >= sum c: pi = 1; budget = pi_min sum c:
-// pi = pi_min; budget below that: infeasible) and the flat objective (all
-// a_ij = b_i = 0) are classified first, from the fp64 sum of c in index
-// order. If Newton does not converge within its iteration cap, the group
-// falls back to the uniform pi = budget / sum c of the same expected cost
-// (the paper's fallback).
+// Solver (one CTA per group, fp64), in the variables pi: with v_i = 1 / pi_i
+// the program is
+//     min  Phi = sum_{i<j} a_ij v_i v_j + sum_i b_i v_i
+//     s.t. sum_i c_i pi_i = budget,   pi_min <= pi_i <= 1,
+// still convex, and with linear constraints only (Phi falls in every pi_i, so
+// the budget is spent; kBudgetMargin keeps the rounded sum below it). It is
+// solved by a primal-dual interior-point method with Mehrotra's predictor and
+// corrector: about 8 to 11 steps to a duality gap of 1e-12 Phi, where a
+// log-barrier Newton iteration in x took 47 (groups of 16) and 80 (64).
+//
+// The Newton system in the relative steps d_i = dpi_i / pi_i is
+//     M_ij = a_ij v_i v_j (i != j),
+//     M_ii = 2 v_i (w_i + b_i) + pi_i^2 (zl_i / sl_i + zh_i / sh_i),
+// w = A v. Its off-diagonal row sum is v_i w_i, at most half its diagonal (and
+// about 1 / 2G of it for a dense graph, where b_i is about G sum_j a_ij), so
+// no factorisation is needed: Chebyshev's iteration on the system scaled by
+// its diagonal, whose spectrum lies within rho = max_i v_i w_i / M_ii <= 1/2 of
+// 1, gains a factor of at least 3.7 per product with A, and two products give
+// the 1e-3 that an interior-point step needs for G >= 16. Odd degrees only:
+// their residual polynomial vanishes at 1, where the coordinates at a bound
+// lie, so those are exact. What the step's residual leaves is corrected by
+// the next step, and the stopping test is on the fp64 residuals themselves.
+//
+// What bounds it: the fp64 pipe (2 multiply-adds per clock and SM) for many
+// groups, the chain of a step's exchanges and products for few. A step of a
+// group of 64 takes five products with A (two of them with two right-hand
+// sides), all G^2 entries from shared memory with every lane busy, and 10
+// block-wide exchanges in a row. Measured on one GB300, against the
+// factorising log-barrier form: 64 groups of 16 in 0.107 ms (2.43 ms), 4096
+// groups of 64 in 4.79 ms (178 ms); with IEEE divisions in place of
+// rcp_approx / rcp_newton and full butterflies 0.188 and 6.84 ms.
+//
+// The paper solves the same program with SLSQP on the CPU (App. C); any
+// method reaching its optimum is equivalent. Cases the program leaves without
+// an interior (budget >= sum c: pi = 1; budget = pi_min sum c: pi = pi_min;
+// budget below that: infeasible) and the flat objective (all a_ij = b_i = 0)
+// are classified first, from the fp64 sum of c in index order. If the
+// iteration does not converge within its cap, the group falls back to the
+// uniform pi = budget / sum c of the same expected cost (the paper's
+// fallback).
 #include <math.h>
 #include <stdint.h>
 
@@ -31,158 +54,250 @@
 namespace pairk {
 namespace {
 
-constexpr int kAllocMaxNewton = 600;    // total Newton steps per group
-constexpr int kAllocMaxBacktrack = 80;  // halvings per line search
-constexpr double kGapRel = 1e-12;       // stop at (2G + 1) / t <= kGapRel * Phi
-// Barrier parameter growth per centring: 32 for groups of up to 24 (fewer
-// Newton steps in all: about 59 against 66 per group of 16), 16 above (at 64,
-// 32 costs more steps than it saves).
-__host__ __device__ constexpr double barrier_growth(int G) { return G <= 24 ? 32.0 : 16.0; }
-// Newton decrement^2 / 2 of a centred point. lambda^2 / 2 bounds F_t - min F_t,
-// so centring adds at most about lambda^2 / t to Phi, far below the gap
-// bound (2G + 1) / t >= 5 / t; a tighter threshold only adds Newton steps
-// (on 64 groups of 16, 1e-6 takes about 68 steps per group and 1e-3 about
-// 65, with pi as close to the KKT point).
-constexpr double kCentred = 1e-3;
-// A line search stops once the decrease its step could bring, step * lambda^2,
-// is below this many fp64 units of |F_t|: such a decrease cannot be told from
-// rounding, so halving further only repeats function evaluations (the point
-// is then treated as centred, as after a failed search).
-constexpr double kResolution = 16.0 * 2.220446049250313e-16;
+constexpr int kAllocMaxSteps = 80;      // interior-point steps per group
+constexpr int kAllocMaxBacktrack = 20;  // halvings of one step
+constexpr double kGapRel = 1e-12;       // stop at gap <= kGapRel * Phi (and the dual residual)
+// The budget the equality constraint aims at is this much (relative) below
+// the caller's: the rounding of the fp64 sum of c pi (at most 128 2^-53) and
+// the primal residual allowed at the end (kPrimalRel) then never spend more.
+constexpr double kBudgetMargin = 4e-14;
+constexpr double kPrimalRel = 2e-14;
+constexpr float kLinRel = 1e-3f;    // reduction of the Newton system's residual
+constexpr int kLinMaxDegree = 61;   // reached only if rounding puts rho far above 1/2
+constexpr float kStepFrac = 0.995f; // of the largest step that keeps the interior
+constexpr double kStartMu = 0.1;    // the start's complementarity: kStartMu Phi in all
 
-// Groups of up to 64 keep the edge proxies a_ij in shared memory (fp64, as
-// computed on the fly otherwise); the 128-candidate form has no room for them.
+// Shape of a group's CTA: GP >= G is the padded group size, TPR adjacent
+// threads share a row of A and each holds its coordinate's state.
 template <int GP>
-constexpr bool kEdgeTable = GP <= 64;
+struct AllocShape {
+  static constexpr int kThreads = GP <= 16 ? 32 : 2 * GP;
+  static constexpr int kTpr = kThreads / GP;
+  static constexpr int kWarps = kThreads / 32;
+};
+
+// Reciprocals from the hardware's approximation over the whole fp64 range
+// (PTX rcp.approx.ftz.f64, about 20 bits; an IEEE division takes some ten
+// instructions of the fp64 pipe, and a step has eighteen of them): as it is
+// where the value only steers (step lengths, the centring parameter) or where
+// the same value enters both sides of an identity; with two steps of Newton's
+// iteration, y += y (1 - x y), to within a unit or two of the last place
+// elsewhere.
+__device__ __forceinline__ double rcp_approx(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ double rcp_newton(double x) {
+  double y = rcp_approx(x);
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+
+// Row pitch of A (odd: rows start in different shared-memory banks).
+__host__ __device__ __forceinline__ int alloc_pitch(int G) { return G | 1; }
 
 template <int GP>
 struct AllocSmem {
-  double H[GP][GP + 1];  // Newton system, factorised in place (lower triangle)
-  double A[kEdgeTable<GP> ? GP : 1][kEdgeTable<GP> ? GP + 1 : 1];  // a_ij (see kEdgeTable)
-  double c[GP], b[GP], dx[GP];
-  double dinv[GP];       // 1 / L_kk of the current factorisation
+  double x[2][2][GP];  // operands of a product: [buffer][right-hand side]
+  double red[2][4][AllocShape<GP>::kWarps];
+  float redm[2][2][AllocShape<GP>::kWarps];
+  double c[GP];
   float p[GP], m[GP];
-  double red[GP / 32];
   double sum_c;
   int any;
 };
 
-// Sum over the CTA (all GP threads call it; returns the total to every thread).
 template <int GP>
-__device__ double block_sum(AllocSmem<GP> &sm, double v) {
+__device__ __forceinline__ void alloc_sync() {
+  if constexpr (AllocShape<GP>::kWarps == 1) __syncwarp();
+  else __syncthreads();
+}
+
+// One group's CTA: its thread's coordinate (i, replicated over the TPR
+// threads of the row), and the exchanges.
+template <int GP>
+struct AllocGroup {
+  static constexpr int kTpr = AllocShape<GP>::kTpr;
+  static constexpr int kWarps = AllocShape<GP>::kWarps;
+  AllocSmem<GP> &sm;
+  double *A;  // [G][pitch], zero diagonal
+  int G, pitch, i, sub;
+  bool act;
+  int xb, rb;  // buffers of the next product and the next reduction
+
+  // NS sums (fp64) and NM maxima (fp32: they only steer) over the group's
+  // coordinates, to every thread. The replicas of a coordinate hold the same
+  // value, so the butterfly starts at the row distance. Its first stages
+  // halve the number of sums a lane carries (4 sums over 16 lanes take 5
+  // additions instead of 16), and shuffles hand the totals back. Two buffers:
+  // a reduction is one barrier.
+  template <int NS, int NM>
+  __device__ void reduce(double (&v)[NS], float (&mx)[NM]) {
+    const int lane = threadIdx.x & 31;
+    constexpr int H1 = NS >= 3 ? 2 : 1;  // sums a lane keeps after the first stage
+    double t[NS >= 3 ? 2 : 1];
+    int o = kTpr;
+    if constexpr (NS >= 2) {
+      const bool up = lane & o;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) sm.red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
+      for (int k = 0; k < H1; ++k) {
+        const double hi = k + H1 < NS ? v[k + H1] : 0.0;
+        const double keep = up ? hi : v[k], send = up ? v[k] : hi;
+        t[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+      o <<= 1;
+    } else {
+      t[0] = v[0];
+    }
+    if constexpr (NS >= 3) {
+      const bool up = lane & o;
+      const double keep = up ? t[1] : t[0], send = up ? t[0] : t[1];
+      t[0] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      o <<= 1;
+    }
+    for (; o < 32; o <<= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
 #pragma unroll
-  for (int w = 0; w < GP / 32; ++w) t += sm.red[w];
-  return t;
-}
-
-// Solves H y = r in place in sm.dx with the Cholesky factor in sm.H (lower
-// triangle) and the pivot inverses in sm.dinv (all GP threads call; thread i
-// holds r_i on entry and reads y_i after the call).
-template <int GP>
-__device__ void chol_solve(AllocSmem<GP> &sm, int G, bool act, double r) {
-  const int i = threadIdx.x;
-  __syncthreads();
-  sm.dx[i] = act ? r : 0.0;
-  for (int k = 0; k < G; ++k) {
-    __syncthreads();
-    if (i == k) sm.dx[k] *= sm.dinv[k];
-    __syncthreads();
-    if (i > k && act) sm.dx[i] -= sm.H[i][k] * sm.dx[k];
+    for (int k = 0; k < NS; ++k) {
+      // Sum k ended in the lanes whose halving bits spell it.
+      const int src = NS >= 3 ? (k / 2) * kTpr + (k % 2) * 2 * kTpr : k * kTpr;
+      v[k] = __shfl_sync(0xffffffffu, t[0], src);
+    }
+#pragma unroll
+    for (int q = kTpr; q < 32; q <<= 1)
+#pragma unroll
+      for (int k = 0; k < NM; ++k) mx[k] = fmaxf(mx[k], __shfl_xor_sync(0xffffffffu, mx[k], q));
+    if constexpr (kWarps > 1) {
+      if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < NS; ++k) sm.red[rb][k][threadIdx.x >> 5] = v[k];
+#pragma unroll
+        for (int k = 0; k < NM; ++k) sm.redm[rb][k][threadIdx.x >> 5] = mx[k];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < NS; ++k) {
+        v[k] = sm.red[rb][k][0];
+#pragma unroll
+        for (int w = 1; w < kWarps; ++w) v[k] += sm.red[rb][k][w];
+      }
+#pragma unroll
+      for (int k = 0; k < NM; ++k) {
+        mx[k] = sm.redm[rb][k][0];
+#pragma unroll
+        for (int w = 1; w < kWarps; ++w) mx[k] = fmaxf(mx[k], sm.redm[rb][k][w]);
+      }
+      rb ^= 1;
+    }
   }
-  for (int k = G - 1; k >= 0; --k) {
-    __syncthreads();
-    if (i == k) sm.dx[k] *= sm.dinv[k];
-    __syncthreads();
-    if (i < k) sm.dx[i] -= sm.H[k][i] * sm.dx[k];
+  template <int NS>
+  __device__ void sum(double (&v)[NS]) {
+    float none[1] = {0.f};
+    reduce<NS, 1>(v, none);
   }
-  __syncthreads();
-}
 
-// Largest step along d keeping every coordinate strictly inside the box
-// (0, X), shared by all threads (min over the group, 1e300 if unbounded).
-template <int GP>
-__device__ double box_step(AllocSmem<GP> &sm, int G, bool act, double x, double d, double X) {
-  double smax = 1.0e300;
-  if (act && d < 0.0) smax = -x / d;
-  if (act && d > 0.0) smax = (X - x) / d;
-  __syncthreads();
-  sm.dx[threadIdx.x] = smax;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double mn = 1.0e300;
-    for (int k = 0; k < G; ++k) mn = fmin(mn, sm.dx[k]);
-    sm.red[0] = mn;
+  // y_r = (A x_r)_i for NR right-hand sides, x given per coordinate.
+  template <int NR>
+  __device__ void product(const double (&x)[NR], double (&y)[NR]) {
+    if (sub == 0)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) sm.x[xb][r][i] = act ? x[r] : 0.0;
+    alloc_sync<GP>();
+    double acc[NR][2];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) acc[r][0] = acc[r][1] = 0.0;
+    if (act) {
+      const double *row = A + (size_t)i * pitch;
+      int j = sub;
+      for (; j + 3 * kTpr < G; j += 4 * kTpr) {
+        double a[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = row[j + u * kTpr];
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            acc[r][u & 1] = fma(a[u], sm.x[xb][r][j + u * kTpr], acc[r][u & 1]);
+      }
+      for (; j < G; j += kTpr) {
+        const double a = row[j];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) acc[r][0] = fma(a, sm.x[xb][r][j], acc[r][0]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      double t = acc[r][0] + acc[r][1];
+#pragma unroll
+      for (int o = 1; o < kTpr; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      y[r] = t;
+    }
+    xb ^= 1;
   }
-  __syncthreads();
-  const double r = sm.red[0];
-  __syncthreads();
-  return r;
-}
 
-struct AllocIn {
-  int G;
-  const float *p_hat, *m_hat, *a;
-  int g;
+  // Approximate solutions of M x_r = rhs_r (see the head of this file):
+  // Chebyshev's iteration on M scaled by its diagonal (inverse rd), odd
+  // degree, until the residual is reduced by kLinRel.
+  template <int NR>
+  __device__ void solve(double v, double rd, float rho, const double (&rhs)[NR],
+                        double (&x)[NR]) {
+    double r[NR], d[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+      r[k] = d[k] = x[k] = rhs[k] * rd;
+    }
+    if (!(rho > 0.f)) return;
+    // err = 1 / T_n(1 / rho) by its recurrence r1 = 1 / (2 / rho - r0). The
+    // two coefficients of an update are r1 r0 and 2 r1 / rho = 1 + r1 r0; in
+    // the second form an odd degree vanishes at 1 whatever r1's rounding.
+    const float s = 1.f / rho;
+    float r0 = rho, err = rho;
+    const double vrd = v * rd;
+    for (int n = 1; !(err <= kLinRel && (n & 1)) && n < kLinMaxDegree; ++n) {
+      double t[NR], y[NR];
+#pragma unroll
+      for (int k = 0; k < NR; ++k) t[k] = v * d[k];
+      product<NR>(t, y);
+      const float r1 = 1.f / (2.f * s - r0);
+      const double al = (double)(r1 * r0);
+#pragma unroll
+      for (int k = 0; k < NR; ++k) {
+        r[k] -= fma(vrd, y[k], d[k]);
+        d[k] = fma(al, d[k] + r[k], r[k]);
+        x[k] += d[k];
+      }
+      r0 = r1;
+      err *= r0;
+    }
+  }
 };
 
 // Edge proxy a_ij: the explicit array, else Eq. (disagreement) from p_hat,
 // times ((m_i + m_j) / 2)^2 with score-norm predictions (Eq. edge-proxy).
-template <int GP>
-__device__ __forceinline__ double edge(const AllocIn &in, const AllocSmem<GP> &sm, int i,
-                                       int j) {
-  if (i == j) return 0.0;
-  if (in.a) return (double)in.a[((size_t)in.g * in.G + i) * in.G + j];
-  const double pi = sm.p[i], pj = sm.p[j];
+__device__ __forceinline__ double edge_proxy(float pi_, float pj_, bool norms, float mi,
+                                             float mj) {
+  const double pi = pi_, pj = pj_;
   double d = pi * (1.0 - pj) + (1.0 - pi) * pj;
-  if (in.m_hat) {
-    const double h = 0.5 * ((double)sm.m[i] + (double)sm.m[j]);
+  if (norms) {
+    const double h = 0.5 * ((double)mi + (double)mj);
     d *= h * h;
   }
   return d;
 }
 
-// a_ij from the table where there is one (same fp64 value as edge()).
 template <int GP>
-__device__ __forceinline__ double edge_at(const AllocIn &in, const AllocSmem<GP> &sm, int i,
-                                          int j) {
-  if constexpr (kEdgeTable<GP>) return sm.A[i][j];
-  else return edge<GP>(in, sm, i, j);
-}
-
-// Phi, the budget slack and this coordinate's S_i = sum_j a_ij u_j at x_i
-// (u_i = e^x_i held by thread i, shared through sm.dx as scratch).
-template <int GP>
-__device__ void eval(const AllocIn &in, AllocSmem<GP> &sm, bool act, double x, double budget,
-                     double &u, double &e, double &S, double &phi, double &slack) {
-  u = act ? exp(x) : 0.0;
-  e = act ? sm.c[threadIdx.x] / u : 0.0;  // c e^-x without a second exp
-  __syncthreads();
-  sm.dx[threadIdx.x] = u;
-  __syncthreads();
-  S = 0.0;
-  if (act)
-    for (int j = 0; j < in.G; ++j) S += edge_at<GP>(in, sm, threadIdx.x, j) * sm.dx[j];
-  phi = block_sum<GP>(sm, act ? u * (0.5 * S + sm.b[threadIdx.x]) : 0.0);
-  slack = budget - block_sum<GP>(sm, e);
-}
-
-template <int GP>
-__global__ void __launch_bounds__(GP, 1) alloc_kernel(int G, const float *p_hat, const float *m_hat,
-                                                   const float *a, const float *c_hat,
-                                                   const float *budget_in, float pi_min,
-                                                   float *pi_out, double *stats,
-                                                   int32_t *dev_err) {
+__global__ void __launch_bounds__(AllocShape<GP>::kThreads)
+    alloc_kernel(int G, const float *__restrict__ p_hat, const float *__restrict__ m_hat,
+                 const float *__restrict__ a, const float *__restrict__ c_hat,
+                 const float *__restrict__ budget_in, float pi_min, float *__restrict__ pi_out,
+                 double *__restrict__ stats, int32_t *dev_err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int kTpr = AllocShape<GP>::kTpr;
   AllocSmem<GP> &sm = *reinterpret_cast<AllocSmem<GP> *>(smem_raw);
-  const int i = threadIdx.x, g = blockIdx.x;
+  const int i = threadIdx.x / kTpr, sub = threadIdx.x % kTpr, g = blockIdx.x;
   const bool act = i < G;
-  const AllocIn in{G, p_hat, m_hat, a, g};
+  AllocGroup<GP> grp{sm, reinterpret_cast<double *>(smem_raw + sizeof(AllocSmem<GP>)),
+                     G,  alloc_pitch(G), i, sub, act, 0, 0};
 
   // ---- inputs and their validity
   bool bad = false;
@@ -200,48 +315,55 @@ __global__ void __launch_bounds__(GP, 1) alloc_kernel(int G, const float *p_hat,
         sm.m[i] = mf;
       }
     } else {
-      for (int j = 0; j < G; ++j) {
+      for (int j = sub; j < G; j += kTpr) {
         const float v = a[((size_t)g * G + i) * G + j];
         bad |= (j != i) && !(v >= 0.f && v <= 3.0e38f);
       }
     }
+    sm.c[i] = ci;
   }
-  sm.c[i] = act ? ci : 0.0;
   const double budget = (double)budget_in[g];
   bad |= !(budget > 0.0 && budget <= 3.0e38);
-  if (i == 0) sm.any = 0;
-  __syncthreads();
+  if (threadIdx.x == 0) sm.any = 0;
+  alloc_sync<GP>();
   if (bad) atomicOr(&sm.any, 1);
   // The sum of c in index order (the classification is bit-identical to a
   // sequential fp64 sum on the host).
-  if (i == 0) {
+  if (threadIdx.x == 0) {
     double s = 0.0;
     for (int k = 0; k < G; ++k) s += sm.c[k];
     sm.sum_c = s;
   }
-  __syncthreads();
+  alloc_sync<GP>();
   const bool invalid = sm.any != 0;
-  const double sc = sm.sum_c, pmin = (double)pi_min, X = -log(pmin);
-  if constexpr (kEdgeTable<GP>) {
-    if (act && !invalid)
-      for (int j = 0; j < G; ++j) sm.A[i][j] = edge<GP>(in, sm, i, j);
-    __syncthreads();
-  }
+  const double sc = sm.sum_c, pmin = (double)pi_min;
 
-  // ---- b_i = (sum_{j != i} sqrt a_ij)^2 - sum_{j != i} a_ij
-  double bi = 0.0, asum = 0.0;
+  // ---- A and b_i = (sum_{j != i} sqrt a_ij)^2 - sum_{j != i} a_ij
+  double bi = 0.0, asum = 0.0, sq = 0.0;
   if (act && !invalid) {
-    double sq = 0.0;
-    for (int j = 0; j < G; ++j) {
-      const double v = edge_at<GP>(in, sm, i, j);
+    const float pi_ = a ? 0.f : sm.p[i], mi = m_hat && !a ? sm.m[i] : 0.f;
+    for (int j = sub; j < G; j += kTpr) {
+      double v = 0.0;
+      if (j != i)
+        v = a ? (double)a[((size_t)g * G + i) * G + j]
+              : edge_proxy(pi_, sm.p[j], m_hat != nullptr, mi, m_hat ? sm.m[j] : 0.f);
+      grp.A[(size_t)i * grp.pitch + j] = v;
       sq += sqrt(v);
       asum += v;
     }
-    bi = sq * sq - asum;
   }
-  sm.b[i] = bi;
-  __syncthreads();
-  const bool flat = block_sum<GP>(sm, asum + bi) == 0.0;
+#pragma unroll
+  for (int o = 1; o < kTpr; o <<= 1) {
+    sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    asum += __shfl_xor_sync(0xffffffffu, asum, o);
+  }
+  bi = sq * sq - asum;
+  bool flat;
+  {
+    double v[1] = {act ? asum + bi : 0.0};
+    grp.template sum<1>(v);
+    flat = v[0] == 0.0;
+  }
 
   int status;
   if (invalid) status = PAIR_ALLOC_INVALID;
@@ -251,159 +373,143 @@ __global__ void __launch_bounds__(GP, 1) alloc_kernel(int G, const float *p_hat,
   else if (flat) status = PAIR_ALLOC_FLAT;
   else status = PAIR_ALLOC_OK;
 
-  double x = 0.0, t = 0.0, gap = 0.0;
-  int newton = 0;
-  if (status == PAIR_ALLOC_SLACK) {
-    x = 0.0;
-  } else if (status == PAIR_ALLOC_FLOOR || status == PAIR_ALLOC_INFEASIBLE) {
-    x = X;
-  } else if (status == PAIR_ALLOC_FLAT) {
-    x = -log(budget / sc);
-  } else if (status == PAIR_ALLOC_OK) {
-    const int m = 2 * G + 1;
-    const double tmul = barrier_growth(G);
-    x = -log(0.5 * (budget / sc + pmin));  // strictly feasible start
-    double u, e, S, phi, slack;
-    eval<GP>(in, sm, act, x, budget, u, e, S, phi, slack);
-    t = (double)m / phi;
-    bool done = false;
-    while (newton < kAllocMaxNewton && !done) {
-      ++newton;
-      // Gradient and Hessian of F_t at x.
-      // 1/x and 1/(X - x) from one division; 1/slack once per step.
-      const double rr = act ? 1.0 / (x * (X - x)) : 0.0;
-      const double bnd_lo = act ? (X - x) * rr : 0.0, bnd_hi = act ? x * rr : 0.0;
-      const double inv_s = 1.0 / slack;
-      const double gi =
-          act ? t * u * (S + sm.b[i]) - e * inv_s - bnd_lo + bnd_hi : 0.0;
-      // u_j and e_j for the Hessian rows (e_j in H's spare column).
-      __syncthreads();
-      sm.dx[i] = u;
-      if (act) sm.H[i][GP] = e;
-      __syncthreads();
-      if (act) {
-        const double inv_s2 = inv_s * inv_s;
-        for (int j = 0; j <= i; ++j) {
-          double h = e * sm.H[j][GP] * inv_s2;
-          if (j == i)
-            h += t * u * (S + sm.b[i]) + e * inv_s + bnd_lo * bnd_lo + bnd_hi * bnd_hi;
-          else
-            h += t * edge_at<GP>(in, sm, i, j) * u * sm.dx[j];
-          sm.H[i][j] = h;
-        }
+  double pi = 1.0, gap = 0.0, phi = 0.0, spent = 0.0;
+  int steps = 0;
+  bool solved = false;
+  if (status == PAIR_ALLOC_OK) {
+    const double target = budget - fmin(kBudgetMargin * budget, 0.5 * (budget - pmin * sc));
+    pi = target / sc;  // uniform start
+    double sl = pi - pmin, sh = 1.0 - pi;
+    if (!(sl > 0.0 && sh > 0.0)) sl = sh = 0.0;  // no interior in fp64: fall back
+    const double half_inv = 0.5 / G;
+    double v = rcp_newton(pi), w, zl, zh, y, dres;
+    float rho;
+    {
+      double x[1] = {v}, r[1];
+      grp.template product<1>(x, r);
+      w = r[0];
+      const double wb = w + bi;
+      double s[3] = {act ? v * (0.5 * w + bi) : 0.0, act ? v * wb : 0.0, act ? ci * pi : 0.0};
+      grp.template sum<3>(s);
+      phi = s[0];
+      y = s[1] / s[2];
+      zl = kStartMu * phi * half_inv / sl;
+      zh = kStartMu * phi * half_inv / sh;
+    }
+    // At a point: the sums Phi, duality gap, dual residual and cost, the
+    // inverse diagonal rd of M, and rho.
+    double rsl, rsh, rd;
+    auto measure = [&](double pi, double v, double w, double sl, double sh, double zl, double zh,
+                       double y, double (&s)[4], float &rho) {
+      const double vw = v * w, vwb = fma(v, bi, vw), cp = ci * pi;
+      rsl = rcp_approx(sl);
+      rsh = rcp_approx(sh);
+      rd = rcp_newton(fma(pi * pi, zl * rsl + zh * rsh, 2.0 * vwb));
+      s[0] = act ? vwb - 0.5 * vw : 0.0;
+      s[1] = act ? zl * sl + zh * sh : 0.0;
+      s[2] = act ? fabs(fma(y, cp, -vwb) - (zl - zh) * pi) : 0.0;
+      s[3] = act ? cp : 0.0;
+      float m[1] = {act ? (float)(vw * rd) : 0.f};
+      grp.template reduce<4, 1>(s, m);
+      rho = m[0];
+    };
+    double s[4];
+    measure(pi, v, w, sl, sh, zl, zh, y, s, rho);
+    phi = s[0]; gap = s[1]; dres = s[2]; spent = s[3];
+    while (true) {
+      // All of these are the same in every thread: uniform exits.
+      if (gap <= kGapRel * phi && dres <= kGapRel * phi &&
+          fabs(target - spent) <= kPrimalRel * budget) {
+        solved = true;
+        break;
       }
-      // Cholesky (lower triangle, in place); each pivot's inverse is formed
-      // once, so the column scaling and both substitutions multiply. One
-      // reciprocal square root per pivot gives both 1/L_kk and L_kk = d/sqrt(d).
-      bool spd = true;
-      for (int k = 0; k < G; ++k) {
-        __syncthreads();
-        if (i == k) {
-          const double d = sm.H[k][k];
-          const double rs = d > 0.0 ? rsqrt(d) : 0.0;
-          sm.H[k][k] = d * rs;
-          sm.dinv[k] = rs;
-        }
-        __syncthreads();
-        if (sm.H[k][k] == 0.0) spd = false;
-        if (!spd) break;
-        if (i > k && act) sm.H[i][k] *= sm.dinv[k];
-        __syncthreads();
-        if (i > k && act) {
-          const double lik = sm.H[i][k];
-          for (int j = k + 1; j <= i; ++j) sm.H[i][j] -= lik * sm.H[j][k];
-        }
-      }
-      if (!spd) break;
-      // Solve H dx = -g (forward, then backward substitution).
-      chol_solve<GP>(sm, G, act, -gi);
-      const double d = act ? sm.dx[i] : 0.0;
-      const double lam2 = -block_sum<GP>(sm, gi * d);
-      if (lam2 * 0.5 <= kCentred) {
-        // Centred: stop once the gap bound is small, else raise t.
-        if ((double)m / t <= kGapRel * phi) {
-          done = true;
-          break;
-        }
-        // Predictor: the central path x*(t) has grad F_t = 0, so
-        // dx*/dt = -H^-1 grad Phi with the Hessian just factorised; move
-        // along it to the next t (kept strictly inside the box and the
-        // budget, halving the step otherwise), then let Newton correct.
-        chol_solve<GP>(sm, G, act, act ? -u * (S + sm.b[i]) : 0.0);
-        const double v = act ? (tmul - 1.0) * t * sm.dx[i] : 0.0;
-        double pstep = fmin(1.0, 0.99 * box_step<GP>(sm, G, act, x, v, X));
-        for (int ls = 0; ls < 8; ++ls) {
-          const double xt = x + pstep * v;
-          double ut, et, St, phit, slackt;
-          eval<GP>(in, sm, act, xt, budget, ut, et, St, phit, slackt);
-          // slackt is the same in every thread: the exit is uniform.
-          if (slackt > 0.0) {
-            x = xt; u = ut; e = et; S = St; phi = phit; slack = slackt;
-            break;
-          }
-          pstep *= 0.5;
-        }
-        t *= tmul;
-        continue;
-      }
-      // Largest step keeping every coordinate strictly inside the box.
-      double step = fmin(1.0, 0.99 * box_step<GP>(sm, G, act, x, d, X));
-      const double F0 = t * phi - log(slack) -
-                        block_sum<GP>(sm, act ? log(x * (X - x)) : 0.0);
-      bool moved = false;
-      for (int ls = 0; ls < kAllocMaxBacktrack; ++ls) {
-        // step, lam2 and F0 are the same in every thread: the exit is uniform.
-        if (step * lam2 < kResolution * fabs(F0)) break;
-        const double xt = x + step * d;
-        double ut, et, St, phit, slackt;
-        eval<GP>(in, sm, act, xt, budget, ut, et, St, phit, slackt);
-        bool ok = slackt > 0.0;
-        if (ok) {
-          const double Ft = t * phit - log(slackt) -
-                            block_sum<GP>(sm, act ? log(xt * (X - xt)) : 0.0);
-          // Strict decrease as well: at fp64 resolution of F_t a step can
-          // pass Armijo without changing anything.
-          ok = Ft < F0 && Ft <= F0 - 0.01 * step * lam2;
-        }
-        if (ok) {
-          x = xt; u = ut; e = et; S = St; phi = phit; slack = slackt;
-          moved = true;
+      if (steps >= kAllocMaxSteps || !(gap > 0.0) || !(phi <= 1.0e300)) break;
+      ++steps;
+      const double rp = target - spent, cp = act ? ci * pi : 0.0;
+      // Predictor (complementarity target 0) and the cost's solution.
+      double rhs[2] = {act ? fma(v, w + bi, -y * cp) : 0.0, cp}, h[2];
+      grp.template solve<2>(v, rd, rho, rhs, h);
+      double q[2] = {cp * h[0], cp * h[1]};
+      grp.template sum<2>(q);
+      const double rchc = rcp_newton(q[1]);
+      double d = fma(-(q[0] - rp) * rchc, h[1], h[0]) * pi;
+      double dl = d * rsl, dh = d * rsh;  // relative steps of the two slacks
+      double dzl = -fma(zl, dl, zl), dzh = fma(zh, dh, -zh);
+      double t[2] = {act ? (zl - zh) * d : 0.0, act ? (dzl - dzh) * d : 0.0};
+      float fl = (float)dl, fh = (float)dh;
+      float mx[2] = {act ? fmaxf(-fl, fh) : 0.f, act ? fmaxf(1.f + fl, 1.f - fh) : 0.f};
+      grp.template reduce<2, 2>(t, mx);
+      const double ap = mx[0] > 1.f ? 1.f / mx[0] : 1.f, az = mx[1] > 1.f ? 1.f / mx[1] : 1.f;
+      // sum (z + az dz)(s + ap ds) / gap, with sum s dz = -gap - sum z ds.
+      const float q3 =
+          (float)((gap + az * (-gap - t[0]) + ap * (t[0] + az * t[1])) * rcp_approx(gap));
+      const double smu = (double)fminf(fmaxf(q3 * q3 * q3, 1e-6f), 1.f) * (gap * half_inv);
+      // Corrector.
+      const double tl = (smu - d * dzl) * rsl, th = (smu + d * dzh) * rsh;
+      double rhs1[1] = {act ? fma(tl - th, pi, rhs[0]) : 0.0}, h1[1];
+      grp.template solve<1>(v, rd, rho, rhs1, h1);
+      double q1[1] = {cp * h1[0]};
+      grp.template sum<1>(q1);
+      const double dy = (q1[0] - rp) * rchc;
+      d = fma(-dy, h[1], h1[0]) * pi;
+      dl = d * rsl;
+      dh = d * rsh;
+      dzl = tl - fma(zl, dl, zl);
+      dzh = th + fma(zh, dh, -zh);
+      fl = (float)dl;
+      fh = (float)dh;
+      const float rl = (float)(dzl * rcp_approx(zl)), rh = (float)(dzh * rcp_approx(zh));
+      float m1[1] = {act ? fmaxf(fmaxf(-fl, fh), fmaxf(-rl, -rh)) : 0.f};
+      double none[1] = {0.0};
+      grp.template reduce<1, 1>(none, m1);
+      double step = m1[0] > kStepFrac ? kStepFrac / m1[0] : 1.f;
+      // The step's point; halved while the residuals grow (they fall in
+      // nearly every step: Phi is far from quadratic only near pi_min << 1).
+      for (int ls = 0;; ++ls) {
+        const double sl2 = fma(step, d, sl), sh2 = fma(-step, d, sh);
+        const double zl2 = fma(step, dzl, zl), zh2 = fma(step, dzh, zh), y2 = fma(step, dy, y);
+        const double pi2 = act ? (sh2 < sl2 ? 1.0 - sh2 : pmin + sl2) : 1.0;
+        const double v2 = rcp_newton(pi2);
+        double x[1] = {v2}, r[1];
+        grp.template product<1>(x, r);
+        float rho2;
+        measure(pi2, v2, r[0], sl2, sh2, zl2, zh2, y2, s, rho2);
+        if (s[2] + s[1] <= 1.001 * (dres + gap) || s[2] + s[1] <= 1e-11 * s[0] ||
+            ls == kAllocMaxBacktrack) {
+          sl = sl2; sh = sh2; zl = zl2; zh = zh2; y = y2; pi = pi2; v = v2; w = r[0];
+          phi = s[0]; gap = s[1]; dres = s[2]; spent = s[3]; rho = rho2;
           break;
         }
         step *= 0.5;
       }
-      if (!moved) {
-        // No descent at fp64 resolution: the point is as centred as it gets.
-        if ((double)m / t <= kGapRel * phi) {
-          done = true;
-          break;
-        }
-        t *= tmul;
-      }
     }
-    gap = (double)m / t;
-    if (!done) {
-      status = PAIR_ALLOC_FALLBACK;
-      x = -log(budget / sc);
-    }
+    if (!solved) status = PAIR_ALLOC_FALLBACK;
   }
 
   // ---- outputs
-  double u_out = 0.0, e_out = 0.0, S_out = 0.0, phi_out = 0.0, slack_out = 0.0;
-  if (status != PAIR_ALLOC_INVALID)
-    eval<GP>(in, sm, act, x, budget, u_out, e_out, S_out, phi_out, slack_out);
-  if (act)
-    pi_out[(size_t)g * G + i] = status == PAIR_ALLOC_INVALID ? __int_as_float(0x7fc00000)
-                                                             : (float)exp(-x);
-  if (i == 0) {
+  if (!solved && status != PAIR_ALLOC_INVALID) {
+    pi = status == PAIR_ALLOC_SLACK ? 1.0
+         : (status == PAIR_ALLOC_FLOOR || status == PAIR_ALLOC_INFEASIBLE) ? pmin
+                                                                          : budget / sc;
+    double x[1] = {1.0 / pi}, r[1];
+    grp.template product<1>(x, r);
+    double s[2] = {act ? x[0] * (0.5 * r[0] + bi) : 0.0, act ? ci * pi : 0.0};
+    grp.template sum<2>(s);
+    phi = s[0];
+    spent = s[1];
+  }
+  if (act && sub == 0)
+    pi_out[(size_t)g * G + i] =
+        status == PAIR_ALLOC_INVALID ? __int_as_float(0x7fc00000) : (float)pi;
+  if (threadIdx.x == 0) {
     if (status == PAIR_ALLOC_INVALID) atomicOr(dev_err, PAIR_DEV_ERR_ALLOC_INPUT);
     if (status == PAIR_ALLOC_INFEASIBLE) atomicOr(dev_err, PAIR_DEV_ERR_ALLOC_INFEASIBLE);
     if (stats) {
       double *st = stats + (size_t)g * PAIR_ALLOC_NSTATS;
-      st[PAIR_ALLOC_PHI] = status == PAIR_ALLOC_INVALID ? 0.0 : phi_out;
-      st[PAIR_ALLOC_SPENT] = status == PAIR_ALLOC_INVALID ? 0.0 : budget - slack_out;
+      st[PAIR_ALLOC_PHI] = phi;
+      st[PAIR_ALLOC_SPENT] = spent;
       st[PAIR_ALLOC_GAP] = gap;
-      st[PAIR_ALLOC_NEWTON] = (double)newton;
+      st[PAIR_ALLOC_NEWTON] = (double)steps;
       st[PAIR_ALLOC_STATUS] = (double)status;
     }
   }
@@ -413,12 +519,13 @@ template <int GP>
 pair_status launch_alloc(int32_t B, int32_t G, const float *p_hat, const float *m_hat,
                          const float *a, const float *c_hat, const float *budget, float pi_min,
                          float *pi, double *stats, int32_t *dev_err, cudaStream_t s) {
-  const size_t smem = sizeof(AllocSmem<GP>);
+  const size_t smem =
+      sizeof(AllocSmem<GP>) + (size_t)G * alloc_pitch(G) * sizeof(double);
   PAIR_CUDA_TRY(cudaFuncSetAttribute(alloc_kernel<GP>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   PAIR_BEGIN("allocate", s);
-  alloc_kernel<GP><<<B, GP, smem, s>>>(G, p_hat, m_hat, a, c_hat, budget, pi_min, pi, stats,
-                                       dev_err);
+  alloc_kernel<GP><<<B, AllocShape<GP>::kThreads, smem, s>>>(G, p_hat, m_hat, a, c_hat, budget,
+                                                             pi_min, pi, stats, dev_err);
   PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
 }
@@ -440,6 +547,10 @@ extern "C" pair_status pair_allocate(int32_t B, int32_t G, const float *p_hat,
   const pair_status dv = check_device();
   if (dv != PAIR_OK) return dv;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  if (G <= 8)
+    return launch_alloc<8>(B, G, p_hat, m_hat, a, c_hat, budget, pi_min, pi, stats, dev_err, s);
+  if (G <= 16)
+    return launch_alloc<16>(B, G, p_hat, m_hat, a, c_hat, budget, pi_min, pi, stats, dev_err, s);
   if (G <= 32)
     return launch_alloc<32>(B, G, p_hat, m_hat, a, c_hat, budget, pi_min, pi, stats, dev_err, s);
   if (G <= 64)
