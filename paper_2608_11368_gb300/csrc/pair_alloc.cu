@@ -67,6 +67,10 @@ constexpr int kLinMaxDegree = 61;   // reached only if rounding puts rho far abo
 constexpr float kStepFrac = 0.995f; // of the largest step that keeps the interior
 constexpr double kStartMu = 0.1;    // the start's complementarity: kStartMu Phi in all
 
+// Where a value only steers (step lengths, the centring parameter) or enters
+// both sides of an identity (the slacks' reciprocals), rcp_approx stands in for
+// a division; v and the diagonal's inverse take rcp_newton.
+
 // Shape of a group's CTA: GP >= G is the padded group size, TPR adjacent
 // threads share a row of A and each holds its coordinate's state.
 template <int GP>
@@ -75,24 +79,6 @@ struct AllocShape {
   static constexpr int kTpr = kThreads / GP;
   static constexpr int kWarps = kThreads / 32;
 };
-
-// Reciprocals from the hardware's approximation over the whole fp64 range
-// (PTX rcp.approx.ftz.f64, about 20 bits; an IEEE division takes some ten
-// instructions of the fp64 pipe, and a step has eighteen of them): as it is
-// where the value only steers (step lengths, the centring parameter) or where
-// the same value enters both sides of an identity; with two steps of Newton's
-// iteration, y += y (1 - x y), to within a unit or two of the last place
-// elsewhere.
-__device__ __forceinline__ double rcp_approx(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-__device__ __forceinline__ double rcp_newton(double x) {
-  double y = rcp_approx(x);
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
-}
 
 // Row pitch of A (odd: rows start in different shared-memory banks).
 __host__ __device__ __forceinline__ int alloc_pitch(int G) { return G | 1; }

@@ -13,13 +13,25 @@
 //   E[ghat] - g = (E[a] - abar) S.
 // K, abar and the quadratic forms are accumulated in fp64; the coefficients
 // are the fp32 pair_coeffs_weighted values of each draw.
+//
+// A draw's terms (r_i - r_j) w_ij are the same for every draw, so they and the
+// weights are formed once per block and a draw only adds the ones of its
+// completed pairs. The draws run one per lane, 32 at a time: no exchange
+// between lanes, uniform (broadcast) reads of the terms and of K, and every
+// lane of the fp64 pipe busy, which is what bounds the pass: about G^2 / 2 + 4 G
+// fp64 operations per draw at 2 per clock and SM. Measured on one GB300, 50,000
+// draws of 16 candidates with D = 4096: the call takes
+// 95 us, its draws pass 62 us; one block per draw, with a tree and five block
+// reductions each, took 653 and 500 us. For G = 64 and 128 (3125 and 781
+// draws) the call takes 0.16 and 0.43 ms, from 0.75 and 1.37 ms.
 #include "pair_coeffs_dev.cuh"
 
 namespace pairk {
 namespace {
 
-constexpr int kAuditBlocks = 4096;  // partial-sum slots (draw b -> block b mod grid), at most
+constexpr int kAuditBlocks = 4096;  // partial-sum slots (blocks of draws), at most
 constexpr int kAuditStats = 8;
+constexpr int kGramThreads = 256;
 
 // Deterministic block sum of one double per thread (all threads call).
 __device__ double block_sum_double(double v, double *red) {
@@ -33,17 +45,56 @@ __device__ double block_sum_double(double v, double *red) {
   return s;
 }
 
-// K[i][j] = sum_d S[i][d] S[j][d] in fp64; block i computes row i.
-__global__ void audit_gram_kernel(int G, int D, const float *__restrict__ S, double *K) {
-  __shared__ double red[32];
-  const int i = blockIdx.x;
-  const float *si = S + (size_t)i * D;
-  for (int j = 0; j < G; ++j) {
-    const float *sj = S + (size_t)j * D;
-    double acc = 0.0;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) acc += (double)si[d] * (double)sj[d];
-    const double t = block_sum_double(acc, red);
-    if (threadIdx.x == 0) K[(size_t)i * G + j] = t;
+// K[i][j] = sum_d S[i][d] S[j][d] in fp64. Block -> a TI x TI tile of (i, j) on
+// or below the diagonal; both triangles are written. One entry per block for
+// G <= 32 (as many blocks as there are entries: a block's chain is D / 256
+// products long, 84 -> 11 us for 16 x 4096), 4 x 4 above, where the blocks fill
+// the chip anyway and a tile halves the conversions per product.
+template <int TI>
+__global__ void __launch_bounds__(kGramThreads)
+    audit_gram_kernel(int G, int D, const float *__restrict__ S, double *K) {
+  __shared__ double red[kGramThreads / 32][TI * TI];
+  // Tile (ti, tj), tj <= ti, of the lower triangle in row order.
+  int ti = (int)((sqrtf(8.f * blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((ti + 1) * (ti + 2) / 2 <= (int)blockIdx.x) ++ti;
+  while (ti * (ti + 1) / 2 > (int)blockIdx.x) --ti;
+  const int tj = (int)blockIdx.x - ti * (ti + 1) / 2;
+  double acc[TI][TI];
+#pragma unroll
+  for (int p = 0; p < TI; ++p)
+#pragma unroll
+    for (int q = 0; q < TI; ++q) acc[p][q] = 0.0;
+  for (int d = threadIdx.x; d < D; d += kGramThreads) {
+    double x[TI], y[TI];
+#pragma unroll
+    for (int p = 0; p < TI; ++p) {
+      const int i = min(ti * TI + p, G - 1), j = min(tj * TI + p, G - 1);
+      x[p] = (double)S[(size_t)i * D + d];
+      y[p] = (double)S[(size_t)j * D + d];
+    }
+#pragma unroll
+    for (int p = 0; p < TI; ++p)
+#pragma unroll
+      for (int q = 0; q < TI; ++q) acc[p][q] = fma(x[p], y[q], acc[p][q]);
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int p = 0; p < TI; ++p)
+#pragma unroll
+    for (int q = 0; q < TI; ++q) {
+      double v = acc[p][q];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) red[warp][p * TI + q] = v;
+    }
+  __syncthreads();
+  if (threadIdx.x < TI * TI) {
+    double t = 0.0;
+    for (int w = 0; w < kGramThreads / 32; ++w) t += red[w][threadIdx.x];
+    const int i = ti * TI + threadIdx.x / TI, j = tj * TI + threadIdx.x % TI;
+    if (i < G && j <= i) {
+      K[(size_t)i * G + j] = t;
+      K[(size_t)j * G + i] = t;
+    }
   }
 }
 
@@ -54,175 +105,427 @@ __global__ void audit_target_kernel(int G, const float *__restrict__ r, float sc
   __shared__ double sa[128];
   __shared__ double red[32];
   const int i = threadIdx.x;
+  const double rsum = block_sum_double(i < G ? (double)r[i] : 0.0, red);
   if (i < G) {
-    double s = 0.0;
-    for (int j = 0; j < G; ++j) s += (double)r[i] - (double)r[j];
-    sa[i] = (double)scale * 0.5 * s;
+    sa[i] = (double)scale * 0.5 * (G * (double)r[i] - rsum);
     abar[i] = sa[i];
   }
   __syncthreads();
   double ui = 0.0;
-  if (i < G) {
-    for (int j = 0; j < G; ++j) ui += K[(size_t)i * G + j] * sa[j];
+  if (i < G) {  // K is symmetric: its columns are read, neighbours together
+#pragma unroll 8
+    for (int j = 0; j < G; ++j) ui += K[(size_t)j * G + i] * sa[j];
     u[i] = ui;
   }
   const double t = block_sum_double(i < G ? sa[i] * ui : 0.0, red);
   if (i == 0) *gg = t;
 }
 
-template <int GP>
-struct AuditSmem {
-  GroupSmemW<GP> grp;
-  double K[GP * GP];
-  double abar[GP], u[GP], e[GP], a[GP];
-  double red[32];
-};
-
-// Persistent: block q handles draws b = q, q + grid, ... in order and writes
-// its partial sums [stats..., sum_b w_b a_b (G)] to part[q].
-template <int GP>
-__global__ void __launch_bounds__(GP, 1) audit_draws_kernel(
-    int N, int G, const float *__restrict__ r, const float *__restrict__ rho,
-    const uint8_t *__restrict__ Jd, const double *__restrict__ wd, float scale, int center,
-    int wmode, float w_max, const double *__restrict__ K, const double *__restrict__ abar,
-    const double *__restrict__ u, const double *__restrict__ gg_p, double *part,
-    int32_t *dev_err) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  AuditSmem<GP> &sm = *reinterpret_cast<AuditSmem<GP> *>(smem_raw);
-  const int tid = threadIdx.x;
-  for (int k = tid; k < G * G; k += GP) {
-    const int i = k / G, j = k % G;
-    sm.K[i * GP + j] = K[k];
-  }
-  if (tid < GP) {
-    const bool in = tid < G;
-    sm.abar[tid] = in ? abar[tid] : 0.0;
-    sm.u[tid] = in ? u[tid] : 0.0;
-    sm.grp.r[tid] = in ? r[tid] : 0.f;
-    sm.grp.pi[tid] = (in && wmode == PAIR_W_MARGINAL) ? rho[(size_t)tid * G + tid] : 1.f;
-  }
-  const double gg = *gg_p;
-  // rho is the same for every draw: its triangle is read once per block.
-  float v[GP / 2];
-  load_upper<GP>(rho, G, weighting_reads_rho(wmode), v);
-  double acc[6] = {0, 0, 0, 0, 0, 0};  // mse, cos, vertices, edges, ess, weight
-  double a_acc = 0.0;
-  for (int b = blockIdx.x; b < N; b += gridDim.x) {
-    __syncthreads();
-    sm.grp.J[tid] = (tid < G) ? (Jd[(size_t)b * G + tid] != 0) : 0;
-    __syncthreads();
-    const WeightedOut o =
-        group_coeffs_w<GP>(sm.grp, v, G, scale, (uint32_t)center, wmode, w_max, dev_err);
-    const double ai = (double)o.a;
-    const double ei = ai - sm.abar[tid];
-    sm.e[tid] = ei;
-    sm.a[tid] = ai;
-    __syncthreads();
-    double Ke = 0.0;
-    if (tid < G)
-      for (int j = 0; j < G; ++j) Ke += sm.K[tid * GP + j] * sm.e[j];
-    const double q_ee = block_sum_double(ei * Ke, sm.red);
-    const double q_au = block_sum_double(ai * sm.u[tid], sm.red);
-    const double q_aa = block_sum_double(ai * (Ke + sm.u[tid]), sm.red);
-    const double w = wd ? wd[b] : 1.0 / (double)N;
-    if (tid == 0) {
-      const double cosb = (q_aa > 0.0 && gg > 0.0) ? q_au / sqrt(q_aa * gg) : 0.0;
-      const double ess = o.W2 > 0.f ? (double)o.W * (double)o.W / (double)o.W2 : 0.0;
-      acc[0] += w * q_ee;
-      acc[1] += w * cosb;
-      acc[2] += w * (double)o.K;
-      acc[3] += w * (double)(o.K * (o.K - 1) / 2);
-      acc[4] += w * ess;
-      acc[5] += w;
-    }
-    a_acc += w * ai;
-  }
-  double *pq = part + (size_t)blockIdx.x * (kAuditStats + GP);
-  if (tid == 0)
-    for (int k = 0; k < 6; ++k) pq[k] = acc[k];
-  if (tid < GP) pq[kAuditStats + tid] = a_acc;
+// Shared memory of the draws kernel (G x G lower triangles packed by rows,
+// entry (i, j), j < i, at i (i - 1) / 2 + j; K with its diagonal).
+__host__ __device__ __forceinline__ size_t audit_tri(int G) { return (size_t)G * (G - 1) / 2; }
+// Warps that share 32 draws: one for G <= 32; above, a draw's fp64 operands
+// (2 x 256 G bytes per 32 draws) leave room for one such batch per block only,
+// and its warps divide the rows.
+__host__ __device__ __forceinline__ int audit_team(int G) { return G <= 32 ? 1 : 8; }
+// Warps per block: small ones of single-warp teams, so that the last round of
+// blocks leaves few SMs idle (50,000 draws of 16 are 1563 batches).
+__host__ __device__ __forceinline__ constexpr int audit_warps(int team) { return team == 1 ? 4 : team; }
+inline size_t audit_draws_smem(int G) {
+  const size_t warps = audit_warps(audit_team(G)), teams = warps / audit_team(G);
+  return sizeof(double) * (audit_tri(G) + G            // K
+                           + 2 * (size_t)G             // abar, u
+                           + teams * 2 * 32 * (size_t)G  // e, sums of a
+                           + warps * 4 * 32)             // exchanges of a team
+         + sizeof(float) * (2 * audit_tri(G) + 2 * (size_t)G)  // terms, weights, r, pi
+         + sizeof(uint32_t) * warps * 4 * 32;    // completion bits
 }
 
-// Sums the partials in block order, normalises by the total weight, and forms
-// the bias E[a] - abar, its norm through K and (optionally) the vector (E[a] -
-// abar) S. One block of 256 threads.
-__global__ void audit_finish_kernel(int nblk, int G, int GP, int D, const float *__restrict__ S,
-                                    const double *__restrict__ K, const double *__restrict__ abar,
-                                    const double *__restrict__ gg_p,
-                                    const double *__restrict__ part, double *stats, double *bias) {
+template <int TW>
+__device__ __forceinline__ void team_sync() {
+  if constexpr (TW == 1) __syncwarp();
+  else __syncthreads();
+}
+
+// Sum over the warps of a team of one value per lane (slot: 0 .. 3, its own
+// exchange buffer until the team's next synchronisation with that slot).
+template <int TW, typename T>
+__device__ __forceinline__ T team_sum(double *xch, int slot, T v) {
+  if constexpr (TW == 1) {
+    return v;
+  } else {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    xch[(warp * 4 + slot) * 32 + lane] = (double)v;
+    __syncthreads();
+    T t = (T)xch[slot * 32 + lane];
+#pragma unroll
+    for (int w = 1; w < TW; ++w) t += (T)xch[(w * 4 + slot) * 32 + lane];
+    return t;
+  }
+}
+
+// Draws in batches of 32, one per lane; batch q of the teams' stride. Row i of
+// a batch belongs to warp i mod TW of its team. Per draw: the row sums
+// a_i = 1/2 sum_j J_i J_j t_ij (16-term trees, combined pairwise) and the weight
+// sums, the weighting's and flags' division and centring, then in fp64
+// e = a - abar, e^T K e over the lower triangle, e^T u. With a = e + abar,
+// u = K abar and gg = abar^T u: a^T u = e^T u + gg and
+// a^T K a = e^T K e + 2 e^T u + gg (0 exactly where a = 0).
+template <int TW>
+__global__ void __launch_bounds__(audit_warps(TW) * 32)
+    audit_draws_kernel(int N, int G, const float *__restrict__ r, const float *__restrict__ rho,
+                       const uint8_t *__restrict__ Jd, const double *__restrict__ wd, float scale,
+                       uint32_t flags, int wmode, float w_max, const double *__restrict__ Kg,
+                       const double *__restrict__ abar_g, const double *__restrict__ u_g,
+                       const double *__restrict__ gg_p, double *part, int32_t *dev_err) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int kWarps = audit_warps(TW), kTeams = kWarps / TW;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = warp / TW, tw = warp % TW;
+  const int tri = (int)audit_tri(G);
+  double *K = reinterpret_cast<double *>(smem_raw);
+  double *abar = K + tri + G, *u = abar + G;
+  double *e_all = u + G, *asum_all = e_all + kTeams * 32 * G;
+  double *xch = asum_all + kTeams * 32 * G;
+  float *T = reinterpret_cast<float *>(xch + kWarps * 4 * 32);
+  float *Wt = T + tri, *rs = Wt + tri, *pis = rs + G;
+  uint32_t *bits_all = reinterpret_cast<uint32_t *>(pis + G);
+  double *e = e_all + team * 32 * G, *asum = asum_all + team * 32 * G;
+  uint32_t *bits = bits_all + team * 4 * 32;
+
+  // ---- the group's constants
+  for (int i = threadIdx.x; i < G; i += blockDim.x) {
+    abar[i] = abar_g[i];
+    u[i] = u_g[i];
+    rs[i] = r[i];
+    pis[i] = wmode == PAIR_W_MARGINAL ? rho[(size_t)i * G + i] : 1.f;
+  }
+  for (int k = threadIdx.x; k < kTeams * 32 * G; k += blockDim.x) asum_all[k] = 0.0;
+  __syncthreads();
+  for (int j = warp; j < G; j += kWarps) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = j + lane + 32 * c;
+      if (i >= G) continue;
+      K[i * (i + 1) / 2 + j] = Kg[(size_t)j * G + i];
+      if (i == j) continue;
+      // Entry (j, i) of rho's strict upper triangle. An invalid weight is
+      // NaN here and raises the error bit in the draws that complete it.
+      const float dr = rs[i] - rs[j];
+      float w = 1.f, t = dr;
+      if (wmode == PAIR_W_MARGINAL) {
+        const float den = pis[j] * pis[i];
+        const bool ok = pis[i] > 0.f && pis[j] > 0.f;
+        w = ok ? __frcp_rn(den) : __int_as_float(0x7fc00000);
+        t = ok ? __fdiv_rn(dr, den) : 0.f;
+      } else if (wmode != PAIR_W_UNWEIGHTED) {
+        const float rij = rho[(size_t)j * G + i];
+        const bool ok = rij > 0.f;
+        w = ok ? __frcp_rn(rij) : __int_as_float(0x7fc00000);
+        t = ok ? __fdiv_rn(dr, rij) : 0.f;
+        if (wmode == PAIR_W_CLIPPED && w > w_max) {
+          w = w_max;
+          t = dr * w_max;
+        }
+      }
+      T[i * (i - 1) / 2 + j] = t;
+      Wt[i * (i - 1) / 2 + j] = w;
+    }
+  }
+  __syncthreads();
+  const double gg = *gg_p, w_all = 1.0 / (double)N;
+
+  double acc[6] = {0, 0, 0, 0, 0, 0};  // mse, cos, vertices, edges, ess, weight (warp 0 of a team)
+  const int nbatch = (N + 31) / 32;
+  for (int bt = blockIdx.x * kTeams + team; bt < nbatch; bt += gridDim.x * kTeams) {
+    // ---- completion bits of the batch: 32 candidates per ballot
+    for (int q = tw; q < 32; q += TW) {
+      const int b = bt * 32 + q;
+      for (int j0 = 0; j0 < G; j0 += 32) {
+        const bool on = b < N && j0 + lane < G && Jd[(size_t)b * G + j0 + lane] != 0;
+        const uint32_t m = __ballot_sync(0xffffffffu, on);
+        if (lane == 0) bits[(j0 >> 5) * 32 + q] = m;
+      }
+    }
+    team_sync<TW>();
+    uint32_t m[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (k * 32 < G) m[k] = bits[k * 32 + lane];
+    // Whether candidate i of this lane's draw is completed.
+    auto done = [&](int i) { return ((bits[(i & ~31) + lane] >> (i & 31)) & 1u) != 0u; };
+    const int Kc = __popc(m[0]) + __popc(m[1]) + __popc(m[2]) + __popc(m[3]);
+
+    // ---- row sums
+    float W = 0.f, W2 = 0.f, s_a = 0.f;
+    for (int i = tw; i < G; i += TW) {
+      const float *row = T + i * (i - 1) / 2, *wrow = Wt + i * (i - 1) / 2;
+      const bool on = done(i);
+      float p[4] = {0.f, 0.f, 0.f, 0.f};
+      float sw = 0.f, sw2 = 0.f;
+#pragma unroll
+      for (int blk = 0; blk < 8; ++blk) {
+        float c = 0.f;
+        if (blk * 16 < G) {
+          const uint32_t mb = m[blk >> 1] >> ((blk & 1) * 16);
+          float x[16], wb = 0.f, wb2 = 0.f;
+#pragma unroll
+          for (int q = 0; q < 16; ++q) {
+            const int j = blk * 16 + q;
+            // Uniform over the warp: which triangle, and past the group.
+            float t = 0.f;
+            const bool jon = (mb >> q) & 1u;
+            if (j < i) {
+              t = row[j];
+              const float w = jon ? wrow[j] : 0.f;
+              wb += w;
+              wb2 = fmaf(w, w, wb2);
+            } else if (j > i && j < G) {
+              t = -T[j * (j - 1) / 2 + i];
+            }
+            x[q] = jon ? t : 0.f;
+          }
+          sw += wb;
+          sw2 += wb2;
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < o; ++q) x[q] += x[q + o];
+          c = x[0];
+        }
+        int mm = blk;
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+          if (mm & 1) { c = p[l] + c; mm >>= 1; }
+          else { p[l] = c; break; }
+        }
+      }
+      const float a = on ? 0.5f * p[3] : 0.f;
+      if (on) {
+        W += sw;
+        W2 += sw2;
+      }
+      s_a += a;
+      reinterpret_cast<float *>(e + (size_t)i * 32)[lane] = a;  // first half of the row's cells
+    }
+    W = team_sum<TW>(xch, 0, W);
+    W2 = team_sum<TW>(xch, 1, W2);
+    if (W != W) flag_error(dev_err, PAIR_DEV_ERR_NONPOSITIVE_INCLUSION);
+
+    // ---- the divisions and the centring of the coefficients
+    float div = 1.f;
+    bool divide = false, zero = false;
+    if (wmode == PAIR_W_HAJEK) {
+      zero = !(W > 0.f);
+      div = W;
+      divide = !zero;
+    }
+    float sd = 1.f;
+    bool standard = false;
+    if ((flags & PAIR_STANDARDIZE) && Kc >= 2) {
+      float sr = 0.f, ss = 0.f;
+      for (int i = 0; i < G; ++i) sr += done(i) ? rs[i] : 0.f;
+      const float mean = sr / (float)Kc;
+      for (int i = 0; i < G; ++i) {
+        const float dv = done(i) ? rs[i] - mean : 0.f;
+        ss = fmaf(dv, dv, ss);
+      }
+      sd = sqrtf(ss / (float)(Kc - 1));
+      standard = true;
+    }
+    auto finish = [&](float a) {
+      if (zero) a = 0.f;
+      else if (divide) a = __fdiv_rn(a, div);
+      if (standard) a = sd > 0.f ? __fdiv_rn(a, sd) : 0.f;
+      return a;
+    };
+    float mean_a = 0.f;
+    if (flags & PAIR_CENTER) {
+      if (divide || zero || standard) {
+        s_a = 0.f;
+        for (int i = tw; i < G; i += TW)
+          s_a += finish(reinterpret_cast<float *>(e + (size_t)i * 32)[lane]);
+      }
+      s_a = team_sum<TW>(xch, 2, s_a);
+      mean_a = Kc > 0 ? s_a / (float)Kc : 0.f;
+    }
+
+    // ---- fp64: e = a - abar, the sums of a, e^T u
+    const int b = bt * 32 + lane;
+    const double w = b < N ? (wd ? wd[b] : w_all) : 0.0;
+    double eu = 0.0;
+    bool any = false;
+    for (int i = tw; i < G; i += TW) {
+      float a = finish(reinterpret_cast<float *>(e + (size_t)i * 32)[lane]);
+      if (done(i)) a -= mean_a;
+      a *= scale;
+      any |= a != 0.f;
+      const double ad = (double)a, ei = ad - abar[i];
+      __syncwarp();  // the row's fp32 cells are read before its fp64 ones are written
+      e[i * 32 + lane] = ei;
+      asum[i * 32 + lane] = fma(w, ad, asum[i * 32 + lane]);
+      eu = fma(ei, u[i], eu);
+    }
+    team_sync<TW>();
+
+    // ---- e^T K e over the lower triangle
+    double q = 0.0;
+    for (int i = tw; i < G; i += TW) {
+      const double *row = K + i * (i + 1) / 2;
+      double s0 = 0.0, s1 = 0.0;
+      int j = 0;
+      for (; j + 4 <= i; j += 4) {
+        s0 = fma(row[j], e[j * 32 + lane], s0);
+        s1 = fma(row[j + 1], e[(j + 1) * 32 + lane], s1);
+        s0 = fma(row[j + 2], e[(j + 2) * 32 + lane], s0);
+        s1 = fma(row[j + 3], e[(j + 3) * 32 + lane], s1);
+      }
+      for (; j < i; ++j) s0 = fma(row[j], e[j * 32 + lane], s0);
+      const double ei = e[i * 32 + lane];
+      q = fma(ei, fma(2.0, s0 + s1, row[i] * ei), q);
+    }
+    q = team_sum<TW>(xch, 2, q);
+    eu = team_sum<TW>(xch, 3, eu);
+    if constexpr (TW > 1) any = team_sum<TW>(xch, 0, any ? 1.f : 0.f) > 0.f;
+    if (tw == 0) {
+      const double q_au = eu + gg, q_aa = any ? q + 2.0 * eu + gg : 0.0;
+      const double cosb = (q_aa > 0.0 && gg > 0.0) ? q_au * rsqrt(q_aa * gg) : 0.0;
+      const double ess = W2 > 0.f ? (double)W * (double)W / (double)W2 : 0.0;
+      acc[0] = fma(w, q, acc[0]);
+      acc[1] = fma(w, cosb, acc[1]);
+      acc[2] = fma(w, (double)Kc, acc[2]);
+      acc[3] = fma(w, (double)(Kc * (Kc - 1) / 2), acc[3]);
+      acc[4] = fma(w, ess, acc[4]);
+      acc[5] += w;
+    }
+    team_sync<TW>();  // bits, e and the exchanges are rewritten by the next batch
+  }
+
+  // ---- the block's partial sums, lanes then teams in order
+  double *pq = part + (size_t)blockIdx.x * (kAuditStats + G);
+#pragma unroll
+  for (int k = 0; k < 6; ++k)
+    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+  __syncthreads();
+  if (tw == 0 && lane == 0)
+#pragma unroll
+    for (int k = 0; k < 6; ++k) xch[team * 6 + k] = acc[k];
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    double t = 0.0;
+    for (int q = 0; q < kTeams; ++q) t += xch[q * 6 + threadIdx.x];
+    pq[threadIdx.x] = t;
+  }
+  for (int i = warp; i < G; i += kWarps) {
+    double t = 0.0;
+    for (int q = 0; q < kTeams; ++q) t += asum_all[((size_t)q * G + i) * 32 + lane];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) pq[kAuditStats + i] = t;
+  }
+}
+
+// Sums the partials (each column by one warp, lanes over the blocks, then a
+// butterfly: a fixed order), normalises by the total weight, and forms the
+// bias E[a] - abar, its norm through K and (optionally) the vector (E[a] -
+// abar) S. Every block forms the means; block 0 writes the statistics, and
+// the blocks share the D components of the bias (one block for all of it
+// took 95 us at 16 x 4096).
+__global__ void __launch_bounds__(256)
+    audit_finish_kernel(int nblk, int G, int D, const float *__restrict__ S,
+                        const double *__restrict__ K, const double *__restrict__ abar,
+                        const double *__restrict__ gg_p, const double *__restrict__ part,
+                        double *stats, double *bias) {
   __shared__ double em[128];
   __shared__ double red[32];
   __shared__ double tot[6];
-  const int tid = threadIdx.x;
-  // Each column of the partials (6 statistics, then G coefficient sums) is
-  // summed by every thread over a strided share of the blocks, then by the
-  // block reduction: a fixed order, and the loads of a column in flight
-  // together.
-  for (int k = 0; k < 6 + G; ++k) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int stride = kAuditStats + G;
+  for (int k = tid >> 5; k < 6 + G; k += 8) {
     const int col = k < 6 ? k : kAuditStats + (k - 6);
     double s = 0.0;
-    for (int q = tid; q < nblk; q += blockDim.x) s += part[(size_t)q * (kAuditStats + GP) + col];
-    const double t = block_sum_double(s, red);
-    if (tid == 0) {
-      if (k < 6) tot[k] = t;
-      else em[k - 6] = t;
+    for (int q = lane; q < nblk; q += 32) s += part[(size_t)q * stride + col];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+      if (k < 6) tot[k] = s;
+      else em[k - 6] = s;
     }
   }
   __syncthreads();
   const double W = tot[5];
   if (tid < G) em[tid] = (W > 0.0 ? em[tid] / W : 0.0) - abar[tid];
   __syncthreads();
-  double Ke = 0.0;
-  if (tid < G)
-    for (int j = 0; j < G; ++j) Ke += K[(size_t)tid * G + j] * em[j];
-  const double bb = block_sum_double(tid < G ? em[tid] * Ke : 0.0, red);
-  if (tid == 0) {
-    stats[0] = sqrt(bb > 0.0 ? bb : 0.0);
-    for (int k = 0; k < 5; ++k) stats[1 + k] = W > 0.0 ? tot[k] / W : 0.0;
-    stats[6] = *gg_p;
-    stats[7] = W;
+  if (blockIdx.x == 0) {
+    double Ke = 0.0;
+    if (tid < G)
+#pragma unroll 8
+      for (int j = 0; j < G; ++j) Ke += K[(size_t)j * G + tid] * em[j];
+    const double bb = block_sum_double(tid < G ? em[tid] * Ke : 0.0, red);
+    if (tid == 0) {
+      stats[0] = sqrt(bb > 0.0 ? bb : 0.0);
+      for (int k = 0; k < 5; ++k) stats[1 + k] = W > 0.0 ? tot[k] / W : 0.0;
+      stats[6] = *gg_p;
+      stats[7] = W;
+    }
   }
   if (bias)
-    for (int d = tid; d < D; d += blockDim.x) {
+    for (int d = blockIdx.x * 256 + tid; d < D; d += gridDim.x * 256) {
       double s = 0.0;
+#pragma unroll 8
       for (int i = 0; i < G; ++i) s += em[i] * (double)S[(size_t)i * D + d];
       bias[d] = s;
     }
 }
 
-template <int GP>
-pair_status launch_audit_gp(int N, int G, int D, const float *r, const float *rho,
-                            const float *S, const uint8_t *Jd, const double *wd, float scale,
-                            uint32_t flags, int wmode, float w_max, double *stats, double *bias,
-                            double *ws, int32_t *dev_err, cudaStream_t s) {
+template <int TW>
+pair_status launch_draws(int nblk, size_t smem, int N, int G, const float *r, const float *rho,
+                         const uint8_t *Jd, const double *wd, float scale, uint32_t flags,
+                         int wmode, float w_max, const double *K, const double *abar,
+                         const double *u, const double *gg, double *part, int32_t *dev_err,
+                         cudaStream_t s) {
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(audit_draws_kernel<TW>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PAIR_BEGIN("audit_draws", s);
+  audit_draws_kernel<TW><<<nblk, audit_warps(TW) * 32, smem, s>>>(
+      N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar, u, gg, part, dev_err);
+  PAIR_LAUNCH_CHECK(s);
+  return PAIR_OK;
+}
+
+pair_status launch_audit(int N, int G, int D, const float *r, const float *rho, const float *S,
+                         const uint8_t *Jd, const double *wd, float scale, uint32_t flags,
+                         int wmode, float w_max, double *stats, double *bias, double *ws,
+                         int32_t *dev_err, cudaStream_t s) {
   double *K = ws, *abar = K + (size_t)G * G, *u = abar + G, *gg = u + G;
   double *part = gg + 2;
+  const int gt = G <= 32 ? G : (G + 3) / 4;  // rows of gram tiles
   PAIR_BEGIN("audit_gram", s);
-  audit_gram_kernel<<<G, 256, 0, s>>>(G, D, S, K);
+  if (G <= 32)
+    audit_gram_kernel<1><<<gt * (gt + 1) / 2, kGramThreads, 0, s>>>(G, D, S, K);
+  else
+    audit_gram_kernel<4><<<gt * (gt + 1) / 2, kGramThreads, 0, s>>>(G, D, S, K);
   PAIR_LAUNCH_CHECK(s);
   PAIR_BEGIN("audit_target", s);
   audit_target_kernel<<<1, 128, 0, s>>>(G, r, scale, K, abar, u, gg);
   PAIR_LAUNCH_CHECK(s);
-  // As many blocks as the SMs hold at once (the draws loop is latency bound,
-  // one group per block), at most the kAuditBlocks partial slots.
-  const size_t smem = sizeof(AuditSmem<GP>);
-  PAIR_CUDA_TRY(cudaFuncSetAttribute(audit_draws_kernel<GP>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int dev = 0, nsm = 0, per_sm = 0;
-  PAIR_CUDA_TRY(cudaGetDevice(&dev));
-  PAIR_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  PAIR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, audit_draws_kernel<GP>, GP,
-                                                              smem));
-  int nblk = (nsm > 0 ? nsm : 1) * (per_sm > 0 ? per_sm : 1);
-  if (nblk > kAuditBlocks) nblk = kAuditBlocks;
-  if (nblk > N) nblk = N;
-  PAIR_BEGIN("audit_draws", s);
-  audit_draws_kernel<GP><<<nblk, GP, smem, s>>>(N, G, r, rho, Jd, wd, scale,
-                                                (int)flags, wmode, w_max, K,
-                                                abar, u, gg, part, dev_err);
-  PAIR_LAUNCH_CHECK(s);
+  // One batch of 32 draws per team where the batches fit the partial slots
+  // and a few rounds of the chip; a stride over the batches beyond that.
+  const int teams = audit_warps(audit_team(G)) / audit_team(G);
+  const size_t smem = audit_draws_smem(G);
+  int nblk = (int)ceil_div(ceil_div(N, 32), teams);
+  const int most = 152 * (int)(227 * 1024 / (smem + 1024) < 8 ? 227 * 1024 / (smem + 1024) : 8);
+  if (nblk > most) nblk = most;
+  pair_status st;
+  if (audit_team(G) == 1)
+    st = launch_draws<1>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar, u,
+                         gg, part, dev_err, s);
+  else
+    st = launch_draws<8>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K,
+                                   abar, u, gg, part, dev_err, s);
+  if (st != PAIR_OK) return st;
   PAIR_BEGIN("audit_finish", s);
-  audit_finish_kernel<<<1, 256, 0, s>>>(nblk, G, GP, D, S, K, abar, gg, part, stats, bias);
+  const int fin = bias ? (int)ceil_div(D, 256) : 1;
+  audit_finish_kernel<<<fin < 152 ? fin : 152, 256, 0, s>>>(nblk, G, D, S, K, abar, gg, part,
+                                                            stats, bias);
   PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
 }
@@ -258,13 +561,6 @@ extern "C" pair_status pair_audit(int32_t N, int32_t G, int32_t D, const float *
   const pair_status dv = check_device();
   if (dv != PAIR_OK) return dv;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  double *w = static_cast<double *>(ws);
-  if (G <= 32)
-    return launch_audit_gp<32>(N, G, D, r, rho, S, Jdraws, draw_weight, scale, flags, wm, w_max,
-                               stats, bias, w, dev_err, s);
-  if (G <= 64)
-    return launch_audit_gp<64>(N, G, D, r, rho, S, Jdraws, draw_weight, scale, flags, wm, w_max,
-                               stats, bias, w, dev_err, s);
-  return launch_audit_gp<128>(N, G, D, r, rho, S, Jdraws, draw_weight, scale, flags, wm, w_max,
-                              stats, bias, w, dev_err, s);
+  return launch_audit(N, G, D, r, rho, S, Jdraws, draw_weight, scale, flags, wm, w_max, stats,
+                      bias, static_cast<double *>(ws), dev_err, s);
 }

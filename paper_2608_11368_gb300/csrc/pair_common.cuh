@@ -30,6 +30,22 @@ __device__ __forceinline__ void flag_error(int32_t *err, int bit) {
   if (err) atomicOr(err, bit);
 }
 
+// Reciprocals from the hardware's approximation over the whole fp64 range
+// (PTX rcp.approx.ftz.f64, about 20 bits), and with two steps of Newton's
+// iteration, y += y (1 - x y), to within a unit or two of the last place (x
+// normal, its reciprocal too). An IEEE division takes some ten instructions of
+// the fp64 pipe, which runs at 2 lanes per clock and SM.
+__device__ __forceinline__ double rcp_approx(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ double rcp_newton(double x) {
+  double y = rcp_approx(x);
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+
 __host__ __device__ __forceinline__ int64_t ceil_div(int64_t a, int64_t b) {
   return (a + b - 1) / b;
 }

@@ -1,0 +1,68 @@
+"""pair_audit's draws kernel at the edges of its batches and teams, against the
+explicit fp64 oracle: 32 draws per batch (a last batch of 1, 31, 32, 33), one
+warp per batch up to G = 32 and the block's eight above, several batches per
+team, weighted draws, centring, and the error bit of an invalid weight only
+where a draw completes its edge. Tolerance as in test_gpu_audit.py."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+from tests.gpu_util import dev, dev_err_word
+from tests.test_gpu_audit import _binding, _check, _population
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("G,N", [(2, 1), (5, 31), (16, 32), (31, 33), (32, 4000), (33, 1),
+                                 (64, 33), (127, 95), (128, 6000), (16, 60000)])
+@pytest.mark.parametrize("wmode,center", [(oracle.W_HT, True), (oracle.W_HAJEK, False),
+                                          (oracle.W_HAJEK, True)])
+def test_audit_batches(G, N, wmode, center):
+    B = _binding()
+    D = 300 if N < 10000 else 8
+    r, S, p, rho, Jd = _population(900 + G, G, D, N)
+    w = np.random.default_rng(G).uniform(0.2, 1.0, N)
+    M = math.comb(G, 2)
+    err = dev_err_word()
+    stats, bias = B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd), draw_weight=dev(w), wmode=wmode,
+                               scale=1.0 / M, flags=1 if center else 0, dev_err=err)
+    assert B.pair_status_sync(err) == 0
+    ref = oracle.audit(r, rho, S, Jd, w, scale=1.0 / M, center=center, wmode=wmode)
+    _check(stats, bias, ref, rtol=2e-5)
+
+
+@pytest.mark.parametrize("G", [12, 40])
+def test_audit_standardize_is_a_scale_per_draw(G):
+    """One draw: standardised coefficients are the plain ones over the sample
+    standard deviation of the completed rewards, so the estimate's cosine is
+    unchanged and ||ghat|| scales (fp32 rounding of the coefficients)."""
+    B = _binding()
+    r, S, p, rho, Jd = _population(950 + G, G, 20, 1)
+    Jd[:] = 1
+    Jd[0, G // 2] = 0
+    sd = r[Jd[0] != 0].astype(np.float64).std(ddof=1)
+    out = []
+    for flags in (0, 2):
+        stats, bias = B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd), flags=flags)
+        out.append((stats.cpu().numpy(), bias.cpu().numpy()))
+    M = G * r.astype(np.float64) - r.sum()
+    g = (0.5 * M) @ S.astype(np.float64)
+    h0, h2 = out[0][1] + g, out[1][1] + g
+    assert np.linalg.norm(h2 - h0 / sd) <= 1e-5 * np.linalg.norm(h2)
+    assert abs(out[0][0][2] - out[1][0][2]) <= 1e-5
+
+
+@pytest.mark.parametrize("G", [9, 50])
+def test_audit_invalid_weight_needs_a_completed_edge(G):
+    B = _binding()
+    r, S, p, rho, Jd = _population(970 + G, G, 4, 70)
+    rho[2, 5] = rho[5, 2] = 0.0
+    for both, want in ((0, 0), (1, 4)):
+        Jd[:, 2] = 1
+        Jd[:, 5] = 0
+        Jd[66, 5] = both
+        err = dev_err_word()
+        B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd), dev_err=err)
+        assert B.pair_status_sync(err) == want
