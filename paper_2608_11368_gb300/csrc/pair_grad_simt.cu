@@ -36,7 +36,9 @@ namespace cg = cooperative_groups;
 // shared memory, and S parts of B, whose outputs are added at the end the same
 // way, in rank order: 1075 tokens are 34 row tiles, too few for 304 CTA slots.
 // What bounds it: fp32 multiply-adds (128 per clock and SM).
-// SIMT_MEASURED
+// Measured on one GB300, 4 x 8 rollouts of 32 to 64 tokens, d = 256, V = 4096:
+// dH with the log-sum-exp 151 us (597 + 962 row by row, a block per token),
+// dW 182 us (856): 30 and 25 TFLOP/s counting the recomputed logits.
 constexpr int kBM = 32, kBN = 32, kTileThreads = 128;
 constexpr int kSliceMax = 256;               // columns of d per CTA, at most
 constexpr int kTileDMax = 8 * kSliceMax;     // largest d of this form
@@ -53,8 +55,11 @@ struct TileArgs {
 __host__ __device__ __forceinline__ int tile_slice(int d, int C) {
   return ((d / 16 + C - 1) / C) * 16;
 }
+// 64-column groups of a slice: outputs per thread, and the pitch of a tile's
+// rows (columns past the slice hold anything; their outputs are not used).
+__host__ __device__ __forceinline__ int tile_groups(int slice) { return (slice + 63) / 64; }
 inline size_t tile_smem(int d, int C) {
-  const size_t pitch = tile_slice(d, C) + 4;
+  const size_t pitch = tile_groups(tile_slice(d, C)) * 64 + 4;
   return sizeof(float) * ((kBM + 2 * kBN) * pitch   // A, B (two buffers)
                           + kBN * kGPitch           // g, n-major
                           + 2 * kBM * kBN           // partial logits (two buffers)
@@ -88,7 +93,7 @@ __device__ __forceinline__ void load_tile(float *dst, int pitch, const float *sr
   }
 }
 
-template <int MODE>
+template <int MODE, int NJ>
 __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileArgs g) {
   const int Teff = g.counters[0];
   const int C = g.C, S = g.S, cs = C * S;
@@ -99,7 +104,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
   const int rank = (int)cluster.block_rank(), ci = rank % C, si = rank / C;
   const int d = g.d, ds = tile_slice(d, C), k0 = ci * ds;
   const int dn = max(min(ds, d - k0), 0);  // this CTA's columns (a multiple of 16)
-  const int pitch = ds + 4;
+  constexpr int pitch = NJ * 64 + 4;
   const float *A = MODE == kModeDw ? g.W : g.Hc, *B = MODE == kModeDw ? g.Hc : g.W;
 
   extern __shared__ __align__(16) float smem[];
@@ -125,11 +130,11 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
   // The target of softmax row tid / 4.
   const int ytile =
       MODE != kModeDw && m0 + tid / 4 < Teff ? g.tok_y[m0 + tid / 4] : -1;
-  float acc[4][4][4];
+  float acc[4][NJ][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < NJ; ++j)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
 
@@ -150,28 +155,35 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
 #pragma unroll
     for (int i = 0; i < 4; ++i) z[i][0] = z[i][1] = 0.f;
     if (live) {
-      // 16-column pieces summed apart: shorter chains of roundings.
+      // 16-column pieces summed apart (shorter chains of roundings); the
+      // operands of the next 4 columns are loaded while these are multiplied.
+      const float *ap = As + zm * 4 * pitch, *bp = Bt + zn * pitch;
+      float4 a[2][4], b[2][2];
+      auto fetch = [&](int k, int q) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          a[q][i] = *reinterpret_cast<const float4 *>(ap + i * pitch + k);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          b[q][j] = *reinterpret_cast<const float4 *>(bp + 16 * j * pitch + k);
+      };
+      fetch(0, 0);
       for (int k = 0; k < dn; k += 16) {
         float zc[4][2];
 #pragma unroll
         for (int i = 0; i < 4; ++i) zc[i][0] = zc[i][1] = 0.f;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          float4 a[4], b[2];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            a[i] = *reinterpret_cast<const float4 *>(As + (zm * 4 + i) * pitch + k + 4 * u);
-#pragma unroll
-          for (int j = 0; j < 2; ++j)
-            b[j] = *reinterpret_cast<const float4 *>(Bt + (zn + 16 * j) * pitch + k + 4 * u);
+          // (Past the slice's end: still inside the row's pitch.)
+          fetch(k + 4 * u + 4, (u + 1) & 1);
 #pragma unroll
           for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-              zc[i][j] = fmaf(a[i].x, b[j].x, zc[i][j]);
-              zc[i][j] = fmaf(a[i].y, b[j].y, zc[i][j]);
-              zc[i][j] = fmaf(a[i].z, b[j].z, zc[i][j]);
-              zc[i][j] = fmaf(a[i].w, b[j].w, zc[i][j]);
+              zc[i][j] = fmaf(a[u & 1][i].x, b[u & 1][j].x, zc[i][j]);
+              zc[i][j] = fmaf(a[u & 1][i].y, b[u & 1][j].y, zc[i][j]);
+              zc[i][j] = fmaf(a[u & 1][i].z, b[u & 1][j].z, zc[i][j]);
+              zc[i][j] = fmaf(a[u & 1][i].w, b[u & 1][j].w, zc[i][j]);
             }
         }
 #pragma unroll
@@ -259,30 +271,35 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
         for (int i = 0; i < 4; ++i) {
           const float f = rf[om * 4 + i];
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
+          for (int j = 0; j < NJ; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[i][j][e] *= f;
         }
       }
-      // Column groups of the slice's width only (uniform over a warp but for
-      // the last group).
+      const float *gp = Gs + om * 4, *bp = Bt + oc * 4;
+      float4 gv = *reinterpret_cast<const float4 *>(gp), b[NJ];
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) b[j] = *reinterpret_cast<const float4 *>(bp + 64 * j);
 #pragma unroll 4
       for (int n = 0; n < kBN; ++n) {
-        const float4 gv = *reinterpret_cast<const float4 *>(Gs + n * kGPitch + om * 4);
         const float gi[4] = {gv.x, gv.y, gv.z, gv.w};
+        float4 c[NJ];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (64 * j + oc * 4 < dn) {
-            const float4 b = *reinterpret_cast<const float4 *>(Bt + n * pitch + oc * 4 + 64 * j);
+        for (int j = 0; j < NJ; ++j) c[j] = b[j];
+        const int nn = n + 1 < kBN ? n + 1 : n;  // the next row, while this one is multiplied
+        gv = *reinterpret_cast<const float4 *>(gp + nn * kGPitch);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              acc[i][j][0] = fmaf(gi[i], b.x, acc[i][j][0]);
-              acc[i][j][1] = fmaf(gi[i], b.y, acc[i][j][1]);
-              acc[i][j][2] = fmaf(gi[i], b.z, acc[i][j][2]);
-              acc[i][j][3] = fmaf(gi[i], b.w, acc[i][j][3]);
-            }
+        for (int j = 0; j < NJ; ++j)
+          b[j] = *reinterpret_cast<const float4 *>(bp + nn * pitch + 64 * j);
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            acc[i][j][0] = fmaf(gi[i], c[j].x, acc[i][j][0]);
+            acc[i][j][1] = fmaf(gi[i], c[j].y, acc[i][j][1]);
+            acc[i][j][2] = fmaf(gi[i], c[j].z, acc[i][j][2]);
+            acc[i][j][3] = fmaf(gi[i], c[j].w, acc[i][j][3]);
           }
-        }
       }
     }
   }
@@ -296,10 +313,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (64 * j + oc * 4 < dn)
-          *reinterpret_cast<float4 *>(Os + (om * 4 + i) * pitch + oc * 4 + 64 * j) =
-              make_float4(acc[i][j][0], acc[i][j][1], acc[i][j][2], acc[i][j][3]);
+      for (int j = 0; j < NJ; ++j)
+        *reinterpret_cast<float4 *>(Os + (om * 4 + i) * pitch + oc * 4 + 64 * j) =
+            make_float4(acc[i][j][0], acc[i][j][1], acc[i][j][2], acc[i][j][3]);
   }
   cluster.sync();
   const int r0 = si * kBM / S, r1 = (si + 1) * kBM / S;
@@ -382,10 +398,32 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
   cluster.sync();  // the peers' shared memory stays up while it is read
 }
 
-// M, N: row and column counts as far as the host knows them (T for tokens).
+template <int MODE, int NJ>
+pair_status launch_tile_nj(const char *name, const TileArgs &a, int64_t ctas, size_t smem,
+                           cudaStream_t s) {
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(simt_tile_kernel<MODE, NJ>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ctas, 1, 1);
+  cfg.blockDim = dim3(kTileThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = a.C * a.S;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  PAIR_BEGIN(name, s);
+  PAIR_CUDA_TRY(cudaLaunchKernelEx(&cfg, simt_tile_kernel<MODE, NJ>, a));
+  PAIR_LAUNCH_CHECK(s);
+  return PAIR_OK;
+}
+
 template <int MODE>
 pair_status launch_tile(const char *name, const GradArgs &g, const GradWorkspace &w, float *out,
                         cudaStream_t s) {
+  // Row and column counts as far as the host knows them (T for tokens).
   const int64_t M = MODE == kModeDw ? g.V : g.T, N = MODE == kModeDw ? g.T : g.V;
   int C = 1;
   while (tile_slice(g.d, C) > kSliceMax) C *= 2;
@@ -395,26 +433,16 @@ pair_status launch_tile(const char *name, const GradArgs &g, const GradWorkspace
   int S = 1;
   while (S * C < 8 && tiles * C * S < 304 && 2 * S <= ceil_div(N, kBN)) S *= 2;
   const size_t smem = tile_smem(g.d, C);
-  PAIR_CUDA_TRY(cudaFuncSetAttribute(simt_tile_kernel<MODE>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles * C * S), 1, 1);
-  cfg.blockDim = dim3(kTileThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = C * S;
-  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   const TileArgs a{g.d, g.V, C, S, w.counters, w.tok_idx, w.tok_y, w.tok_c,
                    static_cast<const float *>(w.Hc), static_cast<const float *>(g.W),
                    w.lse, w.zy, out};
-  PAIR_BEGIN(name, s);
-  PAIR_CUDA_TRY(cudaLaunchKernelEx(&cfg, simt_tile_kernel<MODE>, a));
-  PAIR_LAUNCH_CHECK(s);
-  return PAIR_OK;
+  const int64_t ctas = tiles * C * S;
+  switch (tile_groups(tile_slice(g.d, C))) {
+    case 1: return launch_tile_nj<MODE, 1>(name, a, ctas, smem, s);
+    case 2: return launch_tile_nj<MODE, 2>(name, a, ctas, smem, s);
+    case 3: return launch_tile_nj<MODE, 3>(name, a, ctas, smem, s);
+    default: return launch_tile_nj<MODE, 4>(name, a, ctas, smem, s);
+  }
 }
 
 // ------------------------------------------------ any d (above 2048)
