@@ -46,6 +46,40 @@ __device__ __forceinline__ void lse_unit(int u, int n_pairs, int nsplit, int &pa
   sp = gi * sg + (w - pair * sg);
 }
 
+// Vocabulary splits of a launch over n_pairs pairs of token blocks and ncl
+// clusters (a whole warp calls; every kernel of the launch gets the same
+// answer). Long launches, of eight rounds of units or more, take nsplit: units
+// of unequal length interleave there, and other counts measured the same.
+// Shorter ones take the count whose last round is fullest, by the makespan
+// rounds x (tiles of a split + half a tile for a unit's start and end), of up
+// to 64 splits and up to what the partials' array holds: five pairs in 16
+// splits are 80 units for 76 clusters, two rounds with the second nearly empty
+// (1.2 k tokens, d = 2048, V = 151,936: 733 us, in 15 splits 430 us; d = 2560
+// and 2.8 k tokens: 1376 and 1089 us).
+// The partials of a split are `stride` entries apart, the active tokens
+// rounded up to a block: nsplit strides of Tpad then hold more splits of fewer
+// tokens.
+constexpr int kLseMaxSplit = 64;
+struct LseSplits {
+  int ns;
+  int64_t stride;
+};
+__device__ __forceinline__ LseSplits lse_splits(int n_pairs, int n_vt, int ncl, int nsplit,
+                                                int64_t Tpad, int Teff) {
+  LseSplits o{nsplit < n_vt ? nsplit : n_vt, ((int64_t)Teff + 127) / 128 * 128};
+  if (n_pairs == 0 || (int64_t)n_pairs * nsplit >= 8 * (int64_t)ncl) return o;
+  const int64_t room = nsplit * Tpad / o.stride;
+  const int most = (int)min((int64_t)min(kLseMaxSplit, n_vt), room);
+  unsigned best = 0xffffffffu;
+  for (int ns = 1 + (threadIdx.x & 31); ns <= most; ns += 32) {
+    const unsigned rounds = (n_pairs * ns + ncl - 1) / ncl, tiles = (n_vt + ns - 1) / ns;
+    best = min(best, rounds * (2 * tiles + 1) * (2 * kLseMaxSplit) + ns);
+  }
+  for (int k = 16; k > 0; k >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, k));
+  o.ns = (int)(best % (2 * kLseMaxSplit));
+  return o;
+}
+
 // CTA pairs (2-CTA clusters) work on two token blocks of the same vocabulary
 // split in lockstep, as one M = 256 tile: the even CTA issues every MMA of
 // the pair (cta_group::2), over the 256 token rows of both CTAs' A stages and
@@ -63,7 +97,7 @@ template <bool kImage>
 __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
     lse_kernel(const __grid_constant__ CUtensorMap tmH,
                const __grid_constant__ CUtensorMap tmW, int d, int V,
-               int nsplit, int64_t Tpad, const int32_t *counters,
+               int nsplit_base, int64_t Tpad, const int32_t *counters,
                const int32_t *tok_y, const float *ref, float2 *part, float *zy, int rb0,
                int cap, uint8_t *gimg, int s_blocks, int fix, int32_t *dev_err) {
   // The fix-up launch redoes the pass only if the first one flagged a row
@@ -93,6 +127,9 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
   // lse_unit). (A split-major order, where every pair running at once reads
   // the same split, measured 4 % slower.)
   const int n_pairs = (n_tb + 1) / 2;
+  const LseSplits spl =
+      lse_splits(n_pairs, n_vt, (int)num_clusters_x(), nsplit_base, Tpad, Teff);
+  const int nsplit = spl.ns;
   const int n_units = n_pairs * nsplit;
   const int nk = d / 64;
   const int r = (int)cluster_rank();
@@ -319,7 +356,7 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
       }
       if (!ok) break;
       if (valid) {
-        part[(int64_t)sp * Tpad + p] = make_float2(m2, l);
+        part[sp * spl.stride + p] = make_float2(m2, l);
         if (found) zy[p] = zt;
       }
     }
@@ -350,20 +387,25 @@ constexpr float kImgFixLog2 = 64.f;
 // in counters[2] for the fix-up pass; the fix-up pass (fix = 1) runs only if
 // some row was counted.
 template <bool kImage>
-__global__ void lse_combine_kernel(int nsplit, int64_t Tpad, int32_t *counters,
-                                   const float2 *part, float *lse, float *ref, float *lsum,
-                                   int rb0, int cap, int fix) {
+__global__ void lse_combine_kernel(int V, int ncl, int nsplit_base, int64_t Tpad,
+                                   int32_t *counters, const float2 *part, float *lse, float *ref,
+                                   float *lsum, int rb0, int cap, int fix) {
   if (kImage && fix && counters[2] == 0) return;
   const int Teff = counters[0];
+  const int n_tb = min(max((Teff + 127) / 128 - rb0, 0), cap);
+  const LseSplits spl = lse_splits((n_tb + 1) / 2, (V + kLseBN - 1) / kLseBN, ncl, nsplit_base,
+                                   Tpad, Teff);
+  const int nsplit = spl.ns;
+  const int64_t stride = spl.stride;
   const int64_t hi64 = (int64_t)(rb0 + (int64_t)cap) * 128;
   const int p1 = (int)(hi64 < Teff ? hi64 : Teff);
   for (int p = rb0 * 128 + blockIdx.x * blockDim.x + threadIdx.x; p < p1;
        p += gridDim.x * blockDim.x) {
     float M = -INFINITY;
-    for (int s = 0; s < nsplit; ++s) M = fmaxf(M, part[(int64_t)s * Tpad + p].x);
+    for (int s = 0; s < nsplit; ++s) M = fmaxf(M, part[s * stride + p].x);
     float L = 0.f;
     if (kImage) {
-      for (int s = 0; s < nsplit; ++s) L += part[(int64_t)s * Tpad + p].y;
+      for (int s = 0; s < nsplit; ++s) L += part[s * stride + p].y;
       const float R = ref[p];
       if (!fix && M - R > kImgFixLog2) {
         ref[p] = M;
@@ -374,7 +416,7 @@ __global__ void lse_combine_kernel(int nsplit, int64_t Tpad, int32_t *counters,
       }
     } else {
       for (int s = 0; s < nsplit; ++s) {
-        const float2 q = part[(int64_t)s * Tpad + p];
+        const float2 q = part[s * stride + p];
         if (q.y > 0.f) L += q.y * exp2f(q.x - M);
       }
       lse[p] = (M + log2f(L)) * 0.6931471805599453f;
@@ -449,8 +491,9 @@ pair_status launch_lse(const GradArgs &g, const GradWorkspace &w, cudaStream_t s
         cap, nullptr, 0, 0, g.dev_err);
     PAIR_LAUNCH_CHECK(s);
     PAIR_BEGIN("lse_combine", s);
-    lse_combine_kernel<false><<<nsm * 4, 256, 0, s>>>(w.nsplit, w.Tpad, w.counters, w.part,
-                                                      w.lse, nullptr, nullptr, rb0, cap, 0);
+    lse_combine_kernel<false><<<nsm * 4, 256, 0, s>>>(g.V, grid / kLsePair, w.nsplit, w.Tpad,
+                                                      w.counters, w.part, w.lse, nullptr,
+                                                      nullptr, rb0, cap, 0);
     PAIR_LAUNCH_CHECK(s);
     return PAIR_OK;
   }
@@ -463,8 +506,9 @@ pair_status launch_lse(const GradArgs &g, const GradWorkspace &w, cudaStream_t s
         cap, gimg, s_blocks, fix, g.dev_err);
     PAIR_LAUNCH_CHECK(s);
     PAIR_BEGIN("lse_combine", s);
-    lse_combine_kernel<true><<<nsm * 4, 256, 0, s>>>(w.nsplit, w.Tpad, w.counters, w.part,
-                                                     w.lse, w.ref, w.lsum, rb0, cap, fix);
+    lse_combine_kernel<true><<<nsm * 4, 256, 0, s>>>(g.V, grid / kLsePair, w.nsplit, w.Tpad,
+                                                     w.counters, w.part, w.lse, w.ref, w.lsum,
+                                                     rb0, cap, fix);
     PAIR_LAUNCH_CHECK(s);
   }
   return PAIR_OK;
