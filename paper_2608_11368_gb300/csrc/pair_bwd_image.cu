@@ -87,23 +87,41 @@ constexpr uint32_t kIdescDh = idesc_bf16(256, 256, 0, 1);
 
 // Work list of the persistent backward GEMMs (dh_gemm_kernel,
 // dw_gemm_kernel): the units that fill whole rounds of the grid (ncl
-// clusters) run over all of their K extent; the R < ncl units left for the
-// last round are cut into S parts of K each (R S <= ncl, at most `cap`
-// partial tiles of scratch), so that round takes a part's time instead of a
-// unit's. Work item i < full_end is unit i; item full_end + j is part j % S
-// of unit full_end + j / S, over K steps [part nks / S, (part + 1) nks / S);
-// its fp32 tile goes to scratch slot j and the kernel's tail-combine pass
-// adds the S parts in order (deterministic).
+// clusters) run over all of their K extent; the R < ncl units left over are
+// cut into S parts of K each, which run in as many rounds as they need. Work
+// item i < full_end is unit i; item full_end + j is part j / R of unit
+// full_end + j % R, over K steps [part nks / S, (part + 1) nks / S): the units
+// that read the same rows of the K-indexed operand in a part run next to each
+// other and share them in L2. The item's fp32 tile goes to scratch slot j and
+// the kernel's tail-combine pass adds the S parts in order (deterministic).
+//
+// S is the count of the smallest makespan, rounds x (steps of a part +
+// overhead) + the combine pass's share per tile, of up to 64 and up to the
+// scratch's `cap` tiles; S = 1 needs none. One round of S = ncl / R parts
+// leaves up to half of the clusters idle: 55 units on 76 clusters in one part
+// each take 2374 steps of 64 vocabulary rows, in four 3 x 594 (d = 2560, 11
+// token pairs: 1321 and 1093 us). (Equal contiguous ranges of all R nks steps, one
+// per cluster, leave none idle but read each W row at R different times:
+// 1.35 times as slow as whole parts, from DRAM.)
 struct TailSplit {
   int full_end, R, S;
 };
-__host__ __device__ __forceinline__ TailSplit tail_split(int n_units, int ncl, int cap, int nks) {
-  const int rem = n_units % ncl;
-  int S = rem ? ncl / rem : 1;
-  if (rem && S * rem > cap) S = cap / rem;
-  if (S > nks) S = nks;
-  if (S < 2) return TailSplit{n_units, 0, 1};
-  return TailSplit{n_units - rem, rem, S};
+constexpr int kTailMaxParts = 64;
+// A whole warp calls (every lane gets the answer).
+__device__ __forceinline__ TailSplit tail_split(int n_units, int ncl, int cap, int nks,
+                                                int overhead) {
+  const int R = n_units % ncl;
+  if (R == 0 || nks == 0) return TailSplit{n_units, 0, 1};
+  unsigned long long best = ~0ull;
+  for (int S = 1 + (threadIdx.x & 31); S <= min(kTailMaxParts, nks); S += 32) {
+    if (S > 1 && R * S > cap) break;
+    const long long rounds = (R * S + ncl - 1) / ncl, steps = (nks + S - 1) / S;
+    const long long cost = 8 * rounds * (steps + overhead) + (S > 1 ? 2 * R * S : 0);
+    best = min(best, (unsigned long long)cost * (2 * kTailMaxParts) + S);
+  }
+  for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
+  const int S = (int)(best % (2 * kTailMaxParts));
+  return S < 2 ? TailSplit{n_units, 0, 1} : TailSplit{n_units - R, R, S};
 }
 // Work item i of a TailSplit -> unit u, its K steps [k0, k1) and scratch
 // slot (-1: a whole unit).
@@ -112,13 +130,28 @@ __device__ __forceinline__ void tail_item(const TailSplit &tl, int nks, int i, i
   if (i < tl.full_end) {
     u = i; k0 = 0; k1 = nks; slot = -1;
   } else {
-    const int j = i - tl.full_end, part = j % tl.S;
-    u = tl.full_end + j / tl.S;
+    const int j = i - tl.full_end, part = j / tl.R;
+    u = tl.full_end + (j - part * tl.R);
     k0 = (int)((int64_t)part * nks / tl.S);
     k1 = (int)((int64_t)(part + 1) * nks / tl.S);
     slot = j;
   }
 }
+// Sum of unit full_end + v's parts at float4 `at` of their tiles (`tile`
+// float4 each), in part order.
+__device__ __forceinline__ float4 tail_sum(const TailSplit &tl, int v, const float4 *src,
+                                           int64_t tile, int64_t at) {
+  float4 acc = src[v * tile + at];
+  for (int p = 1; p < tl.S; ++p) {
+    const float4 x = src[((int64_t)p * tl.R + v) * tile + at];
+    acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
+  }
+  return acc;
+}
+// An item's start and drain in K steps: a step of dh is 64 vocabulary rows,
+// about 0.6 us, of dw 32 tokens, half of that; filling the pipeline and
+// writing a 2 x 128 x 512 tile take about twelve microseconds.
+constexpr int kDhOverhead = 20, kDwOverhead = 40;
 
 // Pacing of dh_gemm_kernel's whole units: the CTA pairs of a round read the
 // same W rows (all of them read all of W, in step order) and four at a time
@@ -177,7 +210,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int nks = 2 * n_vt;  // 64-wide vocabulary steps (image atoms)
   const int nq = d / kDhN;
   const int n_units = (nrb + 1) / 2 * nq;
-  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks);
+  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDhOverhead);
   const int n_items = tl.full_end + tl.R * tl.S;
 
   if (threadIdx.x == 0) {
@@ -357,7 +390,7 @@ __global__ void __launch_bounds__(256)
   if (nrb == 0) return;
   const int nks = 2 * ((V + 127) / 128);
   const int nq = d / kDhN;
-  const TailSplit tl = tail_split((nrb + 1) / 2 * nq, ncl, scratch_cap, nks);
+  const TailSplit tl = tail_split((nrb + 1) / 2 * nq, ncl, scratch_cap, nks, kDhOverhead);
   constexpr int kQ = kDhN / 4;  // float4 per tile row
   const int64_t n4 = (int64_t)tl.R * 2 * 128 * kQ;
   const float4 *src = reinterpret_cast<const float4 *>(scratch);
@@ -371,11 +404,7 @@ __global__ void __launch_bounds__(256)
     const int tp = u / nq, q = u - tp * nq;
     const int t = (rb0 + 2 * tp + r) * 128 + row;
     if (2 * tp + r >= nrb || t >= Teff) continue;
-    float4 acc = src[(((int64_t)uj * tl.S * 2 + r) * 128 + row) * kQ + c4];
-    for (int p = 1; p < tl.S; ++p) {
-      const float4 v = src[((((int64_t)uj * tl.S + p) * 2 + r) * 128 + row) * kQ + c4];
-      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-    }
+    const float4 acc = tail_sum(tl, uj, src, 256 * kQ, (int64_t)(r * 128 + row) * kQ + c4);
     const float sc = row_scale(tok_c, lsum, t);
     reinterpret_cast<float4 *>(dH + (int64_t)tok_idx[t] * d + q * kDhN)[c4] =
         make_float4(sc * acc.x, sc * acc.y, sc * acc.z, sc * acc.w);
@@ -439,7 +468,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int nq = d / kDwN;
   const int n_units = (n_vb + 1) / 2 * nq;
   const int nks = nrb * (128 / kDwKS);
-  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks);
+  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDwOverhead);
   const int n_items = tl.full_end + tl.R * tl.S;
 
   if (threadIdx.x == 0) {
@@ -622,7 +651,8 @@ __global__ void __launch_bounds__(256)
   const int nrb = min(max((Teff + 127) / 128 - rb0, 0), cap);
   const int n_vb = (V + 127) / 128;
   const int nq = d / kDwN;
-  const TailSplit tl = tail_split((n_vb + 1) / 2 * nq, ncl, scratch_cap, nrb * (128 / kDwKS));
+  const int nks = nrb * (128 / kDwKS);
+  const TailSplit tl = tail_split((n_vb + 1) / 2 * nq, ncl, scratch_cap, nks, kDwOverhead);
   constexpr int kQ = kDwN / 4;  // float4 per tile row
   const int64_t n4 = (int64_t)tl.R * 2 * 128 * kQ;
   const float4 *src = reinterpret_cast<const float4 *>(scratch);
@@ -636,11 +666,7 @@ __global__ void __launch_bounds__(256)
     const int vp = u / nq, q = u - vp * nq;
     const int v = (2 * vp + r) * 128 + row;
     if (2 * vp + r >= n_vb || v >= V) continue;
-    float4 acc = src[(((int64_t)uj * tl.S * 2 + r) * 128 + row) * kQ + c4];
-    for (int p = 1; p < tl.S; ++p) {
-      const float4 x = src[((((int64_t)uj * tl.S + p) * 2 + r) * 128 + row) * kQ + c4];
-      acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
-    }
+    float4 acc = tail_sum(tl, uj, src, 256 * kQ, (int64_t)(r * 128 + row) * kQ + c4);
     float4 *dst = reinterpret_cast<float4 *>(dW + (int64_t)v * d + q * kDwN) + c4;
     if (accumulate) {
       const float4 o = *dst;
@@ -681,38 +707,42 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
       g.d, rb0, cap, w.counters, w.tok_c, w.lsum, static_cast<const __nv_bfloat16 *>(w.Hc),
       static_cast<__nv_bfloat16 *>(w.hs));
   PAIR_LAUNCH_CHECK(s);
-  // Scratch for the split last round of dH: the cluster path's tail rows
-  // (unused by this path), in 2 x 128 x kDhN fp32 tiles.
+  // Scratch for the split last rounds, in 2 x 128 x 512 fp32 tiles: the
+  // cluster path's ring and, behind it, its tail rows (neither used by this
+  // path); for the first chunk's dH also dW, which nothing has written yet,
+  // where that is larger (at d = 512 the two hold 48 tiles, dW 593 at V =
+  // 151,936).
+  constexpr size_t kTile = 2 * 128 * kDhN * sizeof(float);
+  const size_t ring = (size_t)kMaxClusters * kRingBytesPerCluster;
+  const size_t tail = w.tailbuf ? (size_t)kMaxClusters * 2 * 128 * g.d * sizeof(float) : 0;
+  float *dw_scratch = static_cast<float *>(w.gring);
+  const int dw_scratch_cap = (int)((ring + tail) / kTile);
+  const size_t out = (size_t)g.V * g.d * sizeof(float) / kTile;
+  const bool use_out = c == 0 && out > (size_t)dw_scratch_cap;
+  float *dh_scratch = use_out ? g.dW : dw_scratch;
+  const int scratch_cap = use_out ? (int)(out < 1024 ? out : 1024) : dw_scratch_cap;
   const int dh_grid = pair_grid((const void *)dh_gemm_kernel, dh_smem, &dh_cache);
-  const int scratch_cap =
-      w.tailbuf ? (int)((int64_t)kMaxClusters * 2 * 128 * g.d / (2 * 128 * kDhN)) : 0;
   PAIR_BEGIN("dh_gemm_tc", s);
   dh_gemm_kernel<<<dh_grid, kThreads, dh_smem, s>>>(mGA, mW3, g.d, g.V, rb0, cap, w.counters,
-                                                    w.tok_idx, w.tok_c, w.lsum, g.dH, w.tailbuf,
+                                                    w.tok_idx, w.tok_c, w.lsum, g.dH, dh_scratch,
                                                     scratch_cap, w.prog, g.dev_err);
   PAIR_LAUNCH_CHECK(s);
-  if (scratch_cap > 0) {
-    PAIR_BEGIN("dh_tail", s);
-    dh_tail_combine_kernel<<<num_sms() * 2, 256, 0, s>>>(g.d, g.V, rb0, cap, dh_grid / 2,
-                                                         scratch_cap, w.counters, w.tok_idx,
-                                                         w.tok_c, w.lsum, w.tailbuf, g.dH);
-    PAIR_LAUNCH_CHECK(s);
-  }
+  PAIR_BEGIN("dh_tail", s);
+  dh_tail_combine_kernel<<<num_sms() * 2, 256, 0, s>>>(g.d, g.V, rb0, cap, dh_grid / 2,
+                                                       scratch_cap, w.counters, w.tok_idx,
+                                                       w.tok_c, w.lsum, dh_scratch, g.dH);
+  PAIR_LAUNCH_CHECK(s);
   const int dw_grid = pair_grid((const void *)dw_gemm_kernel, dw_smem, &dw_cache);
-  const int dw_scratch_cap =
-      w.tailbuf ? (int)((int64_t)kMaxClusters * 2 * 128 * g.d / (2 * 128 * kDwN)) : 0;
   PAIR_BEGIN("dw_gemm_tc", s);
   dw_gemm_kernel<<<dw_grid, kThreads, dw_smem, s>>>(mG, mH3, g.d, g.V, rb0, cap, c > 0 ? 1 : 0,
-                                                    w.counters, g.dW, w.tailbuf, dw_scratch_cap,
+                                                    w.counters, g.dW, dw_scratch, dw_scratch_cap,
                                                     g.dev_err);
   PAIR_LAUNCH_CHECK(s);
-  if (dw_scratch_cap > 0) {
-    PAIR_BEGIN("dw_tail", s);
-    dw_tail_combine_kernel<<<num_sms() * 2, 256, 0, s>>>(g.d, g.V, rb0, cap, c > 0 ? 1 : 0,
-                                                         dw_grid / 2, dw_scratch_cap, w.counters,
-                                                         w.tailbuf, g.dW);
-    PAIR_LAUNCH_CHECK(s);
-  }
+  PAIR_BEGIN("dw_tail", s);
+  dw_tail_combine_kernel<<<num_sms() * 2, 256, 0, s>>>(g.d, g.V, rb0, cap, c > 0 ? 1 : 0,
+                                                       dw_grid / 2, dw_scratch_cap, w.counters,
+                                                       dw_scratch, g.dW);
+  PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
 }
 
