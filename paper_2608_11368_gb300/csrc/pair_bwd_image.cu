@@ -428,11 +428,22 @@ __global__ void __launch_bounds__(256)
 // own 128 vocabulary rows) and each 256-column half's four Hs column atoms,
 // two in each CTA. Work unit = (vocabulary block pair, 512-column chunk of
 // d); CTA r accumulates dW[block 2 p + r, chunk] (128 x 512 fp32 = all of
-// TMEM) over the chunk's tokens, 32 token rows per stage, and drains it with
-// plain stores (first chunk) or read-add-writes (later chunks; this CTA owns
-// those rows). An odd last block is computed twice (the pair's other CTA
-// repeats the last block) so both CTAs run the same stage sequence; only one
-// stores it.
+// TMEM) over the chunk's tokens, 32 token rows per stage. An odd last block is
+// computed twice (the pair's other CTA repeats the last block) so both CTAs run
+// the same stage sequence; only one stores it.
+//
+// The accumulator takes all of TMEM, so the next unit's MMAs wait for the
+// drain, which counts on short token batches: a unit's MMAs take 9.6 us per
+// 1000 tokens. Each warp drains its lane quadrant through two shared-memory
+// buffers, 32 rows x 32 columns at a time, written by one tensor-map store
+// (first chunk; later chunks read, add and write their own rows): 5.8 us of a
+// unit, the fabric's time for the 40 MB that all CTAs write at once, where
+// 16-byte stores to 32 rows at a time took 11. The pass takes 547 us at 1280
+// tokens of the 152k vocabulary, d = 2048 (725), 374 at 640 (570). Eight
+// draining warps measured the same. Units of 256 columns with two accumulators,
+// whose drain overlaps the next unit's MMAs, measured slower at every length
+// (625 us at 1280 tokens, 4.7 ms against 3.5 at 10,240): each P^T row is
+// fetched by twice as many units, 60 instead of 45 bytes per clock and SM.
 constexpr int kDwKS = 32;                                 // token rows per stage
 constexpr int kDwStages = 5;
 constexpr int kDwN = 512;                                 // output columns per CTA
@@ -443,6 +454,7 @@ constexpr uint32_t kIdescDw = idesc_bf16(256, 256, 1, 1); // both operands MN-ma
 struct DwSmem {
   uint8_t g[kDwStages][kDwGBytes];  // P^T: MN-major A, atoms 4 KB apart
   uint8_t h[kDwStages][kDwHBytes];  // Hs[t, chunk]: MN-major B, atoms 4 KB apart
+  uint8_t stg[4][2][32 * 128];  // drain, per epilogue warp: 32 rows x 32 fp32, SWIZZLE_128B
   uint64_t full[kDwStages], empty[kDwStages];
   uint64_t acc_full, acc_empty, mma_done;
   uint32_t tmem_base;
@@ -451,7 +463,8 @@ struct DwSmem {
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     dw_gemm_kernel(const __grid_constant__ CUtensorMap tmG,
-                   const __grid_constant__ CUtensorMap tmH, int d, int V, int rb0, int cap,
+                   const __grid_constant__ CUtensorMap tmH,
+                   const __grid_constant__ CUtensorMap tmD, int d, int V, int rb0, int cap,
                    int accumulate, const int32_t *counters, float *dW, float *scratch,
                    int scratch_cap, int32_t *dev_err) {
   const int Teff = counters[0];
@@ -483,6 +496,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     fence_mbar_init();
     prefetch_tmap(&tmG);
     prefetch_tmap(&tmH);
+    prefetch_tmap(&tmD);
   }
   if (warp == 1) {
     tmem_alloc_pair(&sm.tmem_base, 512);
@@ -586,14 +600,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const int row = quad * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
     uint32_t acc_ph = 0;
+    int sbuf = 0;
     bool ok = true;
     for (int i = pid; i < n_items && ok; i += npairs) {
       int u, k0, k1, slot;
       tail_item(tl, nks, i, u, k0, k1, slot);
       const int vp = u / nq, q = u - vp * nq;
-      const int v = (2 * vp + r) * 128 + row;
-      const bool valid = 2 * vp + r < n_vb && v < V;
-      float4 *dst = valid ? reinterpret_cast<float4 *>(dW + (int64_t)v * d + q * kDwN) : nullptr;
+      const int v_warp = (2 * vp + r) * 128 + quad * 32;  // the warp's first row
+      const bool mine = 2 * vp + r < n_vb && v_warp < V;  // uniform over the warp
+      const bool valid = mine && v_warp + lane < V;
+      float4 *dst =
+          valid ? reinterpret_cast<float4 *>(dW + (int64_t)(v_warp + lane) * d + q * kDwN) : nullptr;
       float4 *part_dst =
           slot >= 0
               ? reinterpret_cast<float4 *>(scratch + (((int64_t)slot * 2 + r) * 128 + row) * kDwN)
@@ -614,14 +631,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int e = 0; e < 8; ++e)
             part_dst[c * 8 + e] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+        } else if (!accumulate) {
+          if (!mine) continue;
+          // The store that last read this buffer is done; rows past V are
+          // not stored.
+          if (lane == 0) bulk_wait_group_read<1>();
+          __syncwarp();
+          uint8_t *buf = sm.stg[quad][sbuf];
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            *reinterpret_cast<float4 *>(buf + lane * 128 + ((e ^ (lane & 7)) << 4)) =
+                make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            tma_store_2d(&tmD, buf, q * kDwN + c * 32, v_warp);
+            bulk_commit_group();
+          }
+          sbuf ^= 1;
         } else if (valid) {
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             float4 o = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
-            if (accumulate) {
-              const float4 p = dst[c * 8 + e];
-              o.x += p.x; o.y += p.y; o.z += p.z; o.w += p.w;
-            }
+            const float4 p = dst[c * 8 + e];
+            o.x += p.x; o.y += p.y; o.z += p.z; o.w += p.w;
             dst[c * 8 + e] = o;
           }
         }
@@ -629,6 +662,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       tc_fence_before();
       mbar_arrive_cluster(mapa(smem_u32(&sm.acc_empty), 0));
     }
+    // Every store has completed before the CTA leaves.
+    if (lane == 0) bulk_wait_group<0>();
+    __syncwarp();
   }
 
   tc_fence_before();
@@ -685,7 +721,7 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
   const int cap = w.gimg_rb;
   const int rb0 = (int)(c * cap);
   const int n_vt = (g.V + 127) / 128;
-  CUtensorMap mG, mGA, mH3, mW3;
+  CUtensorMap mG, mGA, mH3, mW3, mD;
   if (!make_map3(&mG, w.gimg, {64, 128, (cuuint64_t)2 * cap * n_vt}, {128, 16384}, {64, 32, 2},
                  CU_TENSOR_MAP_SWIZZLE_NONE) ||
       !make_map3(&mGA, w.gimg, {64, 128, (cuuint64_t)2 * cap * n_vt}, {128, 16384}, {64, 128, 1},
@@ -694,7 +730,8 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
                  {(cuuint64_t)g.d * 2, 128}, {64, (cuuint32_t)kDwKS, 2},
                  CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_map3(&mW3, g.W, {64, (cuuint64_t)g.V, (cuuint64_t)g.d / 64},
-                 {(cuuint64_t)g.d * 2, 128}, {64, 64, 2}, CU_TENSOR_MAP_SWIZZLE_128B))
+                 {(cuuint64_t)g.d * 2, 128}, {64, 64, 2}, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_map_f32(&mD, g.dW, g.V, g.d))
     return PAIR_ERR_CUDA;
   const size_t dh_smem = sizeof(DhSmem) + 1024, dw_smem = sizeof(DwSmem) + 1024;
   PAIR_CUDA_TRY(cudaFuncSetAttribute(dh_gemm_kernel,
@@ -734,9 +771,9 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
   PAIR_LAUNCH_CHECK(s);
   const int dw_grid = pair_grid((const void *)dw_gemm_kernel, dw_smem, &dw_cache);
   PAIR_BEGIN("dw_gemm_tc", s);
-  dw_gemm_kernel<<<dw_grid, kThreads, dw_smem, s>>>(mG, mH3, g.d, g.V, rb0, cap, c > 0 ? 1 : 0,
-                                                    w.counters, g.dW, dw_scratch, dw_scratch_cap,
-                                                    g.dev_err);
+  dw_gemm_kernel<<<dw_grid, kThreads, dw_smem, s>>>(mG, mH3, mD, g.d, g.V, rb0, cap,
+                                                    c > 0 ? 1 : 0, w.counters, g.dW, dw_scratch,
+                                                    dw_scratch_cap, g.dev_err);
   PAIR_LAUNCH_CHECK(s);
   PAIR_BEGIN("dw_tail", s);
   dw_tail_combine_kernel<<<num_sms() * 2, 256, 0, s>>>(g.d, g.V, rb0, cap, c > 0 ? 1 : 0,

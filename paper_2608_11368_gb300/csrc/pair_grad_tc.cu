@@ -49,6 +49,20 @@ bool make_map(CUtensorMap *m, const void *ptr, int64_t rows, int64_t cols,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 2-D fp32 row-major [rows][cols] map with 32 x 32 SWIZZLE_128B boxes.
+bool make_map_f32(CUtensorMap *m, const void *ptr, int64_t rows, int64_t cols) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
+  cuuint32_t box[2] = {32, 32};
+  cuuint32_t estr[2] = {1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(ptr), dims, strides, box,
+            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+         CUDA_SUCCESS;
+}
+
 // 3-D bf16 map: dims (innermost first) with byte strides of dims 1 and 2,
 // box `box`, swizzle `sw`.
 bool make_map3(CUtensorMap *m, const void *ptr, const cuuint64_t (&dims)[3],

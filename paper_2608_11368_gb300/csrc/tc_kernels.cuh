@@ -89,6 +89,8 @@ __device__ __forceinline__ void fence_proxy_async_global() {
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn();
 // 2-D bf16 row-major [rows][cols] map with 64 x box_rows SWIZZLE_128B boxes.
 bool make_map(CUtensorMap *m, const void *ptr, int64_t rows, int64_t cols, int box_rows);
+// 2-D fp32 row-major [rows][cols] map with 32 x 32 SWIZZLE_128B boxes (stores).
+bool make_map_f32(CUtensorMap *m, const void *ptr, int64_t rows, int64_t cols);
 // 3-D bf16 map: dims (innermost first), byte strides of dims 1 and 2, box, swizzle.
 bool make_map3(CUtensorMap *m, const void *ptr, const cuuint64_t (&dims)[3],
                const cuuint64_t (&strides)[2], const cuuint32_t (&box)[3],
