@@ -14,6 +14,7 @@ namespace pairk {
 namespace {
 
 constexpr int kNSplit = 16;  // vocabulary splits of the log-sum-exp pass
+constexpr int kTicket = 3;   // counters[]: blocks of finalize_kernel that are done
 
 __device__ __forceinline__ bool coef_nonzero(float a) {
   return (__float_as_uint(a) & 0x7fffffffu) != 0u;
@@ -24,11 +25,14 @@ __device__ __forceinline__ int clamp_i(int v, int lo, int hi) {
 }
 
 // Counts the active tokens of each rollout; validates every mask=1 target.
+// Clears the one-hot part's n_bkt bucket counters and the finalize ticket.
 __global__ void seg_count_kernel(int R, int T, int V, const int32_t *cu,
                                  const uint8_t *mask, const int32_t *y,
-                                 const float *a, int32_t *seg_cnt,
-                                 int32_t *dev_err) {
+                                 const float *a, int32_t *seg_cnt, int32_t *counters,
+                                 int32_t *bkt, int n_bkt, int32_t *dev_err) {
   const int i = blockIdx.x;
+  if (i == 0 && threadIdx.x == 0) counters[kTicket] = 0;
+  for (int k = i * blockDim.x + threadIdx.x; k < n_bkt; k += gridDim.x * blockDim.x) bkt[k] = 0;
   const int beg = clamp_i(cu[i], 0, T), end = clamp_i(cu[i + 1], beg, T);
   const bool on = coef_nonzero(a[i]);
   int n = 0, bad = 0;
@@ -51,7 +55,8 @@ __global__ void seg_count_kernel(int R, int T, int V, const int32_t *cu,
   }
 }
 
-// Exclusive prefix over rollouts (one block, sequential chunks of 1024).
+// Exclusive prefix over rollouts (one block, sequential chunks of 1024), for
+// more than kGatherScanMax of them.
 __global__ void seg_scan_kernel(int R, const int32_t *seg_cnt, int32_t *seg_off,
                                 int32_t *counters) {
   __shared__ int buf[1024];
@@ -80,21 +85,42 @@ __global__ void seg_scan_kernel(int R, const int32_t *seg_cnt, int32_t *seg_off,
   }
 }
 
-// In-order compaction of each active rollout's mask=1 tokens.
-__global__ void gather_kernel(int R, int T, const int32_t *cu,
-                              const uint8_t *mask, const int32_t *y,
-                              const float *a, const int32_t *seg_off,
-                              int32_t *tok_idx, int32_t *tok_y, float *tok_c) {
+// Rollouts up to which gather_kernel's blocks each sum the counts before their
+// own (a few coalesced loads, instead of a launch of its own for the scan).
+constexpr int kGatherScanMax = 2048;
+
+// In-order compaction of each active rollout's mask=1 tokens; with `sum` also
+// the rollout offsets and the total. Targets out of range (reported by
+// seg_count) are taken as 0, so that no later kernel reads past W. Counts the
+// tokens per target bucket in cnt (nullable).
+__global__ void __launch_bounds__(1024)
+    gather_kernel(int R, int T, int V, const int32_t *cu, const uint8_t *mask, const int32_t *y,
+                  const float *a, const int32_t *seg_cnt, bool sum, int32_t *seg_off,
+                  int32_t *counters, int32_t *tok_idx, int32_t *tok_y, float *tok_c,
+                  int32_t *cnt) {
   const int i = blockIdx.x;
-  if (!coef_nonzero(a[i])) return;
-  const int beg = clamp_i(cu[i], 0, T), end = clamp_i(cu[i + 1], beg, T);
-  const float c = a[i];
   __shared__ int wsum[32];
-  __shared__ int carry;
-  if (threadIdx.x == 0) carry = seg_off[i];
-  __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
+  int carry;
+  if (sum) {
+    int n = 0;
+    for (int k = threadIdx.x; k < i; k += blockDim.x) n += seg_cnt[k];
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) wsum[w] = n;
+    __syncthreads();
+    carry = __reduce_add_sync(0xffffffffu, lane < nw ? wsum[lane] : 0);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      seg_off[i] = carry;
+      if (i == R - 1) seg_off[R] = counters[0] = carry + seg_cnt[i];
+    }
+  } else {
+    carry = seg_off[i];
+  }
+  const float c = a[i];
+  if (!coef_nonzero(c)) return;
+  const int beg = clamp_i(cu[i], 0, T), end = clamp_i(cu[i + 1], beg, T);
   for (int base = beg; base < end; base += blockDim.x) {
     const int t = base + threadIdx.x;
     const int f = (t < end && mask[t]) ? 1 : 0;
@@ -102,59 +128,88 @@ __global__ void gather_kernel(int R, int T, const int32_t *cu,
     const int rank_w = __popc(bal & ((1u << lane) - 1u));
     if (lane == 0) wsum[w] = __popc(bal);
     __syncthreads();
-    int before = 0, total = 0;
-    for (int k = 0; k < nw; ++k) {
-      before += (k < w) ? wsum[k] : 0;
-      total += wsum[k];
-    }
+    const int mine = lane < nw ? wsum[lane] : 0;
+    const int before = __reduce_add_sync(0xffffffffu, lane < w ? mine : 0);
+    const int total = __reduce_add_sync(0xffffffffu, mine);
     if (f) {
       const int p = carry + before + rank_w;
+      int yt = y[t];
+      if (yt < 0 || yt >= V) yt = 0;
       tok_idx[p] = t;
-      tok_y[p] = y[t];
+      tok_y[p] = yt;
       tok_c[p] = c;
+      if (cnt) atomicAdd(&cnt[yt / kOneHotBucket], 1);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) carry += total;
+    carry += total;
     __syncthreads();
   }
 }
 
-// Hc[p] = H[tok_idx[p]] for p < T_eff; zero rows up to the next multiple of
-// 128 (the token-tile height), so tail tiles carry finite zeros.
-template <typename Tin>
-__global__ void copy_rows_kernel(int64_t Tpad, int d, const int32_t *counters,
-                                 const int32_t *tok_idx, const Tin *H, Tin *Hc) {
-  const int Teff = counters[0];
-  const int64_t Tz = ((int64_t)Teff + 127) / 128 * 128;
-  const int vec = 16 / (int)sizeof(Tin);
-  const int dv = d / vec;
-  for (int64_t p = blockIdx.x; p < Tz && p < Tpad; p += gridDim.x) {
-    uint4 *dst = reinterpret_cast<uint4 *>(Hc + p * d);
-    if (p < Teff) {
-      const uint4 *src = reinterpret_cast<const uint4 *>(H + (int64_t)tok_idx[p] * d);
-      for (int k = threadIdx.x; k < dv; k += blockDim.x) dst[k] = src[k];
-    } else {
-      for (int k = threadIdx.x; k < dv; k += blockDim.x) dst[k] = make_uint4(0, 0, 0, 0);
-    }
-  }
-}
-
-// Zero the dH rows of tokens outside the objective (mask = 0 or a = 0).
 constexpr int kZeroCuSmem = 8192;  // rollout offsets staged in shared memory, at most
 
-__global__ void zero_inactive_rows_kernel(int64_t T, int d, int R,
-                                          const int32_t *cu,
-                                          const uint8_t *mask, const float *a,
-                                          float *dH) {
-  // The rollout offsets are searched once per row by every thread: from
-  // shared memory when they fit, so the search costs no global round trips.
+// One warp per row, two independent parts:
+// - Hc[p] = H[tok_idx[p]] for p < T_eff, and zero rows up to the next multiple
+//   of 128 (the token-tile height), so tail tiles carry finite zeros. With ref,
+//   the reference of the image path's log-sum-exp pass from the same loads:
+//   ref[p] = <h, W[y]> log2 e, fp32 sums of the products in a fixed order
+//   (lane-strided 8-element pieces, then the warp's butterfly).
+// - the dH rows of tokens outside the objective (mask = 0 or a = 0) are zeroed.
+// As three kernels (copy, zero, reference) this took 8 us more per call at 1.3
+// k tokens and read Hc once more.
+template <typename Tin>
+__global__ void __launch_bounds__(256)
+    rows_kernel(int64_t T, int64_t Tpad, int d, int R, const int32_t *counters,
+                const int32_t *tok_idx, const int32_t *tok_y, const Tin *H, const Tin *W,
+                Tin *Hc, float *ref, const int32_t *cu, const uint8_t *mask, const float *a,
+                float *dH) {
+  // The rollout offsets are searched once per row by every lane: from shared
+  // memory when they fit, so the search costs no global round trips.
   extern __shared__ int32_t cu_s[];
   const bool staged = R + 1 <= kZeroCuSmem;
   if (staged)
     for (int i = threadIdx.x; i <= R; i += blockDim.x) cu_s[i] = cu[i];
   __syncthreads();
   const int32_t *cs = staged ? cu_s : cu;
-  for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+
+  const int Teff = counters[0];
+  const int64_t Tz = min(((int64_t)Teff + 127) / 128 * 128, Tpad);
+  constexpr int kVec = 16 / (int)sizeof(Tin);
+  const int dv = d / kVec;
+  for (int64_t p = w0; p < Tz; p += nw) {
+    uint4 *dst = reinterpret_cast<uint4 *>(Hc + p * d);
+    if (p >= Teff) {
+      for (int k = lane; k < dv; k += 32) dst[k] = make_uint4(0u, 0u, 0u, 0u);
+      continue;
+    }
+    const uint4 *src = reinterpret_cast<const uint4 *>(H + (int64_t)tok_idx[p] * d);
+    if (sizeof(Tin) == 2 && ref) {
+      const uint4 *wr = reinterpret_cast<const uint4 *>(W + (int64_t)tok_y[p] * d);
+      float acc = 0.f;
+#pragma unroll 4
+      for (int k = lane; k < dv; k += 32) {
+        const uint4 hu = src[k], wu = wr[k];
+        dst[k] = hu;
+        const __nv_bfloat162 *hb = reinterpret_cast<const __nv_bfloat162 *>(&hu);
+        const __nv_bfloat162 *wb = reinterpret_cast<const __nv_bfloat162 *>(&wu);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 hf = __bfloat1622float2(hb[i]), wf = __bfloat1622float2(wb[i]);
+          acc = fmaf(hf.x, wf.x, acc);
+          acc = fmaf(hf.y, wf.y, acc);
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) ref[p] = acc * kLog2e;
+    } else {
+#pragma unroll 4
+      for (int k = lane; k < dv; k += 32) dst[k] = src[k];
+    }
+  }
+
+  for (int64_t t = w0; t < T; t += nw) {
     // rollout of t: last i with cu[i] <= t
     int lo = 0, hi = R - 1;
     while (lo < hi) {
@@ -163,46 +218,50 @@ __global__ void zero_inactive_rows_kernel(int64_t T, int d, int R,
     }
     const bool live = mask[t] && coef_nonzero(a[lo]) && cs[lo] <= t && t < cs[lo + 1];
     if (live) continue;
-    float4 *row = reinterpret_cast<float4 *>(dH + t * d);
-    if ((d & 3) == 0) {
-      for (int k = threadIdx.x; k < d / 4; k += blockDim.x)
-        row[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    } else {
-      for (int k = threadIdx.x; k < d; k += blockDim.x) dH[t * d + k] = 0.f;
-    }
+    float4 *row = reinterpret_cast<float4 *>(dH + t * d);  // d is a multiple of 16
+    for (int k = lane; k < d / 4; k += 32) row[k] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 
-// Per-rollout sum of logp_t = zy - lse over the rollout's compacted range
-// (fp64, fixed tree order).
-__global__ void seg_logp_kernel(int R, const int32_t *seg_off, const float *zy,
-                                const float *lse, double *seg_logp) {
-  const int i = blockIdx.x;
-  const int beg = seg_off[i], end = seg_off[i + 1];
+// Sum of logp_t = zy - lse over a rollout's compacted range (fp64, fixed tree
+// order), by a block; the result in thread 0.
+__device__ double seg_logp_sum(int beg, int end, const float *zy, const float *lse) {
   double s = 0.0;
-  for (int p = beg + threadIdx.x; p < end; p += blockDim.x)
-    s += (double)zy[p] - (double)lse[p];
+  for (int p = beg + threadIdx.x; p < end; p += blockDim.x) s += (double)zy[p] - (double)lse[p];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   __shared__ double red[32];
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
+  double t = 0.0;
+  if (threadIdx.x == 0)
     for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[k];
-    seg_logp[i] = t;
-  }
+  return t;
 }
 
-// Jobj = sum_i a_i * logp_seq_i (fp64, fixed order); logp_seq out.
-__global__ void objective_kernel(int R, const float *a, const double *seg_logp,
-                                 double *Jobj, float *logp_seq) {
+// Per-rollout log-probabilities, and by the last block to finish the
+// objective Jobj = sum_i a_i * logp_seq_i (fp64, fixed order); logp_seq out.
+__global__ void __launch_bounds__(256)
+    finalize_kernel(int R, const int32_t *seg_off, const float *zy, const float *lse,
+                    const float *a, double *seg_logp, int32_t *counters, double *Jobj,
+                    float *logp_seq) {
+  const int i = blockIdx.x;
+  const double lp_i = seg_logp_sum(seg_off[i], seg_off[i + 1], zy, lse);
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    seg_logp[i] = lp_i;
+    __threadfence();
+    last = atomicAdd(&counters[kTicket], 1) == R - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
   __shared__ double red[32];
   double s = 0.0;
-  for (int i = threadIdx.x; i < R; i += blockDim.x) {
-    const bool on = coef_nonzero(a[i]);
-    const double lp = on ? seg_logp[i] : 0.0;
-    if (logp_seq) logp_seq[i] = (float)lp;
-    s += on ? (double)a[i] * lp : 0.0;
+  for (int k = threadIdx.x; k < R; k += blockDim.x) {
+    const bool on = coef_nonzero(a[k]);
+    const double lp = on ? __ldcg(seg_logp + k) : 0.0;
+    if (logp_seq) logp_seq[k] = (float)lp;
+    s += on ? (double)a[k] * lp : 0.0;
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -325,45 +384,29 @@ __device__ __forceinline__ void axpy_row(int d, float c, const Tin *__restrict__
   }
 }
 
-__global__ void onehot_count_kernel(const int32_t *counters, const int32_t *tok_y,
-                                    int32_t *cnt) {
-  const int Teff = counters[0];
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < Teff; p += gridDim.x * blockDim.x)
-    atomicAdd(&cnt[tok_y[p] / kOneHotBucket], 1);
-}
-
-// off[b] = sum of cnt[< b] for b <= nb (one block of 1024 threads).
+// off[b] = sum of cnt[< b] for b <= nb (one block of 1024 threads, each over a
+// contiguous run of buckets).
 __global__ void __launch_bounds__(1024) onehot_scan_kernel(int nb, const int32_t *cnt,
                                                            int32_t *off) {
   __shared__ int32_t wsum[32];
-  __shared__ int32_t carry;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) carry = 0;
+  const int per = (nb + 1024) / 1024;  // of nb + 1 offsets
+  const int b0 = threadIdx.x * per, b1 = min(b0 + per, nb + 1);
+  int v = 0;
+#pragma unroll 8
+  for (int b = b0; b < b1; ++b) v += b < nb ? cnt[b] : 0;
+  int x = v;  // inclusive warp scan
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[warp] = x;
   __syncthreads();
-  for (int base = 0; base <= nb; base += 1024) {
-    const int b = base + threadIdx.x;
-    const int v = b < nb ? cnt[b] : 0;
-    int x = v;  // inclusive warp scan
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-      int w = wsum[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w += y;
-      }
-      wsum[lane] = w;
-    }
-    __syncthreads();
-    const int excl = carry + (warp ? wsum[warp - 1] : 0) + x - v;
-    if (b <= nb) off[b] = excl;
-    __syncthreads();
-    if (threadIdx.x == 1023) carry = excl + v;
-    __syncthreads();
+  int run = __reduce_add_sync(0xffffffffu, lane < warp ? wsum[lane] : 0) + x - v;
+#pragma unroll 8
+  for (int b = b0; b < b1; ++b) {
+    off[b] = run;
+    run += b < nb ? cnt[b] : 0;
   }
 }
 
@@ -499,15 +542,22 @@ __global__ void __launch_bounds__(256)
 // and the gradient coefficient c_i = A_i rho_i where the unclipped term is the
 // minimum (A_i > 0: rho_i <= 1 + eps; A_i < 0: rho_i >= 1 - eps), else 0.
 // The ratio is formed in fp64 from the fp64 per-rollout log-probability.
-__global__ void ppo_coef_kernel(int R, const float *a, const double *seg_logp,
-                                const float *logp_old, float eps, float *c, double *L,
-                                float *coef_out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < R; i += gridDim.x * blockDim.x) {
+// One block per rollout: its summed log-probability, its coefficient, and
+// tok_c[p] = c_i for its compacted tokens p.
+__global__ void __launch_bounds__(256)
+    ppo_coef_kernel(int R, const int32_t *seg_off, const float *zy, const float *lse,
+                    const float *a, const float *logp_old, float eps, double *seg_logp, float *c,
+                    double *L, float *coef_out, float *tok_c) {
+  const int i = blockIdx.x;
+  const int beg = seg_off[i], end = seg_off[i + 1];
+  const double lp = seg_logp_sum(beg, end, zy, lse);
+  __shared__ float c_s;
+  if (threadIdx.x == 0) {
     const double A = (double)a[i];
     float ci = 0.f;
     double li = 0.0;
     if (coef_nonzero(a[i])) {
-      const double ratio = exp(seg_logp[i] - (double)logp_old[i]);
+      const double ratio = exp(lp - (double)logp_old[i]);
       const double lo = 1.0 - (double)eps, hi = 1.0 + (double)eps;
       const double clipped = ratio < lo ? lo : (ratio > hi ? hi : ratio);
       const double u = ratio * A, v = clipped * A;
@@ -515,21 +565,18 @@ __global__ void ppo_coef_kernel(int R, const float *a, const double *seg_logp,
       const bool unclipped = A > 0.0 ? ratio <= hi : ratio >= lo;
       ci = unclipped ? (float)(A * ratio) : 0.f;
     }
+    seg_logp[i] = lp;
     c[i] = ci;
     L[i] = li;
     if (coef_out) coef_out[i] = ci;
+    c_s = ci;
   }
-}
-
-// tok_c[p] = c_i for every compacted token p of rollout i.
-__global__ void retarget_c_kernel(int R, const int32_t *seg_off, const float *c, float *tok_c) {
-  const int i = blockIdx.x;
-  const int beg = seg_off[i], end = seg_off[i + 1];
-  const float ci = c[i];
+  __syncthreads();
+  const float ci = c_s;
   for (int p = beg + threadIdx.x; p < end; p += blockDim.x) tok_c[p] = ci;
 }
 
-// Jobj = sum_i L_i (fp64, fixed order); logp_seq out as in objective_kernel.
+// Jobj = sum_i L_i (fp64, fixed order); logp_seq out as in finalize_kernel.
 __global__ void ppo_objective_kernel(int R, const float *a, const double *seg_logp,
                                      const double *L, double *Jobj, float *logp_seq) {
   __shared__ double red[32];
@@ -665,44 +712,51 @@ int grad_gimg_rows_fit(int64_t T, int32_t d, int32_t V, int32_t R, pair_dtype dt
 
 pair_status grad_prepare(const GradArgs &g, const GradWorkspace &w,
                          cudaStream_t s) {
+  // Bucket counters of the one-hot dW part (bf16 path): counts, then the
+  // offsets the scan writes, then the fill counters; cleared with one pass.
+  const int nb = (g.V + kOneHotBucket - 1) / kOneHotBucket;
+  const bool bf16 = g.dt == PAIR_BF16;
   PAIR_BEGIN("seg_count", s);
-  seg_count_kernel<<<g.R, 256, 0, s>>>(g.R, (int)g.T, g.V, g.cu, g.mask, g.y,
-                                       g.a, w.seg_cnt, g.dev_err);
+  seg_count_kernel<<<g.R, 256, 0, s>>>(g.R, (int)g.T, g.V, g.cu, g.mask, g.y, g.a, w.seg_cnt,
+                                       w.counters, w.bkt, bf16 ? 3 * (nb + 1) : 0, g.dev_err);
   PAIR_LAUNCH_CHECK(s);
-  PAIR_BEGIN("seg_scan", s);
-  seg_scan_kernel<<<1, 1024, 0, s>>>(g.R, w.seg_cnt, w.seg_off, w.counters);
-  PAIR_LAUNCH_CHECK(s);
+  const bool sum = g.R <= kGatherScanMax;
+  if (!sum) {
+    PAIR_BEGIN("seg_scan", s);
+    seg_scan_kernel<<<1, 1024, 0, s>>>(g.R, w.seg_cnt, w.seg_off, w.counters);
+    PAIR_LAUNCH_CHECK(s);
+  }
+  // Threads for the mean rollout (a block walks its rollout in steps of them).
+  const int64_t mean = g.T / g.R;
+  const int threads = mean > 512 ? 1024 : mean > 256 ? 512 : 256;
   PAIR_BEGIN("gather", s);
-  gather_kernel<<<g.R, 256, 0, s>>>(g.R, (int)g.T, g.cu, g.mask, g.y, g.a,
-                                    w.seg_off, w.tok_idx, w.tok_y, w.tok_c);
+  gather_kernel<<<g.R, threads, 0, s>>>(g.R, (int)g.T, g.V, g.cu, g.mask, g.y, g.a, w.seg_cnt,
+                                        sum, w.seg_off, w.counters, w.tok_idx, w.tok_y, w.tok_c,
+                                        bf16 ? w.bkt : nullptr);
   PAIR_LAUNCH_CHECK(s);
-  const int rows_grid = 152 * 16;
-  PAIR_BEGIN("copy_rows", s);
-  if (g.dt == PAIR_BF16)
-    copy_rows_kernel<uint16_t><<<rows_grid, 128, 0, s>>>(
-        w.Tpad, g.d, w.counters, w.tok_idx,
-        static_cast<const uint16_t *>(g.H), static_cast<uint16_t *>(w.Hc));
-  else
-    copy_rows_kernel<float><<<rows_grid, 128, 0, s>>>(
-        w.Tpad, g.d, w.counters, w.tok_idx, static_cast<const float *>(g.H),
-        static_cast<float *>(w.Hc));
-  PAIR_LAUNCH_CHECK(s);
-  PAIR_BEGIN("zero_inactive", s);
   const size_t cu_smem = g.R + 1 <= kZeroCuSmem ? (size_t)(g.R + 1) * sizeof(int32_t) : 0;
-  zero_inactive_rows_kernel<<<rows_grid, 128, cu_smem, s>>>(g.T, g.d, g.R, g.cu,
-                                                            g.mask, g.a, g.dH);
+  const int grid = (int)(ceil_div(g.T, 8) < 152 * 8 ? ceil_div(g.T, 8) : 152 * 8);
+  PAIR_BEGIN("rows", s);
+  if (bf16)
+    rows_kernel<__nv_bfloat16><<<grid, 256, cu_smem, s>>>(
+        g.T, w.Tpad, g.d, g.R, w.counters, w.tok_idx, w.tok_y,
+        static_cast<const __nv_bfloat16 *>(g.H), static_cast<const __nv_bfloat16 *>(g.W),
+        static_cast<__nv_bfloat16 *>(w.Hc), w.gimg_rb > 0 ? w.ref : nullptr, g.cu, g.mask, g.a,
+        g.dH);
+  else
+    rows_kernel<float><<<grid, 256, cu_smem, s>>>(
+        g.T, w.Tpad, g.d, g.R, w.counters, w.tok_idx, w.tok_y, static_cast<const float *>(g.H),
+        static_cast<const float *>(g.W), static_cast<float *>(w.Hc), nullptr, g.cu, g.mask, g.a,
+        g.dH);
   PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
 }
 
 pair_status grad_finalize(const GradArgs &g, const GradWorkspace &w,
                           cudaStream_t s) {
-  PAIR_BEGIN("seg_logp", s);
-  seg_logp_kernel<<<g.R, 256, 0, s>>>(g.R, w.seg_off, w.zy, w.lse, w.seg_logp);
-  PAIR_LAUNCH_CHECK(s);
-  PAIR_BEGIN("objective", s);
-  objective_kernel<<<1, 1024, 0, s>>>(g.R, g.a, w.seg_logp, g.Jobj,
-                                      g.logp_seq);
+  PAIR_BEGIN("finalize", s);
+  finalize_kernel<<<g.R, 256, 0, s>>>(g.R, w.seg_off, w.zy, w.lse, g.a, w.seg_logp, w.counters,
+                                      g.Jobj, g.logp_seq);
   PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
 }
@@ -721,15 +775,9 @@ pair_status grad_token_logp(int64_t T, const GradWorkspace &w, float *logp_tok,
 pair_status grad_ppo_coefficients(const GradArgs &g, const GradWorkspace &w,
                                   const float *logp_old, float eps, float *coef_out,
                                   cudaStream_t s) {
-  PAIR_BEGIN("seg_logp", s);
-  seg_logp_kernel<<<g.R, 256, 0, s>>>(g.R, w.seg_off, w.zy, w.lse, w.seg_logp);
-  PAIR_LAUNCH_CHECK(s);
   PAIR_BEGIN("ppo_coef", s);
-  ppo_coef_kernel<<<(int)ceil_div(g.R, 256), 256, 0, s>>>(g.R, g.a, w.seg_logp, logp_old, eps,
-                                                          w.ppo_c, w.ppo_L, coef_out);
-  PAIR_LAUNCH_CHECK(s);
-  PAIR_BEGIN("retarget_c", s);
-  retarget_c_kernel<<<g.R, 256, 0, s>>>(g.R, w.seg_off, w.ppo_c, w.tok_c);
+  ppo_coef_kernel<<<g.R, 256, 0, s>>>(g.R, w.seg_off, w.zy, w.lse, g.a, logp_old, eps,
+                                      w.seg_logp, w.ppo_c, w.ppo_L, coef_out, w.tok_c);
   PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
 }
@@ -745,11 +793,6 @@ pair_status grad_onehot(const GradArgs &g, const GradWorkspace &w,
                         cudaStream_t s) {
   const int nb = (g.V + kOneHotBucket - 1) / kOneHotBucket;
   int32_t *cnt = w.bkt, *off = w.bkt + (nb + 1), *fill = w.bkt + 2 * (nb + 1);
-  PAIR_CUDA_TRY(cudaMemsetAsync(cnt, 0, (size_t)(nb + 1) * sizeof(int32_t), s));
-  PAIR_CUDA_TRY(cudaMemsetAsync(fill, 0, (size_t)(nb + 1) * sizeof(int32_t), s));
-  PAIR_BEGIN("onehot_count", s);
-  onehot_count_kernel<<<152 * 4, 256, 0, s>>>(w.counters, w.tok_y, cnt);
-  PAIR_LAUNCH_CHECK(s);
   PAIR_BEGIN("onehot_scan", s);
   onehot_scan_kernel<<<1, 1024, 0, s>>>(nb, cnt, off);
   PAIR_LAUNCH_CHECK(s);

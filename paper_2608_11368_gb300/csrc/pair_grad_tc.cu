@@ -115,10 +115,7 @@ using namespace tck;
 // token (with an image, relative to each token's reference, and the first
 // chunk's softmax terms are kept for the backward).
 pair_status grad_lse_tc(const GradArgs &g, const GradWorkspace &w, cudaStream_t s) {
-  if (image_path(w)) {
-    const pair_status st = launch_ref(g, w, s);
-    return st != PAIR_OK ? st : launch_lse(g, w, s, 0, kAllBlocks, true, w.gimg_rb);
-  }
+  if (image_path(w)) return launch_lse(g, w, s, 0, kAllBlocks, true, w.gimg_rb);
   return launch_lse(g, w, s, 0, kAllBlocks, false, 0);
 }
 
@@ -160,8 +157,6 @@ pair_status grad_bwd_tc(const GradArgs &g, const GradWorkspace &w, cudaStream_t 
 // HBM), else forward, then the recomputing backward.
 pair_status grad_head_tc(const GradArgs &g, const GradWorkspace &w, cudaStream_t s) {
   if (image_path(w)) {
-    const pair_status st = launch_ref(g, w, s);
-    if (st != PAIR_OK) return st;
     const int64_t nc = image_chunks(g, w);
     for (int64_t c = 0; c < nc; ++c) {
       pair_status st = launch_lse(g, w, s, (int)(c * w.gimg_rb), w.gimg_rb, true, w.gimg_rb);

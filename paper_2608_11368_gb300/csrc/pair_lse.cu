@@ -424,19 +424,6 @@ __global__ void lse_combine_kernel(int V, int ncl, int nsplit_base, int64_t Tpad
   }
 }
 
-// Reference of the image pass: R_p = z_p[y_p] log2 e for every compacted
-// active token p (target_logit_dot).
-__global__ void ref_logit_kernel(int d, const int32_t *counters, const int32_t *tok_y,
-                                 const __nv_bfloat16 *Hc, const __nv_bfloat16 *W, float *ref) {
-  const int Teff = counters[0];
-  const int lane = threadIdx.x & 31;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < Teff; p += nw) {
-    const float z = target_logit_dot(d, Hc + (int64_t)p * d, W + (int64_t)tok_y[p] * d, lane);
-    if (lane == 0) ref[p] = z * kLog2e;
-  }
-}
-
 // CTAs of the LSE grid: every 2-CTA cluster that fits at once (persistent).
 int lse_grid(size_t smem) {
   static int cached = 0;
@@ -458,15 +445,6 @@ int lse_grid(size_t smem) {
 }  // namespace
 
 namespace tck {
-
-pair_status launch_ref(const GradArgs &g, const GradWorkspace &w, cudaStream_t s) {
-  PAIR_BEGIN("ref_logit", s);
-  ref_logit_kernel<<<num_sms() * 8, 256, 0, s>>>(
-      g.d, w.counters, w.tok_y, static_cast<const __nv_bfloat16 *>(w.Hc),
-      static_cast<const __nv_bfloat16 *>(g.W), w.ref);
-  PAIR_LAUNCH_CHECK(s);
-  return PAIR_OK;
-}
 
 // Log-sum-exp pass over token blocks [rb0, rb0 + cap) (clipped to the active
 // ones), then lse for those tokens. With image, the terms are relative to

@@ -100,12 +100,9 @@ int num_sms();
 int pair_grid(const void *kernel, size_t smem, int *cache);
 
 // ---- stages of the head
-// Per-token reference of the image path's log-sum-exp pass: R_t = z_t[y_t]
-// log2 e for every active token (pair_lse.cu).
-pair_status launch_ref(const GradArgs &g, const GradWorkspace &w, cudaStream_t s);
 // Log-sum-exp pass over token blocks [rb0, rb0 + cap), then lse of those
 // tokens. With image, the softmax terms are taken relative to the reference
-// (launch_ref first), the bf16 terms of its first s_blocks blocks are kept as
+// (rows_kernel, pair_grad_prep.cu), the bf16 terms of its first s_blocks blocks are kept as
 // the image, and rows too far above their reference are redone (pair_lse.cu).
 pair_status launch_lse(const GradArgs &g, const GradWorkspace &w, cudaStream_t s, int rb0,
                        int cap, bool image, int s_blocks);
