@@ -125,23 +125,27 @@ def pair_timing_read(max_launches: int = 4096):
     return [(names[i].decode(), float(ms[i])) for i in range(n)]
 
 
+# Device pointers and streams go to the library as plain integers (the
+# functions' argtypes convert them; None is a null pointer). A call on a small
+# batch is over in a few microseconds on the GPU, so the path to it is kept
+# short: coefficients of 8 x 8 groups took 24 us with a context manager for the
+# device, a stream object and a c_void_p per argument, 17 us without.
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return (torch.cuda.current_stream() if stream is None else stream).cuda_stream
 
 
 def _need(t, name, dtype, shape=None):
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError("%s must be a CUDA tensor" % name)
-    if t.dtype != dtype:
+    if t.dtype is not dtype:
         raise TypeError("%s must be %s, got %s" % (name, dtype, t.dtype))
     if not t.is_contiguous():
         raise ValueError("%s must be contiguous" % name)
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError("%s must have shape %s, got %s" % (name, tuple(shape),
                                                             tuple(t.shape)))
 
@@ -155,6 +159,22 @@ def _on_device(t):
     """Context manager making t's device current for the call: the library
     launches on the current device and takes its stream from there."""
     return torch.cuda.device(t.device)
+
+
+def _call(where, t, stream, *args):
+    """Library function `where` with args and the stream, on t's device (made
+    current for the call if it is not): `stream`, or that device's current
+    one. Raises PairError for any status but PAIR_OK."""
+    fn = getattr(_lib or lib(), where)
+    dev = t.get_device()
+    if dev == torch._C._cuda_getDevice():
+        st = fn(*args, torch._C._cuda_getCurrentRawStream(dev) if stream is None
+                else stream.cuda_stream)
+    else:
+        with _on_device(t):
+            st = fn(*args, _stream(stream))
+    if st != PAIR_OK:
+        raise PairError(st, where)
 
 
 def _out(t, name, shape, dtype, dev):
@@ -180,11 +200,8 @@ def pair_coeffs(r, J, rho, scale=1.0, flags=0, a=None, active=None, edges=None,
     active = _out(active, "active", (B, G), torch.uint8, dev)
     edges = _out(edges, "edges", (B,), torch.int32, dev)
     contrast_edges = _out(contrast_edges, "contrast_edges", (B,), torch.int32, dev)
-    with _on_device(r):
-        st = lib().pair_coeffs(B, G, _p(r), _p(J), _p(rho), float(scale), int(flags),
-                               _p(a), _p(active), _p(edges), _p(contrast_edges),
-                               _p(dev_err), _stream(stream))
-    _check(st, "pair_coeffs")
+    _call("pair_coeffs", r, stream, B, G, _p(r), _p(J), _p(rho), float(scale), int(flags),
+          _p(a), _p(active), _p(edges), _p(contrast_edges), _p(dev_err))
     return a, active, edges, contrast_edges
 
 
@@ -211,11 +228,8 @@ def pair_coeffs_weighted(r, J, rho, wmode=PAIR_W_HT, w_max=0.0, scale=1.0, flags
     if rho is not None:
         _need(rho, "rho", torch.float32, (B, G, G))
     outs = _coeffs_outputs(B, G, r.device, a, active, edges, contrast_edges, ess, max_w)
-    with _on_device(r):
-        st = lib().pair_coeffs_weighted(B, G, _p(r), _p(J), _p(rho), float(scale), int(flags),
-                                        int(wmode), float(w_max), *[_p(t) for t in outs],
-                                        _p(dev_err), _stream(stream))
-    _check(st, "pair_coeffs_weighted")
+    _call("pair_coeffs_weighted", r, stream, B, G, _p(r), _p(J), _p(rho), float(scale),
+          int(flags), int(wmode), float(w_max), *[_p(t) for t in outs], _p(dev_err))
     return outs
 
 
@@ -228,10 +242,8 @@ def pair_coeffs_product(r, J, p, scale=1.0, flags=0, a=None, active=None, edges=
     _need(J, "J", torch.uint8, (B, G))
     _need(p, "p", torch.float32, (B, G))
     outs = _coeffs_outputs(B, G, r.device, a, active, edges, contrast_edges, ess, max_w)
-    with _on_device(r):
-        st = lib().pair_coeffs_product(B, G, _p(r), _p(J), _p(p), float(scale), int(flags),
-                                       *[_p(t) for t in outs], _p(dev_err), _stream(stream))
-    _check(st, "pair_coeffs_product")
+    _call("pair_coeffs_product", r, stream, B, G, _p(r), _p(J), _p(p), float(scale), int(flags),
+          *[_p(t) for t in outs], _p(dev_err))
     return outs
 
 
@@ -256,14 +268,12 @@ def pair_audit(r, rho, S, Jdraws, draw_weight=None, wmode=PAIR_W_HT, w_max=0.0, 
     stats = _out(stats, "stats", (8,), torch.float64, dev)
     bias = _out(bias, "bias", (D,), torch.float64, dev)
     need = int(lib().pair_audit_workspace_size(N, G, D))
-    with _on_device(r):
-        if ws is None:
-            ws = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
-        _need(ws, "ws", torch.uint8)
-        st = lib().pair_audit(N, G, D, _p(r), _p(rho), _p(S), _p(Jdraws), _p(draw_weight),
-                              float(scale), int(flags), int(wmode), float(w_max), _p(stats),
-                              _p(bias), _p(ws), ws.numel(), _p(dev_err), _stream(stream))
-    _check(st, "pair_audit")
+    if ws is None:
+        ws = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+    _need(ws, "ws", torch.uint8)
+    _call("pair_audit", r, stream, N, G, D, _p(r), _p(rho), _p(S), _p(Jdraws), _p(draw_weight),
+          float(scale), int(flags), int(wmode), float(w_max), _p(stats), _p(bias), _p(ws),
+          ws.numel(), _p(dev_err))
     return stats, bias
 
 
@@ -292,11 +302,8 @@ def pair_allocate(c_hat, budget, pi_min, p_hat=None, m_hat=None, a=None, pi=None
     stats = _out(stats, "stats", (B, 5), torch.float64, dev)
     if dev_err is None:
         dev_err = torch.zeros(1, dtype=torch.int32, device=dev)
-    with _on_device(c_hat):
-        st = lib().pair_allocate(B, G, _p(p_hat), _p(m_hat), _p(a), _p(c_hat), _p(budget),
-                                 float(pi_min), _p(pi), _p(stats), _p(dev_err),
-                                 _stream(stream))
-    _check(st, "pair_allocate")
+    _call("pair_allocate", c_hat, stream, B, G, _p(p_hat), _p(m_hat), _p(a), _p(c_hat),
+          _p(budget), float(pi_min), _p(pi), _p(stats), _p(dev_err))
     return pi, stats
 
 
@@ -311,11 +318,8 @@ def pair_estimate_dense(r, J, rho, S, scale=1.0, g=None, a=None, dev_err=None,
     g = _out(g, "g", (B, D), torch.float32, S.device)
     if a is not None:
         a = _out(a, "a", (B, G), torch.float32, S.device)
-    with _on_device(S):
-        st = lib().pair_estimate_dense(B, G, D, _p(r), _p(J), _p(rho), _p(S),
-                                       float(scale), _p(g), _p(a), _p(dev_err),
-                                       _stream(stream))
-    _check(st, "pair_estimate_dense")
+    _call("pair_estimate_dense", S, stream, B, G, D, _p(r), _p(J), _p(rho), _p(S), float(scale),
+          _p(g), _p(a), _p(dev_err))
     return g, a
 
 
@@ -368,16 +372,12 @@ def pair_grad(H, W, y, mask, cu_seqlens, a, dH=None, dW=None, Jobj=None,
     T, d, V, R, dt = _grad_inputs(H, W, y, mask, cu_seqlens, a)
     dev = H.device
     dH, dW, Jobj, logp_seq = _grad_outputs(T, d, V, R, dev, dH, dW, Jobj, logp_seq)
-    with _on_device(H):
-        if ws is None:
-            need = pair_grad_workspace_size(T, d, V, R, dt)
-            ws = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
-        _need(ws, "ws", torch.uint8)
-        st = lib().pair_grad(T, d, V, dt, _p(H), _p(W), _p(y), _p(mask),
-                             _p(cu_seqlens), R, _p(a), _p(dH), _p(dW), _p(Jobj),
-                             _p(logp_seq), _p(ws), ws.numel(), _p(dev_err),
-                             _stream(stream))
-    _check(st, "pair_grad")
+    if ws is None:
+        need = pair_grad_workspace_size(T, d, V, R, dt)
+        ws = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+    _need(ws, "ws", torch.uint8)
+    _call("pair_grad", H, stream, T, d, V, dt, _p(H), _p(W), _p(y), _p(mask), _p(cu_seqlens), R,
+          _p(a), _p(dH), _p(dW), _p(Jobj), _p(logp_seq), _p(ws), ws.numel(), _p(dev_err))
     return Jobj, dH, dW, logp_seq
 
 
@@ -387,10 +387,8 @@ def pair_grad_token_logp(T, d, V, R, dtype, ws, logp_tok=None, stream=None):
     tokens, 0 elsewhere."""
     _need(ws, "ws", torch.uint8)
     logp_tok = _out(logp_tok, "logp_tok", (int(T),), torch.float32, ws.device)
-    with _on_device(ws):
-        st = lib().pair_grad_token_logp(int(T), int(d), int(V), int(R), int(dtype), _p(ws),
-                                        ws.numel(), _p(logp_tok), _stream(stream))
-    _check(st, "pair_grad_token_logp")
+    _call("pair_grad_token_logp", ws, stream, int(T), int(d), int(V), int(R), int(dtype), _p(ws),
+          ws.numel(), _p(logp_tok))
     return logp_tok
 
 
@@ -403,16 +401,13 @@ def pair_grad_clipped(H, W, y, mask, cu_seqlens, a, logp_old, clip_eps=0.2, dH=N
     dev = H.device
     dH, dW, Jobj, logp_seq = _grad_outputs(T, d, V, R, dev, dH, dW, Jobj, logp_seq)
     coef = _out(coef, "coef", (R,), torch.float32, dev)
-    with _on_device(H):
-        if ws is None:
-            need = pair_grad_workspace_size(T, d, V, R, dt)
-            ws = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
-        _need(ws, "ws", torch.uint8)
-        st = lib().pair_grad_clipped(T, d, V, dt, _p(H), _p(W), _p(y), _p(mask), _p(cu_seqlens),
-                                     R, _p(a), _p(logp_old), float(clip_eps), _p(dH), _p(dW),
-                                     _p(Jobj), _p(logp_seq), _p(coef), _p(ws), ws.numel(),
-                                     _p(dev_err), _stream(stream))
-    _check(st, "pair_grad_clipped")
+    if ws is None:
+        need = pair_grad_workspace_size(T, d, V, R, dt)
+        ws = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+    _need(ws, "ws", torch.uint8)
+    _call("pair_grad_clipped", H, stream, T, d, V, dt, _p(H), _p(W), _p(y), _p(mask),
+          _p(cu_seqlens), R, _p(a), _p(logp_old), float(clip_eps), _p(dH), _p(dW), _p(Jobj),
+          _p(logp_seq), _p(coef), _p(ws), ws.numel(), _p(dev_err))
     return Jobj, dH, dW, logp_seq, coef
 
 
@@ -429,12 +424,8 @@ def pair_grad_noalloc(H, W, y, mask, cu_seqlens, a, dH=None, dW=None,
     T, d, V, R, dt = _grad_inputs(H, W, y, mask, cu_seqlens, a)
     dev = H.device
     dH, dW, Jobj, logp_seq = _grad_outputs(T, d, V, R, dev, dH, dW, Jobj, logp_seq)
-    with _on_device(H):
-        st = lib().pair_grad_noalloc(T, d, V, dt, _p(H), _p(W), _p(y), _p(mask),
-                                     _p(cu_seqlens), R, _p(a), _p(dH), _p(dW),
-                                     _p(Jobj), _p(logp_seq), _p(dev_err),
-                                     _stream(stream))
-    _check(st, "pair_grad_noalloc")
+    _call("pair_grad_noalloc", H, stream, T, d, V, dt, _p(H), _p(W), _p(y), _p(mask),
+          _p(cu_seqlens), R, _p(a), _p(dH), _p(dW), _p(Jobj), _p(logp_seq), _p(dev_err))
     return Jobj, dH, dW, logp_seq
 
 
