@@ -1314,20 +1314,27 @@ pair_status grad_bwd_recompute(const GradArgs &g, const GradWorkspace &w, cudaSt
       default: return grad_bwd_cluster<64>(g, w, s, mH, mW128);
     }
   }
+  bool slab_dh = false, slab_dw = false;
+  const pair_status st = grad_bwd_slabs(g, w, s, slab_dh, slab_dw);
+  if (st != PAIR_OK) return st;
   const int nsm = num_sms();
   const size_t bwd_smem = sizeof(BwdSmem) + 1024;
   PAIR_CUDA_TRY(cudaFuncSetAttribute(bwd_kernel<true>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem));
   PAIR_CUDA_TRY(cudaFuncSetAttribute(bwd_kernel<false>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem));
-  PAIR_BEGIN("bwd_dh_tc", s);
-  bwd_kernel<true><<<nsm, kThreads, bwd_smem, s>>>(
-      mH, mW128, g.d, g.V, w.counters, w.tok_idx, w.tok_c, w.lse, g.dH, g.dev_err);
-  PAIR_LAUNCH_CHECK(s);
-  PAIR_BEGIN("bwd_dw_tc", s);
-  bwd_kernel<false><<<nsm, kThreads, bwd_smem, s>>>(
-      mW128, mH, g.d, g.V, w.counters, w.tok_idx, w.tok_c, w.lse, g.dW, g.dev_err);
-  PAIR_LAUNCH_CHECK(s);
+  if (!slab_dh) {
+    PAIR_BEGIN("bwd_dh_tc", s);
+    bwd_kernel<true><<<nsm, kThreads, bwd_smem, s>>>(
+        mH, mW128, g.d, g.V, w.counters, w.tok_idx, w.tok_c, w.lse, g.dH, g.dev_err);
+    PAIR_LAUNCH_CHECK(s);
+  }
+  if (!slab_dw) {
+    PAIR_BEGIN("bwd_dw_tc", s);
+    bwd_kernel<false><<<nsm, kThreads, bwd_smem, s>>>(
+        mW128, mH, g.d, g.V, w.counters, w.tok_idx, w.tok_c, w.lse, g.dW, g.dev_err);
+    PAIR_LAUNCH_CHECK(s);
+  }
   return PAIR_OK;
 }
 

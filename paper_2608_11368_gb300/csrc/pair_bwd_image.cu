@@ -7,6 +7,8 @@
 //     dW[v, :] = sum_t P_tv (s_t Hc[t, :])   (dw_gemm on pre-scaled rows)
 // as plain tcgen05 GEMMs (no logit recomputation, no pass over the image
 // between them), one token chunk at a time.
+#include <math.h>
+
 #include "tc_kernels.cuh"
 
 namespace pairk {
@@ -54,8 +56,14 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Row scale of the softmax part of dH: s_t = -c_t / lsum_t.
+// 256-column halves of the 512-column unit q of d columns: the last unit of a
+// hidden size that is no multiple of 512 may have one. (Columns past d are
+// loaded as zeros and not stored.)
+__device__ __forceinline__ int unit_halves(int d, int q) { return d - q * 512 > 256 ? 2 : 1; }
+
+// Row scale of the softmax part of dH: s_t = -c_t / lsum_t (image of terms).
 __device__ __forceinline__ float row_scale(const float *tok_c, const float *lsum, int t) {
+  if (!lsum) return 1.f;  // the image holds the gradient itself
   const float c = tok_c[t];
   return c != 0.f ? -c / lsum[t] : 0.f;
 }
@@ -208,7 +216,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int pid = (int)cluster_id_x(), npairs = (int)num_clusters_x();
   const int n_vt = (V + 127) / 128;
   const int nks = 2 * n_vt;  // 64-wide vocabulary steps (image atoms)
-  const int nq = d / kDhN;
+  const int nq = (d + kDhN - 1) / kDhN;
   const int n_units = (nrb + 1) / 2 * nq;
   const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDhOverhead);
   const int n_items = tl.full_end + tl.R * tl.S;
@@ -252,6 +260,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int tp = u / nq, q = u - tp * nq;
         const int b = min(2 * tp + r, nrb - 1);
         const int atom0 = b * nks;  // the block's first image atom
+        const int hv = unit_halves(d, q);
         const bool whole = pacing && slot < 0;
         if (pacing && !whole && lane == 0) pace_publish(prog, pid, 0x7fffffff);
         for (int ks = k0; ks < k1; ++ks) {
@@ -262,13 +271,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
           if (!(ok = wait_cluster(&sm.empty[stage], ph ^ 1, abort, dev_err))) break;
           if (elect_one()) {
-            if (r == 0) mbar_expect_tx(&sm.full[stage], 2 * (kDhABytes + kDhBBytes));
+            if (r == 0)
+              mbar_expect_tx(&sm.full[stage], 2 * (kDhABytes + hv * (kDhBBytes / 2)));
             const uint32_t fb = mapa(smem_u32(&sm.full[stage]), 0);
             tma_load_3d_pair(sm.a[stage], &tmG, fb, 0, 0, atom0 + ks);
             // Column atoms 2r, 2r + 1 of each 256-column half of the chunk.
             tma_load_3d_pair(sm.b[stage], &tmW, fb, 0, 64 * ks, q * (kDhN / 64) + 2 * r);
-            tma_load_3d_pair(sm.b[stage] + kDhBBytes / 2, &tmW, fb, 0, 64 * ks,
-                             q * (kDhN / 64) + 4 + 2 * r);
+            if (hv == 2)
+              tma_load_3d_pair(sm.b[stage] + kDhBBytes / 2, &tmW, fb, 0, 64 * ks,
+                               q * (kDhN / 64) + 4 + 2 * r);
           }
           __syncwarp();
           last_ph[stage] = (int)ph;
@@ -301,6 +312,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (int i = pid; i < n_items && ok; i += npairs) {
         int u, k0, k1, slot;
         tail_item(tl, nks, i, u, k0, k1, slot);
+        const int hv = unit_halves(d, u % nq);
         if (!(ok = wait_cluster(&sm.acc_empty, acc_ph ^ 1, abort, dev_err))) break;
         acc_ph ^= 1;
         tc_fence_after();
@@ -314,9 +326,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
               for (int nh = 0; nh < 2; ++nh)
-                mma_bf16_pair(tmem + nh * 256, da + 2 * kk,
-                              db + nh * ((kDhBBytes / 2) >> 4) + kk * (2048 >> 4), kIdescDh,
-                              (ks != k0) | (kk != 0));
+                if (nh < hv)
+                  mma_bf16_pair(tmem + nh * 256, da + 2 * kk,
+                                db + nh * ((kDhBBytes / 2) >> 4) + kk * (2048 >> 4), kIdescDh,
+                                (ks != k0) | (kk != 0));
             mma_commit_pair(&sm.empty[stage], (uint16_t)3);
           }
           __syncwarp();
@@ -354,7 +367,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       acc_ph ^= 1;
       tc_fence_after();
 #pragma unroll 1
-      for (int c = 0; c < kDhN / 32; ++c) {
+      for (int c = 0; c < min(kDhN, d - q * kDhN) / 32; ++c) {
         float x[32];
         tmem_ld32(tmem + lane_off + c * 32, x);
         if (dst) {
@@ -389,7 +402,7 @@ __global__ void __launch_bounds__(256)
   const int nrb = min(max((Teff + 127) / 128 - rb0, 0), cap);
   if (nrb == 0) return;
   const int nks = 2 * ((V + 127) / 128);
-  const int nq = d / kDhN;
+  const int nq = (d + kDhN - 1) / kDhN;
   const TailSplit tl = tail_split((nrb + 1) / 2 * nq, ncl, scratch_cap, nks, kDhOverhead);
   constexpr int kQ = kDhN / 4;  // float4 per tile row
   const int64_t n4 = (int64_t)tl.R * 2 * 128 * kQ;
@@ -403,7 +416,7 @@ __global__ void __launch_bounds__(256)
     const int u = tl.full_end + uj;
     const int tp = u / nq, q = u - tp * nq;
     const int t = (rb0 + 2 * tp + r) * 128 + row;
-    if (2 * tp + r >= nrb || t >= Teff) continue;
+    if (2 * tp + r >= nrb || t >= Teff || q * kDhN + 4 * c4 >= d) continue;
     const float4 acc = tail_sum(tl, uj, src, 256 * kQ, (int64_t)(r * 128 + row) * kQ + c4);
     const float sc = row_scale(tok_c, lsum, t);
     reinterpret_cast<float4 *>(dH + (int64_t)tok_idx[t] * d + q * kDhN)[c4] =
@@ -464,9 +477,11 @@ struct DwSmem {
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     dw_gemm_kernel(const __grid_constant__ CUtensorMap tmG,
                    const __grid_constant__ CUtensorMap tmH,
-                   const __grid_constant__ CUtensorMap tmD, int d, int V, int rb0, int cap,
-                   int accumulate, const int32_t *counters, float *dW, float *scratch,
-                   int scratch_cap, int32_t *dev_err) {
+                   const __grid_constant__ CUtensorMap tmD, int d, int V, int vb0, int n_vb,
+                   int rb0, int cap, int row0, int accumulate, const int32_t *counters, float *dW,
+                   float *scratch, int scratch_cap, int32_t *dev_err) {
+  // Vocabulary blocks [vb0, vb0 + n_vb); tokens [128 rb0, 128 (rb0 + cap)),
+  // whose rows of tmH start at row0.
   const int Teff = counters[0];
   const int nrb = min(max((Teff + 127) / 128 - rb0, 0), cap);
   // A chunk past the last token adds nothing (the first chunk always runs:
@@ -477,8 +492,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = (int)cluster_rank();
   const int pid = (int)cluster_id_x(), npairs = (int)num_clusters_x();
-  const int n_vb = (V + 127) / 128;
-  const int nq = d / kDwN;
+  const int nq = (d + kDwN - 1) / kDwN;
   const int n_units = (n_vb + 1) / 2 * nq;
   const int nks = nrb * (128 / kDwKS);
   const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDwOverhead);
@@ -521,18 +535,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tail_item(tl, nks, i, u, k0, k1, slot);
         const int vp = u / nq, q = u - vp * nq;
         const int vb = min(2 * vp + r, n_vb - 1);
+        const int hv = unit_halves(d, q);
         for (int ks = k0; ks < k1; ++ks) {
           const int rbl = ks >> 2, j = ks & 3;
           if (!(ok = wait_cluster(&sm.empty[stage], ph ^ 1, abort, dev_err))) break;
           if (elect_one()) {
-            if (r == 0) mbar_expect_tx(&sm.full[stage], 2 * (kDwGBytes + kDwHBytes));
+            if (r == 0)
+              mbar_expect_tx(&sm.full[stage], 2 * (kDwGBytes + hv * (kDwHBytes / 2)));
             const uint32_t fb = mapa(smem_u32(&sm.full[stage]), 0);
-            const int t0 = rbl * 128 + kDwKS * j;  // chunk row of Hs
+            const int t0 = row0 + rbl * 128 + kDwKS * j;
             tma_load_3d_pair(sm.g[stage], &tmG, fb, 0, kDwKS * j, 2 * (rbl * n_vb + vb));
             // Column atoms 2r, 2r + 1 of each 256-column half of the chunk.
             tma_load_3d_pair(sm.h[stage], &tmH, fb, 0, t0, q * (kDwN / 64) + 2 * r);
-            tma_load_3d_pair(sm.h[stage] + kDwHBytes / 2, &tmH, fb, 0, t0,
-                             q * (kDwN / 64) + 4 + 2 * r);
+            if (hv == 2)
+              tma_load_3d_pair(sm.h[stage] + kDwHBytes / 2, &tmH, fb, 0, t0,
+                               q * (kDwN / 64) + 4 + 2 * r);
           }
           __syncwarp();
           last_ph[stage] = (int)ph;
@@ -565,6 +582,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (int i = pid; i < n_items && ok && nks > 0; i += npairs) {
         int u, k0, k1, slot;
         tail_item(tl, nks, i, u, k0, k1, slot);
+        const int hv = unit_halves(d, u % nq);
         if (!(ok = wait_cluster(&sm.acc_empty, acc_ph ^ 1, abort, dev_err))) break;
         acc_ph ^= 1;
         tc_fence_after();
@@ -578,9 +596,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             for (int kk = 0; kk < kDwKS / 16; ++kk)
 #pragma unroll
               for (int nh = 0; nh < 2; ++nh)
-                mma_bf16_pair(tmem + nh * 256, dg + kk * (2048 >> 4),
-                              dh + nh * ((kDwHBytes / 2) >> 4) + kk * (2048 >> 4), kIdescDw,
-                              (ks != k0) | (kk != 0));
+                if (nh < hv)
+                  mma_bf16_pair(tmem + nh * 256, dg + kk * (2048 >> 4),
+                                dh + nh * ((kDwHBytes / 2) >> 4) + kk * (2048 >> 4), kIdescDw,
+                                (ks != k0) | (kk != 0));
             mma_commit_pair(&sm.empty[stage], (uint16_t)3);
           }
           __syncwarp();
@@ -606,7 +625,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       int u, k0, k1, slot;
       tail_item(tl, nks, i, u, k0, k1, slot);
       const int vp = u / nq, q = u - vp * nq;
-      const int v_warp = (2 * vp + r) * 128 + quad * 32;  // the warp's first row
+      const int v_warp = (vb0 + 2 * vp + r) * 128 + quad * 32;  // the warp's first row
+      const int uc = min(kDwN, d - q * kDwN);                   // the unit's columns
       const bool mine = 2 * vp + r < n_vb && v_warp < V;  // uniform over the warp
       const bool valid = mine && v_warp + lane < V;
       float4 *dst =
@@ -617,14 +637,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               : nullptr;
       if (nks == 0) {
         if (valid)
-          for (int c = 0; c < kDwN / 4; ++c) dst[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int c = 0; c < uc / 4; ++c) dst[c] = make_float4(0.f, 0.f, 0.f, 0.f);
         continue;
       }
       if (!(ok = wait_sleepy_cluster(&sm.acc_full, acc_ph, abort, dev_err))) break;
       acc_ph ^= 1;
       tc_fence_after();
 #pragma unroll 1
-      for (int c = 0; c < kDwN / 32; ++c) {
+      for (int c = 0; c < uc / 32; ++c) {
         float x[32];
         tmem_ld32(tmem + lane_off + c * 32, x);
         if (part_dst) {
@@ -680,13 +700,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 // TailSplit): the sum of their S partial tiles in part order, stored or
 // (later token chunks) added.
 __global__ void __launch_bounds__(256)
-    dw_tail_combine_kernel(int d, int V, int rb0, int cap, int accumulate, int ncl,
+    dw_tail_combine_kernel(int d, int V, int vb0, int n_vb, int rb0, int cap, int accumulate, int ncl,
                            int scratch_cap, const int32_t *counters,
                            const float *__restrict__ scratch, float *dW) {
   const int Teff = counters[0];
   const int nrb = min(max((Teff + 127) / 128 - rb0, 0), cap);
-  const int n_vb = (V + 127) / 128;
-  const int nq = d / kDwN;
+  const int nq = (d + kDwN - 1) / kDwN;
   const int nks = nrb * (128 / kDwKS);
   const TailSplit tl = tail_split((n_vb + 1) / 2 * nq, ncl, scratch_cap, nks, kDwOverhead);
   constexpr int kQ = kDwN / 4;  // float4 per tile row
@@ -700,8 +719,8 @@ __global__ void __launch_bounds__(256)
     const int uj = (int)(e / (kQ * 256));
     const int u = tl.full_end + uj;
     const int vp = u / nq, q = u - vp * nq;
-    const int v = (2 * vp + r) * 128 + row;
-    if (2 * vp + r >= n_vb || v >= V) continue;
+    const int v = (vb0 + 2 * vp + r) * 128 + row;
+    if (2 * vp + r >= n_vb || v >= V || q * kDwN + 4 * c4 >= d) continue;
     float4 acc = tail_sum(tl, uj, src, 256 * kQ, (int64_t)(r * 128 + row) * kQ + c4);
     float4 *dst = reinterpret_cast<float4 *>(dW + (int64_t)v * d + q * kDwN) + c4;
     if (accumulate) {
@@ -771,18 +790,209 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
   PAIR_LAUNCH_CHECK(s);
   const int dw_grid = pair_grid((const void *)dw_gemm_kernel, dw_smem, &dw_cache);
   PAIR_BEGIN("dw_gemm_tc", s);
-  dw_gemm_kernel<<<dw_grid, kThreads, dw_smem, s>>>(mG, mH3, mD, g.d, g.V, rb0, cap,
+  dw_gemm_kernel<<<dw_grid, kThreads, dw_smem, s>>>(mG, mH3, mD, g.d, g.V, 0, n_vt, rb0, cap, 0,
                                                     c > 0 ? 1 : 0, w.counters, g.dW, dw_scratch,
                                                     dw_scratch_cap, g.dev_err);
   PAIR_LAUNCH_CHECK(s);
   PAIR_BEGIN("dw_tail", s);
-  dw_tail_combine_kernel<<<num_sms() * 2, 256, 0, s>>>(g.d, g.V, rb0, cap, c > 0 ? 1 : 0,
+  dw_tail_combine_kernel<<<num_sms() * 2, 256, 0, s>>>(g.d, g.V, 0, n_vt, rb0, cap, c > 0 ? 1 : 0,
                                                        dw_grid / 2, dw_scratch_cap, w.counters,
                                                        dw_scratch, g.dW);
   PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
 }
 
+// ------------------------- backward without an image workspace, by slabs
+//
+// For hidden sizes whose workspace holds no image (d not a multiple of 512, and
+// d > 3072 with the minimum one), the recomputing kernel (bwd_kernel) forms the
+// logits again for each 256-column slice of d, in each of the two products: 2
+// (1 + d / 256) logit-sized products, and few rows leave most SMs idle. Here they are formed once for each
+// product, as gradient tiles in the image's layout in memory that is free at
+// the time, and the two products are the image form's GEMMs: 4 in all.
+//   dH: token chunks, the tiles over the whole vocabulary in dW, which nothing
+//       has written yet, or in the workspace's ring if that holds more blocks.
+//   dW: vocabulary slabs in ascending order, the tiles over all tokens in the
+//       rows of dW behind the slab (or in the ring); a slab is as large as that
+//       allows. Where even two vocabulary blocks of all tokens fit neither, the
+//       slab's tokens run in chunks that fit the ring, each adding its part.
+// If the ring holds all tiles, they are formed once for both.
+//
+// Each chunk and each slab costs its launches, short K loops and drains, about
+// kSlabUs, so each product takes the cheaper form by a model: bwd_kernel's units
+// (128 rows x 256 columns) at 1/152 of 1.28 PFLOP/s each, in rounds of 152, or
+// two logit-sized products at 1.6 PFLOP/s and kSlabUs per part. Measured on one
+// GB300: d = 2432, V = 60,000, 1.5 k tokens (one chunk, four slabs) 9.2 -> 1.33
+// ms for both; d = 1216, V = 30,000, 7 k tokens (5 chunks, 18 slabs) 5.4 -> 2.76;
+// d = 768, V = 32,000, 6 k tokens in 7 chunks 0.99 -> 1.01 for dH alone, and dW
+// would take 23 slabs (1.83 against 0.96).
+constexpr double kSlabUs = 75.0;
+
+struct SlabPlan {
+  size_t ring, vt, row;  // bytes of the ring; of one vocabulary block's tiles of
+                         // all tokens; of one vocabulary block's dW rows
+  int n_rb, n_vt;        // token blocks (of T) and vocabulary blocks
+  bool one;              // all tiles fit the ring
+  bool in_dw;            // dH's tiles lie in dW
+  int chunk;             // token blocks per dH chunk
+};
+SlabPlan slab_plan(const GradArgs &g) {
+  SlabPlan p;
+  p.ring = (size_t)kMaxClusters * kRingBytesPerCluster;
+  p.n_rb = (int)((g.T + 127) / 128);
+  p.n_vt = (g.V + 127) / 128;
+  p.vt = (size_t)p.n_rb * kGImgTileBytes;
+  p.row = (size_t)128 * g.d * sizeof(float);
+  const size_t block = (size_t)p.n_vt * kGImgTileBytes;
+  p.one = block * p.n_rb <= p.ring;
+  const size_t out = (size_t)g.V * g.d * sizeof(float);
+  p.in_dw = !p.one && out > p.ring;
+  const size_t fit = (p.in_dw ? out : p.ring) / block;
+  p.chunk = (int)(fit < (size_t)p.n_rb ? fit : (size_t)p.n_rb);
+  return p;
+}
+
+// The dW slab at vocabulary block vb0: x blocks (even, but for the last), their
+// tiles in dW behind them or in the ring, in chunks of `chunk` token blocks.
+struct Slab {
+  int x, chunk;
+  bool in_dw;
+};
+Slab slab_at(const GradArgs &g, const SlabPlan &p, int vb0) {
+  // x blocks' tiles behind them in dW: x vt <= (bytes behind the slab).
+  const size_t rest = (size_t)g.V * g.d * sizeof(float) - (size_t)vb0 * p.row;
+  const int x_dw = (int)(rest / (p.vt + p.row)) & ~1, x_ring = (int)(p.ring / p.vt) & ~1;
+  Slab o{x_dw > x_ring ? x_dw : x_ring, p.n_rb, x_dw > x_ring};
+  if (o.x < 2) {
+    o.x = 2;
+    o.chunk = (int)(p.ring / (2 * (size_t)kGImgTileBytes));
+  }
+  if (o.x > p.n_vt - vb0) o.x = p.n_vt - vb0;
+  return o;
+}
+
+// Whether dH, and dW, take the slabs (see kSlabUs; two thirds of the packed
+// tokens taken as active).
+void slabs_choose(const GradArgs &g, const SlabPlan &p, bool &dh, bool &dw) {
+  dh = dw = false;
+  if (p.chunk < 1) return;
+  const double tokens = 2.0 / 3.0 * g.T, slices = (g.d + 255) / 256;
+  const double per_row = 2.0 * (g.d + (g.d < 256 ? g.d : 256)) * 128 / (1.28e9 / 152);  // us
+  const double old_dh = per_row * g.V * ceil(ceil(tokens / 128) * slices / 152);
+  const double old_dw = per_row * tokens * ceil(p.n_vt * slices / 152);
+  const double two = 4.0 * tokens * g.V * g.d / 1.6e9;
+  const int chunks = (p.n_rb + p.chunk - 1) / p.chunk;
+  dh = two + kSlabUs * chunks < old_dh;
+  if (two + kSlabUs >= old_dw) return;
+  int parts = 0;
+  const int most = (int)((old_dw - two) / kSlabUs) + 1;
+  for (int vb0 = 0; vb0 < p.n_vt && parts <= most;) {
+    const Slab o = slab_at(g, p, vb0);
+    parts += (p.n_rb + o.chunk - 1) / o.chunk;
+    vb0 += o.x;
+  }
+  dw = two + kSlabUs * parts < old_dw;
+}
+
+namespace {
+// dH rows of token blocks [rb0, rb0 + cap) from their gradient tiles.
+pair_status slab_dh(const GradArgs &g, const GradWorkspace &w, cudaStream_t s, int rb0, int cap,
+                    void *img, float *scratch, int scratch_cap) {
+  const int n_vt = (g.V + 127) / 128;
+  CUtensorMap mGA, mW3;
+  if (!make_map3(&mGA, img, {64, 128, (cuuint64_t)2 * cap * n_vt}, {128, 16384}, {64, 128, 1},
+                 CU_TENSOR_MAP_SWIZZLE_NONE) ||
+      !make_map3(&mW3, g.W, {64, (cuuint64_t)g.V, (cuuint64_t)g.d / 64},
+                 {(cuuint64_t)g.d * 2, 128}, {64, 64, 2}, CU_TENSOR_MAP_SWIZZLE_128B))
+    return PAIR_ERR_CUDA;
+  const size_t smem = sizeof(DhSmem) + 1024;
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(dh_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)smem));
+  static int cache = 0;
+  const int grid = pair_grid((const void *)dh_gemm_kernel, smem, &cache);
+  PAIR_BEGIN("dh_gemm_tc", s);
+  dh_gemm_kernel<<<grid, kThreads, smem, s>>>(mGA, mW3, g.d, g.V, rb0, cap, w.counters, w.tok_idx,
+                                              w.tok_c, nullptr, g.dH, scratch, scratch_cap,
+                                              nullptr, g.dev_err);
+  PAIR_LAUNCH_CHECK(s);
+  PAIR_BEGIN("dh_tail", s);
+  dh_tail_combine_kernel<<<num_sms() * 2, 256, 0, s>>>(g.d, g.V, rb0, cap, grid / 2, scratch_cap,
+                                                       w.counters, w.tok_idx, w.tok_c, nullptr,
+                                                       scratch, g.dH);
+  PAIR_LAUNCH_CHECK(s);
+  return PAIR_OK;
+}
+
+// dW rows of vocabulary blocks [vb0, vb0 + n_vb) over token blocks [rb0, rb0 +
+// cap), from their gradient tiles.
+pair_status slab_dw(const GradArgs &g, const GradWorkspace &w, cudaStream_t s, int vb0, int n_vb,
+                    int rb0, int cap, bool accumulate, void *img, float *scratch,
+                    int scratch_cap) {
+  CUtensorMap mG, mH3, mD;
+  if (!make_map3(&mG, img, {64, 128, (cuuint64_t)2 * cap * n_vb}, {128, 16384}, {64, 32, 2},
+                 CU_TENSOR_MAP_SWIZZLE_NONE) ||
+      !make_map3(&mH3, w.Hc, {64, (cuuint64_t)w.Tpad, (cuuint64_t)g.d / 64},
+                 {(cuuint64_t)g.d * 2, 128}, {64, (cuuint32_t)kDwKS, 2},
+                 CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_map_f32(&mD, g.dW, g.V, g.d))
+    return PAIR_ERR_CUDA;
+  const size_t smem = sizeof(DwSmem) + 1024;
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(dw_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)smem));
+  static int cache = 0;
+  const int grid = pair_grid((const void *)dw_gemm_kernel, smem, &cache);
+  PAIR_BEGIN("dw_gemm_tc", s);
+  dw_gemm_kernel<<<grid, kThreads, smem, s>>>(mG, mH3, mD, g.d, g.V, vb0, n_vb, rb0, cap,
+                                              rb0 * 128, accumulate ? 1 : 0, w.counters, g.dW,
+                                              scratch, scratch_cap, g.dev_err);
+  PAIR_LAUNCH_CHECK(s);
+  if (scratch_cap > 0) {
+    PAIR_BEGIN("dw_tail", s);
+    dw_tail_combine_kernel<<<num_sms() * 2, 256, 0, s>>>(g.d, g.V, vb0, n_vb, rb0, cap,
+                                                         accumulate ? 1 : 0, grid / 2,
+                                                         scratch_cap, w.counters, scratch, g.dW);
+    PAIR_LAUNCH_CHECK(s);
+  }
+  return PAIR_OK;
+}
+}  // namespace
+
+// The softmax parts of dH and dW that take the slabs, after grad_lse_tc (dh and
+// dw say which; dH runs first: its tiles may lie in dW). The number of chunks
+// and slabs follows from T and V; those past the last active token exit at once.
+pair_status grad_bwd_slabs(const GradArgs &g, const GradWorkspace &w, cudaStream_t s, bool &dh,
+                           bool &dw) {
+  const SlabPlan p = slab_plan(g);
+  slabs_choose(g, p, dh, dw);
+  const int n_tile = (p.n_vt + 1) / 2;  // 256-row tiles of the gradient pass
+  constexpr size_t kTile = 2 * 128 * kDhN * sizeof(float);
+  float *ring = static_cast<float *>(w.gring);
+  const int ring_cap = (int)(p.ring / kTile);
+  char *out = reinterpret_cast<char *>(g.dW);
+
+  for (int rb0 = 0; dh && rb0 < p.n_rb; rb0 += p.chunk) {
+    void *img = p.in_dw ? g.dW : w.gring;
+    pair_status st = launch_grad_image(g, w, s, rb0, p.chunk, 0, n_tile, img);
+    if (st == PAIR_OK)
+      st = slab_dh(g, w, s, rb0, p.chunk, img, ring, p.in_dw ? ring_cap : 0);
+    if (st != PAIR_OK) return st;
+  }
+  if (dw && dh && p.one) return slab_dw(g, w, s, 0, p.n_vt, 0, p.n_rb, false, w.gring, nullptr, 0);
+
+  for (int vb0 = 0; dw && vb0 < p.n_vt;) {
+    const Slab o = slab_at(g, p, vb0);
+    void *img = o.in_dw ? static_cast<void *>(out + (size_t)(vb0 + o.x) * p.row) : w.gring;
+    for (int rb0 = 0; rb0 < p.n_rb; rb0 += o.chunk) {
+      const int cap = o.chunk < p.n_rb - rb0 ? o.chunk : p.n_rb - rb0;
+      pair_status st = launch_grad_image(g, w, s, rb0, cap, vb0 / 2, (o.x + 1) / 2, img);
+      if (st == PAIR_OK)
+        st = slab_dw(g, w, s, vb0, o.x, rb0, cap, rb0 > 0, img, ring, o.in_dw ? ring_cap : 0);
+      if (st != PAIR_OK) return st;
+    }
+    vb0 += o.x;
+  }
+  return PAIR_OK;
+}
 
 }  // namespace tck
 

@@ -93,16 +93,25 @@ __device__ __forceinline__ LseSplits lse_splits(int n_pairs, int n_vt, int ncl, 
 // measured slower over the whole step (deeper pipelines let the pairs drift
 // apart in the vocabulary, so fewer of them share W rows in L2), four starve
 // the MMA.
-template <bool kImage>
+//
+// Modes: kLsePlain, the maximum and sum of each token's logits; kLseTerms, also
+// the image of softmax terms relative to the reference; kLseGrad, no sums: the
+// image of the logit gradient -c_t 2^(z log2 e - lse_t log2 e) itself (ref holds
+// lse), of the vocabulary tiles [tile0, tile0 + n_vt) only.
+enum { kLsePlain = 0, kLseTerms = 1, kLseGrad = 2 };
+template <int kMode>
 __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
     lse_kernel(const __grid_constant__ CUtensorMap tmH,
-               const __grid_constant__ CUtensorMap tmW, int d, int V,
+               const __grid_constant__ CUtensorMap tmW, int d, int V, int tile0, int n_vt,
                int nsplit_base, int64_t Tpad, const int32_t *counters,
-               const int32_t *tok_y, const float *ref, float2 *part, float *zy, int rb0,
-               int cap, uint8_t *gimg, int s_blocks, int fix, int32_t *dev_err) {
+               const int32_t *tok_y, const float *ref, const float *tok_c, float2 *part,
+               float *zy, int rb0, int cap, uint8_t *gimg, int s_blocks, int fix,
+               int32_t *dev_err) {
+  constexpr bool kImage = kMode != kLsePlain, kTerms = kMode == kLseTerms;
+  constexpr bool kGrad = kMode == kLseGrad;
   // The fix-up launch redoes the pass only if the first one flagged a row
   // (the same value for every CTA: uniform exit before any cluster step).
-  if (kImage && fix && counters[2] == 0) return;
+  if (kTerms && fix && counters[2] == 0) return;
   extern __shared__ uint8_t smem_raw[];
   LseSmem &sm = *reinterpret_cast<LseSmem *>(align1k(smem_raw));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -117,9 +126,8 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
   // columns in that layout and writes the 4 KB with one bulk copy). Columns
   // in [V, 128 n_vt128) and rows past T_eff are exact zeros.
   const int n_tb = min(max((Teff + 127) / 128 - rb0, 0), cap);
-  const int n_vt128 = (V + 127) / 128;
+  const int n_vt128 = min((V + 127) / 128 - 2 * tile0, 2 * n_vt);  // image tiles per block
   const int s_lim = min(n_tb, s_blocks);
-  const int n_vt = (V + kLseBN - 1) / kLseBN;
   // Work unit = (pair of token blocks, vocabulary split); CTA r of the pair
   // takes token block 2 * pair + r (past the last block for an odd count:
   // in-bounds padding rows whose results are never written).
@@ -181,7 +189,8 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
               if (r == 0) mbar_expect_tx(&sm.full[stage], kLseStageTx);
               const uint32_t fb = mapa(smem_u32(&sm.full[stage]), 0);
               tma_load_2d_pair(sm.a[stage], &tmH, fb, k * 64, tb * 128);
-              tma_load_2d_pair(sm.b[stage], &tmW, fb, k * 64, vt * kLseBN + r * (kLseBN / 2));
+              tma_load_2d_pair(sm.b[stage], &tmW, fb, k * 64,
+                               (tile0 + vt) * kLseBN + r * (kLseBN / 2));
             }
             __syncwarp();
             last_ph[stage] = (int)ph;
@@ -246,7 +255,8 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
     const int quad = warp & 3;
     const int row = quad * 32 + lane;
     const uint32_t lane_addr = tmem + (static_cast<uint32_t>(quad * 32) << 16);
-    const int img_cols = n_vt128 * 128;  // image columns: V rounded up to a tile
+    // End of the image's columns: V rounded up to a tile.
+    const int img_cols = tile0 * kLseBN + n_vt128 * 128;
     int acc = 0, sbuf_i = 0;
     uint32_t acc_ph = 0;
     bool ok = true;
@@ -260,7 +270,8 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
       const int p = tb * 128 + row;
       const bool valid = p < Teff;
       const bool keep = kImage && tbl < s_lim;  // uniform over the CTA
-      const float R = (kImage && valid) ? ref[p] : 0.f;
+      const float R = (kImage && valid) ? (kGrad ? ref[p] * kLog2e : ref[p]) : 0.f;
+      const float nc = kGrad && valid ? -tok_c[p] : 0.f;
       const int yt = valid ? tok_y[p] : -1;
       float m2 = -INFINITY, l = 0.f, zt = 0.f;
       bool found = false;
@@ -269,12 +280,12 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
         tc_fence_after();
 #pragma unroll 1
         for (int c = 0; c < kLseBN / 32; ++c) {
-          const int col0 = vt * kLseBN + c * 32;
+          const int col0 = (tile0 + vt) * kLseBN + c * 32;
           if (kImage ? col0 >= img_cols : col0 >= V) break;  // the rest lies past V
           float v[32];
           tmem_ld32(lane_addr + acc * kLseBN + c * 32, v);
           const int off = yt - col0;
-          if (off >= 0 && off < 32) {
+          if (!kGrad && off >= 0 && off < 32) {
             found = true;
 #pragma unroll
             for (int j = 0; j < 32; ++j)
@@ -285,9 +296,12 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             v[j] = (j < nvalid) ? v[j] * kLog2e : -INFINITY;
-            mc = fmaxf(mc, v[j]);
+            if (!kGrad) mc = fmaxf(mc, v[j]);
           }
-          if (kImage) {
+          if (kGrad) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = nc * ex2_approx(v[j] - R);
+          } else if (kImage) {
             // Terms relative to the token's reference: v[j] becomes P_j.
             m2 = fmaxf(m2, mc);
             float sum = 0.f;
@@ -338,7 +352,7 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
               fence_async_smem();
               __syncwarp();
               if (lane == 0) {
-                const int acol = col0 & ~63;  // the atom's first column
+                const int acol = (col0 & ~63) - tile0 * kLseBN;  // the atom's first column
                 uint8_t *dst = gimg +
                                (((size_t)tbl * n_vt128 + (acol >> 7)) * 2 + ((acol >> 6) & 1)) *
                                    kAtom128 +
@@ -355,7 +369,7 @@ __global__ void __cluster_dims__(kLsePair, 1, 1) __launch_bounds__(kThreads, 1)
         if (++acc == 2) { acc = 0; acc_ph ^= 1; }
       }
       if (!ok) break;
-      if (valid) {
+      if (!kGrad && valid) {
         part[sp * spl.stride + p] = make_float2(m2, l);
         if (found) zy[p] = zt;
       }
@@ -433,7 +447,7 @@ int lse_grid(size_t smem) {
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, (const void *)lse_kernel<true>, &cfg) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveClusters(&n, (const void *)lse_kernel<kLseTerms>, &cfg) != cudaSuccess ||
       n <= 0) {
     cudaGetLastError();
     n = num_sms() / kLsePair;
@@ -457,16 +471,17 @@ pair_status launch_lse(const GradArgs &g, const GradWorkspace &w, cudaStream_t s
     return PAIR_ERR_CUDA;
   const int nsm = num_sms();
   const size_t lse_smem = sizeof(LseSmem) + 1024;
-  PAIR_CUDA_TRY(cudaFuncSetAttribute(lse_kernel<true>,
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(lse_kernel<kLseTerms>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lse_smem));
-  PAIR_CUDA_TRY(cudaFuncSetAttribute(lse_kernel<false>,
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(lse_kernel<kLsePlain>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lse_smem));
+  const int n_vt = (g.V + kLseBN - 1) / kLseBN;
   const int grid = lse_grid(lse_smem);
   if (!image) {
     PAIR_BEGIN("lse_tc", s);
-    lse_kernel<false><<<grid, kThreads, lse_smem, s>>>(
-        mH, mW128, g.d, g.V, w.nsplit, w.Tpad, w.counters, w.tok_y, nullptr, w.part, w.zy, rb0,
-        cap, nullptr, 0, 0, g.dev_err);
+    lse_kernel<kLsePlain><<<grid, kThreads, lse_smem, s>>>(
+        mH, mW128, g.d, g.V, 0, n_vt, w.nsplit, w.Tpad, w.counters, w.tok_y, nullptr, nullptr,
+        w.part, w.zy, rb0, cap, nullptr, 0, 0, g.dev_err);
     PAIR_LAUNCH_CHECK(s);
     PAIR_BEGIN("lse_combine", s);
     lse_combine_kernel<false><<<nsm * 4, 256, 0, s>>>(g.V, grid / kLsePair, w.nsplit, w.Tpad,
@@ -479,9 +494,9 @@ pair_status launch_lse(const GradArgs &g, const GradWorkspace &w, cudaStream_t s
   PAIR_CUDA_TRY(cudaMemsetAsync(w.counters + 2, 0, sizeof(int32_t), s));
   for (int fix = 0; fix < 2; ++fix) {
     PAIR_BEGIN(fix ? "lse_fix" : "lse_tc", s);
-    lse_kernel<true><<<grid, kThreads, lse_smem, s>>>(
-        mH, mW128, g.d, g.V, w.nsplit, w.Tpad, w.counters, w.tok_y, w.ref, w.part, w.zy, rb0,
-        cap, gimg, s_blocks, fix, g.dev_err);
+    lse_kernel<kLseTerms><<<grid, kThreads, lse_smem, s>>>(
+        mH, mW128, g.d, g.V, 0, n_vt, w.nsplit, w.Tpad, w.counters, w.tok_y, w.ref, nullptr,
+        w.part, w.zy, rb0, cap, gimg, s_blocks, fix, g.dev_err);
     PAIR_LAUNCH_CHECK(s);
     PAIR_BEGIN("lse_combine", s);
     lse_combine_kernel<true><<<nsm * 4, 256, 0, s>>>(g.V, grid / kLsePair, w.nsplit, w.Tpad,
@@ -489,6 +504,25 @@ pair_status launch_lse(const GradArgs &g, const GradWorkspace &w, cudaStream_t s
                                                      rb0, cap, fix);
     PAIR_LAUNCH_CHECK(s);
   }
+  return PAIR_OK;
+}
+
+// Logit-gradient image of token blocks [rb0, rb0 + cap) x vocabulary tiles of
+// 256 rows [tile0, tile0 + n_vt), from the settled log-sum-exp (w.lse) and
+// coefficients (w.tok_c).
+pair_status launch_grad_image(const GradArgs &g, const GradWorkspace &w, cudaStream_t s, int rb0,
+                              int cap, int tile0, int n_vt, void *img) {
+  CUtensorMap mH, mW128;
+  if (!make_map(&mH, w.Hc, w.Tpad, g.d, 128) || !make_map(&mW128, g.W, g.V, g.d, 128))
+    return PAIR_ERR_CUDA;
+  const size_t smem = sizeof(LseSmem) + 1024;
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(lse_kernel<kLseGrad>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PAIR_BEGIN("grad_image", s);
+  lse_kernel<kLseGrad><<<lse_grid(smem), kThreads, smem, s>>>(
+      mH, mW128, g.d, g.V, tile0, n_vt, w.nsplit, w.Tpad, w.counters, w.tok_y, w.lse, w.tok_c,
+      nullptr, nullptr, rb0, cap, static_cast<uint8_t *>(img), cap, 0, g.dev_err);
+  PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
 }
 

@@ -110,6 +110,13 @@ pair_status launch_lse(const GradArgs &g, const GradWorkspace &w, cudaStream_t s
 // dw_gemm (pair_bwd_image.cu).
 pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStream_t s,
                              int64_t c);
+// Gradient tiles of token blocks x vocabulary tiles (pair_lse.cu), and the
+// backward that uses them where the workspace holds no image
+// (pair_bwd_image.cu).
+pair_status launch_grad_image(const GradArgs &g, const GradWorkspace &w, cudaStream_t s, int rb0,
+                              int cap, int tile0, int n_vt, void *img);
+pair_status grad_bwd_slabs(const GradArgs &g, const GradWorkspace &w, cudaStream_t s, bool &dh,
+                           bool &dw);
 // Backward without an image, recomputing the logits (pair_bwd_cluster.cu).
 pair_status grad_bwd_recompute(const GradArgs &g, const GradWorkspace &w, cudaStream_t s);
 // Whole head without an image: fused log-sum-exp + dH, then dW (cluster
