@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(256, 4) dense_staged_kernel(
     __syncwarp();
     WarpCoeffs o = {};
     if (ok)
-      o = warp_group_coeffs<PAIR_W_HT, false>(sm.stage, sm.Qt, stream_diag(G, sm.Qt), G, scale,
+      o = warp_group_coeffs<PAIR_W_HT, false, false>(sm.stage, sm.Qt, stream_diag(G, sm.Qt), G, scale,
                                               0u, 0.f, sm.aux, dev_err);
     sm.a[tid] = o.a0;
     sm.a[tid + 32] = o.a1;
@@ -612,8 +612,13 @@ pair_status launch_coeffs_weighted(int32_t B, int32_t G, const float *r, const u
                                    float w_max, float *a, uint8_t *active, int32_t *edges,
                                    int32_t *contrast, float *ess, float *max_w,
                                    int32_t *dev_err, cudaStream_t s) {
-  if ((wmode == PAIR_W_HT || wmode == PAIR_W_CLIPPED || wmode == PAIR_W_HAJEK) &&
-      coeffs_stream_applies(G, r, J, rho))
+  // Clipped and self-normalised weighting take the streaming kernel for every G
+  // up to 64 (1000 groups of 50: 20 -> 13 us, 4096: 55 -> 27); HT only where
+  // pair_coeffs does, whose terms it returns bit for bit (the block kernel is
+  // faster for plain HT without the diagnostics: 4096 groups of 30 in 12 us
+  // against 20).
+  if (((wmode == PAIR_W_CLIPPED || wmode == PAIR_W_HAJEK) && G <= kGMax) ||
+      (wmode == PAIR_W_HT && coeffs_stream_applies(G, r, J, rho)))
     return launch_coeffs_stream(B, G, r, J, rho, scale, flags, wmode, true, w_max, a, active,
                                 edges, contrast, ess, max_w, dev_err, s);
   if (G <= 32)

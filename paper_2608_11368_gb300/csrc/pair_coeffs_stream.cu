@@ -2,8 +2,8 @@
 // Eq. pair-advantage) with the observed-edge counts of Algorithm 1 and, for
 // the weighting variants of the practical estimator (clipped,
 // self-normalised), the group's weight diagnostics, for groups of at most 64
-// candidates with G a multiple of 4 (the collapse itself is
-// pair_coeffs_stream.cuh).
+// candidates (the collapse itself, and its form for group sizes that are no
+// multiple of 4 or inputs without the alignment, is pair_coeffs_stream.cuh).
 //
 // Shape: a persistent grid of kSW-warp blocks, one per SM; every warp owns a
 // stream of groups and stages them in its own shared memory (kStages at a
@@ -28,7 +28,7 @@ struct StreamSmem {
   __align__(16) unsigned char warp[kSW][kStages * kStageBytes + kWarpAux];
 };
 
-template <int WM, bool DIAG>
+template <int WM, bool DIAG, bool kAny>
 __global__ void __launch_bounds__(kSW * 32, 1) coeffs_stream_kernel(
     int B, int G, const float *__restrict__ r, const uint8_t *__restrict__ J,
     const float *__restrict__ rho, float scale, uint32_t flags, float w_max,
@@ -69,6 +69,38 @@ __global__ void __launch_bounds__(kSW * 32, 1) coeffs_stream_kernel(
   // has completed and its writes are visible.
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
+  auto store = [&](int b, const WarpCoeffs &o) {
+    const size_t gb = (size_t)b * G;
+    if (lane < G) {
+      a[gb + lane] = o.a0;
+      if (active) active[gb + lane] = o.act0 ? 1 : 0;
+    }
+    if (lane + 32 < G) {
+      a[gb + lane + 32] = o.a1;
+      if (active) active[gb + lane + 32] = o.act1 ? 1 : 0;
+    }
+    if (lane == 0) {
+      if (edges) edges[b] = o.K * (o.K - 1) / 2;
+      if (contrast) contrast[b] = o.C;
+      if (DIAG) {
+        if (ess) ess[b] = o.W2 > 0.f ? __fdiv_rn(o.W * o.W, o.W2) : 0.f;
+        if (max_w) max_w[b] = o.Wmax;
+      }
+    }
+  };
+  if constexpr (kAny) {
+    uint32_t jv = load_j_any(J, b0, B, G);
+    for (int b = b0; b < B; b += nw) {
+      issue_any(wbase, rho, r, jv, b, G, sm.Qt);
+      jv = load_j_any(J, b + nw, B, G);
+      wait_any();
+      store(b, warp_group_coeffs<WM, DIAG, true>(wbase, sm.Qt, dg, G, scale, flags, w_max, aux,
+                                                 dev_err));
+      __syncwarp();  // the stage and the packed lists are rewritten next
+    }
+    return;
+  }
+
   uint32_t ph = 0;       // bit s: parity of the next completion of stage s
   uint32_t pending = 0;  // bit s: stage s has copies issued and not yet waited for
 #pragma unroll
@@ -100,25 +132,8 @@ __global__ void __launch_bounds__(kSW * 32, 1) coeffs_stream_kernel(
     ph ^= 1u << s;
     pending &= ~(1u << s);
     __syncwarp();
-    const WarpCoeffs o = warp_group_coeffs<WM, DIAG>(wbase + s * kStageBytes, sm.Qt, dg, G,
-                                                     scale, flags, w_max, aux, dev_err);
-    const size_t gb = (size_t)b * G;
-    if (lane < G) {
-      a[gb + lane] = o.a0;
-      if (active) active[gb + lane] = o.act0 ? 1 : 0;
-    }
-    if (lane + 32 < G) {
-      a[gb + lane + 32] = o.a1;
-      if (active) active[gb + lane + 32] = o.act1 ? 1 : 0;
-    }
-    if (lane == 0) {
-      if (edges) edges[b] = o.K * (o.K - 1) / 2;
-      if (contrast) contrast[b] = o.C;
-      if (DIAG) {
-        if (ess) ess[b] = o.W2 > 0.f ? __fdiv_rn(o.W * o.W, o.W2) : 0.f;
-        if (max_w) max_w[b] = o.Wmax;
-      }
-    }
+    store(b, warp_group_coeffs<WM, DIAG, false>(wbase + s * kStageBytes, sm.Qt, dg, G, scale,
+                                                flags, w_max, aux, dev_err));
     __syncwarp();  // the stage and the packed lists are rewritten next
   }
   // After a timed-out wait, let the copies already issued land (bounded)
@@ -128,13 +143,13 @@ __global__ void __launch_bounds__(kSW * 32, 1) coeffs_stream_kernel(
     if (pending & (1u << s)) drain_wait(&bar[s], (ph >> s) & 1u);
 }
 
-template <int WM, bool DIAG>
+template <int WM, bool DIAG, bool kAny>
 pair_status launch_stream(int32_t B, int32_t G, const float *r, const uint8_t *J,
                           const float *rho, float scale, uint32_t flags, float w_max, float *a,
                           uint8_t *active, int32_t *edges, int32_t *contrast, float *ess,
                           float *max_w, int32_t *dev_err, cudaStream_t s) {
   const int smem = (int)sizeof(StreamSmem);
-  PAIR_CUDA_TRY(cudaFuncSetAttribute(coeffs_stream_kernel<WM, DIAG>,
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(coeffs_stream_kernel<WM, DIAG, kAny>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   int nsm = 0, dev = 0;
   PAIR_CUDA_TRY(cudaGetDevice(&dev));
@@ -153,7 +168,7 @@ pair_status launch_stream(int32_t B, int32_t G, const float *r, const uint8_t *J
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   PAIR_BEGIN(DIAG ? "coeffs_w" : "coeffs", s);
-  PAIR_CUDA_TRY(cudaLaunchKernelEx(&cfg, coeffs_stream_kernel<WM, DIAG>, B, G, r, J, rho, scale,
+  PAIR_CUDA_TRY(cudaLaunchKernelEx(&cfg, coeffs_stream_kernel<WM, DIAG, kAny>, B, G, r, J, rho, scale,
                                    flags, w_max, a, active, edges, contrast, ess, max_w, dev_err,
                                    make_stream_geom(G)));
   PAIR_LAUNCH_CHECK(s);
@@ -173,18 +188,21 @@ pair_status launch_coeffs_stream(int32_t B, int32_t G, const float *r, const uin
                                  bool diag, float w_max, float *a, uint8_t *active,
                                  int32_t *edges, int32_t *contrast, float *ess, float *max_w,
                                  int32_t *dev_err, cudaStream_t s) {
-  if (wmode == PAIR_W_HT && !diag)
-    return launch_stream<PAIR_W_HT, false>(B, G, r, J, rho, scale, flags, w_max, a, active,
-                                           edges, contrast, ess, max_w, dev_err, s);
-  if (wmode == PAIR_W_HT)
-    return launch_stream<PAIR_W_HT, true>(B, G, r, J, rho, scale, flags, w_max, a, active,
-                                          edges, contrast, ess, max_w, dev_err, s);
+  // The bulk-copy form where rows can be copied whole (HT: only there).
+  const bool whole = coeffs_stream_applies(G, r, J, rho);
+  auto go = [&](auto launch) {
+    return launch(B, G, r, J, rho, scale, flags, w_max, a, active, edges, contrast, ess, max_w,
+                  dev_err, s);
+  };
+  if (wmode == PAIR_W_HT && whole)
+    return diag ? go(launch_stream<PAIR_W_HT, true, false>)
+                : go(launch_stream<PAIR_W_HT, false, false>);
   if (wmode == PAIR_W_CLIPPED)
-    return launch_stream<PAIR_W_CLIPPED, true>(B, G, r, J, rho, scale, flags, w_max, a, active,
-                                               edges, contrast, ess, max_w, dev_err, s);
+    return whole ? go(launch_stream<PAIR_W_CLIPPED, true, false>)
+                 : go(launch_stream<PAIR_W_CLIPPED, true, true>);
   if (wmode == PAIR_W_HAJEK)
-    return launch_stream<PAIR_W_HAJEK, true>(B, G, r, J, rho, scale, flags, w_max, a, active,
-                                             edges, contrast, ess, max_w, dev_err, s);
+    return whole ? go(launch_stream<PAIR_W_HAJEK, true, false>)
+                 : go(launch_stream<PAIR_W_HAJEK, true, true>);
   return PAIR_ERR_INVALID_ARG;
 }
 
