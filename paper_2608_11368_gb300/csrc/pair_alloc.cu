@@ -23,20 +23,21 @@
 // about 1 / 2G of it for a dense graph, where b_i is about G sum_j a_ij), so
 // no factorisation is needed: Chebyshev's iteration on the system scaled by
 // its diagonal, whose spectrum lies within rho = max_i v_i w_i / M_ii <= 1/2 of
-// 1, gains a factor of at least 3.7 per product with A, and two products give
-// the 1e-3 that an interior-point step needs for G >= 16. Odd degrees only:
-// their residual polynomial vanishes at 1, where the coordinates at a bound
-// lie, so those are exact. What the step's residual leaves is corrected by
-// the next step, and the stopping test is on the fp64 residuals themselves.
+// 1, gains a factor of at least 3.7 per product with A. A reduction to a tenth is
+// enough: what the solve leaves is in the next step's residual, and the steps
+// are as many as with 1e-12 (10.3 against 9.8 on groups of 64; up to a third
+// more on sparse graphs, with a fifth of the products). So rho <= 1/10, every
+// dense group of 16 or more, needs no product at all: the step solves the
+// diagonal. Odd degrees only: their residual polynomial vanishes at 1, where the
+// coordinates at a bound lie, so those are exact (even degrees stall there). The
+// stopping test is on the fp64 residuals themselves.
 //
 // What bounds it: the fp64 pipe (2 multiply-adds per clock and SM) for many
-// groups, the chain of a step's exchanges and products for few. A step of a
-// group of 64 takes five products with A (two of them with two right-hand
-// sides), all G^2 entries from shared memory with every lane busy, and 10
-// block-wide exchanges in a row. Measured on one GB300, against the
-// factorising log-barrier form: 64 groups of 16 in 0.107 ms (2.43 ms), 4096
-// groups of 64 in 4.79 ms (178 ms); with IEEE divisions in place of
-// rcp_approx / rcp_newton and full butterflies 0.188 and 6.84 ms.
+// groups, the chain of a step's exchanges for few. Measured on one GB300,
+// against the factorising log-barrier form: 64 groups of 16 in 0.078 ms (2.43
+// ms), 4096 groups of 64 in 2.70 ms (178 ms); with kLinRel = 1e-3 0.107 and 4.79
+// ms, with IEEE divisions in place of rcp_approx / rcp_newton and full
+// butterflies besides 0.188 and 6.84 ms.
 //
 // The paper solves the same program with SLSQP on the CPU (App. C); any
 // method reaching its optimum is equivalent. Cases the program leaves without
@@ -62,7 +63,7 @@ constexpr double kGapRel = 1e-12;       // stop at gap <= kGapRel * Phi (and the
 // the primal residual allowed at the end (kPrimalRel) then never spend more.
 constexpr double kBudgetMargin = 4e-14;
 constexpr double kPrimalRel = 2e-14;
-constexpr float kLinRel = 1e-3f;    // reduction of the Newton system's residual
+constexpr float kLinRel = 0.1f;     // reduction of the Newton system's residual
 constexpr int kLinMaxDegree = 61;   // reached only if rounding puts rho far above 1/2
 constexpr float kStepFrac = 0.995f; // of the largest step that keeps the interior
 constexpr double kStartMu = 0.1;    // the start's complementarity: kStartMu Phi in all
