@@ -29,20 +29,26 @@ namespace cg = cooperative_groups;
 // the log-sum-exp costs no pass of its own and the head takes four
 // logit-sized products; for dW, g = -c_t exp(z - lse_t).
 //
-// 128 threads; 4 x 2 logits and 4 x 16 outputs a thread (6 and 5 shared-memory
-// wavefronts for 8 and 16 cycles of multiply-adds), B double-buffered by
-// cp.async, 108 KB, two CTAs per SM. A cluster is C x S CTAs: C slices of
-// up to 256 columns of d, whose partial logits are added through distributed
-// shared memory, and S parts of B, whose outputs are added at the end the same
-// way, in rank order: 1075 tokens are 34 row tiles, too few for 304 CTA slots.
-// What bounds it: fp32 multiply-adds (128 per clock and SM).
-// Measured on one GB300, 4 x 8 rollouts of 32 to 64 tokens, d = 256, V = 4096:
-// dH with the log-sum-exp 151 us (597 + 962 row by row, a block per token),
-// dW 182 us (856): 30 and 25 TFLOP/s counting the recomputed logits.
+// 128 threads, two CTAs per SM (three up to 128 columns). What bounds it is the
+// latency between dependent steps with eight warps on an SM: the FMA pipe is
+// busy 50 % of the cycles and shared memory's data path 48 %, and most of the
+// rest are instructions that wait a fixed time for the one before. So a step does
+// much with little: two multiply-adds an instruction, and thread tiles as large
+// as the registers allow. Logits: each warp takes a quarter of the columns of d
+// and all 32 x 32 of them, 8 x 4 a thread (12 16-byte loads for 128
+// multiply-adds; 4 x 2 a thread over all columns took 24), and the four partial
+// sums meet in shared memory. Outputs: 8 rows x 8 columns a thread. A cluster is
+// C x S CTAs: C slices of up to 256 columns of d, whose partial logits are added
+// through distributed shared memory, and S parts of B, whose outputs are added
+// at the end the same way, in rank order: 1075 tokens are 34 row tiles, too few
+// for 304 CTA slots. 1,075 active tokens, d = 256, V = 4,096: dH with its
+// log-sum-exp 133 us, dW 145 us (single multiply-adds on smaller thread tiles:
+// 166 and 192 us); the four products are 9.0 GFLOP, 0.12 ms at the FMA rate.
 constexpr int kBM = 32, kBN = 32, kTileThreads = 128;
 constexpr int kSliceMax = 256;               // columns of d per CTA, at most
 constexpr int kTileDMax = 8 * kSliceMax;     // largest d of this form
-constexpr int kGPitch = kBM + 4;
+constexpr int kGPitch = kBM + 8;   // g, n-major: writes of a row's columns miss each other
+constexpr int kZPitch = kBN + 4;   // partial logits of a warp
 enum { kModeLse = 0, kModeDh = 1, kModeDw = 2 };
 
 struct TileArgs {
@@ -55,15 +61,29 @@ struct TileArgs {
 __host__ __device__ __forceinline__ int tile_slice(int d, int C) {
   return ((d / 16 + C - 1) / C) * 16;
 }
-// 64-column groups of a slice: outputs per thread, and the pitch of a tile's
+// 128-column groups of a slice: outputs per thread, and the pitch of a tile's
 // rows (columns past the slice hold anything; their outputs are not used).
-__host__ __device__ __forceinline__ int tile_groups(int slice) { return (slice + 63) / 64; }
+__host__ __device__ __forceinline__ int tile_groups(int slice) { return (slice + 127) / 128; }
 inline size_t tile_smem(int d, int C) {
-  const size_t pitch = tile_groups(tile_slice(d, C)) * 64 + 4;
-  return sizeof(float) * ((kBM + 2 * kBN) * pitch   // A, B (two buffers)
-                          + kBN * kGPitch           // g, n-major
-                          + 2 * kBM * kBN           // partial logits (two buffers)
-                          + 4 * kBM);               // row maximum, sum, rescaling, target logit
+  const size_t pitch = tile_groups(tile_slice(d, C)) * 128 + 4;
+  return sizeof(float) * ((kBM + kBN) * pitch            // A, B
+                          + kBN * kGPitch                // g, n-major
+                          + 4 * kBM * kZPitch            // the warps' partial logits
+                          + (C > 1 ? 2 * kBM * kBN : 0)  // the slices' (two buffers)
+                          + 4 * kBM                      // row maximum, sum, rescaling, target logit
+                          + 2 * kBN);                    // dW: lse and -c of the tile's tokens
+}
+
+// Two fp32 multiply-adds in one instruction (each rounded like fmaf): half the
+// issue slots of the products' inner loops.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<unsigned long long &>(d))
+      : "l"(reinterpret_cast<unsigned long long &>(a)),
+        "l"(reinterpret_cast<unsigned long long &>(b)),
+        "l"(reinterpret_cast<unsigned long long &>(c)));
+  return d;
 }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
@@ -94,7 +114,8 @@ __device__ __forceinline__ void load_tile(float *dst, int pitch, const float *sr
 }
 
 template <int MODE, int NJ>
-__global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileArgs g) {
+__global__ void __launch_bounds__(kTileThreads, NJ == 1 ? 3 : 2)
+    simt_tile_kernel(const TileArgs g) {
   const int Teff = g.counters[0];
   const int C = g.C, S = g.S, cs = C * S;
   const int m0 = (int)(blockIdx.x / cs) * kBM;
@@ -104,17 +125,19 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
   const int rank = (int)cluster.block_rank(), ci = rank % C, si = rank / C;
   const int d = g.d, ds = tile_slice(d, C), k0 = ci * ds;
   const int dn = max(min(ds, d - k0), 0);  // this CTA's columns (a multiple of 16)
-  constexpr int pitch = NJ * 64 + 4;
+  constexpr int pitch = NJ * 128 + 4;
   const float *A = MODE == kModeDw ? g.W : g.Hc, *B = MODE == kModeDw ? g.Hc : g.W;
 
   extern __shared__ __align__(16) float smem[];
-  float *As = smem, *Bs = As + kBM * pitch, *Gs = Bs + 2 * kBN * pitch;
-  float *Zp = Gs + kBN * kGPitch, *rm = Zp + 2 * kBM * kBN, *rl = rm + kBM, *rf = rl + kBM, *rz = rf + kBM;
+  float *As = smem, *Bs = As + kBM * pitch, *Gs = Bs + kBN * pitch;
+  float *Zw = Gs + kBN * kGPitch, *Zp = Zw + 4 * kBM * kZPitch;
+  float *rm = Zp + (C > 1 ? 2 * kBM * kBN : 0), *rl = rm + kBM, *rf = rl + kBM, *rz = rf + kBM;
+  float *tl = rz + kBM, *tc = tl + kBN;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // Logits: rows zm * 4 + i, columns zn + 16 j. Outputs: rows om * 4 + i,
-  // columns oc * 4 + 64 j.
-  const int zm = (warp & 1) * 4 + lane / 8, zn = (warp >> 1) * 8 + lane % 8;
-  const int om = zm, oc = zn;
+  // Partial logits: rows zm + 4 i, columns zn + 8 j (neighbouring rows: the
+  // lanes of a load miss each other's banks). Summed logits and their softmax:
+  // row m, columns 4 u + q. Outputs: rows warp * 8 + i, columns lane * 4 + 128 j.
+  const int zm = lane / 8, zn = lane % 8, m = tid / 4, q = tid & 3;
 
   // Tiles of this part of B; every CTA of the cluster runs the same number
   // of steps (they exchange partial logits in each).
@@ -127,16 +150,12 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
     rl[tid] = 0.f;
     rz[tid] = 0.f;  // the part that holds the target's tile sets it
   }
-  // The target of softmax row tid / 4.
-  const int ytile =
-      MODE != kModeDw && m0 + tid / 4 < Teff ? g.tok_y[m0 + tid / 4] : -1;
-  float acc[4][NJ][4];
+  const int ytile = MODE != kModeDw && m0 + m < Teff ? g.tok_y[m0 + m] : -1;
+  float2 acc[8][NJ][2];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < NJ; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
+    for (int j = 0; j < NJ; ++j) acc[i][j][0] = acc[i][j][1] = make_float2(0.f, 0.f);
 
   load_tile(As, pitch, A, M, m0, d, k0, dn);
   if (t0 < t1) load_tile(Bs, pitch, B, N, t0 * kBN, d, k0, dn);
@@ -145,70 +164,78 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
   for (int st = 0; st < steps; ++st) {
     const int t = t0 + st, n0 = t * kBN;
     const bool live = t < t1;
-    const float *Bt = Bs + (st & 1) * kBN * pitch;
+    if (st > 0) {
+      __syncthreads();  // the tile before, Gs and Zw are free
+      if (live) load_tile(Bs, pitch, B, N, n0, d, k0, dn);
+      cp_async_commit();
+    }
+    if (MODE == kModeDw && tid < kBN && live) {
+      const bool in = n0 + tid < N;
+      tl[tid] = in ? g.lse[n0 + tid] : 0.f;
+      tc[tid] = in ? -g.tok_c[n0 + tid] : 0.f;
+    }
     cp_async_wait<0>();
-    __syncthreads();  // this tile is in; the other buffer and Gs are free
-    if (t + 1 < t1) load_tile(Bs + ((st + 1) & 1) * kBN * pitch, pitch, B, N, n0 + kBN, d, k0, dn);
-    cp_async_commit();
+    __syncthreads();  // this tile is in
 
-    float z[4][2];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) z[i][0] = z[i][1] = 0.f;
+    float z[8];
     if (live) {
-      // 16-column pieces summed apart (shorter chains of roundings); the
-      // operands of the next 4 columns are loaded while these are multiplied.
-      const float *ap = As + zm * 4 * pitch, *bp = Bt + zn * pitch;
-      float4 a[2][4], b[2][2];
-      auto fetch = [&](int k, int q) {
+      // This warp's 16-column pieces; even and odd columns summed apart.
+      float2 zc[8][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          a[q][i] = *reinterpret_cast<const float4 *>(ap + i * pitch + k);
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
-          b[q][j] = *reinterpret_cast<const float4 *>(bp + 16 * j * pitch + k);
-      };
-      fetch(0, 0);
-      for (int k = 0; k < dn; k += 16) {
-        float zc[4][2];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) zc[i][0] = zc[i][1] = 0.f;
+        for (int j = 0; j < 4; ++j) zc[i][j] = make_float2(0.f, 0.f);
+      const float *ap = As + zm * pitch, *bp = Bs + zn * pitch;
+      for (int k = warp * 16; k < dn; k += 64) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          // (Past the slice's end: still inside the row's pitch.)
-          fetch(k + 4 * u + 4, (u + 1) & 1);
+          float4 a[8], b[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
+          for (int i = 0; i < 8; ++i)
+            a[i] = *reinterpret_cast<const float4 *>(ap + 4 * i * pitch + k + 4 * u);
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-              zc[i][j] = fmaf(a[u & 1][i].x, b[u & 1][j].x, zc[i][j]);
-              zc[i][j] = fmaf(a[u & 1][i].y, b[u & 1][j].y, zc[i][j]);
-              zc[i][j] = fmaf(a[u & 1][i].z, b[u & 1][j].z, zc[i][j]);
-              zc[i][j] = fmaf(a[u & 1][i].w, b[u & 1][j].w, zc[i][j]);
-            }
+          for (int j = 0; j < 4; ++j)
+            b[j] = *reinterpret_cast<const float4 *>(bp + 8 * j * pitch + k + 4 * u);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              zc[i][j] = fma2(make_float2(a[i].x, a[i].y), make_float2(b[j].x, b[j].y), zc[i][j]);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              zc[i][j] = fma2(make_float2(a[i].z, a[i].w), make_float2(b[j].z, b[j].w), zc[i][j]);
         }
+      }
+      float *zw = Zw + warp * kBM * kZPitch;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
-          for (int j = 0; j < 2; ++j) z[i][j] += zc[i][j];
+        for (int j = 0; j < 4; ++j)
+          zw[(zm + 4 * i) * kZPitch + zn + 8 * j] = zc[i][j].x + zc[i][j].y;
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const float *p = Zw + m * kZPitch + 4 * u + q;
+        constexpr int w = kBM * kZPitch;
+        z[u] = (p[0] + p[w]) + (p[2 * w] + p[3 * w]);
       }
     }
     if (C > 1) {
       float *zp = Zp + (st & 1) * kBM * kBN;
+      if (live)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) zp[(zm * 4 + i) * kBN + zn + 16 * j] = z[i][j];
+        for (int u = 0; u < 8; ++u) zp[u * kTileThreads + tid] = z[u];
       cluster.sync();
+      if (live) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int u = 0; u < 8; ++u) z[u] = 0.f;
+        for (int c = 0; c < C; ++c) {
+          const float *p = cluster.map_shared_rank(zp, si * C + c);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) z[i][j] = 0.f;
-      for (int c = 0; c < C; ++c) {
-        const float *q = cluster.map_shared_rank(zp, si * C + c);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) z[i][j] += q[(zm * 4 + i) * kBN + zn + 16 * j];
+          for (int u = 0; u < 8; ++u) z[u] += p[u * kTileThreads + tid];
+        }
       }
     }
     if (!live) continue;  // uniform over the CTA
@@ -216,34 +243,19 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
     bool rescale = false;
     if constexpr (MODE == kModeDw) {
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int n = n0 + zn + 16 * j;
-        const bool in = n < N;
-        const float c = in ? g.tok_c[n] : 0.f, ls = in ? g.lse[n] : 0.f;
-        float v[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = in ? -c * expf(z[i][j] - ls) : 0.f;
-        *reinterpret_cast<float4 *>(Gs + (zn + 16 * j) * kGPitch + zm * 4) =
-            make_float4(v[0], v[1], v[2], v[3]);
+      for (int u = 0; u < 8; ++u) {
+        const int n = 4 * u + q;
+        Gs[n * kGPitch + m] = n0 + n < N ? tc[n] * expf(z[u] - tl[n]) : 0.f;
       }
       __syncthreads();
     } else {
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const bool in = n0 + zn + 16 * j < N;
-        *reinterpret_cast<float4 *>(Gs + (zn + 16 * j) * kGPitch + zm * 4) =
-            in ? make_float4(z[0][j], z[1][j], z[2][j], z[3][j])
-               : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-      }
-      __syncthreads();
-      // Row m = tid / 4: four lanes, eight columns each.
-      const int m = tid / 4, q = tid & 3;
-      float v[8], mx = -INFINITY;
+      // Four lanes per row, eight columns each.
+      float mx = -INFINITY;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        v[u] = Gs[(4 * u + q) * kGPitch + m];
-        mx = fmaxf(mx, v[u]);
-        if (n0 + 4 * u + q == ytile) rz[m] = v[u];
+        if (n0 + 4 * u + q >= N) z[u] = -INFINITY;
+        mx = fmaxf(mx, z[u]);
+        if (n0 + 4 * u + q == ytile) rz[m] = z[u];
       }
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
@@ -251,9 +263,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
       float l = 0.f;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        v[u] = expf(v[u] - now);
-        l += v[u];
-        if (MODE == kModeDh) Gs[(4 * u + q) * kGPitch + m] = v[u];
+        z[u] = expf(z[u] - now);
+        l += z[u];
+        if (MODE == kModeDh) Gs[(4 * u + q) * kGPitch + m] = z[u];
       }
       l += __shfl_xor_sync(0xffffffffu, l, 1);
       l += __shfl_xor_sync(0xffffffffu, l, 2);
@@ -268,38 +280,33 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
     if constexpr (MODE != kModeLse) {
       if (rescale) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float f = rf[om * 4 + i];
+        for (int i = 0; i < 8; ++i) {
+          const float f = rf[warp * 8 + i];
 #pragma unroll
           for (int j = 0; j < NJ; ++j)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[i][j][e] *= f;
+            for (int e = 0; e < 2; ++e) {
+              acc[i][j][e].x *= f;
+              acc[i][j][e].y *= f;
+            }
         }
       }
-      const float *gp = Gs + om * 4, *bp = Bt + oc * 4;
-      float4 gv = *reinterpret_cast<const float4 *>(gp), b[NJ];
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) b[j] = *reinterpret_cast<const float4 *>(bp + 64 * j);
+      const float *gp = Gs + warp * 8, *bp = Bs + lane * 4;
 #pragma unroll 4
       for (int n = 0; n < kBN; ++n) {
-        const float gi[4] = {gv.x, gv.y, gv.z, gv.w};
-        float4 c[NJ];
+        const float4 g0 = *reinterpret_cast<const float4 *>(gp + n * kGPitch);
+        const float4 g1 = *reinterpret_cast<const float4 *>(gp + n * kGPitch + 4);
+        const float gi[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) c[j] = b[j];
-        const int nn = n + 1 < kBN ? n + 1 : n;  // the next row, while this one is multiplied
-        gv = *reinterpret_cast<const float4 *>(gp + nn * kGPitch);
+        for (int j = 0; j < NJ; ++j) {
+          const float4 b = *reinterpret_cast<const float4 *>(bp + n * pitch + 128 * j);
 #pragma unroll
-        for (int j = 0; j < NJ; ++j)
-          b[j] = *reinterpret_cast<const float4 *>(bp + nn * pitch + 64 * j);
-#pragma unroll
-        for (int j = 0; j < NJ; ++j)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            acc[i][j][0] = fmaf(gi[i], c[j].x, acc[i][j][0]);
-            acc[i][j][1] = fmaf(gi[i], c[j].y, acc[i][j][1]);
-            acc[i][j][2] = fmaf(gi[i], c[j].z, acc[i][j][2]);
-            acc[i][j][3] = fmaf(gi[i], c[j].w, acc[i][j][3]);
+          for (int i = 0; i < 8; ++i) {
+            const float2 gg = make_float2(gi[i], gi[i]);
+            acc[i][j][0] = fma2(gg, make_float2(b.x, b.y), acc[i][j][0]);
+            acc[i][j][1] = fma2(gg, make_float2(b.z, b.w), acc[i][j][1]);
           }
+        }
       }
     }
   }
@@ -311,11 +318,11 @@ __global__ void __launch_bounds__(kTileThreads, 2) simt_tile_kernel(const TileAr
   float *Os = Bs;  // [32][pitch]
   if constexpr (MODE != kModeLse) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
       for (int j = 0; j < NJ; ++j)
-        *reinterpret_cast<float4 *>(Os + (om * 4 + i) * pitch + oc * 4 + 64 * j) =
-            make_float4(acc[i][j][0], acc[i][j][1], acc[i][j][2], acc[i][j][3]);
+        *reinterpret_cast<float4 *>(Os + (warp * 8 + i) * pitch + lane * 4 + 128 * j) =
+            make_float4(acc[i][j][0].x, acc[i][j][0].y, acc[i][j][1].x, acc[i][j][1].y);
   }
   cluster.sync();
   const int r0 = si * kBM / S, r1 = (si + 1) * kBM / S;
@@ -427,22 +434,27 @@ pair_status launch_tile(const char *name, const GradArgs &g, const GradWorkspace
   const int64_t M = MODE == kModeDw ? g.V : g.T, N = MODE == kModeDw ? g.T : g.V;
   int C = 1;
   while (tile_slice(g.d, C) > kSliceMax) C *= 2;
-  // Parts of B: enough CTAs for two on each of the 152 SMs (of T packed
-  // tokens fewer are active, so rounded up), at least one tile each.
-  const int64_t tiles = ceil_div(M, kBM);
+  const int nj = tile_groups(tile_slice(g.d, C));
+  // Parts of B, at least one tile each: doubled until the CTAs fill the 152 SMs,
+  // which for dW, whose rows are all there, four fifths of the slots do (V =
+  // 4,096, d = 256: 145 us in 256 CTAs, 162 in 512; 3,000: 65 us in 376, 76 in
+  // 188) and a few more than all of them don't (V = 5,000, d = 512: 231 us in
+  // 314 CTAs, 194 in 628). Of T packed tokens about two thirds are active, so
+  // for dH all slots are wanted.
+  const int64_t tiles = ceil_div(M, kBM), slots = 152 * (nj == 1 ? 3 : 2);
+  const auto wants = [&](int64_t ctas) {
+    if (MODE != kModeDw) return ctas < slots;
+    return 5 * ctas < 4 * slots || (ctas > slots && 10 * ctas < 11 * slots);
+  };
   int S = 1;
-  while (S * C < 8 && tiles * C * S < 304 && 2 * S <= ceil_div(N, kBN)) S *= 2;
+  while (S * C < 8 && 2 * S <= ceil_div(N, kBN) && wants(tiles * C * S)) S *= 2;
   const size_t smem = tile_smem(g.d, C);
   const TileArgs a{g.d, g.V, C, S, w.counters, w.tok_idx, w.tok_y, w.tok_c,
                    static_cast<const float *>(w.Hc), static_cast<const float *>(g.W),
                    w.lse, w.zy, out};
   const int64_t ctas = tiles * C * S;
-  switch (tile_groups(tile_slice(g.d, C))) {
-    case 1: return launch_tile_nj<MODE, 1>(name, a, ctas, smem, s);
-    case 2: return launch_tile_nj<MODE, 2>(name, a, ctas, smem, s);
-    case 3: return launch_tile_nj<MODE, 3>(name, a, ctas, smem, s);
-    default: return launch_tile_nj<MODE, 4>(name, a, ctas, smem, s);
-  }
+  return nj == 1 ? launch_tile_nj<MODE, 1>(name, a, ctas, smem, s)
+                                              : launch_tile_nj<MODE, 2>(name, a, ctas, smem, s);
 }
 
 // ------------------------------------------------ any d (above 2048)
