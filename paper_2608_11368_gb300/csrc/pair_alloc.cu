@@ -35,8 +35,8 @@
 // What bounds it: the fp64 pipe (2 multiply-adds per clock and SM) for many
 // groups, the chain of a step's exchanges for few. Measured on one GB300,
 // against the factorising log-barrier form: 64 groups of 16 in 0.078 ms (2.43
-// ms), 4096 groups of 64 in 2.70 ms (178 ms); with kLinRel = 1e-3 0.107 and 4.79
-// ms, with IEEE divisions in place of rcp_approx / rcp_newton and full
+// ms), 4096 groups of 64 in 2.45 ms (178 ms); with a root per
+// entry of A 2.70 ms, with kLinRel = 1e-3 too 0.107 and 4.79 ms, with IEEE divisions in place of rcp_approx / rcp_newton and full
 // butterflies besides 0.188 and 6.84 ms.
 //
 // The paper solves the same program with SLSQP on the CPU (App. C); any
@@ -79,6 +79,10 @@ struct AllocShape {
   static constexpr int kThreads = GP <= 16 ? 32 : 2 * GP;
   static constexpr int kTpr = kThreads / GP;
   static constexpr int kWarps = kThreads / 32;
+  // Blocks per SM that the register allocation leaves room for: what shared
+  // memory holds of groups of 64; elsewhere the compiler's choice (0; asking for
+  // 16 warps of the small groups cost 81 us instead of 78 on 64 x 16).
+  static constexpr int kBlocks = GP == 64 ? 5 : 0;
 };
 
 // Row pitch of A (odd: rows start in different shared-memory banks).
@@ -273,7 +277,7 @@ __device__ __forceinline__ double edge_proxy(float pi_, float pj_, bool norms, f
 }
 
 template <int GP>
-__global__ void __launch_bounds__(AllocShape<GP>::kThreads)
+__global__ void __launch_bounds__(AllocShape<GP>::kThreads, AllocShape<GP>::kBlocks)
     alloc_kernel(int G, const float *__restrict__ p_hat, const float *__restrict__ m_hat,
                  const float *__restrict__ a, const float *__restrict__ c_hat,
                  const float *__restrict__ budget_in, float pi_min, float *__restrict__ pi_out,
@@ -325,19 +329,56 @@ __global__ void __launch_bounds__(AllocShape<GP>::kThreads)
   const bool invalid = sm.any != 0;
   const double sc = sm.sum_c, pmin = (double)pi_min;
 
-  // ---- A and b_i = (sum_{j != i} sqrt a_ij)^2 - sum_{j != i} a_ij
+  // ---- A and b_i = (sum_{j != i} sqrt a_ij)^2 - sum_{j != i} a_ij. The
+  // proxies from predictions are symmetric: row i forms the pairs (i, i + s mod
+  // G) for s up to G / 2, a_ij at [j][i] and its square root at [i][j] until the
+  // rows are summed (a square root is some twenty fp64 instructions: 2.70 -> 2.45
+  // ms on 4096 groups of 64). Groups of up to 32, where the extra passes cost as
+  // much, and an explicit array take every entry by itself.
   double bi = 0.0, asum = 0.0, sq = 0.0;
-  if (act && !invalid) {
-    const float pi_ = a ? 0.f : sm.p[i], mi = m_hat && !a ? sm.m[i] : 0.f;
-    for (int j = sub; j < G; j += kTpr) {
-      double v = 0.0;
-      if (j != i)
-        v = a ? (double)a[((size_t)g * G + i) * G + j]
-              : edge_proxy(pi_, sm.p[j], m_hat != nullptr, mi, m_hat ? sm.m[j] : 0.f);
-      grp.A[(size_t)i * grp.pitch + j] = v;
-      sq += sqrt(v);
-      asum += v;
+  if (GP <= 32 || a) {
+    if (act && !invalid) {
+      const float pi_ = a ? 0.f : sm.p[i], mi = m_hat && !a ? sm.m[i] : 0.f;
+      for (int j = sub; j < G; j += kTpr) {
+        double v = 0.0;
+        if (j != i)
+          v = a ? (double)a[((size_t)g * G + i) * G + j]
+                : edge_proxy(pi_, sm.p[j], m_hat != nullptr, mi, m_hat ? sm.m[j] : 0.f);
+        grp.A[(size_t)i * grp.pitch + j] = v;
+        sq += sqrt(v);
+        asum += v;
+      }
     }
+  } else {
+    const float pi_ = act ? sm.p[i] : 0.f, mi = act && m_hat ? sm.m[i] : 0.f;
+    // Row i's pairs: s = 1 .. half (the pairs half the group apart belong to
+    // the first half of the rows).
+    const int half = G % 2 == 0 && i >= G / 2 ? G / 2 - 1 : G / 2;
+    if (act && !invalid) {
+      if (sub == 0) grp.A[(size_t)i * grp.pitch + i] = 0.0;
+      for (int s = 1 + sub; s <= half; s += kTpr) {
+        const int j = i + s < G ? i + s : i + s - G;
+        const double v =
+            edge_proxy(pi_, sm.p[j], m_hat != nullptr, mi, m_hat ? sm.m[j] : 0.f);
+        grp.A[(size_t)j * grp.pitch + i] = v;
+        grp.A[(size_t)i * grp.pitch + j] = sqrt(v);
+      }
+    }
+    alloc_sync<GP>();
+    if (act && !invalid)
+      for (int s = 1 + sub; s < G; s += kTpr) {
+        const int j = i + s < G ? i + s : i + s - G;
+        const double x = grp.A[(size_t)i * grp.pitch + j], y = grp.A[(size_t)j * grp.pitch + i];
+        const bool root = s <= half;  // [i][j] holds the root, [j][i] the proxy
+        sq += root ? x : y;
+        asum += root ? y : x;
+      }
+    alloc_sync<GP>();
+    if (act && !invalid)
+      for (int s = 1 + sub; s <= half; s += kTpr) {
+        const int j = i + s < G ? i + s : i + s - G;
+        grp.A[(size_t)i * grp.pitch + j] = grp.A[(size_t)j * grp.pitch + i];
+      }
   }
 #pragma unroll
   for (int o = 1; o < kTpr; o <<= 1) {
