@@ -21,7 +21,7 @@
 // lane of the fp64 pipe busy, which is what bounds the pass: about G^2 / 2 + 4 G
 // fp64 operations per draw at 2 per clock and SM. Measured on one GB300, 50,000
 // draws of 16 candidates with D = 4096: the call takes
-// 95 us, its draws pass 62 us; one block per draw, with a tree and five block
+// 90 us, its draws pass 57 us; one block per draw, with a tree and five block
 // reductions each, took 653 and 500 us. For G = 64 and 128 (3125 and 781
 // draws) the call takes 0.16 and 0.43 ms, from 0.75 and 1.37 ms.
 #include "pair_coeffs_dev.cuh"
@@ -238,13 +238,28 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
   double acc[6] = {0, 0, 0, 0, 0, 0};  // mse, cos, vertices, edges, ess, weight (warp 0 of a team)
   const int nbatch = (N + 31) / 32;
   for (int bt = blockIdx.x * kTeams + team; bt < nbatch; bt += gridDim.x * kTeams) {
-    // ---- completion bits of the batch: 32 candidates per ballot
-    for (int q = tw; q < 32; q += TW) {
-      const int b = bt * 32 + q;
-      for (int j0 = 0; j0 < G; j0 += 32) {
-        const bool on = b < N && j0 + lane < G && Jd[(size_t)b * G + j0 + lane] != 0;
-        const uint32_t m = __ballot_sync(0xffffffffu, on);
-        if (lane == 0) bits[(j0 >> 5) * 32 + q] = m;
+    // ---- completion bits of the batch: a lane reads its own draw's flags
+    // where one warp has the batch (all loads in flight; ballots, 32 candidates
+    // at a time, chained 32 of them: 10 us of a batch), else by ballots.
+    if constexpr (TW == 1) {
+      const int b = bt * 32 + lane;
+      uint32_t mw = 0u;
+      if (b < N) {
+        const uint8_t *row = Jd + (size_t)b * G;
+#pragma unroll 16
+        for (int j = 0; j < G; ++j) mw |= (row[j] != 0 ? 1u : 0u) << j;
+      }
+      bits[lane] = mw;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 32 / TW; ++k) {
+        const int q = tw + k * TW, b = bt * 32 + q;
+#pragma unroll
+        for (int j0 = 0; j0 < 128; j0 += 32) {
+          const bool on = b < N && j0 + lane < G && Jd[(size_t)b * G + j0 + lane] != 0;
+          const uint32_t m = __ballot_sync(0xffffffffu, on);
+          if (lane == 0) bits[(j0 >> 5) * 32 + q] = m;
+        }
       }
     }
     team_sync<TW>();
