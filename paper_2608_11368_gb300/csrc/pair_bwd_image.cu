@@ -96,12 +96,15 @@ constexpr uint32_t kIdescDh = idesc_bf16(256, 256, 0, 1);
 // Work list of the persistent backward GEMMs (dh_gemm_kernel,
 // dw_gemm_kernel): the units that fill whole rounds of the grid (ncl
 // clusters) run over all of their K extent; the R < ncl units left over are
-// cut into S parts of K each, which run in as many rounds as they need. Work
-// item i < full_end is unit i; item full_end + j is part j / R of unit
-// full_end + j % R, over K steps [part nks / S, (part + 1) nks / S): the units
-// that read the same rows of the K-indexed operand in a part run next to each
-// other and share them in L2. The item's fp32 tile goes to scratch slot j and
-// the kernel's tail-combine pass adds the S parts in order (deterministic).
+// cut into S parts of K each, which run in as many rounds as they need. Of
+// hidden sizes whose last unit per row block is 256 columns wide (every nq-th of
+// all units), these take half the time and get Sh = ceil(S / 2) parts. Work item
+// i < full_end is unit i; then come parts 0 .. Sh - 1 of all R units, then
+// parts Sh .. S - 1 of the wide ones, part-major: the units that read the same
+// rows of the K-indexed operand in a part run next to each other and share them
+// in L2. Part p covers K steps [p nks / P, (p + 1) nks / P) of its unit's P. The
+// item's fp32 tile goes to the scratch slot of its place in the list and the
+// kernel's tail-combine pass adds a unit's parts in order (deterministic).
 //
 // S is the count of the smallest makespan, rounds x (steps of a part +
 // overhead) + the combine pass's share per tile, of up to 64 and up to the
@@ -112,24 +115,49 @@ constexpr uint32_t kIdescDh = idesc_bf16(256, 256, 0, 1);
 // per cluster, leave none idle but read each W row at R different times:
 // 1.35 times as slow as whole parts, from DRAM.)
 struct TailSplit {
-  int full_end, R, S;
+  int full_end, R, S, Sh;
+  int Rh, h0, nq;  // narrow units among the R: at h0, h0 + nq, ...
+
+  __device__ __forceinline__ int items() const { return R * Sh + (R - Rh) * (S - Sh); }
+  __device__ __forceinline__ bool narrow(int v) const {
+    return Rh > 0 && v >= h0 && (v - h0) % nq == 0;
+  }
+  __device__ __forceinline__ int parts(int v) const { return narrow(v) ? Sh : S; }
+  // The j-th wide unit, and the number of wide ones before unit v.
+  __device__ __forceinline__ int wide_at(int j) const {
+    return j < h0 ? j : j + 1 + (j - h0) / (nq - 1);
+  }
+  __device__ __forceinline__ int wide_before(int v) const {
+    return v > h0 ? v - 1 - (v - 1 - h0) / nq : v;
+  }
 };
 constexpr int kTailMaxParts = 64;
-// A whole warp calls (every lane gets the answer).
+// A whole warp calls (every lane gets the answer). d gives the units' widths.
 __device__ __forceinline__ TailSplit tail_split(int n_units, int ncl, int cap, int nks,
-                                                int overhead) {
+                                                int overhead, int d) {
+  TailSplit t{n_units, 0, 1, 1, 0, 0, (d + 511) / 512};
   const int R = n_units % ncl;
-  if (R == 0 || nks == 0) return TailSplit{n_units, 0, 1};
+  if (R == 0 || nks == 0) return t;
+  t.R = R;
+  t.h0 = t.nq - 1 - (n_units - R) % t.nq;
+  if (t.nq > 1 && d % 512 != 0 && d % 512 <= 256 && R > t.h0)
+    t.Rh = 1 + (R - 1 - t.h0) / t.nq;
   unsigned long long best = ~0ull;
   for (int S = 1 + (threadIdx.x & 31); S <= min(kTailMaxParts, nks); S += 32) {
-    if (S > 1 && R * S > cap) break;
-    const long long rounds = (R * S + ncl - 1) / ncl, steps = (nks + S - 1) / S;
-    const long long cost = 8 * rounds * (steps + overhead) + (S > 1 ? 2 * R * S : 0);
+    t.S = S;
+    t.Sh = t.Rh > 0 ? (S + 1) / 2 : S;
+    const int n = t.items();
+    if (S > 1 && n > cap) break;
+    const long long rounds = (n + ncl - 1) / ncl, steps = (nks + S - 1) / S;
+    const long long cost = 8 * rounds * (steps + overhead) + (S > 1 ? 2 * n : 0);
     best = min(best, (unsigned long long)cost * (2 * kTailMaxParts) + S);
   }
   for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
-  const int S = (int)(best % (2 * kTailMaxParts));
-  return S < 2 ? TailSplit{n_units, 0, 1} : TailSplit{n_units - R, R, S};
+  t.S = (int)(best % (2 * kTailMaxParts));
+  t.Sh = t.Rh > 0 ? (t.S + 1) / 2 : t.S;
+  if (t.S < 2) return TailSplit{n_units, 0, 1, 1, 0, 0, t.nq};
+  t.full_end = n_units - R;
+  return t;
 }
 // Work item i of a TailSplit -> unit u, its K steps [k0, k1) and scratch
 // slot (-1: a whole unit).
@@ -138,22 +166,48 @@ __device__ __forceinline__ void tail_item(const TailSplit &tl, int nks, int i, i
   if (i < tl.full_end) {
     u = i; k0 = 0; k1 = nks; slot = -1;
   } else {
-    const int j = i - tl.full_end, part = j / tl.R;
-    u = tl.full_end + (j - part * tl.R);
-    k0 = (int)((int64_t)part * nks / tl.S);
-    k1 = (int)((int64_t)(part + 1) * nks / tl.S);
+    const int j = i - tl.full_end, all = tl.R * tl.Sh, wide = tl.R - tl.Rh;
+    int part, v;
+    if (j < all) {
+      part = j / tl.R;
+      v = j - part * tl.R;
+    } else {
+      part = (j - all) / wide;
+      v = tl.wide_at(j - all - part * wide);
+      part += tl.Sh;
+    }
+    const int parts = tl.parts(v);
+    u = tl.full_end + v;
+    k0 = (int)((int64_t)part * nks / parts);
+    k1 = (int)((int64_t)(part + 1) * nks / parts);
     slot = j;
   }
 }
 // Sum of unit full_end + v's parts at float4 `at` of their tiles (`tile`
-// float4 each), in part order.
+// float4 each), in part order; eight loads in flight.
 __device__ __forceinline__ float4 tail_sum(const TailSplit &tl, int v, const float4 *src,
                                            int64_t tile, int64_t at) {
   float4 acc = src[v * tile + at];
-  for (int p = 1; p < tl.S; ++p) {
-    const float4 x = src[((int64_t)p * tl.R + v) * tile + at];
-    acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
-  }
+  auto add = [&](const float4 *p, int64_t stride, int n) {
+    int k = 0;
+    for (; k + 8 <= n; k += 8, p += 8 * stride) {
+      float4 x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) x[q] = p[q * stride];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        acc.x += x[q].x; acc.y += x[q].y; acc.z += x[q].z; acc.w += x[q].w;
+      }
+    }
+    for (; k < n; ++k, p += stride) {
+      const float4 x = *p;
+      acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
+    }
+  };
+  add(src + (tl.R + v) * tile + at, tl.R * tile, tl.Sh - 1);
+  if (!tl.narrow(v))
+    add(src + ((int64_t)tl.R * tl.Sh + tl.wide_before(v)) * tile + at, (tl.R - tl.Rh) * tile,
+        tl.S - tl.Sh);
   return acc;
 }
 // An item's start and drain in K steps: a step of dh is 64 vocabulary rows,
@@ -218,8 +272,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int nks = 2 * n_vt;  // 64-wide vocabulary steps (image atoms)
   const int nq = (d + kDhN - 1) / kDhN;
   const int n_units = (nrb + 1) / 2 * nq;
-  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDhOverhead);
-  const int n_items = tl.full_end + tl.R * tl.S;
+  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDhOverhead, d);
+  const int n_items = tl.full_end + tl.items();
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kDhStages; ++s) {
@@ -403,7 +457,7 @@ __global__ void __launch_bounds__(256)
   if (nrb == 0) return;
   const int nks = 2 * ((V + 127) / 128);
   const int nq = (d + kDhN - 1) / kDhN;
-  const TailSplit tl = tail_split((nrb + 1) / 2 * nq, ncl, scratch_cap, nks, kDhOverhead);
+  const TailSplit tl = tail_split((nrb + 1) / 2 * nq, ncl, scratch_cap, nks, kDhOverhead, d);
   constexpr int kQ = kDhN / 4;  // float4 per tile row
   const int64_t n4 = (int64_t)tl.R * 2 * 128 * kQ;
   const float4 *src = reinterpret_cast<const float4 *>(scratch);
@@ -495,8 +549,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int nq = (d + kDwN - 1) / kDwN;
   const int n_units = (n_vb + 1) / 2 * nq;
   const int nks = nrb * (128 / kDwKS);
-  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDwOverhead);
-  const int n_items = tl.full_end + tl.R * tl.S;
+  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDwOverhead, d);
+  const int n_items = tl.full_end + tl.items();
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kDwStages; ++s) {
@@ -707,7 +761,7 @@ __global__ void __launch_bounds__(256)
   const int nrb = min(max((Teff + 127) / 128 - rb0, 0), cap);
   const int nq = (d + kDwN - 1) / kDwN;
   const int nks = nrb * (128 / kDwKS);
-  const TailSplit tl = tail_split((n_vb + 1) / 2 * nq, ncl, scratch_cap, nks, kDwOverhead);
+  const TailSplit tl = tail_split((n_vb + 1) / 2 * nq, ncl, scratch_cap, nks, kDwOverhead, d);
   constexpr int kQ = kDwN / 4;  // float4 per tile row
   const int64_t n4 = (int64_t)tl.R * 2 * 128 * kQ;
   const float4 *src = reinterpret_cast<const float4 *>(scratch);
@@ -826,7 +880,9 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
 // ms for both; d = 1216, V = 30,000, 7 k tokens (5 chunks, 18 slabs) 5.4 -> 2.76;
 // d = 768, V = 32,000, 6 k tokens in 7 chunks 0.99 -> 1.01 for dH alone, and dW
 // would take 23 slabs (1.83 against 0.96).
-constexpr double kSlabUs = 75.0;
+constexpr double kSlabUs = 75.0, kSlabDhUs = 35.0;
+constexpr size_t kSlabTile = 2 * 128 * kDhN * sizeof(float);  // a scratch tile
+constexpr size_t kSlabScratch = 1024;
 
 struct SlabPlan {
   size_t ring, vt, row;  // bytes of the ring; of one vocabulary block's tiles of
@@ -835,7 +891,31 @@ struct SlabPlan {
   bool one;              // all tiles fit the ring
   bool in_dw;            // dH's tiles lie in dW
   int chunk;             // token blocks per dH chunk
+  size_t scratch;        // bytes of dW in front of dH's scratch tiles
+  int scratch_cap;       // scratch tiles, at most kSlabScratch (0: in the ring)
+  double dh_us;          // what dH takes by the model
 };
+// dH by chunks of c token blocks with `cap` scratch tiles, two thirds of the
+// packed tokens taken as active: per chunk the tiles at 1.6 PFLOP/s, the GEMM's
+// makespan (tail_split's, a K step 0.7 us) and kSlabDhUs; a chunk without a token
+// costs its launches.
+double slab_dh_us(const GradArgs &g, int n_rb, int n_vt, int c, int cap) {
+  const double wide = g.d % 512 != 0 && g.d % 512 <= 256 ? 0.5 : 0.0;  // the last unit's half
+  const double nks = 2.0 * n_vt, ncl = 76.0;
+  const auto chunk = [&](int rows) {
+    const double units = (rows + 1) / 2 * ((g.d + 511) / 512 - wide);
+    double best = ceil(units / ncl) * (nks + kDhOverhead);
+    for (int S = 2; S <= kTailMaxParts && S * units <= cap; ++S) {
+      const double steps = ceil(S * units / ncl) * (ceil(nks / S) + kDhOverhead) + 0.25 * S * units;
+      if (steps < best) best = steps;
+    }
+    return 2.0 * rows * 128 * 128 * (double)n_vt * g.d / 1.6e9 + 0.7 * best + kSlabDhUs;
+  };
+  const int busy = (2 * n_rb + 2) / 3, full = busy / c, last = busy - full * c;
+  const int idle = (n_rb + c - 1) / c - full - (last > 0);
+  return (full > 0 ? full * chunk(c) : 0.0) + (last > 0 ? chunk(last) : 0.0) + 15.0 * idle;
+}
+
 SlabPlan slab_plan(const GradArgs &g) {
   SlabPlan p;
   p.ring = (size_t)kMaxClusters * kRingBytesPerCluster;
@@ -848,7 +928,27 @@ SlabPlan slab_plan(const GradArgs &g) {
   const size_t out = (size_t)g.V * g.d * sizeof(float);
   p.in_dw = !p.one && out > p.ring;
   const size_t fit = (p.in_dw ? out : p.ring) / block;
-  p.chunk = (int)(fit < (size_t)p.n_rb ? fit : (size_t)p.n_rb);
+  const int most = (int)(fit < (size_t)p.n_rb ? fit : (size_t)p.n_rb);
+  p.chunk = 0;
+  p.scratch = 0;
+  p.scratch_cap = 0;
+  p.dh_us = 0.0;
+  // Larger chunks have fewer launches and drains, smaller ones leave more of dW
+  // for the partial tiles of the GEMM's units, which are few.
+  for (int c = most; c >= 1; c -= c > 1 && c % 2 ? 1 : 2) {
+    const size_t used = p.in_dw ? c * block : 0;
+    size_t cap = (out - used) / kSlabTile;
+    if (cap > kSlabScratch) cap = kSlabScratch;
+    const bool ring = p.in_dw && cap < p.ring / kSlabTile;
+    if (ring) cap = p.ring / kSlabTile;
+    const double us = slab_dh_us(g, p.n_rb, p.n_vt, c, (int)cap);
+    if (p.chunk == 0 || us < p.dh_us) {
+      p.chunk = c;
+      p.scratch = used;
+      p.scratch_cap = ring ? 0 : (int)cap;
+      p.dh_us = us;
+    }
+  }
   return p;
 }
 
@@ -881,8 +981,7 @@ void slabs_choose(const GradArgs &g, const SlabPlan &p, bool &dh, bool &dw) {
   const double old_dh = per_row * g.V * ceil(ceil(tokens / 128) * slices / 152);
   const double old_dw = per_row * tokens * ceil(p.n_vt * slices / 152);
   const double two = 4.0 * tokens * g.V * g.d / 1.6e9;
-  const int chunks = (p.n_rb + p.chunk - 1) / p.chunk;
-  dh = two + kSlabUs * chunks < old_dh;
+  dh = p.dh_us < old_dh;
   if (two + kSlabUs >= old_dw) return;
   int parts = 0;
   const int most = (int)((old_dw - two) / kSlabUs) + 1;
@@ -965,16 +1064,17 @@ pair_status grad_bwd_slabs(const GradArgs &g, const GradWorkspace &w, cudaStream
   const SlabPlan p = slab_plan(g);
   slabs_choose(g, p, dh, dw);
   const int n_tile = (p.n_vt + 1) / 2;  // 256-row tiles of the gradient pass
-  constexpr size_t kTile = 2 * 128 * kDhN * sizeof(float);
   float *ring = static_cast<float *>(w.gring);
-  const int ring_cap = (int)(p.ring / kTile);
+  const int ring_cap = (int)(p.ring / kSlabTile);
   char *out = reinterpret_cast<char *>(g.dW);
 
   for (int rb0 = 0; dh && rb0 < p.n_rb; rb0 += p.chunk) {
     void *img = p.in_dw ? g.dW : w.gring;
+    float *scratch = p.scratch_cap > 0 ? reinterpret_cast<float *>(out + p.scratch) : ring;
     pair_status st = launch_grad_image(g, w, s, rb0, p.chunk, 0, n_tile, img);
     if (st == PAIR_OK)
-      st = slab_dh(g, w, s, rb0, p.chunk, img, ring, p.in_dw ? ring_cap : 0);
+      st = slab_dh(g, w, s, rb0, p.chunk, img, scratch,
+                   p.scratch_cap > 0 ? p.scratch_cap : p.in_dw ? ring_cap : 0);
     if (st != PAIR_OK) return st;
   }
   if (dw && dh && p.one) return slab_dw(g, w, s, 0, p.n_vt, 0, p.n_rb, false, w.gring, nullptr, 0);
