@@ -1,8 +1,10 @@
 // Backward of the bf16 LM-head path without an image of softmax terms (the
 // no-alloc path and minimum workspaces): the logits are recomputed. For
 // d = 512 A (A <= 6), 8-CTA clusters share each Gs tile through an L2 ring
-// (bwd_cluster_kernel); otherwise one CTA per row block and 256-wide d-slice
-// (bwd_kernel).
+// (bwd_cluster_kernel); otherwise a CTA pair per two row blocks and 256-wide
+// d-slice (bwd_kernel).
+#include <math.h>
+
 #include "tc_kernels.cuh"
 
 namespace pairk {
@@ -12,276 +14,368 @@ using namespace tc;
 using namespace tck;
 
 // ------------------------------------------------------------- backward
+//
+// Per 128-row tile of the other side the logits S = R C^T (double-buffered in
+// TMEM), the gradient tile Gs = f(S) in bf16, and out += Gs C[:, slice], for one
+// block of 128 rows (tokens for dH, vocabulary rows for dW) and a 256-column
+// slice of d, whose accumulators stay in TMEM. Recomputing S per slice costs d +
+// 256 multiply-adds per logit and output slice, and every tile is fetched anew.
+//
+// Two forms. For d > 512 an SM's read port bounds it (about 60 bytes a clock): a
+// CTA pair takes two row blocks and each CTA fetches half of C's tile for either
+// product, 24 KB per 64 columns of d and 32 KB of the slice where a CTA by itself
+// takes 32 and 64; S runs two tiles ahead, its buffers free once they are read
+// from TMEM. (d = 768, V = 32,000: dW of 6.4 k tokens 979 -> 875 us, of 24 k 3.80
+// -> 3.24 ms; by single CTAs 1024 us and 4.1 ms.) Below, the chain from S through
+// the conversion to the next product bounds it, which the pair's exchanges only
+// lengthen: one CTA, two Gs tiles, eight warps converting (d = 256, V = 50,000,
+// 6.4 k tokens: dH 747 -> 721, dW 396 -> 305 us; d = 64: 1.58 -> 1.13 ms and 528
+// -> 347 us; in pairs 767 and 408 us at d = 256). Pairs want more than a dozen
+// tiles per unit: with 5 (d = 832, 0.4 k tokens) they take 101 us to 98.
 constexpr int kBwdBN = 128;     // S tile columns
 constexpr int kSlice = 256;     // output columns held in TMEM per unit
-constexpr int kBwdStages = 3;
-constexpr uint32_t kBwdStageTx = 2 * kAtom128;
-constexpr uint32_t kIdescS = idesc_bf16(128, kBwdBN, 0, 0);
+constexpr int kBwdThreads = 320;  // warps 2 .. 9: the epilogue, two per TMEM lane quadrant
 
+template <bool kPair>
 struct BwdSmem {
-  uint8_t a[kBwdStages][kAtom128];   // rows-operand atoms (128 x 64)
-  uint8_t b[kBwdStages][kAtom128];   // cols-operand atoms (128 x 64)
-  uint8_t cs[kSlice / 64][kAtom128]; // cols operand, d-slice (MN-major B)
-  uint8_t g[kBwdBN / 64][kAtom128];  // Gs tile, K-major A (2 atoms along K)
-  float col_c[kBwdBN], col_l[kBwdBN];
-  uint64_t full[kBwdStages], empty[kBwdStages];
-  uint64_t s_full[2], s_empty[2];
-  uint64_t g_full, g_empty, cs_full, cs_empty, o_full, o_empty, mma_done;
+  static constexpr int kStages = kPair ? 4 : 3;
+  static constexpr int kCs = kPair ? 2 : 1;                        // slices of C
+  static constexpr int kAhead = kPair ? 2 : 1;                     // tiles S runs ahead
+  static constexpr uint32_t kBBytes = kPair ? kAtom128 / 2 : kAtom128;  // this CTA's rows of it
+  uint8_t a[kStages][kAtom128];                              // rows-operand atoms (128 x 64)
+  uint8_t b[kStages][kBBytes];                               // cols-operand atoms
+  uint8_t cs[kCs][kSlice / 64 / (kPair ? 2 : 1)][kAtom128];  // cols operand, d-slice (MN-major B)
+  uint8_t g[2][kBwdBN / 64][kAtom128];                       // Gs tiles, K-major A
+  float2 col[kBwdBN];  // dW: -c and lse log2 e of the tile's tokens (c = 0: lse = infinity)
+  uint64_t full[kStages], empty[kStages], cs_full[kCs], cs_empty[kCs];
+  uint64_t s_full[2], s_empty[2], g_full[2], g_empty[2];
+  uint64_t o_full, o_empty, mma_done;
   uint32_t tmem_base;
   int abort;
 };
 
+// Named barrier of the epilogue warps.
+__device__ __forceinline__ void bwd_epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
 // kTokenRows: rows = tokens (output dH), cols = vocabulary.
 // otherwise : rows = vocabulary (output dW), cols = tokens.
-template <bool kTokenRows>
-__global__ void __launch_bounds__(kThreads, 1)
-    bwd_kernel(const __grid_constant__ CUtensorMap tmR,
-               const __grid_constant__ CUtensorMap tmC, int d, int V,
-               const int32_t *counters, const int32_t *tok_idx,
-               const float *tok_c, const float *lse, float *out,
+// tmC / tmCs: the other side with boxes of 128 and (pairs) of 64 rows.
+template <bool kTokenRows, bool kPair>
+__global__ void __launch_bounds__(kBwdThreads, 1)
+    bwd_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmC,
+               const __grid_constant__ CUtensorMap tmCs, int d, int V, const int32_t *counters,
+               const int32_t *tok_idx, const float *tok_c, const float *lse, float *out,
                int32_t *dev_err) {
   extern __shared__ uint8_t smem_raw[];
-  BwdSmem &sm = *reinterpret_cast<BwdSmem *>(align1k(smem_raw));
+  using Smem = BwdSmem<kPair>;
+  constexpr int kCtas = kPair ? 2 : 1, kBwdStages = Smem::kStages, kCs = Smem::kCs, kAhead = Smem::kAhead;
+  Smem &sm = *reinterpret_cast<Smem *>(align1k(smem_raw));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = kPair ? (int)(blockIdx.x & 1) : 0;  // rank in the cluster
+  const int pid = (int)blockIdx.x / kCtas, npairs = (int)gridDim.x / kCtas;
   const int Teff = counters[0];
   const int nsl = (d + kSlice - 1) / kSlice;
   const int n_rb = kTokenRows ? (Teff + 127) / 128 : (V + 127) / 128;
   const int n_ct = kTokenRows ? (V + kBwdBN - 1) / kBwdBN : (Teff + kBwdBN - 1) / kBwdBN;
-  const int n_units = n_rb * nsl;
+  const int n_units = (n_rb + kCtas - 1) / kCtas * nsl;
+  // This pair's tiles, unit after unit. Both products run along them, S two
+  // tiles ahead: what S(i + 2) waits for is that tile i has been read from
+  // TMEM, not that it has been converted.
+  const int n_tiles = n_units > pid ? ((n_units - pid - 1) / npairs + 1) * n_ct : 0;
   const int nk = d / 64;
+  // Columns of slice sl the MMA forms: in a pair a last slice of 64 or 192
+  // columns is rounded up (whole atoms in each CTA; columns past d load as zeros
+  // and are not stored).
+  auto slice_n = [&](int sl) {
+    const int w = min(kSlice, d - sl * kSlice);
+    return kPair ? (w + 127) & ~127 : w;
+  };
+  // Barriers that both CTAs arrive on lie in the even one.
+  auto arrive = [&](uint64_t *bar) {
+    if constexpr (kPair) mbar_arrive_cluster(mapa(smem_u32(bar), 0));
+    else mbar_arrive(bar);
+  };
+  auto commit = [&](uint64_t *bar) {
+    if constexpr (kPair) mma_commit_pair(bar, (uint16_t)3);
+    else mma_commit(bar);
+  };
+  auto mma = [&](uint32_t dst, uint64_t ad, uint64_t bd, uint32_t idesc, bool acc) {
+    if constexpr (kPair) mma_bf16_pair(dst, ad, bd, idesc, acc);
+    else mma_bf16(dst, ad, bd, idesc, acc);
+  };
+  auto load = [&](void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y) {
+    if constexpr (kPair) tma_load_2d_pair(dst, map, mapa(smem_u32(bar), 0), x, y);
+    else tma_load_2d(dst, map, bar, x, y);
+  };
+  volatile int *abort = &sm.abort;
+  auto await = [&](uint64_t *bar, uint32_t parity) {
+    if constexpr (kPair) return wait_cluster(bar, parity, abort, dev_err);
+    else return wait(bar, parity, abort, dev_err);
+  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kBwdStages; ++s) {
-      mbar_init(&sm.full[s], 1);
-      mbar_init(&sm.empty[s], 1);
+      mbar_init(&sm.full[s], 1);   // expect_tx (in a pair the even CTA's, of both CTAs' bytes)
+      mbar_init(&sm.empty[s], 1);  // the MMA's commit
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&sm.s_full[s], 1);
-      mbar_init(&sm.s_empty[s], 128);
+      mbar_init(&sm.s_empty[s], 8 * kCtas);  // the epilogue warps
+      mbar_init(&sm.g_full[s], 8 * kCtas);
+      mbar_init(&sm.g_empty[s], 1);
     }
-    mbar_init(&sm.g_full, 128);
-    mbar_init(&sm.g_empty, 1);
-    mbar_init(&sm.cs_full, 1);
-    mbar_init(&sm.cs_empty, 1);
+    for (int s = 0; s < kCs; ++s) {
+      mbar_init(&sm.cs_full[s], 1);
+      mbar_init(&sm.cs_empty[s], 1);
+    }
     mbar_init(&sm.o_full, 1);
-    mbar_init(&sm.o_empty, 128);
+    mbar_init(&sm.o_empty, 8 * kCtas);
     mbar_init(&sm.mma_done, 1);
     sm.abort = 0;
     fence_mbar_init();
     prefetch_tmap(&tmR);
     prefetch_tmap(&tmC);
+    prefetch_tmap(&tmCs);
   }
   if (warp == 1) {
-    tmem_alloc(&sm.tmem_base, 512);
-    tmem_relinquish();
+    if constexpr (kPair) {
+      tmem_alloc_pair(&sm.tmem_base, 512);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(&sm.tmem_base, 512);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (kPair) cluster_sync();  // the pair's barriers exist before anything lands on them
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   const uint32_t tmem_o = tmem + 2 * kBwdBN;  // columns [256, 512)
-  volatile int *abort = &sm.abort;
 
   if (warp == 0) {
     {  // whole warp: uniform loop state; elected lane issues
       int stage = 0;
-      uint32_t ph = 0, cs_ph = 0;
-      int last_ph[kBwdStages];
+      uint32_t ph = 0, cs_n = 0;
+      int last_ph[kBwdStages], cs_last[kCs];
+      for (int b = 0; b < kCs; ++b) cs_last[b] = -1;
       for (int s = 0; s < kBwdStages; ++s) last_ph[s] = -1;
-      int cs_last = -1;
       bool ok = true;
       auto load_s = [&](int rb, int ct) {
         for (int k = 0; k < nk && ok; ++k) {
-          if (!(ok = wait(&sm.empty[stage], ph ^ 1, abort, dev_err))) break;
+          if (!(ok = await(&sm.empty[stage], ph ^ 1))) break;
           if (elect_one()) {
-            mbar_expect_tx(&sm.full[stage], kBwdStageTx);
-            tma_load_2d(sm.a[stage], &tmR, &sm.full[stage], k * 64, rb * 128);
-            tma_load_2d(sm.b[stage], &tmC, &sm.full[stage], k * 64, ct * kBwdBN);
+            if (r == 0) mbar_expect_tx(&sm.full[stage], kCtas * (kAtom128 + Smem::kBBytes));
+            load(sm.a[stage], &tmR, &sm.full[stage], k * 64, rb * 128);
+            load(sm.b[stage], kPair ? &tmCs : &tmC, &sm.full[stage], k * 64,
+                 ct * kBwdBN + r * 64);
           }
           __syncwarp();
           last_ph[stage] = (int)ph;
           if (++stage == kBwdStages) { stage = 0; ph ^= 1; }
         }
       };
-      auto load_cs = [&](int sl, int w, int ct) {
+      auto load_cs = [&](int sl, int ct) {
         if (!ok) return;
-        if (!(ok = wait(&sm.cs_empty, cs_ph ^ 1, abort, dev_err))) return;
+        const int b = cs_n % kCs;
+        const uint32_t cph = (cs_n / kCs) & 1;
+        if (!(ok = await(&sm.cs_empty[b], cph ^ 1))) return;
         if (elect_one()) {
-          mbar_expect_tx(&sm.cs_full, (uint32_t)(w / 64) * kAtom128);
-          for (int j = 0; j < w / 64; ++j)
-            tma_load_2d(sm.cs[j], &tmC, &sm.cs_full, sl * kSlice + j * 64, ct * kBwdBN);
+          const int n = slice_n(sl);
+          if (r == 0) mbar_expect_tx(&sm.cs_full[b], (uint32_t)(n / 64) * kAtom128);
+          for (int j = 0; j < n / 64 / kCtas; ++j)
+            load(sm.cs[b][j], &tmC, &sm.cs_full[b], sl * kSlice + r * (n / 2) + j * 64,
+                 ct * kBwdBN);
         }
         __syncwarp();
-        cs_last = (int)cs_ph;
-        cs_ph ^= 1;
+        cs_last[b] = (int)cph;
+        ++cs_n;
       };
-      for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
-        const int rb = u / nsl, sl = u % nsl;
-        const int w = min(kSlice, d - sl * kSlice);
-        if (n_ct == 0) continue;
-        load_s(rb, 0);
-        for (int ct = 1; ct < n_ct && ok; ++ct) {
-          load_s(rb, ct);
-          load_cs(sl, w, ct - 1);
-        }
-        load_cs(sl, w, n_ct - 1);
+      int us = pid, cts = 0, uc = pid, ctc = 0;  // next tile of S, of cs
+      auto next_s = [&]() {
+        load_s(kCtas * (us / nsl) + r, cts);
+        if (++cts == n_ct) { cts = 0; us += npairs; }
+      };
+      for (int i = 0; i < kAhead && i < n_tiles; ++i) next_s();
+      for (int i = 0; i < n_tiles && ok; ++i) {
+        if (i + kAhead < n_tiles) next_s();
+        load_cs(uc % nsl, ctc);
+        if (++ctc == n_ct) { ctc = 0; uc += npairs; }
       }
+      // Never leave a copy in flight: wait (bounded) for the last one issued
+      // on every stage: completed on the even CTA, consumed by the pair MMA
+      // on the odd one (both CTAs issue the same sequence).
       volatile int never = 0;
       for (int s = 0; s < kBwdStages; ++s)
-        if (last_ph[s] >= 0) wait(&sm.full[s], (uint32_t)last_ph[s], &never, dev_err);
-      if (cs_last >= 0) wait(&sm.cs_full, (uint32_t)cs_last, &never, dev_err);
+        if (last_ph[s] >= 0)
+          wait_cluster(r == 0 ? &sm.full[s] : &sm.empty[s], (uint32_t)last_ph[s], &never, dev_err);
+      for (int b = 0; b < kCs; ++b)
+        if (cs_last[b] >= 0)
+          wait_cluster(r == 0 ? &sm.cs_full[b] : &sm.cs_empty[b], (uint32_t)cs_last[b], &never,
+                       dev_err);
     }
   } else if (warp == 1) {
-    {  // whole warp: uniform loop state; elected lane issues
+    if (r == 0) {  // whole warp: uniform loop state; elected lane issues
       int stage = 0;
-      uint32_t ph = 0, s_ph[2] = {0, 0}, g_ph = 0, cs_ph = 0, o_ph = 0;
+      uint32_t ph = 0, s_n = 0, g_n = 0, o_ph = 0;  // tiles begun and finished
       bool ok = true;
-      auto issue_s = [&](int ct) {
-        const int buf = ct & 1;
-        if (!(ok = wait(&sm.s_empty[buf], s_ph[buf] ^ 1, abort, dev_err))) return;
+      auto issue_s = [&]() {
+        const int buf = s_n & 1;
+        if (!(ok = await(&sm.s_empty[buf], ((s_n >> 1) & 1) ^ 1))) return;
         tc_fence_after();
         const uint32_t dt = tmem + buf * kBwdBN;
         for (int k = 0; k < nk; ++k) {
-          if (!(ok = wait(&sm.full[stage], ph, abort, dev_err))) return;
+          if (!(ok = await(&sm.full[stage], ph))) return;
+          tc_fence_after();
           const uint32_t sa = smem_u32(sm.a[stage]), sb = smem_u32(sm.b[stage]);
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              mma_bf16(dt, sdesc_sw128(sa + kk * 32, 16, 1024),
-                       sdesc_sw128(sb + kk * 32, 16, 1024), kIdescS,
-                       (k | kk) != 0);
-            mma_commit(&sm.empty[stage]);
+              mma(dt, sdesc_sw128(sa + kk * 32, 16, 1024), sdesc_sw128(sb + kk * 32, 16, 1024),
+                  idesc_bf16(128 * kCtas, kBwdBN, 0, 0), (k | kk) != 0);
+            commit(&sm.empty[stage]);
           }
           __syncwarp();
           if (++stage == kBwdStages) { stage = 0; ph ^= 1; }
         }
-        if (elect_one()) mma_commit(&sm.s_full[buf]);
+        if (elect_one()) commit(&sm.s_full[buf]);
         __syncwarp();
-        s_ph[buf] ^= 1;
+        ++s_n;
       };
-      auto issue_o = [&](int ct, int w) {
+      auto issue_o = [&](int ct, int n) {
         if (!ok) return;
-        if (!(ok = wait(&sm.g_full, g_ph, abort, dev_err))) return;
-        if (!(ok = wait(&sm.cs_full, cs_ph, abort, dev_err))) return;
-        if (ct == 0 && !(ok = wait(&sm.o_empty, o_ph ^ 1, abort, dev_err))) return;
+        const int buf = g_n & 1, b = g_n % kCs;
+        if (!(ok = await(&sm.g_full[buf], (g_n >> 1) & 1))) return;
+        if (!(ok = await(&sm.cs_full[b], (g_n / kCs) & 1))) return;
+        if (ct == 0 && !(ok = await(&sm.o_empty, o_ph ^ 1))) return;
         tc_fence_after();
-        const uint32_t idesc = idesc_bf16(128, w, 0, 1);
-        const uint32_t sg = smem_u32(sm.g[0]), sc = smem_u32(sm.cs[0]);
+        const uint32_t idesc = idesc_bf16(128 * kCtas, n, 0, 1);
+        const uint32_t sg = smem_u32(sm.g[buf][0]), sc = smem_u32(sm.cs[b][0]);
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < kBwdBN / 16; ++kk) {
             const uint64_t ad = sdesc_sw128(sg + (kk >> 2) * kAtom128 + (kk & 3) * 32, 16, 1024);
             const uint64_t bd = sdesc_sw128(sc + kk * 2048, kAtom128, 1024);
-            mma_bf16(tmem_o, ad, bd, idesc, (ct | kk) != 0);
+            mma(tmem_o, ad, bd, idesc, (ct | kk) != 0);
           }
-          mma_commit(&sm.g_empty);
-          mma_commit(&sm.cs_empty);
+          commit(&sm.g_empty[buf]);
+          commit(&sm.cs_empty[b]);
         }
         __syncwarp();
-        g_ph ^= 1;
-        cs_ph ^= 1;
+        ++g_n;
       };
-      for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
-        const int sl = u % nsl;
-        const int w = min(kSlice, d - sl * kSlice);
-        if (n_ct == 0) continue;
-        issue_s(0);
-        for (int ct = 0; ct < n_ct && ok; ++ct) {
-          if (ct + 1 < n_ct) issue_s(ct + 1);
-          issue_o(ct, w);
-        }
+      for (int i = 0; i < kAhead && i < n_tiles && ok; ++i) issue_s();
+      int u = pid, ct = 0;
+      for (int i = 0; i < n_tiles && ok; ++i) {
+        if (i + kAhead < n_tiles) issue_s();
+        issue_o(ct, slice_n(u % nsl));
         if (!ok) break;
-        if (elect_one()) mma_commit(&sm.o_full);
-        __syncwarp();
-        o_ph ^= 1;
+        if (++ct == n_ct) {
+          if (elect_one()) commit(&sm.o_full);
+          __syncwarp();
+          o_ph ^= 1;
+          ct = 0;
+          u += npairs;
+        }
       }
-      if (elect_one()) mma_commit(&sm.mma_done);
+      if (elect_one()) {
+        if constexpr (kPair) mma_commit_pair(&sm.mma_done, (uint16_t)1);
+        else mma_commit(&sm.mma_done);
+      }
       __syncwarp();
       volatile int never = 0;
       wait(&sm.mma_done, 0, &never, dev_err);
     }
   } else {
-    const int quad = warp & 3;
+    // Warp (quad, half): 32 rows, columns [64 half, 64 half + 64) of a tile and
+    // every other 32 of the output.
+    const int quad = warp & 3, half = (warp - 2) >> 2;
     const int row = quad * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-    uint32_t s_ph[2] = {0, 0}, g_ph = 0, o_ph = 0;
+    uint32_t n = 0, o_ph = 0;  // tiles so far
+    // Uniform over the warp; once false the warp only keeps up its barriers.
     bool ok = true;
-    for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
-      const int rb = u / nsl, sl = u % nsl;
+    auto await_all = [&](uint64_t *bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, await(bar, parity)) != 0;
+    };
+    for (int u = pid; u < n_units; u += npairs) {
+      const int rb = kCtas * (u / nsl) + r, sl = u % nsl;
       const int w = min(kSlice, d - sl * kSlice);
       const int rid = rb * 128 + row;  // token position or vocabulary id
-      float rc = 0.f, rl = 0.f;
-      if (kTokenRows && rid < Teff) {
-        rc = tok_c[rid];
-        rl = lse[rid] * kLog2e;
-      }
-      for (int ct = 0; ct < n_ct; ++ct) {
+      // c and lse of a token; terms of tokens with c = 0 underflow to 0.
+      float c = 0.f, l = 0.f;
+      auto token = [&](int p) {
+        c = p < Teff ? tok_c[p] : 0.f;
+        l = p < Teff ? lse[p] : 0.f;
+      };
+      auto term = [&]() { return make_float2(-c, c != 0.f ? l * kLog2e : INFINITY); };
+      token(kTokenRows ? rid : row);  // dW: of the next tile, read while the one before is converted
+      const float2 own = kTokenRows ? term() : make_float2(0.f, 0.f);
+      for (int ct = 0; ct < n_ct; ++ct, ++n) {
         if (!kTokenRows) {
-          epi_sync();
-          const int p = ct * kBwdBN + row;
-          sm.col_c[row] = p < Teff ? tok_c[p] : 0.f;
-          sm.col_l[row] = p < Teff ? lse[p] * kLog2e : 0.f;
-          epi_sync();
+          bwd_epi_sync();
+          if (half == 0) sm.col[row] = term();
+          bwd_epi_sync();
+          token((ct + 1) * kBwdBN + row);
         }
-        const int buf = ct & 1;
-        if (!(ok = wait(&sm.s_full[buf], s_ph[buf], abort, dev_err))) break;
-        s_ph[buf] ^= 1;
-        if (!(ok = wait(&sm.g_empty, g_ph ^ 1, abort, dev_err))) break;
+        const int buf = n & 1;
+        const uint32_t bph = (n >> 1) & 1;
+        if (!(ok = ok && await_all(&sm.s_full[buf], bph))) continue;
         tc_fence_after();
-#pragma unroll 1
-        for (int c = 0; c < kBwdBN / 32; ++c) {
-          float v[32];
-          tmem_ld32(tmem + lane_off + buf * kBwdBN + c * 32, v);
+        float v[2][32];
+        tmem_ld32(tmem + lane_off + buf * kBwdBN + half * 64, v[0]);
+        tmem_ld32(tmem + lane_off + buf * kBwdBN + half * 64 + 32, v[1]);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive(&sm.s_empty[buf]);
+        if (!(ok = await_all(&sm.g_empty[buf], bph ^ 1))) continue;
+        const int lim = V - ct * kBwdBN - half * 64;  // dH: columns of the vocabulary
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          if (kTokenRows && lim < 64) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (c * 32 + j >= lim) v[c][j] = -INFINITY;
+          }
           uint32_t pk[16];
 #pragma unroll
           for (int j = 0; j < 32; j += 2) {
-            float g2[2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const int col = c * 32 + j + e;
-              float cc, ll;
-              bool live;
-              if (kTokenRows) {
-                cc = rc; ll = rl;
-                live = (rc != 0.f) && (ct * kBwdBN + col < V);
-              } else {
-                cc = sm.col_c[col]; ll = sm.col_l[col];
-                live = cc != 0.f;
-              }
-              g2[e] = live ? -cc * ex2_approx(fmaf(v[j + e], kLog2e, -ll)) : 0.f;
-            }
-            __nv_bfloat162 b2 = __floats2bfloat162_rn(g2[0], g2[1]);
+            float4 cl = make_float4(own.x, own.y, own.x, own.y);
+            if (!kTokenRows)
+              cl = *reinterpret_cast<const float4 *>(&sm.col[half * 64 + c * 32 + j]);
+            __nv_bfloat162 b2 =
+                __floats2bfloat162_rn(cl.x * ex2_approx(fmaf(v[c][j], kLog2e, -cl.y)),
+                                      cl.z * ex2_approx(fmaf(v[c][j + 1], kLog2e, -cl.w)));
             pk[j >> 1] = *reinterpret_cast<uint32_t *>(&b2);
           }
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const int k = c * 32 + q * 8;  // first column of this 16-byte piece
-            uint8_t *dst = sm.g[k >> 6] + sw128_offset(row, k & 63);
+            uint8_t *dst = sm.g[buf][half] + sw128_offset(row, k);
             *reinterpret_cast<uint4 *>(dst) =
                 make_uint4(pk[q * 4], pk[q * 4 + 1], pk[q * 4 + 2], pk[q * 4 + 3]);
           }
         }
-        tc_fence_before();
-        mbar_arrive(&sm.s_empty[buf]);
         fence_async_smem();
-        mbar_arrive(&sm.g_full);
-        g_ph ^= 1;
+        __syncwarp();
+        if (lane == 0) arrive(&sm.g_full[buf]);
       }
-      if (!ok) break;
+      if (!ok) continue;
       const bool valid = kTokenRows ? (rid < Teff) : (rid < V);
       float *dst = nullptr;
       if (valid)
         dst = out + (kTokenRows ? (int64_t)tok_idx[rid] : (int64_t)rid) * d + sl * kSlice;
       if (n_ct == 0) {
         if (valid)
-          for (int k = 0; k < w; ++k) dst[k] = 0.f;
+          for (int k = half * 4; k < w; k += 8)
+            *reinterpret_cast<float4 *>(dst + k) = make_float4(0.f, 0.f, 0.f, 0.f);
         continue;
       }
-      if (!(ok = wait(&sm.o_full, o_ph, abort, dev_err))) break;
+      if (!(ok = await_all(&sm.o_full, o_ph))) continue;
       o_ph ^= 1;
       tc_fence_after();
 #pragma unroll 1
-      for (int c = 0; c < w / 32; ++c) {
+      for (int c = half; c < w / 32; c += 2) {
         float v[32];
         tmem_ld32(tmem_o + lane_off + c * 32, v);
         if (valid) {
@@ -292,16 +386,46 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       tc_fence_before();
-      mbar_arrive(&sm.o_empty);
+      __syncwarp();
+      if (lane == 0) arrive(&sm.o_empty);
     }
   }
 
   tc_fence_before();
   __syncthreads();
+  if constexpr (kPair) cluster_sync();  // no CTA leaves while its peer may still signal or fill it
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    if constexpr (kPair) tmem_dealloc_pair(tmem, 512);
+    else tmem_dealloc(tmem, 512);
   }
+}
+
+template <bool kTokenRows, bool kPair>
+pair_status launch_bwd(const char *name, const CUtensorMap &mR, const CUtensorMap &mC,
+                       const CUtensorMap &mCs, const GradArgs &g, const GradWorkspace &w, float *out,
+                       cudaStream_t s) {
+  const size_t smem = sizeof(BwdSmem<kPair>) + 1024;
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(bwd_kernel<kTokenRows, kPair>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(num_sms() & ~1), 1, 1);
+  cfg.blockDim = dim3(kBwdThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kPair ? 2 : 1;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  PAIR_BEGIN(name, s);
+  PAIR_CUDA_TRY(cudaLaunchKernelEx(&cfg, bwd_kernel<kTokenRows, kPair>, mR, mC, mCs, (int)g.d,
+                                   (int)g.V, (const int32_t *)w.counters,
+                                   (const int32_t *)w.tok_idx, (const float *)w.tok_c,
+                                   (const float *)w.lse, out, g.dev_err));
+  PAIR_LAUNCH_CHECK(s);
+  return PAIR_OK;
 }
 
 // ------------------------------------------------- backward, cluster form
@@ -1302,6 +1426,21 @@ pair_status grad_head_onchip(const GradArgs &g, const GradWorkspace &w, cudaStre
   }
 }
 
+// CTA pairs, or single CTAs, of bwd_kernel over `cols` columns (see there).
+bool bwd_pairs(int d, int64_t cols) { return d > 512 && cols >= 2048; }
+
+// Microseconds of bwd_kernel's product with `rows` rows over `cols` columns, by
+// tiles of 128 x 128: in pairs at 1.48 PFLOP/s, else at 2.1 and 0.65 us for the
+// chain (fitted to d = 64 to 1088).
+double bwd_recompute_us(int d, double rows, double cols, int64_t cols_max) {
+  const bool pair = bwd_pairs(d, cols_max);
+  const double flop = 2.0 * 128 * 128 * (d + (d < 256 ? d : 256)) * 152;
+  const double tile = pair ? flop / 1.48e9 : 0.65 + flop / 2.1e9;
+  const double blocks = ceil(rows / 128), slices = (d + 255) / 256;
+  const double rounds = pair ? ceil(ceil(blocks / 2) * slices / 76) : ceil(blocks * slices / 152);
+  return rounds * ceil(cols / 128) * tile;
+}
+
 // Softmax parts of dH and dW, recomputing the logits.
 pair_status grad_bwd_recompute(const GradArgs &g, const GradWorkspace &w, cudaStream_t s) {
   CUtensorMap mH, mW128;
@@ -1317,23 +1456,22 @@ pair_status grad_bwd_recompute(const GradArgs &g, const GradWorkspace &w, cudaSt
   bool slab_dh = false, slab_dw = false;
   const pair_status st = grad_bwd_slabs(g, w, s, slab_dh, slab_dw);
   if (st != PAIR_OK) return st;
-  const int nsm = num_sms();
-  const size_t bwd_smem = sizeof(BwdSmem) + 1024;
-  PAIR_CUDA_TRY(cudaFuncSetAttribute(bwd_kernel<true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem));
-  PAIR_CUDA_TRY(cudaFuncSetAttribute(bwd_kernel<false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem));
+  CUtensorMap mH64, mW64;
+  if (!make_map(&mH64, w.Hc, w.Tpad, g.d, 64) || !make_map(&mW64, g.W, g.V, g.d, 64))
+    return PAIR_ERR_CUDA;
   if (!slab_dh) {
-    PAIR_BEGIN("bwd_dh_tc", s);
-    bwd_kernel<true><<<nsm, kThreads, bwd_smem, s>>>(
-        mH, mW128, g.d, g.V, w.counters, w.tok_idx, w.tok_c, w.lse, g.dH, g.dev_err);
-    PAIR_LAUNCH_CHECK(s);
+    const pair_status e =
+        bwd_pairs(g.d, g.V)
+            ? launch_bwd<true, true>("bwd_dh_tc", mH, mW128, mW64, g, w, g.dH, s)
+            : launch_bwd<true, false>("bwd_dh_tc", mH, mW128, mW64, g, w, g.dH, s);
+    if (e != PAIR_OK) return e;
   }
   if (!slab_dw) {
-    PAIR_BEGIN("bwd_dw_tc", s);
-    bwd_kernel<false><<<nsm, kThreads, bwd_smem, s>>>(
-        mW128, mH, g.d, g.V, w.counters, w.tok_idx, w.tok_c, w.lse, g.dW, g.dev_err);
-    PAIR_LAUNCH_CHECK(s);
+    const pair_status e =
+        bwd_pairs(g.d, g.T)
+            ? launch_bwd<false, true>("bwd_dw_tc", mW128, mH, mH64, g, w, g.dW, s)
+            : launch_bwd<false, false>("bwd_dw_tc", mW128, mH, mH64, g, w, g.dW, s);
+    if (e != PAIR_OK) return e;
   }
   return PAIR_OK;
 }

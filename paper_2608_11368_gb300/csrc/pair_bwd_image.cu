@@ -873,13 +873,13 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
 // If the ring holds all tiles, they are formed once for both.
 //
 // Each chunk and each slab costs its launches, short K loops and drains, about
-// kSlabUs, so each product takes the cheaper form by a model: bwd_kernel's units
-// (128 rows x 256 columns) at 1/152 of 1.28 PFLOP/s each, in rounds of 152, or
-// two logit-sized products at 1.6 PFLOP/s and kSlabUs per part. Measured on one
-// GB300: d = 2432, V = 60,000, 1.5 k tokens (one chunk, four slabs) 9.2 -> 1.33
-// ms for both; d = 1216, V = 30,000, 7 k tokens (5 chunks, 18 slabs) 5.4 -> 2.76;
-// d = 768, V = 32,000, 6 k tokens in 7 chunks 0.99 -> 1.01 for dH alone, and dW
-// would take 23 slabs (1.83 against 0.96).
+// kSlabUs (dH: kSlabDhUs beside the GEMM's makespan), so each product takes the
+// cheaper form by a model: bwd_kernel's rounds of units (bwd_recompute_us), or two
+// logit-sized products at 1.6 PFLOP/s and the parts' cost. Measured on one GB300
+// against bwd_kernel: d = 2432, V = 60,000, 1.5 k tokens (one chunk, four slabs)
+// 9.2 -> 1.15 ms for the call; d = 1216, V = 30,000, 5 k tokens (5 chunks, 13
+// slabs) 2.13 ms; d = 768, V = 32,000, 6.4 k tokens in 10 chunks 0.99 -> 0.81 for
+// dH, and dW would take 23 slabs (1.83 against 0.88).
 constexpr double kSlabUs = 75.0, kSlabDhUs = 35.0;
 constexpr size_t kSlabTile = 2 * 128 * kDhN * sizeof(float);  // a scratch tile
 constexpr size_t kSlabScratch = 1024;
@@ -976,10 +976,9 @@ Slab slab_at(const GradArgs &g, const SlabPlan &p, int vb0) {
 void slabs_choose(const GradArgs &g, const SlabPlan &p, bool &dh, bool &dw) {
   dh = dw = false;
   if (p.chunk < 1) return;
-  const double tokens = 2.0 / 3.0 * g.T, slices = (g.d + 255) / 256;
-  const double per_row = 2.0 * (g.d + (g.d < 256 ? g.d : 256)) * 128 / (1.28e9 / 152);  // us
-  const double old_dh = per_row * g.V * ceil(ceil(tokens / 128) * slices / 152);
-  const double old_dw = per_row * tokens * ceil(p.n_vt * slices / 152);
+  const double tokens = 2.0 / 3.0 * g.T;
+  const double old_dh = bwd_recompute_us(g.d, tokens, g.V, g.V);
+  const double old_dw = bwd_recompute_us(g.d, g.V, tokens, g.T);
   const double two = 4.0 * tokens * g.V * g.d / 1.6e9;
   dh = p.dh_us < old_dh;
   if (two + kSlabUs >= old_dw) return;

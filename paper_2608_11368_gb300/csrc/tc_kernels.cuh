@@ -117,7 +117,9 @@ pair_status launch_grad_image(const GradArgs &g, const GradWorkspace &w, cudaStr
                               int cap, int tile0, int n_vt, void *img);
 pair_status grad_bwd_slabs(const GradArgs &g, const GradWorkspace &w, cudaStream_t s, bool &dh,
                            bool &dw);
-// Backward without an image, recomputing the logits (pair_bwd_cluster.cu).
+// Backward without an image, recomputing the logits (pair_bwd_cluster.cu), and
+// what one of its products takes where no cluster form applies.
+double bwd_recompute_us(int d, double rows, double cols, int64_t cols_max);
 pair_status grad_bwd_recompute(const GradArgs &g, const GradWorkspace &w, cudaStream_t s);
 // Whole head without an image: fused log-sum-exp + dH, then dW (cluster
 // form; d = 512 A, A <= 6). lse, zy and dH, dW softmax parts as the
