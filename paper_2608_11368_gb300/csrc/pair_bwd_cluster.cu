@@ -32,8 +32,15 @@ using namespace tck;
 // 6.4 k tokens: dH 747 -> 721, dW 396 -> 305 us; d = 64: 1.58 -> 1.13 ms and 528
 // -> 347 us; in pairs 767 and 408 us at d = 256). Pairs want more than a dozen
 // tiles per unit: with 5 (d = 832, 0.4 k tokens) they take 101 us to 98.
+//
+// The units of the last, or only, round are cut into parts of C's tiles
+// (TailSplit, at 152 CTAs or 76 pairs): 51 token blocks of d = 256 kept a third of
+// the SMs busy (dH 721 -> 256 us; d = 192, V = 50,000, 5.9 k tokens: 643 -> 160; d =
+// 128, V = 20,000, 0.5 k tokens: 233 -> 20).
 constexpr int kBwdBN = 128;     // S tile columns
 constexpr int kSlice = 256;     // output columns held in TMEM per unit
+// A split unit's start and drain, in tiles.
+constexpr int kBwdOverhead = 3;
 constexpr int kBwdThreads = 320;  // warps 2 .. 9: the epilogue, two per TMEM lane quadrant
 
 template <bool kPair>
@@ -65,7 +72,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
     bwd_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmC,
                const __grid_constant__ CUtensorMap tmCs, int d, int V, const int32_t *counters,
                const int32_t *tok_idx, const float *tok_c, const float *lse, float *out,
-               int32_t *dev_err) {
+               float *scratch, int scratch_cap, int32_t *dev_err) {
   extern __shared__ uint8_t smem_raw[];
   using Smem = BwdSmem<kPair>;
   constexpr int kCtas = kPair ? 2 : 1, kBwdStages = Smem::kStages, kCs = Smem::kCs, kAhead = Smem::kAhead;
@@ -78,10 +85,31 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
   const int n_rb = kTokenRows ? (Teff + 127) / 128 : (V + 127) / 128;
   const int n_ct = kTokenRows ? (V + kBwdBN - 1) / kBwdBN : (Teff + kBwdBN - 1) / kBwdBN;
   const int n_units = (n_rb + kCtas - 1) / kCtas * nsl;
-  // This pair's tiles, unit after unit. Both products run along them, S two
-  // tiles ahead: what S(i + 2) waits for is that tile i has been read from
-  // TMEM, not that it has been converted.
-  const int n_tiles = n_units > pid ? ((n_units - pid - 1) / npairs + 1) * n_ct : 0;
+  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, n_ct, kBwdOverhead, 1, nsl * 512);
+  const int n_items = tl.full_end + tl.items();
+  // This CTA's or pair's tiles, item after item. Both products run along them, S
+  // kAhead tiles ahead: what S(i + 2) waits for is that tile i has been read
+  // from TMEM, not that it has been converted.
+  struct Tile {
+    int i, u, ct, k0, k1, slot;
+    bool live;
+  };
+  auto open_item = [&](Tile &x) {
+    x.live = x.i < n_items && n_ct > 0;
+    if (x.live) tail_item(tl, n_ct, x.i, x.u, x.k0, x.k1, x.slot);
+    x.ct = x.k0;
+  };
+  auto first = [&]() {
+    Tile x{pid, 0, 0, 0, 0, -1, false};
+    open_item(x);
+    return x;
+  };
+  auto advance = [&](Tile &x) {
+    if (++x.ct == x.k1) {
+      x.i += npairs;
+      open_item(x);
+    }
+  };
   const int nk = d / 64;
   // Columns of slice sl the MMA forms: in a pair a last slice of 64 or 192
   // columns is rounded up (whole atoms in each CTA; columns past d load as zeros
@@ -191,16 +219,15 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
         cs_last[b] = (int)cph;
         ++cs_n;
       };
-      int us = pid, cts = 0, uc = pid, ctc = 0;  // next tile of S, of cs
+      Tile ts = first(), tc = ts;  // next tile of S, of cs
       auto next_s = [&]() {
-        load_s(kCtas * (us / nsl) + r, cts);
-        if (++cts == n_ct) { cts = 0; us += npairs; }
+        load_s(kCtas * (ts.u / nsl) + r, ts.ct);
+        advance(ts);
       };
-      for (int i = 0; i < kAhead && i < n_tiles; ++i) next_s();
-      for (int i = 0; i < n_tiles && ok; ++i) {
-        if (i + kAhead < n_tiles) next_s();
-        load_cs(uc % nsl, ctc);
-        if (++ctc == n_ct) { ctc = 0; uc += npairs; }
+      for (int k = 0; k < kAhead && ts.live; ++k) next_s();
+      for (; tc.live && ok; advance(tc)) {
+        if (ts.live) next_s();
+        load_cs(tc.u % nsl, tc.ct);
       }
       // Never leave a copy in flight: wait (bounded) for the last one issued
       // on every stage: completed on the even CTA, consumed by the pair MMA
@@ -242,12 +269,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
         __syncwarp();
         ++s_n;
       };
-      auto issue_o = [&](int ct, int n) {
+      auto issue_o = [&](bool begin, int n) {
         if (!ok) return;
         const int buf = g_n & 1, b = g_n % kCs;
         if (!(ok = await(&sm.g_full[buf], (g_n >> 1) & 1))) return;
         if (!(ok = await(&sm.cs_full[b], (g_n / kCs) & 1))) return;
-        if (ct == 0 && !(ok = await(&sm.o_empty, o_ph ^ 1))) return;
+        if (begin && !(ok = await(&sm.o_empty, o_ph ^ 1))) return;
         tc_fence_after();
         const uint32_t idesc = idesc_bf16(128 * kCtas, n, 0, 1);
         const uint32_t sg = smem_u32(sm.g[buf][0]), sc = smem_u32(sm.cs[b][0]);
@@ -256,7 +283,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
           for (int kk = 0; kk < kBwdBN / 16; ++kk) {
             const uint64_t ad = sdesc_sw128(sg + (kk >> 2) * kAtom128 + (kk & 3) * 32, 16, 1024);
             const uint64_t bd = sdesc_sw128(sc + kk * 2048, kAtom128, 1024);
-            mma(tmem_o, ad, bd, idesc, (ct | kk) != 0);
+            mma(tmem_o, ad, bd, idesc, !begin || kk != 0);
           }
           commit(&sm.g_empty[buf]);
           commit(&sm.cs_empty[b]);
@@ -264,18 +291,19 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
         __syncwarp();
         ++g_n;
       };
-      for (int i = 0; i < kAhead && i < n_tiles && ok; ++i) issue_s();
-      int u = pid, ct = 0;
-      for (int i = 0; i < n_tiles && ok; ++i) {
-        if (i + kAhead < n_tiles) issue_s();
-        issue_o(ct, slice_n(u % nsl));
+      Tile ts = first(), to = ts;  // next tile of S, of the output
+      for (int k = 0; k < kAhead && ts.live && ok; ++k, advance(ts)) issue_s();
+      for (; to.live && ok; advance(to)) {
+        if (ts.live) {
+          issue_s();
+          advance(ts);
+        }
+        issue_o(to.ct == to.k0, slice_n(to.u % nsl));
         if (!ok) break;
-        if (++ct == n_ct) {
+        if (to.ct + 1 == to.k1) {
           if (elect_one()) commit(&sm.o_full);
           __syncwarp();
           o_ph ^= 1;
-          ct = 0;
-          u += npairs;
         }
       }
       if (elect_one()) {
@@ -298,7 +326,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
     auto await_all = [&](uint64_t *bar, uint32_t parity) {
       return __all_sync(0xffffffffu, await(bar, parity)) != 0;
     };
-    for (int u = pid; u < n_units; u += npairs) {
+    for (int i = pid; i < n_items; i += npairs) {
+      int u, k0, k1, slot;
+      tail_item(tl, n_ct, i, u, k0, k1, slot);
       const int rb = kCtas * (u / nsl) + r, sl = u % nsl;
       const int w = min(kSlice, d - sl * kSlice);
       const int rid = rb * 128 + row;  // token position or vocabulary id
@@ -309,9 +339,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
         l = p < Teff ? lse[p] : 0.f;
       };
       auto term = [&]() { return make_float2(-c, c != 0.f ? l * kLog2e : INFINITY); };
-      token(kTokenRows ? rid : row);  // dW: of the next tile, read while the one before is converted
+      token(kTokenRows ? rid : k0 * kBwdBN + row);  // dW: of the next tile, read while the one before is converted
       const float2 own = kTokenRows ? term() : make_float2(0.f, 0.f);
-      for (int ct = 0; ct < n_ct; ++ct, ++n) {
+      for (int ct = k0; ct < k1; ++ct, ++n) {
         if (!kTokenRows) {
           bwd_epi_sync();
           if (half == 0) sm.col[row] = term();
@@ -363,7 +393,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
       if (!ok) continue;
       const bool valid = kTokenRows ? (rid < Teff) : (rid < V);
       float *dst = nullptr;
-      if (valid)
+      if (slot >= 0)
+        dst = scratch + (((int64_t)slot * kCtas + r) * 128 + row) * kSlice;
+      else if (valid)
         dst = out + (kTokenRows ? (int64_t)tok_idx[rid] : (int64_t)rid) * d + sl * kSlice;
       if (n_ct == 0) {
         if (valid)
@@ -378,7 +410,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
       for (int c = half; c < w / 32; c += 2) {
         float v[32];
         tmem_ld32(tmem_o + lane_off + c * 32, v);
-        if (valid) {
+        if (dst) {
 #pragma unroll
           for (int q = 0; q < 8; ++q)
             reinterpret_cast<float4 *>(dst + c * 32)[q] =
@@ -401,10 +433,41 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
   }
 }
 
+// Whether the last round's units may be split: with more than six rounds the
+// partial tiles and their pass cost what that round leaves idle.
+bool bwd_splits(int64_t rows, int d, int ctas) {
+  const int64_t units = ((rows + 127) / 128 + ctas - 1) / ctas * ((d + kSlice - 1) / kSlice);
+  return units <= 6 * (int64_t)(152 / ctas);
+}
+
+// Rows of the units bwd_kernel split (see TailSplit): their parts' sum.
+template <bool kTokenRows, bool kPair>
+__global__ void __launch_bounds__(256)
+    bwd_tail_kernel(int d, int V, int ncl, int scratch_cap, const int32_t *counters,
+                    const int32_t *tok_idx, const float *__restrict__ scratch, float *out) {
+  constexpr int kCtas = kPair ? 2 : 1, kRows = 128 * kCtas, kQ = kSlice / 4;
+  const int Teff = counters[0], rows = kTokenRows ? Teff : V;
+  const int nsl = (d + kSlice - 1) / kSlice;
+  const int n_ct = ((kTokenRows ? V : Teff) + kBwdBN - 1) / kBwdBN;
+  const int n_units = ((rows + 127) / 128 + kCtas - 1) / kCtas * nsl;
+  const TailSplit tl = tail_split(n_units, ncl, scratch_cap, n_ct, kBwdOverhead, 1, nsl * 512);
+  const float4 *src = reinterpret_cast<const float4 *>(scratch);
+  const int64_t n4 = (int64_t)tl.R * kRows * kQ;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n4;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int c4 = (int)(e % kQ), row = (int)(e / kQ % kRows), v = (int)(e / (kQ * kRows));
+    const int u = tl.full_end + v, rid = u / nsl * kRows + row, col = u % nsl * kSlice + 4 * c4;
+    if (rid >= rows || col >= d) continue;
+    const float4 t = tail_sum(tl, v, src, kRows * kQ, (int64_t)row * kQ + c4);
+    *reinterpret_cast<float4 *>(out + (kTokenRows ? (int64_t)tok_idx[rid] : (int64_t)rid) * d +
+                                col) = t;
+  }
+}
+
 template <bool kTokenRows, bool kPair>
 pair_status launch_bwd(const char *name, const CUtensorMap &mR, const CUtensorMap &mC,
                        const CUtensorMap &mCs, const GradArgs &g, const GradWorkspace &w, float *out,
-                       cudaStream_t s) {
+                       float *scratch, size_t scratch_bytes, cudaStream_t s) {
   const size_t smem = sizeof(BwdSmem<kPair>) + 1024;
   PAIR_CUDA_TRY(cudaFuncSetAttribute(bwd_kernel<kTokenRows, kPair>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -419,12 +482,22 @@ pair_status launch_bwd(const char *name, const CUtensorMap &mR, const CUtensorMa
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  const int ncl = (num_sms() & ~1) / (kPair ? 2 : 1);
+  size_t cap = scratch_bytes / ((kPair ? 2 : 1) * 128 * kSlice * sizeof(float));
+  if (cap > 1024) cap = 1024;
+  if (!bwd_splits(kTokenRows ? g.T : (int64_t)g.V, g.d, kPair ? 2 : 1)) cap = 0;
   PAIR_BEGIN(name, s);
   PAIR_CUDA_TRY(cudaLaunchKernelEx(&cfg, bwd_kernel<kTokenRows, kPair>, mR, mC, mCs, (int)g.d,
                                    (int)g.V, (const int32_t *)w.counters,
                                    (const int32_t *)w.tok_idx, (const float *)w.tok_c,
-                                   (const float *)w.lse, out, g.dev_err));
+                                   (const float *)w.lse, out, scratch, (int)cap, g.dev_err));
   PAIR_LAUNCH_CHECK(s);
+  if (cap > 0) {
+    PAIR_BEGIN(kTokenRows ? "bwd_dh_tail" : "bwd_dw_tail", s);
+    bwd_tail_kernel<kTokenRows, kPair><<<num_sms() * 2, 256, 0, s>>>(
+        g.d, g.V, ncl, (int)cap, w.counters, w.tok_idx, scratch, out);
+    PAIR_LAUNCH_CHECK(s);
+  }
   return PAIR_OK;
 }
 
@@ -1431,14 +1504,23 @@ bool bwd_pairs(int d, int64_t cols) { return d > 512 && cols >= 2048; }
 
 // Microseconds of bwd_kernel's product with `rows` rows over `cols` columns, by
 // tiles of 128 x 128: in pairs at 1.48 PFLOP/s, else at 2.1 and 0.65 us for the
-// chain (fitted to d = 64 to 1088).
-double bwd_recompute_us(int d, double rows, double cols, int64_t cols_max) {
+// chain (fitted to d = 64 to 1088), and the last round split as far as the scratch
+// allows, about an eighth above its even share.
+double bwd_recompute_us(int d, double rows, double cols, int64_t rows_max, int64_t cols_max,
+                        size_t scratch_bytes) {
   const bool pair = bwd_pairs(d, cols_max);
+  const int ctas = pair ? 2 : 1, ncl = 152 / ctas, slices = (d + kSlice - 1) / kSlice;
   const double flop = 2.0 * 128 * 128 * (d + (d < 256 ? d : 256)) * 152;
   const double tile = pair ? flop / 1.48e9 : 0.65 + flop / 2.1e9;
-  const double blocks = ceil(rows / 128), slices = (d + 255) / 256;
-  const double rounds = pair ? ceil(ceil(blocks / 2) * slices / 76) : ceil(blocks * slices / 152);
-  return rounds * ceil(cols / 128) * tile;
+  const double units = ceil(ceil(rows / 128) / ctas) * slices, n_ct = ceil(cols / 128);
+  const double full = floor(units / ncl), left = units - full * ncl;
+  double last = left > 0 ? n_ct : 0;
+  const double cap = (double)(scratch_bytes / (ctas * 128 * kSlice * sizeof(float)));
+  if (bwd_splits(rows_max, d, ctas) && 2 * left <= cap) {
+    const double share = left / ncl > left / cap ? left / ncl : left / cap;
+    last = fmin(last, 1.125 * share * n_ct + 2 * kBwdOverhead);
+  }
+  return (full * n_ct + last) * tile + 10.0;
 }
 
 // Softmax parts of dH and dW, recomputing the logits.
@@ -1459,18 +1541,27 @@ pair_status grad_bwd_recompute(const GradArgs &g, const GradWorkspace &w, cudaSt
   CUtensorMap mH64, mW64;
   if (!make_map(&mH64, w.Hc, w.Tpad, g.d, 64) || !make_map(&mW64, g.W, g.V, g.d, 64))
     return PAIR_ERR_CUDA;
+  // Scratch for split units: the ring, or for dH, where nothing has written it yet,
+  // dW if that is larger.
+  float *ring = static_cast<float *>(w.gring);
+  const size_t ring_bytes = (size_t)kMaxClusters * kRingBytesPerCluster;
   if (!slab_dh) {
+    const size_t out = (size_t)g.V * g.d * sizeof(float);
+    const bool use_out = !slab_dw && out > ring_bytes;
+    float *scratch = use_out ? g.dW : ring;
+    const size_t bytes = use_out ? out : ring_bytes;
     const pair_status e =
         bwd_pairs(g.d, g.V)
-            ? launch_bwd<true, true>("bwd_dh_tc", mH, mW128, mW64, g, w, g.dH, s)
-            : launch_bwd<true, false>("bwd_dh_tc", mH, mW128, mW64, g, w, g.dH, s);
+            ? launch_bwd<true, true>("bwd_dh_tc", mH, mW128, mW64, g, w, g.dH, scratch, bytes, s)
+            : launch_bwd<true, false>("bwd_dh_tc", mH, mW128, mW64, g, w, g.dH, scratch, bytes, s);
     if (e != PAIR_OK) return e;
   }
   if (!slab_dw) {
     const pair_status e =
         bwd_pairs(g.d, g.T)
-            ? launch_bwd<false, true>("bwd_dw_tc", mW128, mH, mH64, g, w, g.dW, s)
-            : launch_bwd<false, false>("bwd_dw_tc", mW128, mH, mH64, g, w, g.dW, s);
+            ? launch_bwd<false, true>("bwd_dw_tc", mW128, mH, mH64, g, w, g.dW, ring, ring_bytes, s)
+            : launch_bwd<false, false>("bwd_dw_tc", mW128, mH, mH64, g, w, g.dW, ring, ring_bytes,
+                                       s);
     if (e != PAIR_OK) return e;
   }
   return PAIR_OK;

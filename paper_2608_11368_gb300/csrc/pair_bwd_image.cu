@@ -93,127 +93,11 @@ constexpr uint32_t kDhABytes = kAtom128;               // 128 tokens x 64 vocabu
 constexpr uint32_t kDhBBytes = (kDhN / 128) * 64 * 128; // this CTA's 4 column atoms x 64 rows
 constexpr uint32_t kIdescDh = idesc_bf16(256, 256, 0, 1);
 
-// Work list of the persistent backward GEMMs (dh_gemm_kernel,
-// dw_gemm_kernel): the units that fill whole rounds of the grid (ncl
-// clusters) run over all of their K extent; the R < ncl units left over are
-// cut into S parts of K each, which run in as many rounds as they need. Of
-// hidden sizes whose last unit per row block is 256 columns wide (every nq-th of
-// all units), these take half the time and get Sh = ceil(S / 2) parts. Work item
-// i < full_end is unit i; then come parts 0 .. Sh - 1 of all R units, then
-// parts Sh .. S - 1 of the wide ones, part-major: the units that read the same
-// rows of the K-indexed operand in a part run next to each other and share them
-// in L2. Part p covers K steps [p nks / P, (p + 1) nks / P) of its unit's P. The
-// item's fp32 tile goes to the scratch slot of its place in the list and the
-// kernel's tail-combine pass adds a unit's parts in order (deterministic).
-//
-// S is the count of the smallest makespan, rounds x (steps of a part +
-// overhead) + the combine pass's share per tile, of up to 64 and up to the
-// scratch's `cap` tiles; S = 1 needs none. One round of S = ncl / R parts
-// leaves up to half of the clusters idle: 55 units on 76 clusters in one part
-// each take 2374 steps of 64 vocabulary rows, in four 3 x 594 (d = 2560, 11
-// token pairs: 1321 and 1093 us). (Equal contiguous ranges of all R nks steps, one
-// per cluster, leave none idle but read each W row at R different times:
-// 1.35 times as slow as whole parts, from DRAM.)
-struct TailSplit {
-  int full_end, R, S, Sh;
-  int Rh, h0, nq;  // narrow units among the R: at h0, h0 + nq, ...
-
-  __device__ __forceinline__ int items() const { return R * Sh + (R - Rh) * (S - Sh); }
-  __device__ __forceinline__ bool narrow(int v) const {
-    return Rh > 0 && v >= h0 && (v - h0) % nq == 0;
-  }
-  __device__ __forceinline__ int parts(int v) const { return narrow(v) ? Sh : S; }
-  // The j-th wide unit, and the number of wide ones before unit v.
-  __device__ __forceinline__ int wide_at(int j) const {
-    return j < h0 ? j : j + 1 + (j - h0) / (nq - 1);
-  }
-  __device__ __forceinline__ int wide_before(int v) const {
-    return v > h0 ? v - 1 - (v - 1 - h0) / nq : v;
-  }
-};
-constexpr int kTailMaxParts = 64;
-// A whole warp calls (every lane gets the answer). d gives the units' widths.
-__device__ __forceinline__ TailSplit tail_split(int n_units, int ncl, int cap, int nks,
-                                                int overhead, int d) {
-  TailSplit t{n_units, 0, 1, 1, 0, 0, (d + 511) / 512};
-  const int R = n_units % ncl;
-  if (R == 0 || nks == 0) return t;
-  t.R = R;
-  t.h0 = t.nq - 1 - (n_units - R) % t.nq;
-  if (t.nq > 1 && d % 512 != 0 && d % 512 <= 256 && R > t.h0)
-    t.Rh = 1 + (R - 1 - t.h0) / t.nq;
-  unsigned long long best = ~0ull;
-  for (int S = 1 + (threadIdx.x & 31); S <= min(kTailMaxParts, nks); S += 32) {
-    t.S = S;
-    t.Sh = t.Rh > 0 ? (S + 1) / 2 : S;
-    const int n = t.items();
-    if (S > 1 && n > cap) break;
-    const long long rounds = (n + ncl - 1) / ncl, steps = (nks + S - 1) / S;
-    const long long cost = 8 * rounds * (steps + overhead) + (S > 1 ? 2 * n : 0);
-    best = min(best, (unsigned long long)cost * (2 * kTailMaxParts) + S);
-  }
-  for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
-  t.S = (int)(best % (2 * kTailMaxParts));
-  t.Sh = t.Rh > 0 ? (t.S + 1) / 2 : t.S;
-  if (t.S < 2) return TailSplit{n_units, 0, 1, 1, 0, 0, t.nq};
-  t.full_end = n_units - R;
-  return t;
-}
-// Work item i of a TailSplit -> unit u, its K steps [k0, k1) and scratch
-// slot (-1: a whole unit).
-__device__ __forceinline__ void tail_item(const TailSplit &tl, int nks, int i, int &u, int &k0,
-                                          int &k1, int &slot) {
-  if (i < tl.full_end) {
-    u = i; k0 = 0; k1 = nks; slot = -1;
-  } else {
-    const int j = i - tl.full_end, all = tl.R * tl.Sh, wide = tl.R - tl.Rh;
-    int part, v;
-    if (j < all) {
-      part = j / tl.R;
-      v = j - part * tl.R;
-    } else {
-      part = (j - all) / wide;
-      v = tl.wide_at(j - all - part * wide);
-      part += tl.Sh;
-    }
-    const int parts = tl.parts(v);
-    u = tl.full_end + v;
-    k0 = (int)((int64_t)part * nks / parts);
-    k1 = (int)((int64_t)(part + 1) * nks / parts);
-    slot = j;
-  }
-}
-// Sum of unit full_end + v's parts at float4 `at` of their tiles (`tile`
-// float4 each), in part order; eight loads in flight.
-__device__ __forceinline__ float4 tail_sum(const TailSplit &tl, int v, const float4 *src,
-                                           int64_t tile, int64_t at) {
-  float4 acc = src[v * tile + at];
-  auto add = [&](const float4 *p, int64_t stride, int n) {
-    int k = 0;
-    for (; k + 8 <= n; k += 8, p += 8 * stride) {
-      float4 x[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) x[q] = p[q * stride];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        acc.x += x[q].x; acc.y += x[q].y; acc.z += x[q].z; acc.w += x[q].w;
-      }
-    }
-    for (; k < n; ++k, p += stride) {
-      const float4 x = *p;
-      acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
-    }
-  };
-  add(src + (tl.R + v) * tile + at, tl.R * tile, tl.Sh - 1);
-  if (!tl.narrow(v))
-    add(src + ((int64_t)tl.R * tl.Sh + tl.wide_before(v)) * tile + at, (tl.R - tl.Rh) * tile,
-        tl.S - tl.Sh);
-  return acc;
-}
 // An item's start and drain in K steps: a step of dh is 64 vocabulary rows,
 // about 0.6 us, of dw 32 tokens, half of that; filling the pipeline and
 // writing a 2 x 128 x 512 tile take about twelve microseconds.
-constexpr int kDhOverhead = 20, kDwOverhead = 40;
+// A scratch tile's share of the combine pass: 16/64 of a step.
+constexpr int kDhOverhead = 20, kDwOverhead = 40, kGemmTile = 16;
 
 // Pacing of dh_gemm_kernel's whole units: the CTA pairs of a round read the
 // same W rows (all of them read all of W, in step order) and four at a time
@@ -272,7 +156,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int nks = 2 * n_vt;  // 64-wide vocabulary steps (image atoms)
   const int nq = (d + kDhN - 1) / kDhN;
   const int n_units = (nrb + 1) / 2 * nq;
-  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDhOverhead, d);
+  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDhOverhead, kGemmTile, d);
   const int n_items = tl.full_end + tl.items();
 
   if (threadIdx.x == 0) {
@@ -457,7 +341,7 @@ __global__ void __launch_bounds__(256)
   if (nrb == 0) return;
   const int nks = 2 * ((V + 127) / 128);
   const int nq = (d + kDhN - 1) / kDhN;
-  const TailSplit tl = tail_split((nrb + 1) / 2 * nq, ncl, scratch_cap, nks, kDhOverhead, d);
+  const TailSplit tl = tail_split((nrb + 1) / 2 * nq, ncl, scratch_cap, nks, kDhOverhead, kGemmTile, d);
   constexpr int kQ = kDhN / 4;  // float4 per tile row
   const int64_t n4 = (int64_t)tl.R * 2 * 128 * kQ;
   const float4 *src = reinterpret_cast<const float4 *>(scratch);
@@ -549,7 +433,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int nq = (d + kDwN - 1) / kDwN;
   const int n_units = (n_vb + 1) / 2 * nq;
   const int nks = nrb * (128 / kDwKS);
-  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDwOverhead, d);
+  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, nks, kDwOverhead, kGemmTile, d);
   const int n_items = tl.full_end + tl.items();
 
   if (threadIdx.x == 0) {
@@ -761,7 +645,7 @@ __global__ void __launch_bounds__(256)
   const int nrb = min(max((Teff + 127) / 128 - rb0, 0), cap);
   const int nq = (d + kDwN - 1) / kDwN;
   const int nks = nrb * (128 / kDwKS);
-  const TailSplit tl = tail_split((n_vb + 1) / 2 * nq, ncl, scratch_cap, nks, kDwOverhead, d);
+  const TailSplit tl = tail_split((n_vb + 1) / 2 * nq, ncl, scratch_cap, nks, kDwOverhead, kGemmTile, d);
   constexpr int kQ = kDwN / 4;  // float4 per tile row
   const int64_t n4 = (int64_t)tl.R * 2 * 128 * kQ;
   const float4 *src = reinterpret_cast<const float4 *>(scratch);
@@ -874,7 +758,7 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
 //
 // Each chunk and each slab costs its launches, short K loops and drains, about
 // kSlabUs (dH: kSlabDhUs beside the GEMM's makespan), so each product takes the
-// cheaper form by a model: bwd_kernel's rounds of units (bwd_recompute_us), or two
+// cheaper form by a model: bwd_kernel's (bwd_recompute_us), or two
 // logit-sized products at 1.6 PFLOP/s and the parts' cost. Measured on one GB300
 // against bwd_kernel: d = 2432, V = 60,000, 1.5 k tokens (one chunk, four slabs)
 // 9.2 -> 1.15 ms for the call; d = 1216, V = 30,000, 5 k tokens (5 chunks, 13
@@ -977,8 +861,10 @@ void slabs_choose(const GradArgs &g, const SlabPlan &p, bool &dh, bool &dw) {
   dh = dw = false;
   if (p.chunk < 1) return;
   const double tokens = 2.0 / 3.0 * g.T;
-  const double old_dh = bwd_recompute_us(g.d, tokens, g.V, g.V);
-  const double old_dw = bwd_recompute_us(g.d, g.V, tokens, g.T);
+  const size_t out = (size_t)g.V * g.d * sizeof(float);
+  const double old_dh =
+      bwd_recompute_us(g.d, tokens, g.V, g.T, g.V, out > p.ring ? out : p.ring);
+  const double old_dw = bwd_recompute_us(g.d, g.V, tokens, g.V, g.T, p.ring);
   const double two = 4.0 * tokens * g.V * g.d / 1.6e9;
   dh = p.dh_us < old_dh;
   if (two + kSlabUs >= old_dw) return;

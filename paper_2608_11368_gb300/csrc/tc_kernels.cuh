@@ -85,6 +85,126 @@ __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
+// Work list of the persistent backward kernels (dh_gemm_kernel,
+// dw_gemm_kernel, bwd_kernel): the units that fill whole rounds of the grid (ncl
+// clusters or CTAs) run over all of their K extent; the R < ncl units left over are
+// cut into S parts of K each, which run in as many rounds as they need. Of
+// hidden sizes whose last unit per row block is 256 columns wide (every nq-th of
+// all units), these take half the time and get Sh = ceil(S / 2) parts. Work item
+// i < full_end is unit i; then come parts 0 .. Sh - 1 of all R units, then
+// parts Sh .. S - 1 of the wide ones, part-major: the units that read the same
+// rows of the K-indexed operand in a part run next to each other and share them
+// in L2. Part p covers K steps [p nks / P, (p + 1) nks / P) of its unit's P. The
+// item's fp32 tile goes to the scratch slot of its place in the list and the
+// kernel's tail-combine pass adds a unit's parts in order (deterministic).
+//
+// S is the count of the smallest makespan, rounds x (steps of a part +
+// overhead) + the combine pass's share per tile, of up to 64 and up to the
+// scratch's `cap` tiles; S = 1 needs none. One round of S = ncl / R parts
+// leaves up to half of the clusters idle: 55 units on 76 clusters in one part
+// each take 2374 steps of 64 vocabulary rows, in four 3 x 594 (d = 2560, 11
+// token pairs: 1321 and 1093 us). (Equal contiguous ranges of all R nks steps, one
+// per cluster, leave none idle but read each W row at R different times:
+// 1.35 times as slow as whole parts, from DRAM.)
+struct TailSplit {
+  int full_end, R, S, Sh;
+  int Rh, h0, nq;  // narrow units among the R: at h0, h0 + nq, ...
+
+  __device__ __forceinline__ int items() const { return R * Sh + (R - Rh) * (S - Sh); }
+  __device__ __forceinline__ bool narrow(int v) const {
+    return Rh > 0 && v >= h0 && (v - h0) % nq == 0;
+  }
+  __device__ __forceinline__ int parts(int v) const { return narrow(v) ? Sh : S; }
+  // The j-th wide unit, and the number of wide ones before unit v.
+  __device__ __forceinline__ int wide_at(int j) const {
+    return j < h0 ? j : j + 1 + (j - h0) / (nq - 1);
+  }
+  __device__ __forceinline__ int wide_before(int v) const {
+    return v > h0 ? v - 1 - (v - 1 - h0) / nq : v;
+  }
+};
+constexpr int kTailMaxParts = 64;
+// A whole warp calls (every lane gets the answer). d gives the units' widths (a
+// multiple of 512: all alike); `tile` is the combine pass's share per scratch tile
+// in 1/64 steps.
+__device__ __forceinline__ TailSplit tail_split(int n_units, int ncl, int cap, int nks,
+                                                int overhead, int tile, int d) {
+  TailSplit t{n_units, 0, 1, 1, 0, 0, (d + 511) / 512};
+  const int R = n_units % ncl;
+  if (R == 0 || nks == 0) return t;
+  t.R = R;
+  t.h0 = t.nq - 1 - (n_units - R) % t.nq;
+  if (t.nq > 1 && d % 512 != 0 && d % 512 <= 256 && R > t.h0)
+    t.Rh = 1 + (R - 1 - t.h0) / t.nq;
+  unsigned long long best = ~0ull;
+  for (int S = 1 + (threadIdx.x & 31); S <= min(kTailMaxParts, nks); S += 32) {
+    t.S = S;
+    t.Sh = t.Rh > 0 ? (S + 1) / 2 : S;
+    const int n = t.items();
+    if (S > 1 && n > cap) break;
+    const long long rounds = (n + ncl - 1) / ncl, steps = (nks + S - 1) / S;
+    const long long cost = 64 * rounds * (steps + overhead) + (S > 1 ? (long long)tile * n : 0);
+    best = min(best, (unsigned long long)cost * (2 * kTailMaxParts) + S);
+  }
+  for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
+  t.S = (int)(best % (2 * kTailMaxParts));
+  t.Sh = t.Rh > 0 ? (t.S + 1) / 2 : t.S;
+  if (t.S < 2) return TailSplit{n_units, 0, 1, 1, 0, 0, t.nq};
+  t.full_end = n_units - R;
+  return t;
+}
+// Work item i of a TailSplit -> unit u, its K steps [k0, k1) and scratch
+// slot (-1: a whole unit).
+__device__ __forceinline__ void tail_item(const TailSplit &tl, int nks, int i, int &u, int &k0,
+                                          int &k1, int &slot) {
+  if (i < tl.full_end) {
+    u = i; k0 = 0; k1 = nks; slot = -1;
+  } else {
+    const int j = i - tl.full_end, all = tl.R * tl.Sh, wide = tl.R - tl.Rh;
+    int part, v;
+    if (j < all) {
+      part = j / tl.R;
+      v = j - part * tl.R;
+    } else {
+      part = (j - all) / wide;
+      v = tl.wide_at(j - all - part * wide);
+      part += tl.Sh;
+    }
+    const int parts = tl.parts(v);
+    u = tl.full_end + v;
+    k0 = (int)((int64_t)part * nks / parts);
+    k1 = (int)((int64_t)(part + 1) * nks / parts);
+    slot = j;
+  }
+}
+// Sum of unit full_end + v's parts at float4 `at` of their tiles (`tile`
+// float4 each), in part order; eight loads in flight.
+__device__ __forceinline__ float4 tail_sum(const TailSplit &tl, int v, const float4 *src,
+                                           int64_t tile, int64_t at) {
+  float4 acc = src[v * tile + at];
+  auto add = [&](const float4 *p, int64_t stride, int n) {
+    int k = 0;
+    for (; k + 8 <= n; k += 8, p += 8 * stride) {
+      float4 x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) x[q] = p[q * stride];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        acc.x += x[q].x; acc.y += x[q].y; acc.z += x[q].z; acc.w += x[q].w;
+      }
+    }
+    for (; k < n; ++k, p += stride) {
+      const float4 x = *p;
+      acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
+    }
+  };
+  add(src + (tl.R + v) * tile + at, tl.R * tile, tl.Sh - 1);
+  if (!tl.narrow(v))
+    add(src + ((int64_t)tl.R * tl.Sh + tl.wide_before(v)) * tile + at, (tl.R - tl.Rh) * tile,
+        tl.S - tl.Sh);
+  return acc;
+}
+
 // ---- host helpers (pair_grad_tc.cu)
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn();
 // 2-D bf16 row-major [rows][cols] map with 64 x box_rows SWIZZLE_128B boxes.
@@ -119,7 +239,8 @@ pair_status grad_bwd_slabs(const GradArgs &g, const GradWorkspace &w, cudaStream
                            bool &dw);
 // Backward without an image, recomputing the logits (pair_bwd_cluster.cu), and
 // what one of its products takes where no cluster form applies.
-double bwd_recompute_us(int d, double rows, double cols, int64_t cols_max);
+double bwd_recompute_us(int d, double rows, double cols, int64_t rows_max, int64_t cols_max,
+                        size_t scratch_bytes);
 pair_status grad_bwd_recompute(const GradArgs &g, const GradWorkspace &w, cudaStream_t s);
 // Whole head without an image: fused log-sum-exp + dH, then dW (cluster
 // form; d = 512 A, A <= 6). lse, zy and dH, dW softmax parts as the

@@ -1,8 +1,9 @@
-"""The recomputing backward of bf16 hidden sizes without an image (two row blocks
-and 256 columns of d per CTA pair): last slices of 64, 128, 192 and 256 columns,
-one, odd and even numbers of token and vocabulary blocks, ragged ends of both,
-and more units than pairs. Checked as in test_gpu_grad.py; reruns are
-bit-identical."""
+"""The recomputing backward of bf16 hidden sizes without an image (a row block
+and 256 columns of d per CTA; two row blocks per CTA pair): last slices of 64,
+128, 192 and 256 columns, one, odd and even numbers of token and vocabulary
+blocks, ragged ends of both, units split over parts of the other side (scratch
+in the ring and in dW), and more units than CTAs. Checked as in
+test_gpu_grad.py; reruns are bit-identical."""
 import pytest
 import torch
 
@@ -21,7 +22,9 @@ pytestmark = pytest.mark.gpu
     (448, 257, 1, 8, 0.3),      # of 192
     (640, 2000, 1, 4, 0.06),
     (128, 24000, 1, 4, 0.2),    # dW: more units than pairs
-    (960, 1024, 2, 8, 0.3),     # four slices, the last of 192
+    (256, 16000, 1, 4, 0.3),    # dH split, its scratch in dW
+    (704, 2100, 2, 8, 0.3),     # pairs, an odd number of vocabulary blocks, dW split
+    (960, 1024, 2, 8, 0.3),     # dW in pairs; four slices, the last of 192
 ])
 def test_recompute(d, V, B, G, ls):
     inp = synth.make_head_workload(synth.WORKLOADS["qwen3_1p7b_head"], 17, B=B, G=G, d=d, V=V,
