@@ -20,7 +20,8 @@ CASES = [
     # d, V, B, G, len_scale: the launches the model of the dispatch picks
     (2496, 2050, 1, 4, 0.45),  # all tiles in the ring; last unit 448 columns: two halves
     (1216, 7000, 1, 8, 0.25),  # dH in one chunk, dW recomputed; last unit 192 columns: one half
-    (2496, 5000, 2, 8, 0.28),  # two dH chunks and four dW slabs
+    (2496, 5000, 2, 8, 0.28),  # one dH chunk and three dW slabs
+    (1216, 9000, 2, 8, 0.6),   # five dH chunks, narrow last units split in half as many parts
     (4096, 3000, 1, 8, 0.25),  # d beyond the cluster form, minimum workspace
     (320, 777, 2, 4, 0.1),     # too small for either
 ]
