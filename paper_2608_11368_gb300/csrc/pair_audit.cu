@@ -11,19 +11,23 @@
 //   ||ghat_b - g||^2 = e_b^T K e_b,  e_b = a_b - abar,
 //   <ghat_b, g> = a_b^T K abar,  ||ghat_b||^2 = a_b^T K a_b,
 //   E[ghat] - g = (E[a] - abar) S.
-// K, abar and the quadratic forms are accumulated in fp64; the coefficients
-// are the fp32 pair_coeffs_weighted values of each draw.
+// K, abar, the coefficients' division, centring and scale and the quadratic forms
+// are fp64, on row sums of the terms' fp64 quotients (see audit_draws_kernel).
 //
 // A draw's terms (r_i - r_j) w_ij are the same for every draw, so they and the
 // weights are formed once per block and a draw only adds the ones of its
 // completed pairs. The draws run one per lane, 32 at a time: no exchange
 // between lanes, uniform (broadcast) reads of the terms and of K, and every
-// lane of the fp64 pipe busy, which is what bounds the pass: about G^2 / 2 + 4 G
+// lane of the fp64 pipe busy, which is what bounds the pass: about G^2 / 2 + 5 G
 // fp64 operations per draw at 2 per clock and SM. Measured on one GB300, 50,000
-// draws of 16 candidates with D = 4096: the call takes
-// 90 us, its draws pass 57 us; one block per draw, with a tree and five block
-// reductions each, took 653 and 500 us. For G = 64 and 128 (3125 and 781
-// draws) the call takes 0.16 and 0.43 ms, from 0.75 and 1.37 ms.
+// draws of 16 candidates with D = 4096: the call takes 100 us, its draws pass 73
+// us; one block per draw, with a tree and five block reductions each, took 653 and
+// 500 us. For G = 64 and 128 (3125 and 781 draws) the call takes 0.18 and 0.48
+// ms, from 0.75 and 1.37 ms.
+#include <math.h>
+
+#include <type_traits>
+
 #include "pair_coeffs_dev.cuh"
 
 namespace pairk {
@@ -131,13 +135,15 @@ __host__ __device__ __forceinline__ int audit_team(int G) { return G <= 32 ? 1 :
 // Warps per block: small ones of single-warp teams, so that the last round of
 // blocks leaves few SMs idle (50,000 draws of 16 are 1563 batches).
 __host__ __device__ __forceinline__ constexpr int audit_warps(int team) { return team == 1 ? 4 : team; }
+// Whether the terms' low parts fit in shared memory too.
+inline bool audit_split(int G) { return G <= 120; }
 inline size_t audit_draws_smem(int G) {
   const size_t warps = audit_warps(audit_team(G)), teams = warps / audit_team(G);
   return sizeof(double) * (audit_tri(G) + G            // K
                            + 2 * (size_t)G             // abar, u
                            + teams * 2 * 32 * (size_t)G  // e, sums of a
                            + warps * 4 * 32)             // exchanges of a team
-         + sizeof(float) * (2 * audit_tri(G) + 2 * (size_t)G)  // terms, weights, r, pi
+         + sizeof(float) * ((audit_split(G) ? 3 : 2) * audit_tri(G) + 2 * (size_t)G)  // terms, weights, r, pi
          + sizeof(uint32_t) * warps * 4 * 32;    // completion bits
 }
 
@@ -164,14 +170,30 @@ __device__ __forceinline__ T team_sum(double *xch, int slot, T v) {
   }
 }
 
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("add.rn.f32x2 %0, %1, %2;"
+      : "=l"(reinterpret_cast<unsigned long long &>(d))
+      : "l"(reinterpret_cast<unsigned long long &>(a)),
+        "l"(reinterpret_cast<unsigned long long &>(b)));
+  return d;
+}
+
 // Draws in batches of 32, one per lane; batch q of the teams' stride. Row i of
-// a batch belongs to warp i mod TW of its team. Per draw: the row sums
-// a_i = 1/2 sum_j J_i J_j t_ij (16-term trees, combined pairwise) and the weight
-// sums, the weighting's and flags' division and centring, then in fp64
-// e = a - abar, e^T K e over the lower triangle, e^T u. With a = e + abar,
+// a batch belongs to warp i mod TW of its team. Per draw: the row sums 2 a_i =
+// sum_j J_i J_j t_ij and the weight sums, then in fp64 the weighting's and flags'
+// division and centring, e = a - abar, e^T K e over the lower triangle, e^T u. With a = e + abar,
 // u = K abar and gg = abar^T u: a^T u = e^T u + gg and
 // a^T K a = e^T K e + 2 e^T u + gg (0 exactly where a = 0).
-template <int TW>
+//
+// SPLIT: a term is kept as t = hi + lo, hi a multiple of q = 2^-24 times the power
+// of two above G max |t|, so that fp32 sums of hi are exact in any order, and lo <=
+// q / 2 the rest of the fp64 quotient: the pair is summed by one packed addition,
+// and a is good to some 2^-40 of the largest term where fp32 terms and trees left
+// 1e-6 of the bias, a small remainder of such sums (2.4e-6 -> 5e-8 relative, the
+// rounding of scale; the draws of the size above 57 -> 73 us). Otherwise (G > 120) fp32 terms in 16-term trees, combined
+// pairwise.
+template <int TW, bool SPLIT>
 __global__ void __launch_bounds__(audit_warps(TW) * 32)
     audit_draws_kernel(int N, int G, const float *__restrict__ r, const float *__restrict__ rho,
                        const uint8_t *__restrict__ Jd, const double *__restrict__ wd, float scale,
@@ -187,13 +209,16 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
   double *abar = K + tri + G, *u = abar + G;
   double *e_all = u + G, *asum_all = e_all + kTeams * 32 * G;
   double *xch = asum_all + kTeams * 32 * G;
-  float *T = reinterpret_cast<float *>(xch + kWarps * 4 * 32);
-  float *Wt = T + tri, *rs = Wt + tri, *pis = rs + G;
+  using Term = std::conditional_t<SPLIT, float2, float>;
+  Term *T = reinterpret_cast<Term *>(xch + kWarps * 4 * 32);
+  float *Wt = reinterpret_cast<float *>(T + tri), *rs = Wt + tri, *pis = rs + G;
   uint32_t *bits_all = reinterpret_cast<uint32_t *>(pis + G);
   double *e = e_all + team * 32 * G, *asum = asum_all + team * 32 * G;
   uint32_t *bits = bits_all + team * 4 * 32;
 
   // ---- the group's constants
+  __shared__ unsigned t_max;  // bits of the largest |t|
+  if (threadIdx.x == 0) t_max = 0u;
   for (int i = threadIdx.x; i < G; i += blockDim.x) {
     abar[i] = abar_g[i];
     u[i] = u_g[i];
@@ -202,6 +227,53 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
   }
   for (int k = threadIdx.x; k < kTeams * 32 * G; k += blockDim.x) asum_all[k] = 0.0;
   __syncthreads();
+  // Weight and term of pair (j, i), j < i (entry (j, i) of rho's strict upper
+  // triangle). An invalid weight is NaN here and raises the error bit in the
+  // draws that complete it.
+  auto pair_term = [&](int j, int i, float &w) -> double {
+    const double dr = (double)rs[i] - (double)rs[j];
+    w = 1.f;
+    if (wmode == PAIR_W_MARGINAL) {
+      const bool ok = pis[i] > 0.f && pis[j] > 0.f;
+      w = ok ? __frcp_rn(pis[j] * pis[i]) : __int_as_float(0x7fc00000);
+      return ok ? dr / ((double)pis[j] * (double)pis[i]) : 0.0;
+    }
+    if (wmode == PAIR_W_UNWEIGHTED) return dr;
+    const float rij = rho[(size_t)j * G + i];
+    const bool ok = rij > 0.f;
+    w = ok ? __frcp_rn(rij) : __int_as_float(0x7fc00000);
+    if (wmode == PAIR_W_CLIPPED && w > w_max) {
+      w = w_max;
+      return dr * (double)w_max;
+    }
+    return ok ? dr / (double)rij : 0.0;
+  };
+  // 2^-24 of the power of two above G max |t|, and its reciprocal.
+  double q = 0.0, q_inv = 0.0;
+  if constexpr (SPLIT) {
+    // max |t| from fp32 quotients, which round up to 3 ulp off.
+    float m = 0.f;
+    for (int j = warp; j < G; j += kWarps)
+      for (int i = j + 1 + lane; i < G; i += 32) {
+        float t = fabsf(rs[i] - rs[j]);
+        if (wmode == PAIR_W_MARGINAL) {
+          if (pis[i] > 0.f && pis[j] > 0.f) t = __fdividef(t, pis[j] * pis[i]);
+        } else if (wmode != PAIR_W_UNWEIGHTED) {
+          const float rij = rho[(size_t)j * G + i];
+          if (rij > 0.f) t *= __frcp_rn(rij);
+        }
+        m = fmaxf(m, t);
+      }
+    atomicMax(&t_max, __float_as_uint(m));
+    __syncthreads();
+    const double top = 1.000001 * (double)G * (double)__uint_as_float(t_max);
+    if (top > 1e-30 && top < 1e38) {
+      int e;
+      frexp(top, &e);
+      q = ldexp(1.0, e - 24);
+      q_inv = ldexp(1.0, 24 - e);
+    }
+  }
   for (int j = warp; j < G; j += kWarps) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -209,26 +281,17 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
       if (i >= G) continue;
       K[i * (i + 1) / 2 + j] = Kg[(size_t)j * G + i];
       if (i == j) continue;
-      // Entry (j, i) of rho's strict upper triangle. An invalid weight is
-      // NaN here and raises the error bit in the draws that complete it.
-      const float dr = rs[i] - rs[j];
-      float w = 1.f, t = dr;
-      if (wmode == PAIR_W_MARGINAL) {
-        const float den = pis[j] * pis[i];
-        const bool ok = pis[i] > 0.f && pis[j] > 0.f;
-        w = ok ? __frcp_rn(den) : __int_as_float(0x7fc00000);
-        t = ok ? __fdiv_rn(dr, den) : 0.f;
-      } else if (wmode != PAIR_W_UNWEIGHTED) {
-        const float rij = rho[(size_t)j * G + i];
-        const bool ok = rij > 0.f;
-        w = ok ? __frcp_rn(rij) : __int_as_float(0x7fc00000);
-        t = ok ? __fdiv_rn(dr, rij) : 0.f;
-        if (wmode == PAIR_W_CLIPPED && w > w_max) {
-          w = w_max;
-          t = dr * w_max;
-        }
+      float w;
+      const double t = pair_term(j, i, w);
+      Term &o = T[i * (i - 1) / 2 + j];
+      if constexpr (SPLIT) {
+        // (Where no q serves, the largest term being 0, tiny or beyond fp32's range
+        // over G, hi is t itself.)
+        const double hi = q > 0.0 ? rint(t * q_inv) * q : (double)(float)t;
+        o = make_float2((float)hi, isfinite((float)hi) ? (float)(t - hi) : 0.f);
+      } else {
+        o = (float)t;
       }
-      T[i * (i - 1) / 2 + j] = t;
       Wt[i * (i - 1) / 2 + j] = w;
     }
   }
@@ -272,71 +335,100 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
     const int Kc = __popc(m[0]) + __popc(m[1]) + __popc(m[2]) + __popc(m[3]);
 
     // ---- row sums
-    float W = 0.f, W2 = 0.f, s_a = 0.f;
+    float W = 0.f, W2 = 0.f;
+    double s_a = 0.0;
     for (int i = tw; i < G; i += TW) {
-      const float *row = T + i * (i - 1) / 2, *wrow = Wt + i * (i - 1) / 2;
+      const Term *row = T + i * (i - 1) / 2;
+      const float *wrow = Wt + i * (i - 1) / 2;
       const bool on = done(i);
-      float p[4] = {0.f, 0.f, 0.f, 0.f};
       float sw = 0.f, sw2 = 0.f;
+      double a = 0.0;
+      if constexpr (SPLIT) {
+        float2 x[4];
 #pragma unroll
-      for (int blk = 0; blk < 8; ++blk) {
-        float c = 0.f;
-        if (blk * 16 < G) {
+        for (int q = 0; q < 4; ++q) x[q] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int blk = 0; blk < (TW == 1 ? 2 : 8); ++blk) {
+          if (blk * 16 >= G) break;
           const uint32_t mb = m[blk >> 1] >> ((blk & 1) * 16);
-          float x[16], wb = 0.f, wb2 = 0.f;
+          float wb = 0.f, wb2 = 0.f;
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
             const int j = blk * 16 + q;
-            // Uniform over the warp: which triangle, and past the group.
-            float t = 0.f;
             const bool jon = (mb >> q) & 1u;
+            // Uniform over the warp: which triangle, and past the group.
+            float2 t = make_float2(0.f, 0.f);
             if (j < i) {
               t = row[j];
               const float w = jon ? wrow[j] : 0.f;
               wb += w;
               wb2 = fmaf(w, w, wb2);
             } else if (j > i && j < G) {
-              t = -T[j * (j - 1) / 2 + i];
+              t = T[j * (j - 1) / 2 + i];
+              t = make_float2(-t.x, -t.y);
             }
-            x[q] = jon ? t : 0.f;
+            x[q & 3] = add2(x[q & 3], make_float2(jon ? t.x : 0.f, jon ? t.y : 0.f));
           }
           sw += wb;
           sw2 += wb2;
-#pragma unroll
-          for (int o = 8; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q < o; ++q) x[q] += x[q + o];
-          c = x[0];
         }
-        int mm = blk;
+        const float2 y = add2(add2(x[0], x[1]), add2(x[2], x[3]));
+        if (on) a = (double)y.x + (double)y.y;
+      } else {
+        float p[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int l = 0; l < 4; ++l) {
-          if (mm & 1) { c = p[l] + c; mm >>= 1; }
-          else { p[l] = c; break; }
+        for (int blk = 0; blk < 8; ++blk) {
+          float c = 0.f;
+          if (blk * 16 < G) {
+            const uint32_t mb = m[blk >> 1] >> ((blk & 1) * 16);
+            float x[16], wb = 0.f, wb2 = 0.f;
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+              const int j = blk * 16 + q;
+              const bool jon = (mb >> q) & 1u;
+              float t = 0.f;
+              if (j < i) {
+                t = row[j];
+                const float w = jon ? wrow[j] : 0.f;
+                wb += w;
+                wb2 = fmaf(w, w, wb2);
+              } else if (j > i && j < G) {
+                t = -T[j * (j - 1) / 2 + i];
+              }
+              x[q] = jon ? t : 0.f;
+            }
+            sw += wb;
+            sw2 += wb2;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+              for (int q = 0; q < o; ++q) x[q] += x[q + o];
+            c = x[0];
+          }
+          int mm = blk;
+#pragma unroll
+          for (int l = 0; l < 4; ++l) {
+            if (mm & 1) { c = p[l] + c; mm >>= 1; }
+            else { p[l] = c; break; }
+          }
         }
+        if (on) a = (double)p[3];
       }
-      const float a = on ? 0.5f * p[3] : 0.f;
       if (on) {
         W += sw;
         W2 += sw2;
       }
       s_a += a;
-      reinterpret_cast<float *>(e + (size_t)i * 32)[lane] = a;  // first half of the row's cells
+      e[i * 32 + lane] = a;
     }
     W = team_sum<TW>(xch, 0, W);
     W2 = team_sum<TW>(xch, 1, W2);
     if (W != W) flag_error(dev_err, PAIR_DEV_ERR_NONPOSITIVE_INCLUSION);
 
-    // ---- the divisions and the centring of the coefficients
-    float div = 1.f;
-    bool divide = false, zero = false;
-    if (wmode == PAIR_W_HAJEK) {
-      zero = !(W > 0.f);
-      div = W;
-      divide = !zero;
-    }
-    float sd = 1.f;
-    bool standard = false;
+    // ---- the divisions, the centring and the scale of the coefficients:
+    // a_i -> f (a_i - mean), a half of f being the row sums'
+    double f = 0.5 * (double)scale;
+    if (wmode == PAIR_W_HAJEK) f = W > 0.f ? f / (double)W : 0.0;
     if ((flags & PAIR_STANDARDIZE) && Kc >= 2) {
       float sr = 0.f, ss = 0.f;
       for (int i = 0; i < G; ++i) sr += done(i) ? rs[i] : 0.f;
@@ -345,40 +437,27 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
         const float dv = done(i) ? rs[i] - mean : 0.f;
         ss = fmaf(dv, dv, ss);
       }
-      sd = sqrtf(ss / (float)(Kc - 1));
-      standard = true;
+      const float sd = sqrtf(ss / (float)(Kc - 1));
+      f = sd > 0.f ? f / (double)sd : 0.0;
     }
-    auto finish = [&](float a) {
-      if (zero) a = 0.f;
-      else if (divide) a = __fdiv_rn(a, div);
-      if (standard) a = sd > 0.f ? __fdiv_rn(a, sd) : 0.f;
-      return a;
-    };
-    float mean_a = 0.f;
+    double mean_a = 0.0;
     if (flags & PAIR_CENTER) {
-      if (divide || zero || standard) {
-        s_a = 0.f;
-        for (int i = tw; i < G; i += TW)
-          s_a += finish(reinterpret_cast<float *>(e + (size_t)i * 32)[lane]);
-      }
       s_a = team_sum<TW>(xch, 2, s_a);
-      mean_a = Kc > 0 ? s_a / (float)Kc : 0.f;
+      mean_a = Kc > 0 ? s_a / (double)Kc : 0.0;
     }
 
     // ---- fp64: e = a - abar, the sums of a, e^T u
     const int b = bt * 32 + lane;
-    const double w = b < N ? (wd ? wd[b] : w_all) : 0.0;
+    const double w = b < N ? (wd ? wd[b] : w_all) : 0.0, wf = w * f;
     double eu = 0.0;
-    bool any = false;
+    bool any = false;  // (of a before its factor; f = 0 is checked below)
     for (int i = tw; i < G; i += TW) {
-      float a = finish(reinterpret_cast<float *>(e + (size_t)i * 32)[lane]);
-      if (done(i)) a -= mean_a;
-      a *= scale;
-      any |= a != 0.f;
-      const double ad = (double)a, ei = ad - abar[i];
-      __syncwarp();  // the row's fp32 cells are read before its fp64 ones are written
+      double a = e[i * 32 + lane];
+      if ((flags & PAIR_CENTER) && done(i)) a -= mean_a;
+      any |= a != 0.0;
+      const double ei = fma(a, f, -abar[i]);
       e[i * 32 + lane] = ei;
-      asum[i * 32 + lane] = fma(w, ad, asum[i * 32 + lane]);
+      asum[i * 32 + lane] = fma(wf, a, asum[i * 32 + lane]);
       eu = fma(ei, u[i], eu);
     }
     team_sync<TW>();
@@ -403,7 +482,7 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
     eu = team_sum<TW>(xch, 3, eu);
     if constexpr (TW > 1) any = team_sum<TW>(xch, 0, any ? 1.f : 0.f) > 0.f;
     if (tw == 0) {
-      const double q_au = eu + gg, q_aa = any ? q + 2.0 * eu + gg : 0.0;
+      const double q_au = eu + gg, q_aa = any && f != 0.0 ? q + 2.0 * eu + gg : 0.0;
       const double cosb = (q_aa > 0.0 && gg > 0.0) ? q_au * rsqrt(q_aa * gg) : 0.0;
       const double ess = W2 > 0.f ? (double)W * (double)W / (double)W2 : 0.0;
       acc[0] = fma(w, q, acc[0]);
@@ -491,16 +570,16 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-template <int TW>
+template <int TW, bool SPLIT>
 pair_status launch_draws(int nblk, size_t smem, int N, int G, const float *r, const float *rho,
                          const uint8_t *Jd, const double *wd, float scale, uint32_t flags,
                          int wmode, float w_max, const double *K, const double *abar,
                          const double *u, const double *gg, double *part, int32_t *dev_err,
                          cudaStream_t s) {
-  PAIR_CUDA_TRY(cudaFuncSetAttribute(audit_draws_kernel<TW>,
+  PAIR_CUDA_TRY(cudaFuncSetAttribute(audit_draws_kernel<TW, SPLIT>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   PAIR_BEGIN("audit_draws", s);
-  audit_draws_kernel<TW><<<nblk, audit_warps(TW) * 32, smem, s>>>(
+  audit_draws_kernel<TW, SPLIT><<<nblk, audit_warps(TW) * 32, smem, s>>>(
       N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar, u, gg, part, dev_err);
   PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
@@ -531,11 +610,14 @@ pair_status launch_audit(int N, int G, int D, const float *r, const float *rho, 
   if (nblk > most) nblk = most;
   pair_status st;
   if (audit_team(G) == 1)
-    st = launch_draws<1>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar, u,
-                         gg, part, dev_err, s);
+    st = launch_draws<1, true>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar,
+                               u, gg, part, dev_err, s);
+  else if (audit_split(G))
+    st = launch_draws<8, true>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar,
+                               u, gg, part, dev_err, s);
   else
-    st = launch_draws<8>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K,
-                                   abar, u, gg, part, dev_err, s);
+    st = launch_draws<8, false>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K,
+                                abar, u, gg, part, dev_err, s);
   if (st != PAIR_OK) return st;
   PAIR_BEGIN("audit_finish", s);
   const int fin = bias ? (int)ceil_div(D, 256) : 1;
