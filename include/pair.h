@@ -223,8 +223,9 @@ PAIR_API pair_status pair_coeffs_product(int32_t B, int32_t G, const float *r,
  *                           completed edges, [PAIR_AUDIT_ESS] mean ESS
  *   [PAIR_AUDIT_TARGET_SQ]  || g ||^2,  [PAIR_AUDIT_WEIGHT] W
  * and bias [D] (double, nullable) the vector sum_b w_b ghat_b / W - g.
- * Everything is formed through the Gram matrix S S^T in fp64 (the
- * coefficients themselves are fp32); deterministic. ws: device workspace of
+ * Everything is formed through the Gram matrix S S^T in fp64 (a draw's
+ * coefficients are not rounded to fp32, except their row sums for G > 120, and
+ * the ESS weights); deterministic. ws: device workspace of
  * pair_audit_workspace_size(N, G, D) bytes, 16-byte aligned, no initial
  * contents needed.
  * Errors: as pair_coeffs_weighted; PAIR_ERR_WORKSPACE.
@@ -340,9 +341,11 @@ PAIR_API size_t pair_grad_workspace_size(int64_t T, int32_t d, int32_t V, int32_
  * pair_grad_workspace_min_size -- the smallest workspace pair_grad accepts:
  * pair_grad_workspace_size without the image. Any size from here up to
  * pair_grad_workspace_size is valid; the image then holds the token blocks
- * that fit (more chunks), and with none no logit-sized tensor is kept at all
- * (the on-chip form: the log-sum-exp pass is fused with dH, and dW
- * recomputes the logits). Results agree to bf16/fp32 rounding across sizes
+ * that fit (more chunks), and with none no logit-sized tensor is kept in it
+ * (the on-chip form for d a multiple of 512 up to 3072: the log-sum-exp pass is
+ * fused with dH, and dW recomputes the logits; other bf16 d recompute them or
+ * stage bf16 gradient tiles, a part at a time, in the workspace's exchange buffer
+ * or in rows of dW that are not written yet). Results agree to bf16/fp32 rounding across sizes
  * (the sums run in a different order), and are bit-identical for the same
  * size.
  */
@@ -363,7 +366,10 @@ PAIR_API size_t pair_grad_workspace_min_size(int64_t T, int32_t d, int32_t V, in
  * written as exact zeros. No logit-sized tensor is written in fp32: with the
  * default workspace the log-sum-exp pass keeps the bf16 softmax terms once
  * for the dH and dW GEMMs (see pair_grad_workspace_size); with the minimum
- * workspace nothing logit-sized is written.
+ * workspace nothing logit-sized is written (for bf16 d that are no multiple of
+ * 512 or above 3072, bf16 gradient tiles may pass through dW or the workspace).
+ * dW serves as scratch before its rows are written: it must not overlap any
+ * input or other output.
  *
  * In:  T >= 1 packed tokens; d hidden size; V vocabulary size; dt dtype of
  *      H and W (PAIR_BF16: fp32 accumulation on the tensor cores, requires
@@ -458,8 +464,8 @@ PAIR_API pair_status pair_grad_clipped(int64_t T, int32_t d, int32_t V, pair_dty
  * Arguments, outputs and numerics are those of pair_grad, minus ws and
  * ws_bytes. The workspace is a file-scope device array of
  * PAIR_NOALLOC_MAX_WORKSPACE bytes that every GPU loading this library
- * holds until the process exits. It keeps no image of softmax terms (the
- * backward recomputes the logits); a problem is accepted iff
+ * holds until the process exits. It keeps no image of softmax terms (see
+ * pair_grad_workspace_min_size); a problem is accepted iff
  * pair_grad_workspace_min_size(T, d, V, R, dt) <= PAIR_NOALLOC_MAX_WORKSPACE
  * and rejected with PAIR_ERR_WORKSPACE before any launch otherwise. That
  * size grows with T * d (the compacted hidden rows) plus, for bf16, a fixed
