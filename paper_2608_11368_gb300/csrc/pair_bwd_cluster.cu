@@ -1,8 +1,8 @@
 // Backward of the bf16 LM-head path without an image of softmax terms (the
 // no-alloc path and minimum workspaces): the logits are recomputed. For
 // d = 512 A (A <= 6), 8-CTA clusters share each Gs tile through an L2 ring
-// (bwd_cluster_kernel); otherwise a CTA pair per two row blocks and 256-wide
-// d-slice (bwd_kernel).
+// (bwd_cluster_kernel); otherwise a CTA, or a CTA pair, per row block, or two,
+// and slice of d (bwd_kernel).
 #include <math.h>
 
 #include "tc_kernels.cuh"
@@ -15,47 +15,51 @@ using namespace tck;
 
 // ------------------------------------------------------------- backward
 //
-// Per 128-row tile of the other side the logits S = R C^T (double-buffered in
-// TMEM), the gradient tile Gs = f(S) in bf16, and out += Gs C[:, slice], for one
-// block of 128 rows (tokens for dH, vocabulary rows for dW) and a 256-column
-// slice of d, whose accumulators stay in TMEM. Recomputing S per slice costs d +
-// 256 multiply-adds per logit and output slice, and every tile is fetched anew.
+// Per 128-row tile of the other side the logits S = R C^T (in TMEM), the gradient
+// tile Gs = f(S) in bf16, and out += Gs C[:, slice], for one block of 128 rows
+// (tokens for dH, vocabulary rows for dW) and a slice of d, whose accumulators
+// stay in TMEM. Recomputing S per slice costs d + slice multiply-adds per logit
+// and slice, and every tile is fetched anew.
 //
 // Two forms. For d > 512 an SM's read port bounds it (about 60 bytes a clock): a
 // CTA pair takes two row blocks and each CTA fetches half of C's tile for either
-// product, 24 KB per 64 columns of d and 32 KB of the slice where a CTA by itself
-// takes 32 and 64; S runs two tiles ahead, its buffers free once they are read
-// from TMEM. (d = 768, V = 32,000: dW of 6.4 k tokens 979 -> 875 us, of 24 k 3.80
-// -> 3.24 ms; by single CTAs 1024 us and 4.1 ms.) Below, the chain from S through
-// the conversion to the next product bounds it, which the pair's exchanges only
-// lengthen: one CTA, two Gs tiles, eight warps converting (d = 256, V = 50,000,
-// 6.4 k tokens: dH 747 -> 721, dW 396 -> 305 us; d = 64: 1.58 -> 1.13 ms and 528
-// -> 347 us; in pairs 767 and 408 us at d = 256). Pairs want more than a dozen
-// tiles per unit: with 5 (d = 832, 0.4 k tokens) they take 101 us to 98.
+// product, 24 KB per 64 columns of d where a CTA by itself takes 32; one S tile,
+// free again once it is read from TMEM, leaves room for slices of 384 columns
+// (d = 768: two instead of three). d = 768, V = 32,000: dW of 6.4 k tokens 979 ->
+// 702 us (slices of 256 and two S tiles 860, single CTAs 1024), of 24 k 3.80 -> 2.58
+// ms; six stages and one slice of C in shared memory against four and two: 2.85
+// and 2.97 ms. Below, the chain from S through the conversion to the next product
+// bounds it, which the pair's exchanges only lengthen: one CTA, slices of 256, two
+// S and Gs tiles, eight warps converting (d = 256, V = 50,000, 6.4 k tokens: dW 396
+// -> 306 us; in pairs 408). Pairs want more than a dozen tiles per unit: with 5
+// (d = 832, 0.4 k tokens) they took 101 us to 98.
 //
 // The units of the last, or only, round are cut into parts of C's tiles
-// (TailSplit, at 152 CTAs or 76 pairs): 51 token blocks of d = 256 kept a third of
-// the SMs busy (dH 721 -> 256 us; d = 192, V = 50,000, 5.9 k tokens: 643 -> 160; d =
-// 128, V = 20,000, 0.5 k tokens: 233 -> 20).
+// (TailSplit, at 152 CTAs or 76 pairs; the first part goes to the unit's rows of
+// out, so that the scratch serves more): 51 token blocks of d = 256 kept a third
+// of the SMs busy (dH 721 -> 256 us; d = 192, V = 50,000, 5.9 k tokens: 643 -> 160;
+// d = 128, V = 20,000, 0.5 k tokens: 233 -> 20).
 constexpr int kBwdBN = 128;     // S tile columns
-constexpr int kSlice = 256;     // output columns held in TMEM per unit
+// Output columns held in TMEM per unit, beside two S tiles or (pairs) one.
+constexpr int bwd_slice(bool pair) { return pair ? 384 : 256; }
 // A split unit's start and drain, in tiles.
 constexpr int kBwdOverhead = 3;
 constexpr int kBwdThreads = 320;  // warps 2 .. 9: the epilogue, two per TMEM lane quadrant
 
 template <bool kPair>
 struct BwdSmem {
-  static constexpr int kStages = kPair ? 4 : 3;
-  static constexpr int kCs = kPair ? 2 : 1;                        // slices of C
-  static constexpr int kAhead = kPair ? 2 : 1;                     // tiles S runs ahead
+  static constexpr int kStages = kPair ? 6 : 3;
+  static constexpr int kSlice = bwd_slice(kPair);
+  static constexpr int kS = kPair ? 1 : 2;   // S tiles in TMEM
+  static constexpr int kG = kPair ? 1 : 2;   // Gs tiles
   static constexpr uint32_t kBBytes = kPair ? kAtom128 / 2 : kAtom128;  // this CTA's rows of it
   uint8_t a[kStages][kAtom128];                              // rows-operand atoms (128 x 64)
   uint8_t b[kStages][kBBytes];                               // cols-operand atoms
-  uint8_t cs[kCs][kSlice / 64 / (kPair ? 2 : 1)][kAtom128];  // cols operand, d-slice (MN-major B)
-  uint8_t g[2][kBwdBN / 64][kAtom128];                       // Gs tiles, K-major A
+  uint8_t cs[kSlice / 64 / (kPair ? 2 : 1)][kAtom128];       // cols operand, d-slice (MN-major B)
+  uint8_t g[kG][kBwdBN / 64][kAtom128];                      // Gs tiles, K-major A
   float2 col[kBwdBN];  // dW: -c and lse log2 e of the tile's tokens (c = 0: lse = infinity)
-  uint64_t full[kStages], empty[kStages], cs_full[kCs], cs_empty[kCs];
-  uint64_t s_full[2], s_empty[2], g_full[2], g_empty[2];
+  uint64_t full[kStages], empty[kStages], cs_full, cs_empty;
+  uint64_t s_full[kS], s_empty[kS], g_full[kG], g_empty[kG];
   uint64_t o_full, o_empty, mma_done;
   uint32_t tmem_base;
   int abort;
@@ -75,7 +79,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
                float *scratch, int scratch_cap, int32_t *dev_err) {
   extern __shared__ uint8_t smem_raw[];
   using Smem = BwdSmem<kPair>;
-  constexpr int kCtas = kPair ? 2 : 1, kBwdStages = Smem::kStages, kCs = Smem::kCs, kAhead = Smem::kAhead;
+  constexpr int kCtas = kPair ? 2 : 1, kBwdStages = Smem::kStages, kSlice = Smem::kSlice;
+  constexpr int kS = Smem::kS, kG = Smem::kG;
   Smem &sm = *reinterpret_cast<Smem *>(align1k(smem_raw));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = kPair ? (int)(blockIdx.x & 1) : 0;  // rank in the cluster
@@ -85,11 +90,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
   const int n_rb = kTokenRows ? (Teff + 127) / 128 : (V + 127) / 128;
   const int n_ct = kTokenRows ? (V + kBwdBN - 1) / kBwdBN : (Teff + kBwdBN - 1) / kBwdBN;
   const int n_units = (n_rb + kCtas - 1) / kCtas * nsl;
-  const TailSplit tl = tail_split(n_units, npairs, scratch_cap, n_ct, kBwdOverhead, 1, nsl * 512);
+  const TailSplit tl =
+      tail_split(n_units, npairs, scratch_cap, n_ct, kBwdOverhead, 1, nsl * 512, true);
   const int n_items = tl.full_end + tl.items();
   // This CTA's or pair's tiles, item after item. Both products run along them, S
-  // kAhead tiles ahead: what S(i + 2) waits for is that tile i has been read
-  // from TMEM, not that it has been converted.
+  // one tile ahead: what its buffer waits for is that the tile before has been
+  // read from TMEM, not that it has been converted.
   struct Tile {
     int i, u, ct, k0, k1, slot;
     bool live;
@@ -146,16 +152,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
       mbar_init(&sm.full[s], 1);   // expect_tx (in a pair the even CTA's, of both CTAs' bytes)
       mbar_init(&sm.empty[s], 1);  // the MMA's commit
     }
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < kS; ++s) {
       mbar_init(&sm.s_full[s], 1);
       mbar_init(&sm.s_empty[s], 8 * kCtas);  // the epilogue warps
+    }
+    for (int s = 0; s < kG; ++s) {
       mbar_init(&sm.g_full[s], 8 * kCtas);
       mbar_init(&sm.g_empty[s], 1);
     }
-    for (int s = 0; s < kCs; ++s) {
-      mbar_init(&sm.cs_full[s], 1);
-      mbar_init(&sm.cs_empty[s], 1);
-    }
+    mbar_init(&sm.cs_full, 1);
+    mbar_init(&sm.cs_empty, 1);
     mbar_init(&sm.o_full, 1);
     mbar_init(&sm.o_empty, 8 * kCtas);
     mbar_init(&sm.mma_done, 1);
@@ -179,14 +185,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
   if constexpr (kPair) cluster_sync();  // the pair's barriers exist before anything lands on them
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
-  const uint32_t tmem_o = tmem + 2 * kBwdBN;  // columns [256, 512)
+  const uint32_t tmem_o = tmem + kS * kBwdBN;  // the slice's columns
 
   if (warp == 0) {
     {  // whole warp: uniform loop state; elected lane issues
       int stage = 0;
-      uint32_t ph = 0, cs_n = 0;
-      int last_ph[kBwdStages], cs_last[kCs];
-      for (int b = 0; b < kCs; ++b) cs_last[b] = -1;
+      uint32_t ph = 0, cs_ph = 0;
+      int last_ph[kBwdStages], cs_last = -1;
       for (int s = 0; s < kBwdStages; ++s) last_ph[s] = -1;
       bool ok = true;
       auto load_s = [&](int rb, int ct) {
@@ -205,26 +210,27 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
       };
       auto load_cs = [&](int sl, int ct) {
         if (!ok) return;
-        const int b = cs_n % kCs;
-        const uint32_t cph = (cs_n / kCs) & 1;
-        if (!(ok = await(&sm.cs_empty[b], cph ^ 1))) return;
+        if (!(ok = await(&sm.cs_empty, cs_ph ^ 1))) return;
         if (elect_one()) {
           const int n = slice_n(sl);
-          if (r == 0) mbar_expect_tx(&sm.cs_full[b], (uint32_t)(n / 64) * kAtom128);
-          for (int j = 0; j < n / 64 / kCtas; ++j)
-            load(sm.cs[b][j], &tmC, &sm.cs_full[b], sl * kSlice + r * (n / 2) + j * 64,
-                 ct * kBwdBN);
+          if (r == 0) mbar_expect_tx(&sm.cs_full, (uint32_t)(n / 64) * kAtom128);
+          // (In a pair this CTA's half of the first 256 columns, then of the rest.)
+          const int n1 = min(n, 256);
+          for (int j = 0; j < n / 64 / kCtas; ++j) {
+            const int c = j * 64 < n1 / kCtas ? r * (n1 / 2) + j * 64 : n1 / 2 + r * 64 + j * 64;
+            load(sm.cs[j], &tmC, &sm.cs_full, sl * kSlice + c, ct * kBwdBN);
+          }
         }
         __syncwarp();
-        cs_last[b] = (int)cph;
-        ++cs_n;
+        cs_last = (int)cs_ph;
+        cs_ph ^= 1;
       };
       Tile ts = first(), tc = ts;  // next tile of S, of cs
       auto next_s = [&]() {
         load_s(kCtas * (ts.u / nsl) + r, ts.ct);
         advance(ts);
       };
-      for (int k = 0; k < kAhead && ts.live; ++k) next_s();
+      if (ts.live) next_s();
       for (; tc.live && ok; advance(tc)) {
         if (ts.live) next_s();
         load_cs(tc.u % nsl, tc.ct);
@@ -236,10 +242,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
       for (int s = 0; s < kBwdStages; ++s)
         if (last_ph[s] >= 0)
           wait_cluster(r == 0 ? &sm.full[s] : &sm.empty[s], (uint32_t)last_ph[s], &never, dev_err);
-      for (int b = 0; b < kCs; ++b)
-        if (cs_last[b] >= 0)
-          wait_cluster(r == 0 ? &sm.cs_full[b] : &sm.cs_empty[b], (uint32_t)cs_last[b], &never,
-                       dev_err);
+      if (cs_last >= 0)
+        wait_cluster(r == 0 ? &sm.cs_full : &sm.cs_empty, (uint32_t)cs_last, &never, dev_err);
     }
   } else if (warp == 1) {
     if (r == 0) {  // whole warp: uniform loop state; elected lane issues
@@ -247,8 +251,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
       uint32_t ph = 0, s_n = 0, g_n = 0, o_ph = 0;  // tiles begun and finished
       bool ok = true;
       auto issue_s = [&]() {
-        const int buf = s_n & 1;
-        if (!(ok = await(&sm.s_empty[buf], ((s_n >> 1) & 1) ^ 1))) return;
+        const int buf = s_n % kS;
+        if (!(ok = await(&sm.s_empty[buf], ((s_n / kS) & 1) ^ 1))) return;
         tc_fence_after();
         const uint32_t dt = tmem + buf * kBwdBN;
         for (int k = 0; k < nk; ++k) {
@@ -271,28 +275,35 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
       };
       auto issue_o = [&](bool begin, int n) {
         if (!ok) return;
-        const int buf = g_n & 1, b = g_n % kCs;
-        if (!(ok = await(&sm.g_full[buf], (g_n >> 1) & 1))) return;
-        if (!(ok = await(&sm.cs_full[b], (g_n / kCs) & 1))) return;
+        const int buf = g_n % kG;
+        if (!(ok = await(&sm.g_full[buf], (g_n / kG) & 1))) return;
+        if (!(ok = await(&sm.cs_full, g_n & 1))) return;
         if (begin && !(ok = await(&sm.o_empty, o_ph ^ 1))) return;
         tc_fence_after();
-        const uint32_t idesc = idesc_bf16(128 * kCtas, n, 0, 1);
-        const uint32_t sg = smem_u32(sm.g[buf][0]), sc = smem_u32(sm.cs[b][0]);
+        const int n1 = min(n, 256);  // (one MMA has at most 256 columns)
+        const uint32_t idesc = idesc_bf16(128 * kCtas, n1, 0, 1);
+        const uint32_t sg = smem_u32(sm.g[buf][0]), sc = smem_u32(sm.cs[0]);
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < kBwdBN / 16; ++kk) {
             const uint64_t ad = sdesc_sw128(sg + (kk >> 2) * kAtom128 + (kk & 3) * 32, 16, 1024);
             const uint64_t bd = sdesc_sw128(sc + kk * 2048, kAtom128, 1024);
             mma(tmem_o, ad, bd, idesc, !begin || kk != 0);
+            if (kSlice > 256 && n > 256)
+              mma(tmem_o + 256, ad, sdesc_sw128(sc + 2 * kAtom128 + kk * 2048, kAtom128, 1024),
+                  idesc_bf16(128 * kCtas, 128, 0, 1), !begin || kk != 0);
           }
           commit(&sm.g_empty[buf]);
-          commit(&sm.cs_empty[b]);
+          commit(&sm.cs_empty);
         }
         __syncwarp();
         ++g_n;
       };
       Tile ts = first(), to = ts;  // next tile of S, of the output
-      for (int k = 0; k < kAhead && ts.live && ok; ++k, advance(ts)) issue_s();
+      if (ts.live) {
+        issue_s();
+        advance(ts);
+      }
       for (; to.live && ok; advance(to)) {
         if (ts.live) {
           issue_s();
@@ -348,9 +359,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
           bwd_epi_sync();
           token((ct + 1) * kBwdBN + row);
         }
-        const int buf = n & 1;
-        const uint32_t bph = (n >> 1) & 1;
-        if (!(ok = ok && await_all(&sm.s_full[buf], bph))) continue;
+        const int buf = n % kS, gb = n % kG;
+        if (!(ok = ok && await_all(&sm.s_full[buf], (n / kS) & 1))) continue;
         tc_fence_after();
         float v[2][32];
         tmem_ld32(tmem + lane_off + buf * kBwdBN + half * 64, v[0]);
@@ -358,7 +368,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) arrive(&sm.s_empty[buf]);
-        if (!(ok = await_all(&sm.g_empty[buf], bph ^ 1))) continue;
+        if (!(ok = await_all(&sm.g_empty[gb], ((n / kG) & 1) ^ 1))) continue;
         const int lim = V - ct * kBwdBN - half * 64;  // dH: columns of the vocabulary
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
@@ -381,20 +391,21 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const int k = c * 32 + q * 8;  // first column of this 16-byte piece
-            uint8_t *dst = sm.g[buf][half] + sw128_offset(row, k);
+            uint8_t *dst = sm.g[gb][half] + sw128_offset(row, k);
             *reinterpret_cast<uint4 *>(dst) =
                 make_uint4(pk[q * 4], pk[q * 4 + 1], pk[q * 4 + 2], pk[q * 4 + 3]);
           }
         }
         fence_async_smem();
         __syncwarp();
-        if (lane == 0) arrive(&sm.g_full[buf]);
+        if (lane == 0) arrive(&sm.g_full[gb]);
       }
       if (!ok) continue;
       const bool valid = kTokenRows ? (rid < Teff) : (rid < V);
       float *dst = nullptr;
-      if (slot >= 0)
-        dst = scratch + (((int64_t)slot * kCtas + r) * 128 + row) * kSlice;
+      // (A split unit's first part goes to its rows of out.)
+      if (slot >= tl.R)
+        dst = scratch + (((int64_t)(slot - tl.R) * kCtas + r) * 128 + row) * kSlice;
       else if (valid)
         dst = out + (kTokenRows ? (int64_t)tok_idx[rid] : (int64_t)rid) * d + sl * kSlice;
       if (n_ct == 0) {
@@ -436,7 +447,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
 // Whether the last round's units may be split: with more than six rounds the
 // partial tiles and their pass cost what that round leaves idle.
 bool bwd_splits(int64_t rows, int d, int ctas) {
-  const int64_t units = ((rows + 127) / 128 + ctas - 1) / ctas * ((d + kSlice - 1) / kSlice);
+  const int slice = bwd_slice(ctas == 2);
+  const int64_t units = ((rows + 127) / 128 + ctas - 1) / ctas * ((d + slice - 1) / slice);
   return units <= 6 * (int64_t)(152 / ctas);
 }
 
@@ -445,12 +457,14 @@ template <bool kTokenRows, bool kPair>
 __global__ void __launch_bounds__(256)
     bwd_tail_kernel(int d, int V, int ncl, int scratch_cap, const int32_t *counters,
                     const int32_t *tok_idx, const float *__restrict__ scratch, float *out) {
-  constexpr int kCtas = kPair ? 2 : 1, kRows = 128 * kCtas, kQ = kSlice / 4;
+  constexpr int kSlice = bwd_slice(kPair), kCtas = kPair ? 2 : 1, kRows = 128 * kCtas;
+  constexpr int kQ = kSlice / 4;
   const int Teff = counters[0], rows = kTokenRows ? Teff : V;
   const int nsl = (d + kSlice - 1) / kSlice;
   const int n_ct = ((kTokenRows ? V : Teff) + kBwdBN - 1) / kBwdBN;
   const int n_units = ((rows + 127) / 128 + kCtas - 1) / kCtas * nsl;
-  const TailSplit tl = tail_split(n_units, ncl, scratch_cap, n_ct, kBwdOverhead, 1, nsl * 512);
+  const TailSplit tl =
+      tail_split(n_units, ncl, scratch_cap, n_ct, kBwdOverhead, 1, nsl * 512, true);
   const float4 *src = reinterpret_cast<const float4 *>(scratch);
   const int64_t n4 = (int64_t)tl.R * kRows * kQ;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n4;
@@ -458,9 +472,9 @@ __global__ void __launch_bounds__(256)
     const int c4 = (int)(e % kQ), row = (int)(e / kQ % kRows), v = (int)(e / (kQ * kRows));
     const int u = tl.full_end + v, rid = u / nsl * kRows + row, col = u % nsl * kSlice + 4 * c4;
     if (rid >= rows || col >= d) continue;
-    const float4 t = tail_sum(tl, v, src, kRows * kQ, (int64_t)row * kQ + c4);
-    *reinterpret_cast<float4 *>(out + (kTokenRows ? (int64_t)tok_idx[rid] : (int64_t)rid) * d +
-                                col) = t;
+    float4 *dst = reinterpret_cast<float4 *>(
+        out + (kTokenRows ? (int64_t)tok_idx[rid] : (int64_t)rid) * d + col);
+    *dst = tail_sum(tl, v, *dst, src + v * kRows * kQ, kRows * kQ, (int64_t)row * kQ + c4);
   }
 }
 
@@ -483,7 +497,7 @@ pair_status launch_bwd(const char *name, const CUtensorMap &mR, const CUtensorMa
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const int ncl = (num_sms() & ~1) / (kPair ? 2 : 1);
-  size_t cap = scratch_bytes / ((kPair ? 2 : 1) * 128 * kSlice * sizeof(float));
+  size_t cap = scratch_bytes / ((kPair ? 2 : 1) * 128 * bwd_slice(kPair) * sizeof(float));
   if (cap > 1024) cap = 1024;
   if (!bwd_splits(kTokenRows ? g.T : (int64_t)g.V, g.d, kPair ? 2 : 1)) cap = 0;
   PAIR_BEGIN(name, s);
@@ -1509,15 +1523,17 @@ bool bwd_pairs(int d, int64_t cols) { return d > 512 && cols >= 2048; }
 double bwd_recompute_us(int d, double rows, double cols, int64_t rows_max, int64_t cols_max,
                         size_t scratch_bytes) {
   const bool pair = bwd_pairs(d, cols_max);
-  const int ctas = pair ? 2 : 1, ncl = 152 / ctas, slices = (d + kSlice - 1) / kSlice;
-  const double flop = 2.0 * 128 * 128 * (d + (d < 256 ? d : 256)) * 152;
+  const int slice = bwd_slice(pair);
+  const int ctas = pair ? 2 : 1, ncl = 152 / ctas, slices = (d + slice - 1) / slice;
+  const double flop = 2.0 * 128 * 128 * (d + (d < slice ? d : slice)) * 152;
   const double tile = pair ? flop / 1.48e9 : 0.65 + flop / 2.1e9;
   const double units = ceil(ceil(rows / 128) / ctas) * slices, n_ct = ceil(cols / 128);
   const double full = floor(units / ncl), left = units - full * ncl;
   double last = left > 0 ? n_ct : 0;
-  const double cap = (double)(scratch_bytes / (ctas * 128 * kSlice * sizeof(float)));
-  if (bwd_splits(rows_max, d, ctas) && 2 * left <= cap) {
-    const double share = left / ncl > left / cap ? left / ncl : left / cap;
+  const double cap = (double)(scratch_bytes / (ctas * 128 * slice * sizeof(float)));
+  if (bwd_splits(rows_max, d, ctas) && left <= cap) {
+    const double most = left / (left + cap);  // one part in the output, the others in scratch
+    const double share = left / ncl > most ? left / ncl : most;
     last = fmin(last, 1.125 * share * n_ct + 2 * kBwdOverhead);
   }
   return (full * n_ct + last) * tile + 10.0;

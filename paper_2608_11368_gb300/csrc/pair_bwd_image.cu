@@ -355,7 +355,9 @@ __global__ void __launch_bounds__(256)
     const int tp = u / nq, q = u - tp * nq;
     const int t = (rb0 + 2 * tp + r) * 128 + row;
     if (2 * tp + r >= nrb || t >= Teff || q * kDhN + 4 * c4 >= d) continue;
-    const float4 acc = tail_sum(tl, uj, src, 256 * kQ, (int64_t)(r * 128 + row) * kQ + c4);
+    const int64_t at = (int64_t)(r * 128 + row) * kQ + c4, tile = 256 * kQ;
+    const float4 acc =
+        tail_sum(tl, uj, src[uj * tile + at], src + (tl.R + uj) * tile, tile, at);
     const float sc = row_scale(tok_c, lsum, t);
     reinterpret_cast<float4 *>(dH + (int64_t)tok_idx[t] * d + q * kDhN)[c4] =
         make_float4(sc * acc.x, sc * acc.y, sc * acc.z, sc * acc.w);
@@ -659,7 +661,8 @@ __global__ void __launch_bounds__(256)
     const int vp = u / nq, q = u - vp * nq;
     const int v = (vb0 + 2 * vp + r) * 128 + row;
     if (2 * vp + r >= n_vb || v >= V || q * kDwN + 4 * c4 >= d) continue;
-    float4 acc = tail_sum(tl, uj, src, 256 * kQ, (int64_t)(r * 128 + row) * kQ + c4);
+    const int64_t at = (int64_t)(r * 128 + row) * kQ + c4, tile = 256 * kQ;
+    float4 acc = tail_sum(tl, uj, src[uj * tile + at], src + (tl.R + uj) * tile, tile, at);
     float4 *dst = reinterpret_cast<float4 *>(dW + (int64_t)v * d + q * kDwN) + c4;
     if (accumulate) {
       const float4 o = *dst;
@@ -744,10 +747,10 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
 //
 // For hidden sizes whose workspace holds no image (d not a multiple of 512, and
 // d > 3072 with the minimum one), the recomputing kernel (bwd_kernel) forms the
-// logits again for each 256-column slice of d, in each of the two products: 2
-// (1 + d / 256) logit-sized products, and few rows leave most SMs idle. Here they are formed once for each
-// product, as gradient tiles in the image's layout in memory that is free at
-// the time, and the two products are the image form's GEMMs: 4 in all.
+// logits again for each slice of d (256 or 384 columns), in each of the two
+// products. Here they are formed once for each product, as gradient tiles in the
+// image's layout in memory that is free at the time, and the two products are the
+// image form's GEMMs: 4 logit-sized products in all.
 //   dH: token chunks, the tiles over the whole vocabulary in dW, which nothing
 //       has written yet, or in the workspace's ring if that holds more blocks.
 //   dW: vocabulary slabs in ascending order, the tiles over all tokens in the
@@ -762,8 +765,9 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
 // logit-sized products at 1.6 PFLOP/s and the parts' cost. Measured on one GB300
 // against bwd_kernel: d = 2432, V = 60,000, 1.5 k tokens (one chunk, four slabs)
 // 9.2 -> 1.15 ms for the call; d = 1216, V = 30,000, 5 k tokens (5 chunks, 13
-// slabs) 2.13 ms; d = 768, V = 32,000, 6.4 k tokens in 10 chunks 0.99 -> 0.81 for
-// dH, and dW would take 23 slabs (1.83 against 0.88).
+// slabs) 2.13 ms (2.38 with the GEMM's scratch in the ring alone). d = 768, V =
+// 32,000, 6.4 k tokens, whose dW holds few blocks' tiles, is recomputed: dH in 10
+// chunks takes 0.81 ms to 0.66, dW in 23 slabs 1.83 to 0.71.
 constexpr double kSlabUs = 75.0, kSlabDhUs = 35.0;
 constexpr size_t kSlabTile = 2 * 128 * kDhN * sizeof(float);  // a scratch tile
 constexpr size_t kSlabScratch = 1024;

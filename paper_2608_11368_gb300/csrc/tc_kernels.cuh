@@ -126,9 +126,9 @@ struct TailSplit {
 constexpr int kTailMaxParts = 64;
 // A whole warp calls (every lane gets the answer). d gives the units' widths (a
 // multiple of 512: all alike); `tile` is the combine pass's share per scratch tile
-// in 1/64 steps.
+// in 1/64 steps; own: the units' first parts need no scratch (slots R and up).
 __device__ __forceinline__ TailSplit tail_split(int n_units, int ncl, int cap, int nks,
-                                                int overhead, int tile, int d) {
+                                                int overhead, int tile, int d, bool own = false) {
   TailSplit t{n_units, 0, 1, 1, 0, 0, (d + 511) / 512};
   const int R = n_units % ncl;
   if (R == 0 || nks == 0) return t;
@@ -141,7 +141,7 @@ __device__ __forceinline__ TailSplit tail_split(int n_units, int ncl, int cap, i
     t.S = S;
     t.Sh = t.Rh > 0 ? (S + 1) / 2 : S;
     const int n = t.items();
-    if (S > 1 && n > cap) break;
+    if (S > 1 && n - (own ? R : 0) > cap) break;
     const long long rounds = (n + ncl - 1) / ncl, steps = (nks + S - 1) / S;
     const long long cost = 64 * rounds * (steps + overhead) + (S > 1 ? (long long)tile * n : 0);
     best = min(best, (unsigned long long)cost * (2 * kTailMaxParts) + S);
@@ -177,11 +177,11 @@ __device__ __forceinline__ void tail_item(const TailSplit &tl, int nks, int i, i
     slot = j;
   }
 }
-// Sum of unit full_end + v's parts at float4 `at` of their tiles (`tile`
-// float4 each), in part order; eight loads in flight.
-__device__ __forceinline__ float4 tail_sum(const TailSplit &tl, int v, const float4 *src,
-                                           int64_t tile, int64_t at) {
-  float4 acc = src[v * tile + at];
+// First part `acc` of unit full_end + v plus its others at float4 `at` of their
+// tiles (`tile` float4 each, the second part's being `src`), in part order; eight
+// loads in flight.
+__device__ __forceinline__ float4 tail_sum(const TailSplit &tl, int v, float4 acc,
+                                           const float4 *src, int64_t tile, int64_t at) {
   auto add = [&](const float4 *p, int64_t stride, int n) {
     int k = 0;
     for (; k + 8 <= n; k += 8, p += 8 * stride) {
@@ -198,10 +198,10 @@ __device__ __forceinline__ float4 tail_sum(const TailSplit &tl, int v, const flo
       acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
     }
   };
-  add(src + (tl.R + v) * tile + at, tl.R * tile, tl.Sh - 1);
+  add(src + at, tl.R * tile, tl.Sh - 1);
   if (!tl.narrow(v))
-    add(src + ((int64_t)tl.R * tl.Sh + tl.wide_before(v)) * tile + at, (tl.R - tl.Rh) * tile,
-        tl.S - tl.Sh);
+    add(src + ((int64_t)tl.R * (tl.Sh - 1) + tl.wide_before(v) - v) * tile + at,
+        (tl.R - tl.Rh) * tile, tl.S - tl.Sh);
   return acc;
 }
 

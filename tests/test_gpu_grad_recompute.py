@@ -1,6 +1,6 @@
 """The recomputing backward of bf16 hidden sizes without an image (a row block
-and 256 columns of d per CTA; two row blocks per CTA pair): last slices of 64,
-128, 192 and 256 columns, one, odd and even numbers of token and vocabulary
+and 256 columns of d per CTA; two row blocks and 384 columns per CTA pair): last
+slices of 64 to 256 and 64 to 384 columns, one, odd and even numbers of token and vocabulary
 blocks, ragged ends of both, units split over parts of the other side (scratch
 in the ring and in dW), and more units than CTAs. Checked as in
 test_gpu_grad.py; reruns are bit-identical."""
@@ -24,7 +24,10 @@ pytestmark = pytest.mark.gpu
     (128, 24000, 1, 4, 0.2),    # dW: more units than pairs
     (256, 16000, 1, 4, 0.3),    # dH split, its scratch in dW
     (704, 2100, 2, 8, 0.3),     # pairs, an odd number of vocabulary blocks, dW split
-    (960, 1024, 2, 8, 0.3),     # dW in pairs; four slices, the last of 192
+    (960, 1024, 2, 8, 0.3),     # dW in pairs; three slices, the last of 192
+    (768, 2048, 1, 8, 0.3),     # two whole slices
+    (832, 2500, 1, 8, 0.3),     # a last slice of 64
+    (640, 5000, 2, 8, 0.5),     # of 256
 ])
 def test_recompute(d, V, B, G, ls):
     inp = synth.make_head_workload(synth.WORKLOADS["qwen3_1p7b_head"], 17, B=B, G=G, d=d, V=V,
