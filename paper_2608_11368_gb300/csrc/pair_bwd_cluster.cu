@@ -31,7 +31,10 @@ using namespace tck;
 // and 2.97 ms. Below, the chain from S through the conversion to the next product
 // bounds it, which the pair's exchanges only lengthen: one CTA, slices of 256, two
 // S and Gs tiles, eight warps converting (d = 256, V = 50,000, 6.4 k tokens: dW 396
-// -> 306 us; in pairs 408). Pairs want more than a dozen tiles per unit: with 5
+// -> 306 us; in pairs 408; d = 448, V = 46,000, 12 k tokens: dH 1.15 and dW 1.27 ms,
+// in pairs 1.28 and 1.53), but for 256 < d <= 384, where pairs need one slice
+// instead of two (d = 320, V = 151,936, 6.3 k tokens: dH 1.70 -> 1.14, dW 1.78 -> 1.23
+// ms). Pairs want more than a dozen tiles per unit: with 5
 // (d = 832, 0.4 k tokens) they took 101 us to 98.
 //
 // The units of the last, or only, round are cut into parts of C's tiles
@@ -1514,7 +1517,9 @@ pair_status grad_head_onchip(const GradArgs &g, const GradWorkspace &w, cudaStre
 }
 
 // CTA pairs, or single CTAs, of bwd_kernel over `cols` columns (see there).
-bool bwd_pairs(int d, int64_t cols) { return d > 512 && cols >= 2048; }
+bool bwd_pairs(int d, int64_t cols) {
+  return (d > 512 || (d > 256 && d <= 384)) && cols >= 2048;
+}
 
 // Microseconds of bwd_kernel's product with `rows` rows over `cols` columns, by
 // tiles of 128 x 128: in pairs at 1.48 PFLOP/s, else at 2.1 and 0.65 us for the

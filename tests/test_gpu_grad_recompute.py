@@ -23,6 +23,8 @@ pytestmark = pytest.mark.gpu
     (640, 2000, 1, 4, 0.06),
     (128, 24000, 1, 4, 0.2),    # dW: more units than pairs
     (256, 16000, 1, 4, 0.3),    # dH split, its scratch in dW
+    (320, 2100, 2, 8, 0.3),     # pairs with one slice
+    (384, 4001, 1, 8, 0.4),     # a whole one
     (704, 2100, 2, 8, 0.3),     # pairs, an odd number of vocabulary blocks, dW split
     (960, 1024, 2, 8, 0.3),     # dW in pairs; three slices, the last of 192
     (768, 2048, 1, 8, 0.3),     # two whole slices
