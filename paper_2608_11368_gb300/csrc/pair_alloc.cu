@@ -24,11 +24,18 @@
 // no factorisation is needed: Chebyshev's iteration on the system scaled by
 // its diagonal, whose spectrum lies within rho = max_i v_i w_i / M_ii <= 1/2 of
 // 1, gains a factor of at least 3.7 per product with A. A reduction to a tenth is
-// enough: what the solve leaves is in the next step's residual, and the steps
-// are as many as with 1e-12 (10.3 against 9.8 on groups of 64; up to a third
-// more on sparse graphs, with a fifth of the products). So rho <= 1/10, every
-// dense group of 16 or more, needs no product at all: the step solves the
-// diagonal. Odd degrees only: their residual polynomial vanishes at 1, where the
+// enough as long as whole steps pass the test of the residuals: what the solve
+// leaves is in the next step's residual, and the steps are as many as with 1e-12
+// (10.3 against 9.8 on groups of 64). So rho <= 1/10, every dense group of 16 or
+// more, needs no product at all: the step solves the diagonal. Where rho is near
+// 1/2 (groups of 2, sparse graphs) a direction a tenth off can fail that test again
+// and again; its halved steps then stand still (45 of 100,000 groups of 2 and a few
+// of 100,000 sparse ones of 3 to 8 reached the cap of steps). So from a group's
+// second halving on its systems are solved to 1e-6: none of a million groups each
+// of 2, 3, 4, 5 and 8, dense and sparse, took more than 20 steps then. (A first
+// halving alone says little: switching there cost 4096 groups of 64, a tenth of
+// which have one, 2.93 instead of 2.45 ms.)
+// Odd degrees only: their residual polynomial vanishes at 1, where the
 // coordinates at a bound lie, so those are exact (even degrees stall there). The
 // stopping test is on the fp64 residuals themselves.
 //
@@ -63,7 +70,8 @@ constexpr double kGapRel = 1e-12;       // stop at gap <= kGapRel * Phi (and the
 // the primal residual allowed at the end (kPrimalRel) then never spend more.
 constexpr double kBudgetMargin = 4e-14;
 constexpr double kPrimalRel = 2e-14;
-constexpr float kLinRel = 0.1f;     // reduction of the Newton system's residual
+constexpr float kLinRel = 0.1f;     // reduction of the Newton system's residual,
+constexpr float kLinTight = 1e-6f;  // and from a group's second halving on
 constexpr int kLinMaxDegree = 61;   // reached only if rounding puts rho far above 1/2
 constexpr float kStepFrac = 0.995f; // of the largest step that keeps the interior
 constexpr double kStartMu = 0.1;    // the start's complementarity: kStartMu Phi in all
@@ -116,6 +124,7 @@ struct AllocGroup {
   int G, pitch, i, sub;
   bool act;
   int xb, rb;  // buffers of the next product and the next reduction
+  float lin;   // reduction of a system's residual
 
   // NS sums (fp64) and NM maxima (fp32: they only steer) over the group's
   // coordinates, to every thread. The replicas of a coordinate hold the same
@@ -228,7 +237,7 @@ struct AllocGroup {
 
   // Approximate solutions of M x_r = rhs_r (see the head of this file):
   // Chebyshev's iteration on M scaled by its diagonal (inverse rd), odd
-  // degree, until the residual is reduced by kLinRel.
+  // degree, until the residual is reduced by lin.
   template <int NR>
   __device__ void solve(double v, double rd, float rho, const double (&rhs)[NR],
                         double (&x)[NR]) {
@@ -244,7 +253,7 @@ struct AllocGroup {
     const float s = 1.f / rho;
     float r0 = rho, err = rho;
     const double vrd = v * rd;
-    for (int n = 1; !(err <= kLinRel && (n & 1)) && n < kLinMaxDegree; ++n) {
+    for (int n = 1; !(err <= lin && (n & 1)) && n < kLinMaxDegree; ++n) {
       double t[NR], y[NR];
 #pragma unroll
       for (int k = 0; k < NR; ++k) t[k] = v * d[k];
@@ -288,7 +297,7 @@ __global__ void __launch_bounds__(AllocShape<GP>::kThreads, AllocShape<GP>::kBlo
   const int i = threadIdx.x / kTpr, sub = threadIdx.x % kTpr, g = blockIdx.x;
   const bool act = i < G;
   AllocGroup<GP> grp{sm, reinterpret_cast<double *>(smem_raw + sizeof(AllocSmem<GP>)),
-                     G,  alloc_pitch(G), i, sub, act, 0, 0};
+                     G,  alloc_pitch(G), i, sub, act, 0, 0, kLinRel};
 
   // ---- inputs and their validity
   bool bad = false;
@@ -402,7 +411,7 @@ __global__ void __launch_bounds__(AllocShape<GP>::kThreads, AllocShape<GP>::kBlo
   else status = PAIR_ALLOC_OK;
 
   double pi = 1.0, gap = 0.0, phi = 0.0, spent = 0.0;
-  int steps = 0;
+  int steps = 0, halvings = 0;
   bool solved = false;
   if (status == PAIR_ALLOC_OK) {
     const double target = budget - fmin(kBudgetMargin * budget, 0.5 * (budget - pmin * sc));
@@ -509,6 +518,7 @@ __global__ void __launch_bounds__(AllocShape<GP>::kThreads, AllocShape<GP>::kBlo
           break;
         }
         step *= 0.5;
+        if (++halvings == 2) grp.lin = kLinTight;
       }
     }
     if (!solved) status = PAIR_ALLOC_FALLBACK;

@@ -12,7 +12,8 @@ import pytest
 
 from oracle import allocation as al
 from paper_2608_11368_gb300 import synth
-from tests.test_gpu_allocate import _run
+from tests.gpu_util import dev, dev_err_word
+from tests.test_gpu_allocate import _binding, _run
 
 pytestmark = pytest.mark.gpu
 
@@ -55,3 +56,58 @@ def test_allocate_sparse_proxy(G, scale):
     st, pi, stats = _run(inp, explicit_a=a)
     _check(inp, a.astype(np.float64), st, pi, stats)
     assert np.array_equal(pi, _run(inp, explicit_a=a)[1])
+
+
+def _groups(kind, B, G, cost_sd, rng):
+    """Predicted success probabilities, or an explicit sparse proxy (about two
+    edges a vertex, none without one), and costs."""
+    c = np.exp(cost_sd * rng.standard_normal((B, G))).astype(np.float32)
+    if kind == "predicted":
+        return dict(p_hat=rng.random((B, G)).astype(np.float32)), c
+    keep = np.triu(rng.random((B, G, G)) < 1.5 / G, 1)
+    i = np.arange(G - 1)
+    keep[:, i, i + 1] = True
+    a = np.where(keep, rng.uniform(0.1, 2.0, (B, G, G)), 0.0).astype(np.float32)
+    return dict(a=a + np.swapaxes(a, 1, 2)), c
+
+
+def _solved(proxy, c, budget, pi_min):
+    """Every group between its limits is solved, within its budget and to the
+    duality gap of the contract. Returns the stats."""
+    B = _binding()
+    err = dev_err_word()
+    pi, stats = B.pair_allocate(dev(c), dev(budget), pi_min, dev_err=err,
+                                **{k: dev(v) for k, v in proxy.items()})
+    pi, st = pi.cpu().numpy(), stats.cpu().numpy()
+    total = np.add.accumulate(c.astype(np.float64), axis=1)[:, -1]
+    b = budget.astype(np.float64)
+    inside = (b > np.float64(np.float32(pi_min)) * total) & (b < total)
+    assert inside.mean() > 0.5
+    assert np.count_nonzero(st[inside, 4] != al.ALLOC_OK) == 0
+    assert np.all(st[inside, 1] <= b[inside])
+    assert np.all(st[inside, 2] <= 1e-12 * st[inside, 0])
+    assert np.all(pi[inside] >= np.float32(pi_min)) and np.all(pi[inside] <= 1.0)
+    return st
+
+
+@pytest.mark.parametrize("G", [2, 3, 4, 8])
+@pytest.mark.parametrize("kind", ["predicted", "sparse"])
+@pytest.mark.parametrize("pi_min", [0.02, 0.08, 0.5])
+def test_allocate_solves_every_ordinary_group(G, kind, pi_min):
+    """100,000 groups: where the Newton system's off-diagonal row sums come near
+    half its diagonal, the inner solves have to be tight enough that the steps
+    go on (a tenth of the residual left 40 to 70 of 100,000 groups of 2 at the
+    uniform fallback)."""
+    B = 100000
+    rng = np.random.default_rng(1000 * G + int(100 * pi_min))
+    proxy, c = _groups(kind, B, G, 0.6, rng)
+    frac = rng.uniform(max(0.15, 1.05 * pi_min), 0.9, B)
+    _solved(proxy, c, (frac * c.sum(1, dtype=np.float64)).astype(np.float32), pi_min)
+
+
+def test_allocate_stalled_group_of_two():
+    """A group of 2 that such solves left at the fallback."""
+    p = np.array([[0.97856975, 0.0509815]], np.float32)
+    c = np.array([[0.79262024, 0.51749206]], np.float32)
+    st = _solved(dict(p_hat=p), c, np.array([1.0323904], np.float32), 0.08)
+    assert st[0, 0] < 1.4315 and st[0, 3] <= 20  # 1.497 at the uniform pi
