@@ -72,6 +72,11 @@ constexpr double kBudgetMargin = 4e-14;
 constexpr double kPrimalRel = 2e-14;
 constexpr float kLinRel = 0.1f;     // reduction of the Newton system's residual,
 constexpr float kLinTight = 1e-6f;  // and from a group's second halving on
+// Rounding of the dual residual: its terms y c pi sum to y budget, which exceeds
+// Phi by many powers of ten where costs do and the budget is near pi_min sum c.
+// The residual then stops there, above kGapRel Phi (5 to 17 of 20,000 such groups
+// reached the cap of steps; the log-barrier form, which has no such test, at most 3).
+constexpr double kDualRound = 8e-16;
 constexpr int kLinMaxDegree = 61;   // reached only if rounding puts rho far above 1/2
 constexpr float kStepFrac = 0.995f; // of the largest step that keeps the interior
 constexpr double kStartMu = 0.1;    // the start's complementarity: kStartMu Phi in all
@@ -455,7 +460,7 @@ __global__ void __launch_bounds__(AllocShape<GP>::kThreads, AllocShape<GP>::kBlo
     phi = s[0]; gap = s[1]; dres = s[2]; spent = s[3];
     while (true) {
       // All of these are the same in every thread: uniform exits.
-      if (gap <= kGapRel * phi && dres <= kGapRel * phi &&
+      if (gap <= kGapRel * phi && dres <= fmax(kGapRel * phi, kDualRound * y * budget) &&
           fabs(target - spent) <= kPrimalRel * budget) {
         solved = true;
         break;

@@ -111,3 +111,16 @@ def test_allocate_stalled_group_of_two():
     c = np.array([[0.79262024, 0.51749206]], np.float32)
     st = _solved(dict(p_hat=p), c, np.array([1.0323904], np.float32), 0.08)
     assert st[0, 0] < 1.4315 and st[0, 3] <= 20  # 1.497 at the uniform pi
+
+
+@pytest.mark.parametrize("G", [2, 4, 8, 16])
+@pytest.mark.parametrize("kind", ["predicted", "sparse"])
+def test_allocate_near_the_limits_with_costs_over_decades(G, kind):
+    """Budgets within 1e-6 to 1/2 of the range's ends, costs exp(3 N): the dual
+    residual's rounding is above 1e-12 of the objective in some of these."""
+    B, pi_min = 40000, 0.3
+    rng = np.random.default_rng(77 + G)
+    proxy, c = _groups(kind, B, G, 3.0, rng)
+    eps = np.exp(rng.uniform(np.log(1e-6), np.log(0.5), B))
+    frac = np.where(rng.random(B) < 0.5, pi_min + (1 - pi_min) * eps, 1 - (1 - pi_min) * eps)
+    _solved(proxy, c, (frac * c.sum(1, dtype=np.float64)).astype(np.float32), pi_min)
