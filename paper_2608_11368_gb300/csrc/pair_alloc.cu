@@ -39,6 +39,17 @@
 // coordinates at a bound lie, so those are exact (even degrees stall there). The
 // stopping test is on the fp64 residuals themselves.
 //
+// A vertex without an edge has no curvature but its complementarity's, z / s: once
+// that has shrunk below its dual residual its step points far outside the box and
+// the rest stands still. So after two halvings the corrector's second-order term,
+// which such a step makes as large as the step, is scaled by the predictor's step
+// lengths, and the centring keeps the gap from falling behind the residual
+// (kGapBehind). Without the two up to 2039 of 40,000 groups of 6 with such vertices
+// and costs over decades stopped at the cap. With them all of 9.2 million groups of 2
+// to 64 were solved (dense, sparse, uneven, with such vertices; costs up to exp(6 N);
+// half of them within 1e-6 to 1/2 of the budget's limits), two of them in more than 80
+// steps; the log-barrier form left 12 at its cap.
+//
 // What bounds it: the fp64 pipe (2 multiply-adds per clock and SM) for many
 // groups, the chain of a step's exchanges for few. Measured on one GB300,
 // against the factorising log-barrier form: 64 groups of 16 in 0.078 ms (2.43
@@ -62,7 +73,7 @@
 namespace pairk {
 namespace {
 
-constexpr int kAllocMaxSteps = 80;      // interior-point steps per group
+constexpr int kAllocMaxSteps = 200;     // interior-point steps per group (most take 6 to 17)
 constexpr int kAllocMaxBacktrack = 20;  // halvings of one step
 constexpr double kGapRel = 1e-12;       // stop at gap <= kGapRel * Phi (and the dual residual)
 // The budget the equality constraint aims at is this much (relative) below
@@ -78,6 +89,8 @@ constexpr float kLinTight = 1e-6f;  // and from a group's second halving on
 // reached the cap of steps; the log-barrier form, which has no such test, at most 3).
 constexpr double kDualRound = 8e-16;
 constexpr int kLinMaxDegree = 61;   // reached only if rounding puts rho far above 1/2
+constexpr double kGapBehind = 10.0; // times the gap: a dual residual above it is
+constexpr double kGapHold = 3e-3;   // answered by a complementarity of this part of it
 constexpr float kStepFrac = 0.995f; // of the largest step that keeps the interior
 constexpr double kStartMu = 0.1;    // the start's complementarity: kStartMu Phi in all
 
@@ -485,9 +498,14 @@ __global__ void __launch_bounds__(AllocShape<GP>::kThreads, AllocShape<GP>::kBlo
       // sum (z + az dz)(s + ap ds) / gap, with sum s dz = -gap - sum z ds.
       const float q3 =
           (float)((gap + az * (-gap - t[0]) + ap * (t[0] + az * t[1])) * rcp_approx(gap));
-      const double smu = (double)fminf(fmaxf(q3 * q3 * q3, 1e-6f), 1.f) * (gap * half_inv);
+      double smu = (double)fminf(fmaxf(q3 * q3 * q3, 1e-6f), 1.f) * (gap * half_inv);
+      double d2 = d;
+      if (halvings >= 2) {
+        d2 *= ap * az;
+        if (dres > kGapBehind * gap) smu = fmax(smu, kGapHold * dres * half_inv);
+      }
       // Corrector.
-      const double tl = (smu - d * dzl) * rsl, th = (smu + d * dzh) * rsh;
+      const double tl = (smu - d2 * dzl) * rsl, th = (smu + d2 * dzh) * rsh;
       double rhs1[1] = {act ? fma(tl - th, pi, rhs[0]) : 0.0}, h1[1];
       grp.template solve<1>(v, rd, rho, rhs1, h1);
       double q1[1] = {cp * h1[0]};

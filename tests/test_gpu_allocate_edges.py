@@ -60,13 +60,16 @@ def test_allocate_sparse_proxy(G, scale):
 
 def _groups(kind, B, G, cost_sd, rng):
     """Predicted success probabilities, or an explicit sparse proxy (about two
-    edges a vertex, none without one), and costs."""
+    edges a vertex, none without one; "isolated": some without), and costs."""
     c = np.exp(cost_sd * rng.standard_normal((B, G))).astype(np.float32)
     if kind == "predicted":
         return dict(p_hat=rng.random((B, G)).astype(np.float32)), c
     keep = np.triu(rng.random((B, G, G)) < 1.5 / G, 1)
     i = np.arange(G - 1)
-    keep[:, i, i + 1] = True
+    if kind == "sparse":
+        keep[:, i, i + 1] = True
+    else:  # but for one edge, so that the objective is not flat
+        keep[:, 0, 1] = True
     a = np.where(keep, rng.uniform(0.1, 2.0, (B, G, G)), 0.0).astype(np.float32)
     return dict(a=a + np.swapaxes(a, 1, 2)), c
 
@@ -121,6 +124,19 @@ def test_allocate_near_the_limits_with_costs_over_decades(G, kind):
     B, pi_min = 40000, 0.3
     rng = np.random.default_rng(77 + G)
     proxy, c = _groups(kind, B, G, 3.0, rng)
+    eps = np.exp(rng.uniform(np.log(1e-6), np.log(0.5), B))
+    frac = np.where(rng.random(B) < 0.5, pi_min + (1 - pi_min) * eps, 1 - (1 - pi_min) * eps)
+    _solved(proxy, c, (frac * c.sum(1, dtype=np.float64)).astype(np.float32), pi_min)
+
+
+@pytest.mark.parametrize("G", [3, 6, 12])
+@pytest.mark.parametrize("cost_sd", [0.6, 3.0, 6.0])
+def test_allocate_vertices_without_an_edge(G, cost_sd):
+    """Vertices whose only curvature is the bounds' (any budget they take is as
+    good as any other), budgets and costs as in the test above."""
+    B, pi_min = 40000, 0.01
+    rng = np.random.default_rng(99 + G)
+    proxy, c = _groups("isolated", B, G, cost_sd, rng)
     eps = np.exp(rng.uniform(np.log(1e-6), np.log(0.5), B))
     frac = np.where(rng.random(B) < 0.5, pi_min + (1 - pi_min) * eps, 1 - (1 - pi_min) * eps)
     _solved(proxy, c, (frac * c.sum(1, dtype=np.float64)).astype(np.float32), pi_min)
