@@ -251,7 +251,8 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
   // 2^-24 of the power of two above G max |t|, and its reciprocal.
   double q = 0.0, q_inv = 0.0;
   if constexpr (SPLIT) {
-    // max |t| from fp32 quotients, which round up to 3 ulp off.
+    // max |t| from fp32 quotients, which round up to 3 ulp off (of the weights as
+    // they are used: one rho far below 1 / w_max would else leave all terms to lo).
     float m = 0.f;
     for (int j = warp; j < G; j += kWarps)
       for (int i = j + 1 + lane; i < G; i += 32) {
@@ -260,7 +261,10 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
           if (pis[i] > 0.f && pis[j] > 0.f) t = __fdividef(t, pis[j] * pis[i]);
         } else if (wmode != PAIR_W_UNWEIGHTED) {
           const float rij = rho[(size_t)j * G + i];
-          if (rij > 0.f) t *= __frcp_rn(rij);
+          if (rij > 0.f) {
+            const float w = __frcp_rn(rij);
+            t *= wmode == PAIR_W_CLIPPED ? fminf(w, w_max) : w;
+          }
         }
         m = fmaxf(m, t);
       }

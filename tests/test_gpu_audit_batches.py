@@ -66,3 +66,22 @@ def test_audit_invalid_weight_needs_a_completed_edge(G):
         err = dev_err_word()
         B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd), dev_err=err)
         assert B.pair_status_sync(err) == want
+
+
+@pytest.mark.parametrize("G,tiny", [(8, 1e-9), (16, 1e-9), (16, 1e-39), (60, 1e-9)])
+def test_audit_clipped_with_one_tiny_rho(G, tiny):
+    """Clipped terms keep their split when one 1 / rho is far above w_max: the bias to
+    1e-8 of itself. (With scale a power of two split terms leave some 2^-48 G of the
+    largest one, fp32 sums of whole terms left 2e-8 to 7e-8 of this bias from G = 16 on.)"""
+    B = _binding()
+    N, w_max = 40000, 200.0
+    r, S, p, rho, Jd = _population(990 + G, G, 16, N)
+    r[2], r[3] = 1.0, 0.0
+    rho[2, 3] = rho[3, 2] = tiny
+    Jd[:, 2] = Jd[:, 3] = 0  # never completed: only the split sees it
+    scale = 1.0 / 2 ** int(math.log2(math.comb(G, 2)))  # exact in fp32
+    _, bias = B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd), wmode=oracle.W_CLIPPED, w_max=w_max,
+                           scale=scale)
+    ref = oracle.audit(r, rho, S, Jd, scale=scale, wmode=oracle.W_CLIPPED, w_max=w_max)
+    err = np.linalg.norm(bias.cpu().numpy() - ref["bias"]) / np.linalg.norm(ref["bias"])
+    assert err <= 1e-8, err
