@@ -182,9 +182,11 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
 // Draws in batches of 32, one per lane; batch q of the teams' stride. Row i of
 // a batch belongs to warp i mod TW of its team. Per draw: the row sums 2 a_i =
 // sum_j J_i J_j t_ij and the weight sums, then in fp64 the weighting's and flags'
-// division and centring, e = a - abar, e^T K e over the lower triangle, e^T u. With a = e + abar,
-// u = K abar and gg = abar^T u: a^T u = e^T u + gg and
-// a^T K a = e^T K e + 2 e^T u + gg (0 exactly where a = 0).
+// division and centring, e = a - abar, e^T K e over the lower triangle, a^T u. With a = e + abar,
+// u = K abar and gg = abar^T u: a^T K a = e^T K e + 2 a^T u - gg (0 exactly where a = 0),
+// formed from a itself where that leaves less than gg / 1024, as for weights or
+// standardised rewards that make a small beside abar (a second pass over K, in
+// batches that hold such a draw).
 //
 // SPLIT: a term is kept as t = hi + lo, hi a multiple of q = 2^-24 times the power
 // of two above G max |t|, so that fp32 sums of hi are exact in any order, and lo <=
@@ -450,10 +452,10 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
       mean_a = Kc > 0 ? s_a / (double)Kc : 0.0;
     }
 
-    // ---- fp64: e = a - abar, the sums of a, e^T u
+    // ---- fp64: e = a - abar, the sums of a, a^T u (before its factor)
     const int b = bt * 32 + lane;
     const double w = b < N ? (wd ? wd[b] : w_all) : 0.0, wf = w * f;
-    double eu = 0.0;
+    double au = 0.0;
     bool any = false;  // (of a before its factor; f = 0 is checked below)
     for (int i = tw; i < G; i += TW) {
       double a = e[i * 32 + lane];
@@ -462,31 +464,41 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
       const double ei = fma(a, f, -abar[i]);
       e[i * 32 + lane] = ei;
       asum[i * 32 + lane] = fma(wf, a, asum[i * 32 + lane]);
-      eu = fma(ei, u[i], eu);
+      au = fma(a, u[i], au);
     }
     team_sync<TW>();
 
-    // ---- e^T K e over the lower triangle
-    double q = 0.0;
-    for (int i = tw; i < G; i += TW) {
-      const double *row = K + i * (i + 1) / 2;
-      double s0 = 0.0, s1 = 0.0;
-      int j = 0;
-      for (; j + 4 <= i; j += 4) {
-        s0 = fma(row[j], e[j * 32 + lane], s0);
-        s1 = fma(row[j + 1], e[(j + 1) * 32 + lane], s1);
-        s0 = fma(row[j + 2], e[(j + 2) * 32 + lane], s0);
-        s1 = fma(row[j + 3], e[(j + 3) * 32 + lane], s1);
+    // ---- x^T K x over the lower triangle
+    auto form = [&](auto x) {
+      double q = 0.0;
+      for (int i = tw; i < G; i += TW) {
+        const double *row = K + i * (i + 1) / 2;
+        double s0 = 0.0, s1 = 0.0;
+        int j = 0;
+        for (; j + 4 <= i; j += 4) {
+          s0 = fma(row[j], x(j), s0);
+          s1 = fma(row[j + 1], x(j + 1), s1);
+          s0 = fma(row[j + 2], x(j + 2), s0);
+          s1 = fma(row[j + 3], x(j + 3), s1);
+        }
+        for (; j < i; ++j) s0 = fma(row[j], x(j), s0);
+        const double xi = x(i);
+        q = fma(xi, fma(2.0, s0 + s1, row[i] * xi), q);
       }
-      for (; j < i; ++j) s0 = fma(row[j], e[j * 32 + lane], s0);
-      const double ei = e[i * 32 + lane];
-      q = fma(ei, fma(2.0, s0 + s1, row[i] * ei), q);
-    }
-    q = team_sum<TW>(xch, 2, q);
-    eu = team_sum<TW>(xch, 3, eu);
+      return team_sum<TW>(xch, 2, q);
+    };
+    const double q = form([&](int j) { return e[j * 32 + lane]; });
+    au = team_sum<TW>(xch, 3, au) * f;
     if constexpr (TW > 1) any = team_sum<TW>(xch, 0, any ? 1.f : 0.f) > 0.f;
+    any = any && f != 0.0;
+    double q_aa = any ? fma(2.0, au, q) - gg : 0.0;
+    // (The same answer in every warp of the team.)
+    if (__any_sync(0xffffffffu, any && q_aa < gg * 0x1p-10)) {
+      const double a2 = form([&](int j) { return e[j * 32 + lane] + abar[j]; });
+      if (any && q_aa < gg * 0x1p-10) q_aa = a2;
+    }
     if (tw == 0) {
-      const double q_au = eu + gg, q_aa = any && f != 0.0 ? q + 2.0 * eu + gg : 0.0;
+      const double q_au = any ? au : 0.0;
       const double cosb = (q_aa > 0.0 && gg > 0.0) ? q_au * rsqrt(q_aa * gg) : 0.0;
       const double ess = W2 > 0.f ? (double)W * (double)W / (double)W2 : 0.0;
       acc[0] = fma(w, q, acc[0]);

@@ -85,3 +85,21 @@ def test_audit_clipped_with_one_tiny_rho(G, tiny):
     ref = oracle.audit(r, rho, S, Jd, scale=scale, wmode=oracle.W_CLIPPED, w_max=w_max)
     err = np.linalg.norm(bias.cpu().numpy() - ref["bias"]) / np.linalg.norm(ref["bias"])
     assert err <= 1e-8, err
+
+
+@pytest.mark.parametrize("G,N", [(6, 40), (32, 100), (50, 64), (125, 40)])
+@pytest.mark.parametrize("size", [1e-3, 1e-5, 1e-7])
+def test_audit_cosine_of_small_estimates(G, N, size):
+    """Coefficients far below the target's (weights clipped at `size`; every edge
+    clipped): the cosine does not depend on their size, and ||ghat||^2 is not
+    left to the difference of terms of the target's size. The coefficients' own
+    rounding beside the target leaves 2^-53 / size of a."""
+    B = _binding()
+    r, S, p, rho, Jd = _population(1000 + G, G, 9, N)
+    scale = 1.0 / math.comb(G, 2)
+    st = [B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd), wmode=oracle.W_CLIPPED, w_max=w,
+                       scale=scale)[0].cpu().numpy() for w in (1.0, size)]
+    ref = oracle.audit(r, rho, S, Jd, scale=scale, wmode=oracle.W_CLIPPED, w_max=np.float32(size))
+    assert abs(st[1][2] - ref["cos"]) <= 1e-6 * abs(ref["cos"])
+    assert abs(st[1][2] - st[0][2]) <= 1e-6 * abs(ref["cos"])
+    assert abs(st[1][1] - ref["mse"]) <= 1e-6 * ref["mse"]
