@@ -223,9 +223,10 @@ PAIR_API pair_status pair_coeffs_product(int32_t B, int32_t G, const float *r,
  *                           completed edges, [PAIR_AUDIT_ESS] mean ESS
  *   [PAIR_AUDIT_TARGET_SQ]  || g ||^2,  [PAIR_AUDIT_WEIGHT] W
  * and bias [D] (double, nullable) the vector sum_b w_b ghat_b / W - g.
- * Everything is formed through the Gram matrix S S^T in fp64 (a draw's
- * coefficients are not rounded to fp32, except their row sums for G > 120, and
- * the ESS weights); deterministic. ws: device workspace of
+ * Everything is formed through the Gram matrix S S^T in fp64, a draw's
+ * coefficients too, with these exceptions in fp32: their row sums for G > 120,
+ * and the edge weights and their sums (the ESS and the self-normalised
+ * weighting's divisor). Deterministic. ws: device workspace of
  * pair_audit_workspace_size(N, G, D) bytes, 16-byte aligned, no initial
  * contents needed.
  * Errors: as pair_coeffs_weighted; PAIR_ERR_WORKSPACE.

@@ -436,15 +436,15 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
     double f = 0.5 * (double)scale;
     if (wmode == PAIR_W_HAJEK) f = W > 0.f ? f / (double)W : 0.0;
     if ((flags & PAIR_STANDARDIZE) && Kc >= 2) {
-      float sr = 0.f, ss = 0.f;
-      for (int i = 0; i < G; ++i) sr += done(i) ? rs[i] : 0.f;
-      const float mean = sr / (float)Kc;
+      double sr = 0.0, ss = 0.0;
+      for (int i = 0; i < G; ++i) sr += done(i) ? (double)rs[i] : 0.0;
+      const double mean = sr / (double)Kc;
       for (int i = 0; i < G; ++i) {
-        const float dv = done(i) ? rs[i] - mean : 0.f;
-        ss = fmaf(dv, dv, ss);
+        const double dv = done(i) ? (double)rs[i] - mean : 0.0;
+        ss = fma(dv, dv, ss);
       }
-      const float sd = sqrtf(ss / (float)(Kc - 1));
-      f = sd > 0.f ? f / (double)sd : 0.0;
+      const double sd = sqrt(ss / (double)(Kc - 1));
+      f = sd > 0.0 ? f / sd : 0.0;
     }
     double mean_a = 0.0;
     if (flags & PAIR_CENTER) {

@@ -103,3 +103,19 @@ def test_audit_cosine_of_small_estimates(G, N, size):
     assert abs(st[1][2] - ref["cos"]) <= 1e-6 * abs(ref["cos"])
     assert abs(st[1][2] - st[0][2]) <= 1e-6 * abs(ref["cos"])
     assert abs(st[1][1] - ref["mse"]) <= 1e-6 * ref["mse"]
+
+
+@pytest.mark.parametrize("G", [7, 32, 100])
+def test_audit_standardize_by_the_exact_deviation(G):
+    """Rewards around 1000: the coefficients are the plain ones over the fp64 sample
+    standard deviation (two-pass fp32 sums left 1e-8 to 2e-7 of it)."""
+    B = _binding()
+    r, S, p, rho, Jd = _population(960 + G, G, 20, 1)
+    r = (1000.0 + np.random.default_rng(G).standard_normal(G)).astype(np.float32)
+    Jd[:] = 1
+    Jd[0, G // 2] = 0
+    sd = r[Jd[0] != 0].astype(np.float64).std(ddof=1)
+    g = 0.5 * (G * r.astype(np.float64) - r.astype(np.float64).sum()) @ S.astype(np.float64)
+    h = [B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd), flags=f)[1].cpu().numpy() + g
+         for f in (0, 2)]
+    assert np.linalg.norm(h[1] - h[0] / sd) <= 1e-11 * np.linalg.norm(g)
