@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
   const double gg = *gg_p, w_all = 1.0 / (double)N;
 
   double acc[6] = {0, 0, 0, 0, 0, 0};  // mse, cos, vertices, edges, ess, weight (warp 0 of a team)
-  const int nbatch = (N + 31) / 32;
+  const int nbatch = (int)ceil_div(N, 32);  // (N + 31 may exceed an int)
   for (int bt = blockIdx.x * kTeams + team; bt < nbatch; bt += gridDim.x * kTeams) {
     // ---- completion bits of the batch: a lane reads its own draw's flags
     // where one warp has the batch (all loads in flight; ballots, 32 candidates

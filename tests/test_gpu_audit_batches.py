@@ -7,6 +7,7 @@ import math
 
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from tests.gpu_util import dev, dev_err_word
@@ -119,3 +120,16 @@ def test_audit_standardize_by_the_exact_deviation(G):
     h = [B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd), flags=f)[1].cpu().numpy() + g
          for f in (0, 2)]
     assert np.linalg.norm(h[1] - h[0] / sd) <= 1e-11 * np.linalg.norm(g)
+
+
+def test_audit_largest_draw_count():
+    """N = 2^31 - 1 draws (4.3 GB of flags): the batch count is formed beyond 32 bits."""
+    B = _binding()
+    N = 2 ** 31 - 1
+    r, S, p, rho, _ = _population(991, 2, 3, 1)
+    Jd = torch.ones(N, 2, dtype=torch.uint8, device="cuda")
+    Jd[N - 1] = 0
+    stats, _ = B.pair_audit(dev(r), dev(rho), dev(S), Jd)
+    st = stats.cpu().numpy()
+    assert abs(st[7] - 1.0) <= 1e-6 and abs(st[3] - 2.0 * (N - 1) / N) <= 1e-6
+    assert abs(st[4] - (N - 1) / N) <= 1e-6 and st[1] > 0
