@@ -587,13 +587,22 @@ __global__ void __launch_bounds__(256)
 }
 
 template <int TW, bool SPLIT>
-pair_status launch_draws(int nblk, size_t smem, int N, int G, const float *r, const float *rho,
+pair_status launch_draws(int &nblk, int nsm, size_t smem, int N, int G, const float *r, const float *rho,
                          const uint8_t *Jd, const double *wd, float scale, uint32_t flags,
                          int wmode, float w_max, const double *K, const double *abar,
                          const double *u, const double *gg, double *part, int32_t *dev_err,
                          cudaStream_t s) {
   PAIR_CUDA_TRY(cudaFuncSetAttribute(audit_draws_kernel<TW, SPLIT>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // One batch of 32 draws per team as far as the chip holds the blocks at once (and
+  // the partial slots); a stride over the batches beyond that.
+  int per_sm = 0;
+  PAIR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &per_sm, audit_draws_kernel<TW, SPLIT>, audit_warps(TW) * 32, smem));
+  const int64_t want = ceil_div(ceil_div(N, 32), audit_warps(TW) / TW);
+  const int64_t most = (int64_t)nsm * (per_sm > 0 ? per_sm : 1);
+  nblk = (int)(want < most ? want : most);
+  if (nblk > kAuditBlocks) nblk = kAuditBlocks;
   PAIR_BEGIN("audit_draws", s);
   audit_draws_kernel<TW, SPLIT><<<nblk, audit_warps(TW) * 32, smem, s>>>(
       N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar, u, gg, part, dev_err);
@@ -617,27 +626,24 @@ pair_status launch_audit(int N, int G, int D, const float *r, const float *rho, 
   PAIR_BEGIN("audit_target", s);
   audit_target_kernel<<<1, 128, 0, s>>>(G, r, scale, K, abar, u, gg);
   PAIR_LAUNCH_CHECK(s);
-  // One batch of 32 draws per team where the batches fit the partial slots
-  // and a few rounds of the chip; a stride over the batches beyond that.
-  const int teams = audit_warps(audit_team(G)) / audit_team(G);
+  int dev = 0, nsm = 0, nblk = 0;
+  PAIR_CUDA_TRY(cudaGetDevice(&dev));
+  PAIR_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const size_t smem = audit_draws_smem(G);
-  int nblk = (int)ceil_div(ceil_div(N, 32), teams);
-  const int most = 152 * (int)(227 * 1024 / (smem + 1024) < 8 ? 227 * 1024 / (smem + 1024) : 8);
-  if (nblk > most) nblk = most;
   pair_status st;
   if (audit_team(G) == 1)
-    st = launch_draws<1, true>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar,
+    st = launch_draws<1, true>(nblk, nsm, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar,
                                u, gg, part, dev_err, s);
   else if (audit_split(G))
-    st = launch_draws<8, true>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar,
+    st = launch_draws<8, true>(nblk, nsm, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K, abar,
                                u, gg, part, dev_err, s);
   else
-    st = launch_draws<8, false>(nblk, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K,
+    st = launch_draws<8, false>(nblk, nsm, smem, N, G, r, rho, Jd, wd, scale, flags, wmode, w_max, K,
                                 abar, u, gg, part, dev_err, s);
   if (st != PAIR_OK) return st;
   PAIR_BEGIN("audit_finish", s);
   const int fin = bias ? (int)ceil_div(D, 256) : 1;
-  audit_finish_kernel<<<fin < 152 ? fin : 152, 256, 0, s>>>(nblk, G, D, S, K, abar, gg, part,
+  audit_finish_kernel<<<fin < nsm ? fin : nsm, 256, 0, s>>>(nblk, G, D, S, K, abar, gg, part,
                                                             stats, bias);
   PAIR_LAUNCH_CHECK(s);
   return PAIR_OK;
