@@ -78,3 +78,22 @@ def test_subnormal_and_invalid_rho():
             ref = oracle.coeffs(r, J, rho)
             assert (np.abs(a - ref["a"]) <= 1e-6 * ref["a_mag"]).all()
             assert (np.abs(b - ref["a"]) <= 1e-6 * ref["a_mag"]).all()
+
+
+@pytest.mark.parametrize("dr,p01", [(1e5, 1e-36), (3e38, 0.25), (np.inf, 0.5), (1e-38, 0.3),
+                                    (1e30, 1e-12), (7e-20, 1e25)])
+def test_quotients_beyond_the_range(dr, p01):
+    """Terms that overflow are infinite, not NaN, and tiny ones are rounded like
+    the IEEE quotient: one contrast edge, whose coefficients are +-1/2 of it."""
+    B = _binding()
+    G = 3
+    r = np.array([[dr, 0.0, 0.0]], np.float32)
+    rho = np.full((1, G, G), p01, np.float32)
+    J = np.array([[1, 1, 0]], np.uint8)
+    with np.errstate(over="ignore"):
+        want = np.float32(0.5) * (np.float32(dr) / np.float32(p01))
+    err = dev_err_word()
+    a = B.pair_coeffs_weighted(dev(r), dev(J), dev(rho), wmode=B.PAIR_W_CLIPPED, w_max=3e38,
+                               dev_err=err)[0].cpu().numpy()
+    assert B.pair_status_sync(err) == 0
+    assert a.tolist() == [[float(want), -float(want), 0.0]]
