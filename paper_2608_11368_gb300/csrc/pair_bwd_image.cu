@@ -757,7 +757,7 @@ pair_status launch_chunk_bwd(const GradArgs &g, const GradWorkspace &w, cudaStre
 //       rows of dW behind the slab (or in the ring); a slab is as large as that
 //       allows. Where even two vocabulary blocks of all tokens fit neither, the
 //       slab's tokens run in chunks that fit the ring, each adding its part.
-// If the ring holds all tiles, they are formed once for both.
+// If the ring holds all tiles, and dH runs in one chunk, they are formed once for both.
 //
 // Each chunk and each slab costs its launches, short K loops and drains, about
 // kSlabUs (dH: kSlabDhUs beside the GEMM's makespan), so each product takes the
@@ -966,7 +966,8 @@ pair_status grad_bwd_slabs(const GradArgs &g, const GradWorkspace &w, cudaStream
                    p.scratch_cap > 0 ? p.scratch_cap : p.in_dw ? ring_cap : 0);
     if (st != PAIR_OK) return st;
   }
-  if (dw && dh && p.one) return slab_dw(g, w, s, 0, p.n_vt, 0, p.n_rb, false, w.gring, nullptr, 0);
+  // (In several dH chunks the ring would hold the last one's tiles only.)
+  if (dw && dh && p.one && p.chunk >= p.n_rb) return slab_dw(g, w, s, 0, p.n_vt, 0, p.n_rb, false, w.gring, nullptr, 0);
 
   for (int vb0 = 0; dw && vb0 < p.n_vt;) {
     const Slab o = slab_at(g, p, vb0);
