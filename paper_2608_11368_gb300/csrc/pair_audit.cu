@@ -12,7 +12,8 @@
 //   <ghat_b, g> = a_b^T K abar,  ||ghat_b||^2 = a_b^T K a_b,
 //   E[ghat] - g = (E[a] - abar) S.
 // K, abar, the coefficients' division, centring and scale and the quadratic forms
-// are fp64, on row sums of the terms' fp64 quotients (see audit_draws_kernel).
+// are fp64, on row sums of the terms' fp64 quotients (see audit_draws_kernel); the
+// edge weights and their sums are fp32.
 //
 // A draw's terms (r_i - r_j) w_ij are the same for every draw, so they and the
 // weights are formed once per block and a draw only adds the ones of its
@@ -20,7 +21,7 @@
 // between lanes, uniform (broadcast) reads of the terms and of K, and every
 // lane of the fp64 pipe busy, which is what bounds the pass: about G^2 / 2 + 5 G
 // fp64 operations per draw at 2 per clock and SM. Measured on one GB300, 50,000
-// draws of 16 candidates with D = 4096: the call takes 100 us, its draws pass 73
+// draws of 16 candidates with D = 4096: the call takes 104 us, its draws pass 76
 // us; one block per draw, with a tree and five block reductions each, took 653 and
 // 500 us. For G = 64 and 128 (3125 and 781 draws) the call takes 0.18 and 0.48
 // ms, from 0.75 and 1.37 ms.
@@ -186,14 +187,15 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
 // u = K abar and gg = abar^T u: a^T K a = e^T K e + 2 a^T u - gg (0 exactly where a = 0),
 // formed from a itself where that leaves less than gg / 1024, as for weights or
 // standardised rewards that make a small beside abar (a second pass over K, in
-// batches that hold such a draw).
+// batches that hold such a draw). Self-normalised coefficients are all that small,
+// about 1 / C(G, 2) of abar: there a^T K a comes first and e^T K e from it, the same way.
 //
 // SPLIT: a term is kept as t = hi + lo, hi a multiple of q = 2^-24 times the power
 // of two above G max |t|, so that fp32 sums of hi are exact in any order, and lo <=
 // q / 2 the rest of the fp64 quotient: the pair is summed by one packed addition,
 // and a is good to some 2^-40 of the largest term where fp32 terms and trees left
 // 1e-6 of the bias, a small remainder of such sums (2.4e-6 -> 5e-8 relative, the
-// rounding of scale; the draws of the size above 57 -> 73 us). Otherwise (G > 120) fp32 terms in 16-term trees, combined
+// rounding of scale; the draws of the size above 57 -> 73 us then). Otherwise (G > 120) fp32 terms in 16-term trees, combined
 // pairwise.
 template <int TW, bool SPLIT>
 __global__ void __launch_bounds__(audit_warps(TW) * 32)
@@ -218,11 +220,12 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
   double *e = e_all + team * 32 * G, *asum = asum_all + team * 32 * G;
   uint32_t *bits = bits_all + team * 4 * 32;
 
-  // ---- the group's constants
+  // ---- the group's constants (abar: what e subtracts)
+  const bool small = wmode == PAIR_W_HAJEK;
   __shared__ unsigned t_max;  // bits of the largest |t|
   if (threadIdx.x == 0) t_max = 0u;
   for (int i = threadIdx.x; i < G; i += blockDim.x) {
-    abar[i] = abar_g[i];
+    abar[i] = small ? 0.0 : abar_g[i];
     u[i] = u_g[i];
     rs[i] = r[i];
     pis[i] = wmode == PAIR_W_MARGINAL ? rho[(size_t)i * G + i] : 1.f;
@@ -452,7 +455,7 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
       mean_a = Kc > 0 ? s_a / (double)Kc : 0.0;
     }
 
-    // ---- fp64: e = a - abar, the sums of a, a^T u (before its factor)
+    // ---- fp64: e = a - abar (small: a itself), the sums of a, a^T u (before its factor)
     const int b = bt * 32 + lane;
     const double w = b < N ? (wd ? wd[b] : w_all) : 0.0, wf = w * f;
     double au = 0.0;
@@ -461,8 +464,7 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
       double a = e[i * 32 + lane];
       if ((flags & PAIR_CENTER) && done(i)) a -= mean_a;
       any |= a != 0.0;
-      const double ei = fma(a, f, -abar[i]);
-      e[i * 32 + lane] = ei;
+      e[i * 32 + lane] = fma(a, f, -abar[i]);
       asum[i * 32 + lane] = fma(wf, a, asum[i * 32 + lane]);
       au = fma(a, u[i], au);
     }
@@ -487,16 +489,19 @@ __global__ void __launch_bounds__(audit_warps(TW) * 32)
       }
       return team_sum<TW>(xch, 2, q);
     };
-    const double q = form([&](int j) { return e[j * 32 + lane]; });
+    const double p = form([&](int j) { return e[j * 32 + lane]; });
     au = team_sum<TW>(xch, 3, au) * f;
     if constexpr (TW > 1) any = team_sum<TW>(xch, 0, any ? 1.f : 0.f) > 0.f;
     any = any && f != 0.0;
-    double q_aa = any ? fma(2.0, au, q) - gg : 0.0;
-    // (The same answer in every warp of the team.)
-    if (__any_sync(0xffffffffu, any && q_aa < gg * 0x1p-10)) {
-      const double a2 = form([&](int j) { return e[j * 32 + lane] + abar[j]; });
-      if (any && q_aa < gg * 0x1p-10) q_aa = a2;
+    // The other of the two forms (the conditions are the same in every warp of the team).
+    const double sign = small ? -1.0 : 1.0;
+    double other = fma(sign, fma(2.0, au, -gg), p);
+    const bool redo = (any || small) && other < gg * 0x1p-10;
+    if (__any_sync(0xffffffffu, redo)) {
+      const double x = form([&](int j) { return fma(sign, abar_g[j], e[j * 32 + lane]); });
+      if (redo) other = x;
     }
+    const double q = small ? other : p, q_aa = !any ? 0.0 : small ? p : other;
     if (tw == 0) {
       const double q_au = any ? au : 0.0;
       const double cosb = (q_aa > 0.0 && gg > 0.0) ? q_au * rsqrt(q_aa * gg) : 0.0;

@@ -34,6 +34,29 @@ def test_audit_batches(G, N, wmode, center):
     _check(stats, bias, ref, rtol=2e-5)
 
 
+@pytest.mark.parametrize("G,N,scale", [(2, 40, 1.0), (3, 64, 1.0), (16, 100, 120.0), (50, 70, 1.0)])
+def test_audit_self_normalised_forms(G, N, scale):
+    """Self-normalised estimates are about 1 / C(G, 2) of the target, and equal to it
+    for complete draws of two (one edge, rho = 1): neither ||ghat||^2 nor the error
+    is left to a difference that cancels. 1e-6: the fp32 sum of the weights."""
+    B = _binding()
+    r, S, p, rho, Jd = _population(1100 + G, G, 9, N)
+    if G < 4:
+        rho[:] = 1.0
+        Jd[: N // 2] = 1
+    err = dev_err_word()
+    stats = B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd), wmode=oracle.W_HAJEK, scale=scale,
+                         dev_err=err)[0].cpu().numpy()
+    assert B.pair_status_sync(err) == 0
+    ref = oracle.audit(r, rho, S, Jd, scale=scale, wmode=oracle.W_HAJEK)
+    assert abs(stats[2] - ref["cos"]) <= 1e-6
+    assert abs(stats[1] - ref["mse"]) <= 1e-6 * ref["mse"]
+    if G == 2:  # complete draws alone: the estimate is the target
+        one = B.pair_audit(dev(r), dev(rho), dev(S), dev(Jd[:1]), wmode=oracle.W_HAJEK,
+                           scale=scale)[0].cpu().numpy()
+        assert one[1] <= 1e-24 * one[6] and abs(one[2] - 1.0) <= 1e-12
+
+
 @pytest.mark.parametrize("G", [12, 40])
 def test_audit_standardize_is_a_scale_per_draw(G):
     """One draw: standardised coefficients are the plain ones over the sample
