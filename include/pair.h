@@ -369,8 +369,9 @@ PAIR_API size_t pair_grad_workspace_min_size(int64_t T, int32_t d, int32_t V, in
  * for the dH and dW GEMMs (see pair_grad_workspace_size); with the minimum
  * workspace nothing logit-sized is written (for bf16 d that are no multiple of
  * 512 or above 3072, bf16 gradient tiles may pass through dW or the workspace).
- * dW serves as scratch before its rows are written: it must not overlap any
- * input or other output.
+ * dW serves as scratch before its rows are written, once H, y, mask, cu_seqlens
+ * (and logp_old) have been read: like its rows it must not overlap W, a, ws or
+ * another output.
  *
  * In:  T >= 1 packed tokens; d hidden size; V vocabulary size; dt dtype of
  *      H and W (PAIR_BF16: fp32 accumulation on the tensor cores, requires
